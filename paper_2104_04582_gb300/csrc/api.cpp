@@ -206,6 +206,10 @@ struct SlotPlan {
     std::vector<int> slot_ptr;
     std::vector<int2> contrib;
     std::vector<int2> rows;
+    std::vector<int4> row_slot;  // (first slot, highest n, lowest n, 0) of each row
+    // tensor-core summation: row pairs, K steps, centre of the n range and signed m of the last
+    // pair's second row; pairs 0 where the mode set exceeds its accumulators or basis
+    int tc_pairs = 0, tc_ks = 0, n_mid = 0, m_fin = 0;
 };
 
 few_status plan_slots(const int *l, const int *m, const int *n, int N, SlotPlan &P)
@@ -262,7 +266,17 @@ few_status plan_slots(const int *l, const int *m, const int *n, int N, SlotPlan 
             for (int q = hi[j]; q >= lo[j]; --q) slot_of[std::make_pair(ms, q)] = slot++;
         }
         P.rows.push_back(make_int2(L, j == 0 ? 0 : prev_lo - cur_lo));
+        P.row_slot.push_back(make_int4(slot - L, L ? hi[j] : -1, L ? lo[j] : 0, 0));
         prev_lo = cur_lo;
+    }
+    const int n_lo = *std::min_element(lo.begin(), lo.end());
+    const int n_hi = *std::max_element(hi.begin(), hi.end());
+    P.n_mid = n_lo + (n_hi - n_lo) / 2;
+    const int half = n_hi - P.n_mid;
+    if (n_rows <= kTcMaxRows && half <= kTcMaxHalf) {
+        P.tc_pairs = (n_rows + 1) / 2;
+        P.tc_ks = half / 8 + 1;
+        P.m_fin = mmax - (2 * P.tc_pairs - 1);
     }
     P.n_slots = slot;
     P.m_last = m_last;
@@ -318,17 +332,27 @@ struct few_traj {
     const double *src_phi_phi = nullptr, *src_phi_r = nullptr, *src_re = nullptr, *src_im = nullptr;
 };
 
-struct few_batch {
-    few_ctx *ctx = nullptr;
-    bool fp64 = false;
+// Launch shape of one plan.
+struct LaunchPlan {
     int variant = kVariantFp64;
-    int n = 0;
-    void *blob_dev = nullptr;
-    void *scratch_dev = nullptr;
-    void *jobs_dev = nullptr;
-    int n_jobs = 0, build_blocks = 0, max_knots = 0;
     int grid = 0, threads = 0, R = 0, smem = 0, total_pairs = 0, total_fold = 0;
     int total_anchor_segs = 0;
+    int total_segs = 0, total_tiles = 0;  // kVariantTc
+};
+
+struct few_batch {
+    // The waves of one summation variant: a mixed batch may need both (kVariantTc and
+    // kVariantScalar), which then run one after the other.
+    struct Part {
+        void *blob_dev = nullptr;
+        void *scratch_dev = nullptr;
+        LaunchPlan launch;
+    };
+    few_ctx *ctx = nullptr;
+    int n = 0;
+    std::vector<Part> parts;
+    void *jobs_dev = nullptr;
+    int n_jobs = 0, build_blocks = 0, max_knots = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
 };
@@ -341,11 +365,11 @@ struct PlanImage {
     size_t off_waves = 0, off_cta = 0, off_seg = 0, off_anc = 0;
     size_t scratch_bytes = 0;
     std::vector<size_t> fcoef_off, ylm_off, anchor_off;
+    size_t recs_off = 0;  // kVariantTc: tile records of all waves
     std::vector<std::vector<int64_t>> seg;  // per wave: segment sample ranges [K]
     bool fp64 = false;
-    int variant = kVariantFp64;
-    int grid = 0, threads = 0, R = 0, smem = 0, buf_bytes = 0, total_pairs = 0, total_fold = 0;
-    int total_anchor_segs = 0, stage_slots = 0, ring = 0;
+    LaunchPlan launch;
+    int buf_bytes = 0, stage_slots = 0, ring = 0;
 };
 
 int occupancy(few_ctx *c, int variant, int R, int T, int smem)
@@ -391,47 +415,64 @@ few_status validate_request(const few_request &r, bool need_device_out)
     return FEW_OK;
 }
 
-// Build the host image of a plan for `n` requests of one precision.
-few_status build_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P)
+// Whether a request's mode set fits the tensor-core summation (kTcMaxRows, kTcMaxHalf).
+bool tc_fits(const few_request &r) { return r.prec == FEW_MIXED && r.traj->plan.tc_pairs > 0; }
+
+// Build the host image of a plan for `n` requests of one precision; tc: by the tensor-core
+// summation (every request fits it).
+few_status build_image(few_ctx *c, const few_request *reqs, int n, bool tc, PlanImage &P)
 {
     P.fp64 = reqs[0].prec == FEW_FP64;
+    LaunchPlan &L = P.launch;
     const int pi = P.fp64 ? 0 : 1;
-    P.R = c->tile_R[pi];
-    P.threads = c->tile_T[pi];
+    L.R = c->tile_R[pi];
+    L.threads = c->tile_T[pi];
     int max_slots = 1;
     for (int q = 0; q < n; ++q) max_slots = std::max(max_slots, reqs[q].traj->plan.n_slots);
-    P.variant = P.fp64 ? kVariantFp64 : kVariantScalar;
-    const size_t slot_bytes = (size_t)sum_slot_bytes(P.variant);
+    L.variant = P.fp64 ? kVariantFp64 : kVariantScalar;
+    const size_t slot_bytes = (size_t)sum_slot_bytes(L.variant);
     P.stage_slots = std::min(c->tile_S[pi], max_slots);  // no stage larger than any table
     P.ring = kDefaultRing;
     P.buf_bytes = (int)align_up((size_t)P.stage_slots * slot_bytes, 128);
-    P.smem = P.ring * P.buf_bytes;
-    const int occ = occupancy(c, P.variant, P.R, P.threads, P.smem);
+    L.smem = P.ring * P.buf_bytes;
+    // the tile settings are checked for every variant, also one that does not use them
+    const int occ = occupancy(c, L.variant, L.R, L.threads, L.smem);
     if (occ <= 0) return FEW_ERR_LIMIT;
-    P.grid = c->sm_count * occ;
-
-    // layout of the blob
-    size_t off = align_up(sizeof(PlanHdr), 64);
-    P.off_waves = off;
-    off = align_up(off + sizeof(WaveDev) * n, 64);
-    P.off_cta = off;
-    off = align_up(off + sizeof(CtaStart) * (P.grid + 1), 64);
-    P.off_seg = off;
-    size_t seg_ints = 0;
-    for (int q = 0; q < n; ++q) seg_ints += reqs[q].traj->K;
-    off = align_up(off + sizeof(int) * seg_ints, 64);
-    P.off_anc = off;  // per wave: first anchor of each segment, then the wave's total
-    if (!P.fp64) off += sizeof(int) * seg_ints;
-    off = align_up(off, 256);
-    P.blob.assign(off, 0);
+    L.grid = c->sm_count * occ;
     P.seg.resize(n);
     for (int q = 0; q < n; ++q) {
         const few_request &r = reqs[q];
         P.seg[q].resize(r.traj->K);
         segments(r.traj->t_host.data(), r.traj->K, r.t0, r.dt, r.n_samples, P.seg[q].data());
     }
+    if (tc) {
+        L.variant = kVariantTc;
+        int64_t tiles = 0;
+        for (int q = 0; q < n; ++q)
+            for (int k = 0; k + 1 < reqs[q].traj->K; ++k)
+                tiles += tiles_in_segment((int)P.seg[q][k], (int)P.seg[q][k + 1]);
+        if (tiles > 0x7fffffff) return FEW_ERR_LIMIT;
+        L.total_tiles = (int)tiles;
+        L.grid = (int)std::min<int64_t>(c->sm_count, tiles);
+    }
 
-    // scratch: folded coefficients and harmonic tables per wave
+    // layout of the blob
+    size_t off = align_up(sizeof(PlanHdr), 64);
+    P.off_waves = off;
+    off = align_up(off + sizeof(WaveDev) * n, 64);
+    P.off_cta = off;  // kVariantTc: int first tiles instead
+    off = align_up(off + sizeof(CtaStart) * (L.grid + 1), 64);
+    P.off_seg = off;
+    size_t seg_ints = 0;
+    for (int q = 0; q < n; ++q) seg_ints += reqs[q].traj->K;
+    off = align_up(off + sizeof(int) * seg_ints, 64);
+    P.off_anc = off;  // per wave: first anchor (or tile) of each segment, then the wave's total
+    if (!P.fp64) off += sizeof(int) * seg_ints;
+    off = align_up(off, 256);
+    P.blob.assign(off, 0);
+
+    // scratch: folded coefficients (or operand tables, then their scales) and harmonic tables
+    // per wave
     size_t s_off = 0;
     P.fcoef_off.resize(n);
     P.ylm_off.resize(n);
@@ -439,19 +480,43 @@ few_status build_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P)
     for (int q = 0; q < n; ++q) {
         const few_traj *tr = reqs[q].traj;
         P.fcoef_off[q] = s_off;
-        s_off = align_up(s_off + (size_t)tr->S * tr->plan.n_slots * slot_bytes, 256);
+        if (tc)
+            s_off = align_up(s_off + (size_t)tr->S * (tc_table_bytes(tr->plan.tc_pairs, tr->plan.tc_ks) +
+                                                      sizeof(float)), 256);
+        else
+            s_off = align_up(s_off + (size_t)tr->S * tr->plan.n_slots * slot_bytes, 256);
         P.ylm_off[q] = s_off;
         s_off = align_up(s_off + (size_t)tr->plan.pair_lm.size() * 2 * sizeof(double2), 256);
         P.anchor_off[q] = s_off;
-        if (!P.fp64) {
+        if (L.variant == kVariantScalar) {
             int na = 0;
             for (int k = 0; k + 1 < tr->K; ++k)
                 na += anchors_in_segment((int)P.seg[q][k], (int)P.seg[q][k + 1]);
             s_off = align_up(s_off + sizeof(Anchor) * (size_t)na, 256);
         }
     }
+    P.recs_off = s_off;
+    if (tc) s_off += sizeof(TileRec) * (size_t)L.total_tiles;
     P.scratch_bytes = s_off;
     return FEW_OK;
+}
+
+// First tile of each CTA of a tensor-core plan: contiguous runs of tiles of equal total cost.
+void partition_tiles(const std::vector<int> &tile_begin, const std::vector<double> &tile_cost,
+                     int grid, int *cta)
+{
+    const int n = (int)tile_cost.size();
+    std::vector<double> cum(n + 1, 0.0);
+    for (int q = 0; q < n; ++q)
+        cum[q + 1] = cum[q] + tile_cost[q] * (tile_begin[q + 1] - tile_begin[q]);
+    int q = 0;
+    for (int g = 0; g < grid; ++g) {
+        const double x = cum[n] * g / grid;
+        while (q < n - 1 && cum[q + 1] <= x) ++q;
+        const int k = (int)std::ceil((x - cum[q]) / tile_cost[q]);
+        cta[g] = std::min(tile_begin[q] + k, tile_begin[q + 1]);
+    }
+    cta[grid] = tile_begin[n];
 }
 
 // CTA slices of the concatenated (wave, sample) space of n waves (segs[q]: wave q's K[q]
@@ -509,8 +574,12 @@ void fill_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P, unsign
     CtaStart *cta = reinterpret_cast<CtaStart *>(P.blob.data() + P.off_cta);
     int *seg = reinterpret_cast<int *>(P.blob.data() + P.off_seg);
     int *anc = reinterpret_cast<int *>(P.blob.data() + P.off_anc);
+    LaunchPlan &L = P.launch;
+    const bool tc = L.variant == kVariantTc;
     size_t seg_pos = 0;
-    int pair_begin = 0, fold_begin = 0, anchor_seg_begin = 0;
+    int pair_begin = 0, fold_begin = 0, anchor_seg_begin = 0, seg_begin = 0;
+    std::vector<int> tile_begin(1, 0);
+    std::vector<double> tile_cost;
     for (int q = 0; q < n; ++q) {
         const few_request &r = reqs[q];
         const few_traj *tr = r.traj;
@@ -535,7 +604,23 @@ void fill_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P, unsign
         const std::vector<int64_t> &ss = P.seg[q];
         for (int k = 0; k < tr->K; ++k) seg[seg_pos + k] = (int)ss[k];
         W.seg_start = reinterpret_cast<const int *>(blob_dev + P.off_seg) + seg_pos;
-        if (!P.fp64) {
+        if (tc) {
+            int a = 0;
+            for (int k = 0; k + 1 < tr->K; ++k) {
+                anc[seg_pos + k] = a;
+                a += tiles_in_segment((int)ss[k], (int)ss[k + 1]);
+            }
+            anc[seg_pos + tr->K - 1] = a;
+            W.tab = scratch_dev + P.fcoef_off[q];
+            W.tab_inv = reinterpret_cast<float *>(
+                W.tab + (size_t)tr->S * tc_table_bytes(tr->plan.tc_pairs, tr->plan.tc_ks));
+            W.tile_off = reinterpret_cast<const int *>(blob_dev + P.off_anc) + seg_pos;
+            W.tile_begin = tile_begin[q];
+            W.seg_begin = seg_begin;
+            seg_begin += tr->S;
+            tile_begin.push_back(tile_begin[q] + a);
+            tile_cost.push_back(tc_tile_cost(tr->plan.tc_pairs, tr->plan.tc_ks));
+        } else if (!P.fp64) {
             int a = 0;
             for (int k = 0; k + 1 < tr->K; ++k) {
                 anc[seg_pos + k] = a;
@@ -554,10 +639,13 @@ void fill_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P, unsign
         W.fold_begin = fold_begin;
         fold_begin += tr->S * W.fold_blocks_per_seg;
     }
-    P.total_pairs = pair_begin;
-    P.total_fold = fold_begin;
-    P.total_anchor_segs = anchor_seg_begin;
-    {
+    L.total_pairs = pair_begin;
+    L.total_fold = fold_begin;
+    L.total_anchor_segs = anchor_seg_begin;
+    L.total_segs = seg_begin;
+    if (tc) {
+        partition_tiles(tile_begin, tile_cost, L.grid, reinterpret_cast<int *>(cta));
+    } else {
         std::vector<const int64_t *> segs(n);
         std::vector<int> Ks(n), slots(n);
         for (int q = 0; q < n; ++q) {
@@ -565,63 +653,84 @@ void fill_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P, unsign
             Ks[q] = reqs[q].traj->K;
             slots[q] = reqs[q].traj->plan.n_slots;
         }
-        partition_ctas(n, segs.data(), Ks.data(), slots.data(), P.grid,
-                       (long long)P.threads * P.R, cta);
+        partition_ctas(n, segs.data(), Ks.data(), slots.data(), L.grid,
+                       (long long)L.threads * L.R, cta);
     }
     hdr->n_waves = n;
-    hdr->total_pairs = P.total_pairs;
-    hdr->total_fold_blocks = P.total_fold;
-    hdr->total_anchor_segs = P.total_anchor_segs;
-    hdr->grid_sum = P.grid;
+    hdr->total_pairs = L.total_pairs;
+    hdr->total_fold_blocks = L.total_fold;
+    hdr->total_anchor_segs = L.total_anchor_segs;
+    hdr->total_segs = L.total_segs;
+    hdr->total_tiles = L.total_tiles;
+    hdr->tile_cta = reinterpret_cast<const int *>(blob_dev + P.off_cta);
+    hdr->recs = reinterpret_cast<TileRec *>(scratch_dev + P.recs_off);
+    hdr->grid_sum = L.grid;
     hdr->buf_bytes = P.buf_bytes;
     hdr->stage_slots = P.stage_slots;
     hdr->ring = P.ring;
-    hdr->variant = P.variant;
+    hdr->variant = L.variant;
     hdr->waves = reinterpret_cast<const WaveDev *>(blob_dev + P.off_waves);
     hdr->cta = reinterpret_cast<const CtaStart *>(blob_dev + P.off_cta);
     hdr->err = c->d_err;
 }
 
-few_status launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, int total_pairs, int total_fold,
-                          int total_anchor_segs, int grid, int threads, int R, int smem, int variant,
-                          cudaStream_t st)
+// Queue a plan's kernels on `st`.  Errors are returned after everything queued has been joined.
+cudaError_t launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, const LaunchPlan &P, cudaStream_t st,
+                           bool mark)
 {
+    auto tm = [&](int slot, bool end) {
+        if (mark) tmark(c, slot, end, st);
+    };
+    const bool fp64 = P.variant == kVariantFp64;
+    cudaError_t e;
+    if (P.variant == kVariantTc) {
+        tm(1, false);
+        if ((e = launch_ylm(hdr_dev, P.total_pairs, false, st)) != cudaSuccess) return e;
+        tm(1, true);
+        tm(2, false);
+        if ((e = launch_fold_tc(hdr_dev, P.total_segs, P.total_tiles, st)) != cudaSuccess) return e;
+        tm(2, true);
+        tm(3, false);
+        if ((e = launch_sum_tc(hdr_dev, P.grid, st)) != cudaSuccess) return e;
+        tm(3, true);
+        return cudaSuccess;
+    }
     // the phase anchors depend on the splines only: they run on a side lane beside the
     // harmonics and the fold (FP64-pipe work next to latency-bound work), joined before the sum
-    const bool fork = total_anchor_segs > 0;
+    const bool fork = P.total_anchor_segs > 0;
     auto &L = c->lanes[c->lane_next++ % 4];
     if (fork) {
         // any failure after this point still leaves the side stream's work ordered before what
         // the caller queues next on `st` (the release of the call's scratch)
-        if (cudaEventRecord(L.fork, st) != cudaSuccess ||
-            cudaStreamWaitEvent(L.s, L.fork, 0) != cudaSuccess)
-            return FEW_ERR_CUDA;
-        const cudaError_t ea = launch_anchor(hdr_dev, total_anchor_segs, L.s);
-        if (cudaEventRecord(L.join, L.s) != cudaSuccess) {
+        if ((e = cudaEventRecord(L.fork, st)) != cudaSuccess ||
+            (e = cudaStreamWaitEvent(L.s, L.fork, 0)) != cudaSuccess)
+            return e;
+        const cudaError_t ea = launch_anchor(hdr_dev, P.total_anchor_segs, L.s);
+        if ((e = cudaEventRecord(L.join, L.s)) != cudaSuccess) {
             cudaStreamSynchronize(L.s);
-            return FEW_ERR_CUDA;
+            return e;
         }
         if (ea != cudaSuccess) {
             cudaStreamWaitEvent(st, L.join, 0);
-            return FEW_ERR_CUDA;
+            return ea;
         }
     }
-    auto joined = [&](cudaError_t e) {  // a failed launch: join the side stream, then report
-        if (e == cudaSuccess) return true;
-        if (fork) cudaStreamWaitEvent(st, L.join, 0);
-        return false;
+    auto joined = [&](cudaError_t err) {  // a failed launch: join the side stream, then report
+        if (err != cudaSuccess && fork) cudaStreamWaitEvent(st, L.join, 0);
+        return err;
     };
-    tmark(c, 1, false, st);
-    if (!joined(launch_ylm(hdr_dev, total_pairs, variant == kVariantFp64, st))) return FEW_ERR_CUDA;
-    tmark(c, 1, true, st);
-    tmark(c, 2, false, st);
-    if (!joined(launch_fold(hdr_dev, total_fold, variant == kVariantFp64, st))) return FEW_ERR_CUDA;
-    if (fork) FEW_CUDA_TRY(cudaStreamWaitEvent(st, L.join, 0));
-    tmark(c, 2, true, st);
-    tmark(c, 3, false, st);
-    FEW_CUDA_TRY(launch_sum(hdr_dev, grid, threads, R, smem, variant, st));
-    tmark(c, 3, true, st);
-    return FEW_OK;
+    tm(1, false);
+    if ((e = joined(launch_ylm(hdr_dev, P.total_pairs, fp64, st))) != cudaSuccess) return e;
+    tm(1, true);
+    tm(2, false);
+    if ((e = joined(launch_fold(hdr_dev, P.total_fold, fp64, st))) != cudaSuccess) return e;
+    if (fork && (e = cudaStreamWaitEvent(st, L.join, 0)) != cudaSuccess) return e;
+    tm(2, true);
+    tm(3, false);
+    if ((e = launch_sum(hdr_dev, P.grid, P.threads, P.R, P.smem, P.variant, st)) != cudaSuccess)
+        return e;
+    tm(3, true);
+    return cudaSuccess;
 }
 
 const char *kNames[] = {"FEW_OK",           "FEW_ERR_INVALID_ARG", "FEW_ERR_KNOTS",
@@ -693,7 +802,7 @@ few_status few_ctx_create(few_ctx **out, int device, size_t hbm_budget_bytes)
             return fail(FEW_ERR_CUDA);
     if (cudaMalloc(&c->d_err, sizeof(unsigned)) != cudaSuccess) return fail(FEW_ERR_NOMEM);
     if (cudaMemset(c->d_err, 0, sizeof(unsigned)) != cudaSuccess) return fail(FEW_ERR_CUDA);
-    if (sum_configure() != cudaSuccess) return fail(FEW_ERR_CUDA);
+    if (sum_configure() != cudaSuccess || tc_configure() != cudaSuccess) return fail(FEW_ERR_CUDA);
     for (auto &e : c->tev)
         if (cudaEventCreate(&e) != cudaSuccess) return fail(FEW_ERR_CUDA);
     *out = c;
@@ -789,7 +898,8 @@ few_status few_traj_create(few_ctx *ctx, const double *t_knots, int K, const int
                  o_pair = take(sizeof(int2) * P.pair_lm.size()), o_mp = take(sizeof(int) * N),
                  o_sp = take(sizeof(int) * P.slot_ptr.size()),
                  o_ct = take(sizeof(int2) * std::max<size_t>(1, P.contrib.size())),
-                 o_rows = take(sizeof(int2) * P.rows.size()), o_job = take(sizeof(BuildJob));
+                 o_rows = take(sizeof(int2) * P.rows.size()),
+                 o_rslot = take(sizeof(int4) * P.row_slot.size()), o_job = take(sizeof(BuildJob));
     if ((st = dev_alloc(ctx, off, ctx->internal, &tr->dmem))) {
         delete tr;
         return st;
@@ -807,6 +917,7 @@ few_status few_traj_create(few_ctx *ctx, const double *t_knots, int K, const int
     put(o_sp, P.slot_ptr.data(), sizeof(int) * P.slot_ptr.size());
     put(o_ct, P.contrib.data(), sizeof(int2) * P.contrib.size());
     put(o_rows, P.rows.data(), sizeof(int2) * P.rows.size());
+    put(o_rslot, P.row_slot.data(), sizeof(int4) * P.row_slot.size());
 
     TrajDev &D = tr->dev;
     D.K = K;
@@ -837,6 +948,11 @@ few_status few_traj_create(few_ctx *ctx, const double *t_knots, int K, const int
     D.slot_ptr = reinterpret_cast<const int *>(d + o_sp);
     D.contrib = reinterpret_cast<const int2 *>(d + o_ct);
     D.rows = reinterpret_cast<const int2 *>(d + o_rows);
+    D.row_slot = reinterpret_cast<const int4 *>(d + o_rslot);
+    D.tc_pairs = P.tc_pairs;
+    D.tc_ks = P.tc_ks;
+    D.n_mid = P.n_mid;
+    D.m_fin = P.m_fin;
     tr->job_dev = reinterpret_cast<BuildJob *>(d + o_job);
 
     cudaStream_t s = ctx->internal;
@@ -983,14 +1099,21 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream)
     if (!dev_scope.ok) return FEW_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     PlanImage P;
-    if ((st = build_image(ctx, req, 1, P))) return st;
     const size_t out_bytes = (size_t)req->n_samples * (req->out_c64 ? 8 : 16);
     void *blob = nullptr, *scratch = nullptr, *dout = nullptr;
-    if ((st = dev_alloc(ctx, P.blob.size(), s, &blob))) return st;
-    if ((st = dev_alloc(ctx, P.scratch_bytes, s, &scratch))) {
-        dev_free(ctx, blob, s);
-        return st;
-    }
+    auto plan = [&](bool tc) {
+        P = PlanImage();
+        few_status e = build_image(ctx, req, 1, tc, P);
+        if (e) return e;
+        if ((e = dev_alloc(ctx, P.blob.size(), s, &blob))) return e;
+        if ((e = dev_alloc(ctx, P.scratch_bytes, s, &scratch))) dev_free(ctx, blob, s);
+        return e;
+    };
+    const bool tc = tc_fits(*req);
+    st = plan(tc);
+    // the tensor-core plan may need more scratch than the scalar one (sparse mode sets)
+    if (tc && (st == FEW_ERR_BUDGET || st == FEW_ERR_NOMEM)) st = plan(false);
+    if (st) return st;
     void *out_dev = req->out;
     if (req->out_where == FEW_MEM_HOST) {
         // page-locked host memory is addressable from the device (over NVLink-C2C on a Grace
@@ -1013,9 +1136,10 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream)
     fill_image(ctx, req, 1, P, static_cast<unsigned char *>(blob),
                static_cast<unsigned char *>(scratch), &out_dev);
     st = upload(ctx, blob, P.blob.data(), P.blob.size(), s);
-    if (!st)
-        st = launch_kernels(ctx, static_cast<const PlanHdr *>(blob), P.total_pairs, P.total_fold,
-                            P.total_anchor_segs, P.grid, P.threads, P.R, P.smem, P.variant, s);
+    if (!st && launch_kernels(ctx, static_cast<const PlanHdr *>(blob), P.launch, s, true) != cudaSuccess) {
+        (void)cudaGetLastError();
+        st = FEW_ERR_CUDA;
+    }
     if (!st && dout) {
         cudaError_t e = cudaMemcpyAsync(req->out, dout, out_bytes, cudaMemcpyDeviceToHost, s);
         if (e != cudaSuccess) {
@@ -1267,20 +1391,22 @@ few_status few_batch_plan(few_ctx *ctx, const few_request *reqs, int n, unsigned
     std::lock_guard<std::recursive_mutex> lk(ctx->mu);
     DeviceScope dev_scope(ctx->device);
     if (!dev_scope.ok) return FEW_ERR_CUDA;
-    PlanImage P;
-    few_status st = build_image(ctx, reqs, n, P);
-    if (st) return st;
+    few_status st = FEW_OK;
     few_batch *b = new (std::nothrow) few_batch();
     if (!b) return FEW_ERR_NOMEM;
     b->ctx = ctx;
-    b->fp64 = P.fp64;
-    b->variant = P.variant;
     b->n = n;
     cudaStream_t s = ctx->internal;
+    auto drop_parts = [&]() {
+        for (auto &p : b->parts) {
+            dev_free(ctx, p.scratch_dev, s);
+            dev_free(ctx, p.blob_dev, s);
+        }
+        b->parts.clear();
+    };
     auto fail = [&](few_status e) {
         dev_free(ctx, b->jobs_dev, s);
-        dev_free(ctx, b->scratch_dev, s);
-        dev_free(ctx, b->blob_dev, s);
+        drop_parts();
         cudaStreamSynchronize(s);
         (void)cudaGetLastError();
         if (b->exec) cudaGraphExecDestroy(b->exec);
@@ -1288,13 +1414,34 @@ few_status few_batch_plan(few_ctx *ctx, const few_request *reqs, int n, unsigned
         delete b;
         return e;
     };
-    if ((st = dev_alloc(ctx, P.blob.size(), s, &b->blob_dev))) return fail(st);
-    if ((st = dev_alloc(ctx, P.scratch_bytes, s, &b->scratch_dev))) return fail(st);
-    std::vector<void *> outs(n);
-    for (int q = 0; q < n; ++q) outs[q] = reqs[q].out;
-    fill_image(ctx, reqs, n, P, static_cast<unsigned char *>(b->blob_dev),
-               static_cast<unsigned char *>(b->scratch_dev), outs.data());
-    if ((st = upload(ctx, b->blob_dev, P.blob.data(), P.blob.size(), s))) return fail(st);
+    // one part per summation variant
+    auto add_part = [&](const std::vector<few_request> &rq, bool tc) -> few_status {
+        if (rq.empty()) return FEW_OK;
+        const int nr = (int)rq.size();
+        PlanImage P;
+        few_status e = build_image(ctx, rq.data(), nr, tc, P);
+        if (e) return e;
+        b->parts.emplace_back();
+        few_batch::Part &part = b->parts.back();
+        if ((e = dev_alloc(ctx, P.blob.size(), s, &part.blob_dev))) return e;
+        if ((e = dev_alloc(ctx, P.scratch_bytes, s, &part.scratch_dev))) return e;
+        std::vector<void *> outs(nr);
+        for (int q = 0; q < nr; ++q) outs[q] = rq[q].out;
+        fill_image(ctx, rq.data(), nr, P, static_cast<unsigned char *>(part.blob_dev),
+                   static_cast<unsigned char *>(part.scratch_dev), outs.data());
+        part.launch = P.launch;
+        return upload(ctx, part.blob_dev, P.blob.data(), P.blob.size(), s);
+    };
+    std::vector<few_request> tc_reqs, other;
+    for (int q = 0; q < n; ++q) (tc_fits(reqs[q]) ? tc_reqs : other).push_back(reqs[q]);
+    st = add_part(tc_reqs, true);
+    if (!st) st = add_part(other, false);
+    if ((st == FEW_ERR_BUDGET || st == FEW_ERR_NOMEM) && !tc_reqs.empty()) {
+        // the scalar plan of sparse mode sets needs less scratch
+        drop_parts();
+        st = add_part(std::vector<few_request>(reqs, reqs + n), false);
+    }
+    if (st) return fail(st);
     if (flags & FEW_BATCH_REBUILD_SPLINES) {
         std::vector<BuildJob> jobs;
         std::set<const few_traj *> seen;
@@ -1319,36 +1466,18 @@ few_status few_batch_plan(few_ctx *ctx, const few_request *reqs, int n, unsigned
         b->n_jobs = (int)jobs.size();
         b->build_blocks = blocks;
     }
-    b->grid = P.grid;
-    b->threads = P.threads;
-    b->R = P.R;
-    b->smem = P.smem;
-    b->total_pairs = P.total_pairs;
-    b->total_fold = P.total_fold;
-    b->total_anchor_segs = P.total_anchor_segs;
     if (cudaStreamSynchronize(s) != cudaSuccess) return fail(FEW_ERR_CUDA);
     if (!(flags & FEW_BATCH_NO_GRAPH)) {
         cudaStream_t cap = nullptr;
         if (cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) return fail(FEW_ERR_CUDA);
         cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            const PlanHdr *hd = static_cast<const PlanHdr *>(b->blob_dev);
             if (b->n_jobs)
                 launch_build(static_cast<const BuildJob *>(b->jobs_dev), b->n_jobs, b->build_blocks,
                              b->max_knots, ctx->d_err, cap);
-            // the same fork and join as launch_kernels, recorded into the graph
-            const bool fork = b->total_anchor_segs > 0;
-            auto &L = ctx->lanes[ctx->lane_next++ % 4];
-            if (fork) {
-                cudaEventRecord(L.fork, cap);
-                cudaStreamWaitEvent(L.s, L.fork, 0);
-                launch_anchor(hd, b->total_anchor_segs, L.s);
-                cudaEventRecord(L.join, L.s);
-            }
-            launch_ylm(hd, b->total_pairs, b->fp64, cap);
-            launch_fold(hd, b->total_fold, b->fp64, cap);
-            if (fork) cudaStreamWaitEvent(cap, L.join, 0);
-            launch_sum(hd, b->grid, b->threads, b->R, b->smem, b->variant, cap);
+            // the same forks and joins as a direct run, recorded into the graph
+            for (const auto &p : b->parts)
+                launch_kernels(ctx, static_cast<const PlanHdr *>(p.blob_dev), p.launch, cap, false);
             e = cudaStreamEndCapture(cap, &b->graph);
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
@@ -1372,15 +1501,15 @@ few_status few_batch_run(few_ctx *ctx, few_batch *b, void *stream)
         FEW_CUDA_TRY(cudaGraphLaunch(b->exec, s));
         return FEW_OK;
     }
-    const PlanHdr *hd = static_cast<const PlanHdr *>(b->blob_dev);
     if (b->n_jobs) {
         tmark(ctx, 0, false, s);
         FEW_CUDA_TRY(launch_build(static_cast<const BuildJob *>(b->jobs_dev), b->n_jobs,
                                   b->build_blocks, b->max_knots, ctx->d_err, s));
         tmark(ctx, 0, true, s);
     }
-    return launch_kernels(ctx, hd, b->total_pairs, b->total_fold, b->total_anchor_segs, b->grid,
-                          b->threads, b->R, b->smem, b->variant, s);
+    for (const auto &p : b->parts)
+        FEW_CUDA_TRY(launch_kernels(ctx, static_cast<const PlanHdr *>(p.blob_dev), p.launch, s, true));
+    return FEW_OK;
 }
 
 few_status few_batch_release(few_ctx *ctx, few_batch *b)
@@ -1393,8 +1522,10 @@ few_status few_batch_release(few_ctx *ctx, few_batch *b)
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     dev_free(ctx, b->jobs_dev, ctx->internal);
-    dev_free(ctx, b->scratch_dev, ctx->internal);
-    dev_free(ctx, b->blob_dev, ctx->internal);
+    for (auto &p : b->parts) {
+        dev_free(ctx, p.scratch_dev, ctx->internal);
+        dev_free(ctx, p.blob_dev, ctx->internal);
+    }
     cudaStreamSynchronize(ctx->internal);
     (void)cudaGetLastError();
     ctx->batches.erase(b);
@@ -1552,6 +1683,8 @@ bool ctx_traj_view(few_ctx *ctx, const few_traj *tr, CtxTrajView *v)
     v->K = tr->K;
     v->n_slots = tr->plan.n_slots;
     v->n_pairs = (int)tr->plan.pair_lm.size();
+    v->tc_pairs = tr->plan.tc_pairs;
+    v->tc_ks = tr->plan.tc_ks;
     v->t_host = tr->t_host.data();
     v->dev = tr->dev;
     return true;

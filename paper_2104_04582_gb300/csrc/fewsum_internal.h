@@ -30,8 +30,34 @@ constexpr int kMinStageSlots = 16, kMaxStageSlots = 4096;
 // Summation kernel variants (and the folded-coefficient layout each reads).
 enum : int {
     kVariantFp64 = 0,   // FP64 throughout; slot = 8 doubles
-    kVariantScalar = 1  // mixed: FP64 phases at anchors, FP32 everything else; slot = 8 floats
+    kVariantScalar = 1,  // mixed: FP64 phases at anchors, FP32 everything else; slot = 8 floats
+    kVariantTc = 2       // mixed: the sum over n on the tensor cores (tcsum.cu)
 };
+
+// Tensor-core summation (tcsum.cu): tiles of kTcTile consecutive samples of one segment, starting
+// at multiples of kTcTile (so a sample's arithmetic does not depend on the request's slicing).
+constexpr int kTcTile = 128;    // the MMA's M: one sample per tensor-memory lane
+constexpr int kTcMaxRows = 22;  // rows (signed m): two accumulators of 8 columns per row, beside
+                                //   the operands, in the 512 tensor-memory columns
+constexpr int kTcMaxHalf = 31;  // half-width of the n range: 64 basis values (K)
+constexpr int kTcFoldThreads = 704;
+constexpr int kTcRecThreads = 128;  // threads of a fold block that fill tile records
+// Everything the summation reads for one tile, one 128-byte line.  Phases of sample a + v, a =
+// max(i0, s0): c0 + c1 v + c2 v^2 + c3 v^3 turns modulo 1, each coefficient in units of 2^-64 turn
+// (64-bit wrap-around arithmetic is then the exact reduction modulo one turn).
+struct alignas(128) TileRec {
+    long long phi[4], r[4];
+    int i0, s0, s1;       // first sample of lane 0; the segment's samples [s0, s1)
+    int tile_end;         // first tile after the segment
+    float u0, du;         // u of sample i: u0 + (i - s0) du
+    const float *inv;     // inverse of the segment table's power-of-two scale
+    const unsigned char *tab;  // the segment's operand table
+    void *out;
+    int pairs, ks;        // row pairs, K steps of 16 (8 powers of z_r each)
+    int mids;             // n_mid (low 16 bits, signed) and m_fin (high 16 bits, signed)
+    int c64;
+};
+static_assert(sizeof(TileRec) == 128, "one line");
 
 // Phase anchors of the mixed path: the FP64 phase splines are evaluated and reduced modulo one
 // turn at every kAnchorGroup-th sample (absolute sample index a = kAnchorGroup * q), together
@@ -82,6 +108,9 @@ struct TrajDev {
     const int *slot_ptr;   // [n_slots + 1] CSR into contrib
     const int2 *contrib;   // [n_contrib] (mode * 2 + kind, 2 * pair + kind); kind 0: A Y+,
                            //   1: conj(A) Y-
+    int tc_pairs, tc_ks;   // tensor-core summation: row pairs, K steps (tc_pairs 0: not used)
+    int n_mid, m_fin;      //   centre of the n range; signed m of the last pair's second row
+    const int4 *row_slot;  // [n_rows] (first slot, highest n, lowest n, 0); lowest > highest: empty
     const int2 *rows;      // [n_rows] (slots of the row, lowest n of the previous row minus
                            //   this row's lowest n); a row's slots run from its highest n down
 };
@@ -123,6 +152,11 @@ struct WaveDev {
     Anchor *anchors;      // mixed plans: [n_anchors] phase anchors (segment by segment)
     const int *anchor_off;  // mixed plans: [K] first anchor of each segment, then the total
     int anchor_seg_begin; // first global segment index of this wave (anchor kernel grid)
+    unsigned char *tab;   // tensor-core plans: [S] operand tables of tc_table_bytes
+    float *tab_inv;       //   [S] inverse table scales
+    const int *tile_off;  //   [K] first tile of each segment, then the total
+    int tile_begin;       //   first tile of this wave in the plan
+    int seg_begin;        //   first segment of this wave in the plan
     double2 *ylm;         // [n_pairs][2]: Y+ = -2Y_{l,m}, Y- = (-1)^l -2Y_{l,-m} (0 if m = 0)
     const int *seg_start; // [K] sample range of each segment
     int pair_begin;       // first global pair index of this wave (ylm kernel)
@@ -149,6 +183,9 @@ struct PlanHdr {
     int stage_slots; // slots per ring stage (the mode tile)
     int ring;        // ring stages
     int variant;     // kVariant* of the summation kernel and the folded layout
+    int total_segs, total_tiles;  // tensor-core plans
+    const int *tile_cta;  //   [grid + 1] first tile of each CTA
+    TileRec *recs;        //   [total_tiles]
     const WaveDev *waves;
     const CtaStart *cta;
     unsigned *err;
@@ -175,6 +212,18 @@ inline int anchors_in_segment(int s_begin, int s_end)
 cudaError_t launch_wait_selftest(unsigned *err, unsigned limit_us, cudaStream_t st);
 cudaError_t launch_sum(const PlanHdr *hdr_dev, int grid, int threads, int samples_per_thread,
                        int smem_bytes, int variant, cudaStream_t st);
+// Bytes of one segment's tensor-core operand table: fp16 high and low parts, N = 16 pairs rows of
+// 16 ks columns each.
+__host__ __device__ inline int tc_table_bytes(int pairs, int ks) { return 1024 * pairs * ks; }
+// Relative cost of one tile: the MMAs' cycles plus the per-sample work around them.
+inline double tc_tile_cost(int pairs, int ks) { return 24.0 * pairs * ks + 300.0; }
+inline int tiles_in_segment(int s_begin, int s_end)
+{
+    return s_end > s_begin ? (s_end - 1) / kTcTile - s_begin / kTcTile + 1 : 0;
+}
+cudaError_t tc_configure();
+cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st);
+cudaError_t launch_sum_tc(const PlanHdr *hdr_dev, int grid, cudaStream_t st);
 // Bytes of one folded slot in the layout a variant reads.
 int sum_slot_bytes(int variant);
 cudaError_t launch_phases(const TrajDev &tr, const int *seg_start, double t0, double dt, int n,
@@ -246,7 +295,7 @@ struct CtxTrajView {
     unsigned *d_err;
     int tile_R[2], tile_T[2], tile_S[2];
     bool has_data;
-    int K, n_slots, n_pairs;
+    int K, n_slots, n_pairs, tc_pairs, tc_ks;
     const double *t_host;
     TrajDev dev;
 };

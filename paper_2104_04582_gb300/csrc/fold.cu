@@ -21,6 +21,7 @@
 #include "fewsum_internal.h"
 #include "harmonics.cuh"
 #include "convert.cuh"
+#include "fold_slot.cuh"
 
 namespace fewsum {
 
@@ -116,9 +117,6 @@ cudaError_t launch_ylm(const PlanHdr *hdr_dev, int total_pairs, bool fp64, cudaS
     return cudaGetLastError();
 }
 
-__device__ __forceinline__ double cvt(double v, double) { return v; }
-__device__ __forceinline__ float cvt(double v, float) { return f64_to_f32_fast(v); }
-
 template <typename T> struct Slot8;
 template <> struct Slot8<double> {
     __device__ static void store(double *dst, const double (&re)[4], const double (&im)[4])
@@ -139,11 +137,8 @@ template <> struct Slot8<float> {
     }
 };
 
-// One thread per (wave, segment, slot): K_slot = scale * sum of its contributions, summed on the
-// splines' Hermite data (values and slopes at the segment's two knots) and turned into power
-// coefficients in u once.
-// T is the arithmetic and storage type of the folded coefficients (double for FEW_FP64,
-// float for FEW_MIXED, whose amplitudes are FP32 by design).
+// One thread per (wave, segment, slot).  T is the arithmetic and storage type of the folded
+// coefficients (double for FEW_FP64, float for FEW_MIXED, whose amplitudes are FP32 by design).
 template <typename T>
 __global__ void __launch_bounds__(kFoldThreads) k_fold(const PlanHdr *__restrict__ hp)
 {
@@ -156,39 +151,8 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold(const PlanHdr *__restrict
     const int slot = (local % W.fold_blocks_per_seg) * kFoldThreads + threadIdx.x;
     const TrajDev &tr = W.tr;
     if (s >= tr.S || slot >= tr.n_slots) return;
-    T re[4] = {0, 0, 0, 0}, im[4] = {0, 0, 0, 0};
-    const int c0 = tr.slot_ptr[slot], c1 = tr.slot_ptr[slot + 1];
-    const double *__restrict__ cs = tr.coef + (size_t)s * tr.J * 4;
-    for (int c = c0; c < c1; ++c) {
-        const int2 code = tr.contrib[c];  // (mode * 2 + kind, harmonic-table index)
-        const int i = code.x >> 1, kind = code.x & 1;
-        const double2 Yd = W.ylm[code.y];
-        const T yr = cvt(Yd.x, T()), yi = cvt(Yd.y, T());
-        const double2 *ca = reinterpret_cast<const double2 *>(cs + (size_t)(2 + 2 * i) * 4);
-        const double2 r01 = ca[0], r23 = ca[1], i01 = ca[2], i23 = ca[3];
-        const T ar[4] = {cvt(r01.x, T()), cvt(r01.y, T()), cvt(r23.x, T()), cvt(r23.y, T())};
-        T ai[4] = {cvt(i01.x, T()), cvt(i01.y, T()), cvt(i23.x, T()), cvt(i23.y, T())};
-        if (kind) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) ai[q] = -ai[q];
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            re[q] += ar[q] * yr - ai[q] * yi;
-            im[q] += ar[q] * yi + ai[q] * yr;
-        }
-    }
-    // the folded values are Hermite data (the fold is linear in them): power coefficients in u
-    // once per (segment, slot)
-    const T hk = cvt(tr.h[s], T()), sc = cvt(W.scale, T());
     T pre[4], pim[4];
-    hermite_to_power(re[0], re[1], re[2], re[3], hk, pre);
-    hermite_to_power(im[0], im[1], im[2], im[3], hk, pim);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        pre[q] *= sc;
-        pim[q] *= sc;
-    }
+    fold_slot<T>(tr, W.ylm, tr.coef + (size_t)s * tr.J * 4, slot, tr.h[s], W.scale, pre, pim);
     T *dst = reinterpret_cast<T *>(W.fcoef) + ((size_t)s * tr.n_slots + slot) * 8;
     Slot8<T>::store(dst, pre, pim);
 }

@@ -144,9 +144,20 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     const size_t fcoef_bytes = up((size_t)S * v.n_slots * slot_bytes, 256);
     const size_t ylm_bytes = up((size_t)v.n_pairs * 2 * sizeof(double2), 256);
     const size_t anc_bytes = up(sizeof(Anchor) * (size_t)n_anchors, 256);
+    // what fits is decided by the plain layout; the tensor-core plan (tile records, operand tables
+    // and their scales instead of anchors and folded coefficients) is taken where it fits too
     if (blob_bytes + fcoef_bytes + ylm_bytes + anc_bytes > kScratchBytes) return FEW_ERR_LIMIT;
+    int n_tiles = 0;
+    if (!fp64 && v.tc_pairs > 0)
+        for (int k = 0; k + 1 < K; ++k) n_tiles += tiles_in_segment(seg[k], seg[k + 1]);
+    const size_t tab_bytes = up((size_t)S * tc_table_bytes(v.tc_pairs, v.tc_ks), 256);
+    const size_t inv_bytes = up((size_t)S * sizeof(float), 256);
+    const size_t rec_bytes = sizeof(TileRec) * (size_t)n_tiles;
+    const bool tc = n_tiles > 0 &&
+                    blob_bytes + rec_bytes + tab_bytes + inv_bytes + ylm_bytes <= kScratchBytes;
+    const int grid_tc = n_tiles < v.sm_count ? n_tiles : v.sm_count;
     unsigned char *d_fcoef = base + blob_bytes;
-    unsigned char *d_ylm = d_fcoef + fcoef_bytes;
+    unsigned char *d_ylm = tc ? base + blob_bytes + rec_bytes + tab_bytes + inv_bytes : d_fcoef + fcoef_bytes;
     unsigned char *d_anc = d_ylm + ylm_bytes;
 
     W->tr = v.dev;
@@ -169,28 +180,48 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     W->pair_begin = 0;
     W->fold_begin = 0;
     W->fold_blocks_per_seg = (v.n_slots + kFoldThreads - 1) / kFoldThreads;
-    if (!fp64) {
+    if (tc) {
+        int a = 0;
+        for (int k = 0; k + 1 < K; ++k) {
+            anc[k] = a;
+            a += tiles_in_segment(seg[k], seg[k + 1]);
+        }
+        anc[K - 1] = a;
+        W->tab = base + blob_bytes + rec_bytes;
+        W->tab_inv = reinterpret_cast<float *>(W->tab + tab_bytes);
+        W->tile_off = reinterpret_cast<const int *>(base + off_anc);
+        W->tile_begin = 0;
+        W->seg_begin = 0;
+    } else if (!fp64) {
         W->anchors = reinterpret_cast<Anchor *>(d_anc);
         W->anchor_off = reinterpret_cast<const int *>(base + off_anc);
         W->anchor_seg_begin = 0;
     }
 
-    // equal slices of the samples (one waveform: equal cost per sample)
-    for (int g = 0; g < grid; ++g) {
-        const long double x = (long double)ns * g / grid;
-        cta[g] = CtaStart{0, (int)std::ceil(x)};
+    if (tc) {  // equal runs of tiles (grid_tc <= grid: the table has room)
+        int *first = reinterpret_cast<int *>(cta);
+        for (int g = 0; g <= grid_tc; ++g) first[g] = (int)(((long long)n_tiles * g + grid_tc - 1) / grid_tc);
+    } else {  // equal slices of the samples (one waveform: equal cost per sample)
+        for (int g = 0; g < grid; ++g) {
+            const long double x = (long double)ns * g / grid;
+            cta[g] = CtaStart{0, (int)std::ceil(x)};
+        }
+        cta[grid] = CtaStart{1, 0};
     }
-    cta[grid] = CtaStart{1, 0};
 
     hdr->n_waves = 1;
     hdr->total_pairs = v.n_pairs;
     hdr->total_fold_blocks = S * W->fold_blocks_per_seg;
-    hdr->total_anchor_segs = fp64 ? 0 : S;
-    hdr->grid_sum = grid;
+    hdr->total_anchor_segs = fp64 || tc ? 0 : S;
+    hdr->total_segs = tc ? S : 0;
+    hdr->total_tiles = n_tiles;
+    hdr->tile_cta = reinterpret_cast<const int *>(base + off_cta);
+    hdr->recs = reinterpret_cast<TileRec *>(base + blob_bytes);
+    hdr->grid_sum = tc ? grid_tc : grid;
     hdr->buf_bytes = buf_bytes;
     hdr->stage_slots = stage_slots;
     hdr->ring = kDefaultRing;
-    hdr->variant = variant;
+    hdr->variant = tc ? kVariantTc : variant;
     hdr->waves = reinterpret_cast<const WaveDev *>(base + off_waves);
     hdr->cta = reinterpret_cast<const CtaStart *>(base + off_cta);
     hdr->err = v.d_err;
@@ -204,6 +235,15 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     }
     if (cudaGetLastError() != cudaSuccess) return FEW_ERR_CUDA;
     const PlanHdr *hd = reinterpret_cast<const PlanHdr *>(base);
+    if (tc) {
+        if (launch_ylm(hd, v.n_pairs, false, s) != cudaSuccess ||
+            launch_fold_tc(hd, S, n_tiles, s) != cudaSuccess ||
+            launch_sum_tc(hd, grid_tc, s) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return FEW_ERR_CUDA;
+        }
+        return FEW_OK;
+    }
     if (launch_ylm(hd, v.n_pairs, fp64, s) != cudaSuccess ||
         launch_fold(hd, hdr->total_fold_blocks, fp64, s) != cudaSuccess ||
         launch_anchor(hd, fp64 ? 0 : S, s) != cudaSuccess ||

@@ -1,0 +1,522 @@
+// tcsum.cu -- the mixed-precision mode sum on the tensor cores (arXiv:2104.04582 Sec. 3.C, Sec. 4).
+//
+// With K_{m,n}(u) = sum_d c_{m,n,d} u^d the folded cubic of a signed frequency (fold_slot.cuh),
+// n = n_mid + b and theta = Phi_r, the sum over n of one row m is, degree by degree,
+//     sum_n c_{m,n,d} e^{-i n theta} = e^{-i n_mid theta} [ sum_{b >= 0} X_{m,b,d} cos(b theta)
+//                                                        + Y_{m,b,d} sin(b theta) ],
+//     X = c_{+b} + c_{-b},  Y = -i (c_{+b} - c_{-b})   (b = 0: X = c_0, Y = 0):
+// a real contraction over at most 64 basis values per sample, with 8 real columns (two components,
+// four degrees) per row, whose right-hand side is the same for every sample of a segment.  That
+// is a matrix product, [samples x 64] [64 x 8 rows], and it runs on tcgen05; what is left per
+// sample is the basis (powers of z = e^{i theta}), one cubic in u per row and Horner's rule in
+// z_phi over the rows: ~600 FP32 operations instead of the ~12,800 of the scalar chain (sum.cu) on
+// the 21 x 61 grid.
+//
+// Precision: both operands are split in two fp16 parts, x = hi + lo (11 significant bits each;
+// the table after exact power-of-two scaling of the segment's largest entry into [2^14, 2^15)),
+// and the products lo.hi, hi.lo, hi.hi are accumulated in FP32 in tensor memory; the dropped
+// lo.lo is below 2^-24 of the term.  Phases are 64-bit fixed-point turns: a cubic in the sample
+// number whose coefficients (the FP64 Taylor expansion of the phase splines at the tile's first
+// sample) are in units of 2^-64 turn, so that wrap-around arithmetic is the exact reduction modulo
+// one turn and z_r^8, z_phi^2 and the final factor come from exact integer multiples of the
+// phases instead of powers of rounded exponentials.  Measured error against a 64-bit restatement
+// over the one-year 3843-mode waveform: see the table beside k_sum_tc.
+//
+// Work decomposition: tiles of 128 samples (one per tensor-memory lane) that start at multiples of
+// 128 within a segment; a persistent CTA per SM takes a contiguous run of tiles.  Two warpgroups
+// take its tiles in turn, each with its own accumulator and operand columns in tensor memory: one
+// generates its basis or drains its accumulator while the other's MMAs run.  A ninth warp keeps
+// the operand tables of this and the next segment in shared memory (bulk copies, two buffers).
+#include <cuda_fp16.h>
+
+#include "fewsum_internal.h"
+#include "fold_slot.cuh"
+#include "phase_eval.cuh"
+#include "tcgen05.cuh"
+
+namespace fewsum {
+
+namespace {
+
+constexpr int kTcThreads = 288;          // two warpgroups and the table producer's warp
+constexpr int kTcMaxN = 8 * kTcMaxRows;  // accumulator columns
+constexpr int kTcMaxKs = (kTcMaxHalf + 8) / 8;
+constexpr int kTcMaxTable = 1024 * (kTcMaxRows / 2) * kTcMaxKs;
+constexpr uint32_t kTcDStride = 192, kTcECol = 384, kTcEStride = 64, kTcELo = 32;  // tmem columns
+
+__device__ __forceinline__ float pow2(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
+
+// A value in turns as 2^-64 turn units modulo one turn.
+__device__ __forceinline__ long long turns_fixed(double y)
+{
+    return __double2ll_rn((y - rint(y)) * 18446744073709551616.0);
+}
+
+__device__ int wave_of_seg(const PlanHdr &h, int g)
+{
+    int lo = 0, hi = h.n_waves - 1;
+    while (lo < hi) {  // largest w with seg_begin <= g
+        const int mid = (lo + hi + 1) >> 1;
+        if (h.waves[mid].seg_begin <= g) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// Record of tile T: its segment, the FP64 phases at its first sample and their Taylor expansion.
+__device__ void fill_record(const PlanHdr &h, int T)
+{
+    int lo = 0, hi = h.n_waves - 1;
+    while (lo < hi) {  // largest w with tile_begin <= T
+        const int mid = (lo + hi + 1) >> 1;
+        if (h.waves[mid].tile_begin <= T) lo = mid; else hi = mid - 1;
+    }
+    const WaveDev &W = h.waves[lo];
+    const TrajDev &tr = W.tr;
+    const int t = T - W.tile_begin;
+    int s = 0, e = tr.S - 1;
+    while (s < e) {  // largest s with tile_off[s] <= t: the segment that holds tile t
+        const int mid = (s + e + 1) >> 1;
+        if (W.tile_off[mid] <= t) s = mid; else e = mid - 1;
+    }
+    TileRec r;
+    r.s0 = W.seg_start[s];
+    r.s1 = W.seg_start[s + 1];
+    r.i0 = (r.s0 / kTcTile + (t - W.tile_off[s])) * kTcTile;
+    r.tile_end = W.tile_begin + W.tile_off[s + 1];
+    const SegPhase sp = seg_phase(tr, s, W.dphi_phi, W.dphi_r);
+    const double kInv2Pi = 0.15915494309189533577;
+    const double u = (fma((double)max(r.i0, r.s0), W.dt, W.t0) - sp.tk) * sp.ih, du = W.dt * sp.ih;
+    double all = 0.0;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const double *p = k ? sp.pr : sp.pphi;
+        long long *c = k ? r.r : r.phi;
+        const double f0 = fma(fma(fma(p[2], u, p[1]), u, p[0]), u, k ? sp.c0r : sp.c0phi) * kInv2Pi;
+        c[0] = turns_fixed(f0);
+        c[1] = turns_fixed(fma(fma(3.0 * p[2], u, 2.0 * p[1]), u, p[0]) * du * kInv2Pi);
+        c[2] = turns_fixed(fma(3.0 * p[2], u, p[1]) * du * du * kInv2Pi);
+        c[3] = turns_fixed(p[2] * du * du * du * kInv2Pi);
+        all += f0;
+    }
+    // integers cannot carry a NaN: non-finite phases (latched by the build) reach the output here
+    r.u0 = (float)((fma((double)r.s0, W.dt, W.t0) - sp.tk) * sp.ih) + (float)(all - all);
+    r.du = (float)du;
+    r.inv = W.tab_inv + s;
+    r.tab = W.tab + (size_t)s * tc_table_bytes(tr.tc_pairs, tr.tc_ks);
+    r.out = W.out;
+    r.pairs = tr.tc_pairs;
+    r.ks = tr.tc_ks;
+    r.mids = (tr.n_mid & 0xffff) | (int)((unsigned)tr.m_fin << 16);
+    r.c64 = W.out_c64;
+    h.recs[T] = r;
+}
+
+// Row stride (floats) of the staged table: 16-byte aligned, and 8 consecutive rows start 4 banks
+// apart, so the packing reads of a quarter-warp do not collide.
+__host__ __device__ constexpr int staged_stride(int ks) { return 16 * ks + 4; }
+
+}  // namespace
+
+// Operand tables and tile records.  Block g < total_segs: segment g's table, one thread per (row,
+// b) forming the cubics of the slots n_mid + b and n_mid - b and their X and Y; the block then
+// scales by the power of two that brings the table's largest entry into [2^14, 2^15) and packs
+// high and low fp16 parts as the MMA reads them (K-major without swizzle: 8 x 16 B core matrices,
+// 128 B apart along K).  Column 16 p + 2 x + e of the product is row 2 p + e (signed m descending),
+// x = 4 component + degree; basis value 2 b is cos(b theta), 2 b + 1 sin(b theta).  The blocks
+// after that fill the tile records (FP64 work beside the fold's gathers).
+__global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *__restrict__ hp)
+{
+    extern __shared__ __align__(16) float tcf[];
+    __shared__ float s_max[kTcFoldThreads / 32];
+    const PlanHdr &h = *hp;
+    const int tid = threadIdx.x;
+    if ((int)blockIdx.x >= h.total_segs) {
+        const int T = ((int)blockIdx.x - h.total_segs) * kTcRecThreads + tid;
+        if (tid < kTcRecThreads && T < h.total_tiles) fill_record(h, T);
+        return;
+    }
+    const WaveDev &W = h.waves[wave_of_seg(h, blockIdx.x)];
+    const TrajDev &tr = W.tr;
+    const int s = (int)blockIdx.x - W.seg_begin;
+    if (s >= tr.S || W.tile_off[s] == W.tile_off[s + 1]) return;  // no sample in this segment
+    const int P = tr.tc_pairs, ks = tr.tc_ks, nb = 8 * ks, ld = staged_stride(ks);
+    const double *cs = tr.coef + (size_t)s * tr.J * 4;
+    const double hk = tr.h[s];
+    float mx = 0.0f;
+    for (int it = tid; it < 2 * P * nb; it += blockDim.x) {
+        const int row = it / nb, b = it - row * nb;
+        float X[8], Y[8];  // x = 4 component + degree
+#pragma unroll
+        for (int x = 0; x < 8; ++x) X[x] = Y[x] = 0.0f;
+        if (row < tr.n_rows) {
+            const int4 rs = tr.row_slot[row];  // slots n = rs.y .. rs.z
+#pragma unroll
+            for (int sign = 0; sign < 2; ++sign) {
+                const int n = sign ? tr.n_mid - b : tr.n_mid + b;
+                if ((sign && b == 0) || n > rs.y || n < rs.z) continue;
+                float pr[4], pi[4];
+                fold_slot<float>(tr, W.ylm, cs, rs.x + rs.y - n, hk, W.scale, pr, pi);
+#pragma unroll
+                for (int d = 0; d < 4; ++d) {
+                    X[d] += pr[d];
+                    X[4 + d] += pi[d];
+                    if (b > 0) {  // Y = -i (c_+ - c_-)
+                        Y[d] += sign ? -pi[d] : pi[d];
+                        Y[4 + d] += sign ? pr[d] : -pr[d];
+                    }
+                }
+            }
+        }
+        float *dst = tcf + (16 * (row >> 1) + (row & 1)) * ld + 2 * b;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+            *reinterpret_cast<float2 *>(dst + 2 * x * ld) = make_float2(X[x], Y[x]);
+            mx = fmaxf(mx, fmaxf(fabsf(X[x]), fabsf(Y[x])));
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((tid & 31) == 0) s_max[tid >> 5] = mx;
+    __syncthreads();
+    mx = 0.0f;
+    for (int w = 0; w < (int)blockDim.x / 32; ++w) mx = fmaxf(mx, s_max[w]);
+    int e = 0;
+    if (mx > 0.0f) e = 14 + 127 - (int)(__float_as_uint(mx) >> 23);
+    e = max(-126, min(126, e));
+    const float f = pow2(e);
+    if (tid == 0) W.tab_inv[s] = pow2(-e);
+    unsigned char *hi_dst = W.tab + (size_t)s * tc_table_bytes(P, ks);
+    unsigned char *lo_dst = hi_dst + tc_table_bytes(P, ks) / 2;
+    const int c8n = 2 * ks;
+    for (int id = tid; id < 16 * P * c8n; id += blockDim.x) {  // 16-byte chunks in memory order
+        const int r8 = id & 7, g = id >> 3, c8 = g % c8n, r = (g / c8n) * 8 + r8;
+        const float4 *src = reinterpret_cast<const float4 *>(tcf + r * ld + 8 * c8);
+        const float4 p = src[0], q = src[1];
+        const float v[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+        uint32_t wh[4], wl[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float x0 = v[2 * k] * f, x1 = v[2 * k + 1] * f;
+            const __half2 hi = __floats2half2_rn(x0, x1);
+            const float2 hf = __half22float2(hi);
+            const __half2 lo = __floats2half2_rn(x0 - hf.x, x1 - hf.y);
+            wh[k] = *reinterpret_cast<const uint32_t *>(&hi);
+            wl[k] = *reinterpret_cast<const uint32_t *>(&lo);
+        }
+        reinterpret_cast<uint4 *>(hi_dst)[id] = make_uint4(wh[0], wh[1], wh[2], wh[3]);
+        reinterpret_cast<uint4 *>(lo_dst)[id] = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+    }
+}
+
+namespace {
+
+// cos and sin of 2 pi f 2^-32, f a 32-bit fixed-point turn: the quadrant is split off exactly, so
+// the reduced angle |x| <= pi/4 is rounded once (2^-28 turn at most); Taylor polynomials to x^10
+// and x^9 (truncation below 2e-9).
+__device__ __forceinline__ void sincos_fixed(uint32_t f, float &s, float &c)
+{
+    const uint32_t q = f + 0x20000000u;
+    const int r = (int)(f - (q & 0xc0000000u));
+    const float x = (float)r * 1.4629180792671596e-9f;  // 2 pi 2^-32
+    const float x2 = x * x;
+    float ps = fmaf(x2, 2.7557319e-6f, -1.9841270e-4f);
+    ps = fmaf(ps, x2, 8.3333333e-3f);
+    ps = fmaf(ps, x2, -1.6666667e-1f);
+    ps = fmaf(ps * x2, x, x);
+    float pc = fmaf(x2, -2.7557319e-7f, 2.4801587e-5f);
+    pc = fmaf(pc, x2, -1.3888889e-3f);
+    pc = fmaf(pc, x2, 4.1666667e-2f);
+    pc = fmaf(pc, x2, -0.5f);
+    pc = fmaf(pc, x2, 1.0f);
+    const bool swap = (q & 0x40000000u) != 0;
+    const float a = swap ? pc : ps, b = swap ? ps : pc;
+    s = __uint_as_float(__float_as_uint(a) ^ (q & 0x80000000u));
+    c = __uint_as_float(__float_as_uint(b) ^ ((q + 0x40000000u) & 0x80000000u));
+}
+
+__device__ __forceinline__ unsigned long long horner_fixed(const long long (&c)[4], uint32_t v)
+{
+    unsigned long long a = (unsigned long long)c[3];
+    a = a * v + (unsigned long long)c[2];
+    a = a * v + (unsigned long long)c[1];
+    return a * v + (unsigned long long)c[0];
+}
+
+__device__ __forceinline__ TileRec load_record(const TileRec *p)
+{
+    TileRec r;
+    const int4 *s = reinterpret_cast<const int4 *>(p);
+    int4 *d = reinterpret_cast<int4 *>(&r);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) d[k] = __ldg(s + k);
+    return r;
+}
+
+// Barrier of one warpgroup that also tells every thread whether any of them failed.
+__device__ __forceinline__ bool wg_any(int id, bool bad)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "barrier.cta.red.or.pred q, %2, 128, p;\n\t"
+        "selp.u32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((uint32_t)bad), "r"(id)
+        : "memory");
+    return r != 0;
+}
+
+// Eight complex powers (c, s) as packed fp16 high and low parts into eight columns each.
+__device__ __forceinline__ void store_powers(uint32_t e_addr, const float (&c)[8], const float (&s)[8])
+{
+    uint32_t vh[8], vl[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const __half2 hi = __floats2half2_rn(c[k], s[k]);
+        const float2 hf = __half22float2(hi);
+        const __half2 lo = __floats2half2_rn(c[k] - hf.x, s[k] - hf.y);
+        vh[k] = *reinterpret_cast<const uint32_t *>(&hi);
+        vl[k] = *reinterpret_cast<const uint32_t *>(&lo);
+    }
+    tc_st8(e_addr, vh);
+    tc_st8(e_addr + kTcELo, vl);
+}
+
+// The basis of one sample: powers z^0 .. z^(8 ks - 1) of z = e^{i theta}, eight at a time; z and
+// z^8 from the phase itself, z^2 .. z^7 and z^(8 a) by products.
+__device__ __forceinline__ void write_basis(uint32_t e_addr, unsigned long long fr, int ks)
+{
+    float c[8], s[8];
+    c[0] = 1.0f;
+    s[0] = 0.0f;
+    sincos_fixed((uint32_t)(fr >> 32), s[1], c[1]);
+    auto mul = [](float ac, float as, float bc, float bs, float &oc, float &os) {
+        oc = fmaf(ac, bc, -as * bs);
+        os = fmaf(ac, bs, as * bc);
+    };
+    mul(c[1], s[1], c[1], s[1], c[2], s[2]);
+    mul(c[2], s[2], c[1], s[1], c[3], s[3]);
+#pragma unroll
+    for (int k = 4; k < 8; ++k) mul(c[k / 2], s[k / 2], c[k - k / 2], s[k - k / 2], c[k], s[k]);
+    store_powers(e_addr, c, s);
+    if (ks > 1) {
+        float bc, bs;
+        sincos_fixed((uint32_t)((8 * fr) >> 32), bs, bc);
+        float gc = bc, gs = bs;
+        for (int a = 1; a < ks; ++a) {
+            float pc[8], ps[8];
+            pc[0] = gc;
+            ps[0] = gs;
+#pragma unroll
+            for (int k = 1; k < 8; ++k) mul(gc, gs, c[k], s[k], pc[k], ps[k]);
+            store_powers(e_addr + 8 * a, pc, ps);
+            float nc, ns;
+            mul(gc, gs, bc, bs, nc, ns);
+            gc = nc;
+            gs = ns;
+        }
+    }
+}
+
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+}  // namespace
+
+__global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restrict__ hp)
+{
+    extern __shared__ __align__(128) unsigned char tcs[];  // two operand tables
+    __shared__ __align__(8) uint64_t b_full[2], b_empty[2], d_full[2];
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int s_abort;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const TileRec *__restrict__ recs = hp->recs;
+    const int T0 = hp->tile_cta[blockIdx.x], T1 = hp->tile_cta[blockIdx.x + 1];
+    if (T0 >= T1) return;  // uniform across the CTA: no work
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_u32(&tmem_slot)),
+                     "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&b_full[b], 1);
+            mbar_init(&b_empty[b], 2);
+            mbar_init(&d_full[b], 1);
+        }
+        fence_mbar_init();
+        s_abort = 0;
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    if (warp == 8) {
+        if ((tid & 31) == 0) {  // operand tables of the slice's segments, in order
+            int j = 0, landed = 0;
+            for (int T = T0; T < T1 && !s_abort; ++j) {
+                const TileRec *r = recs + T;
+                const uint32_t bytes = (uint32_t)tc_table_bytes(r->pairs, r->ks);
+                const unsigned char *src = r->tab;
+                const int b = j & 1;
+                if (!mbar_wait_bounded(&b_empty[b], ((j >> 1) & 1) ^ 1)) {
+                    s_abort = 1;
+                    break;
+                }
+                landed = max(landed, j - 1);  // both warpgroups have used table j - 2
+                mbar_arrive_expect_tx(&b_full[b], bytes);
+                for (uint32_t o = 0; o < bytes; o += 16384u)
+                    bulk_g2s(tcs + b * kTcMaxTable + o, src + o, min(16384u, bytes - o), &b_full[b]);
+                T = r->tile_end;
+            }
+            // no copy may land after the CTA's shared memory is gone
+            for (; landed < j; ++landed) mbar_wait_bounded(&b_full[landed & 1], (landed >> 1) & 1);
+        }
+        __syncwarp();
+    } else {
+        const int g = warp >> 2, lane = tid & 127;
+        const bool lead = lane == 0;
+        const uint32_t quarter = (uint32_t)(32 * (warp & 3)) << 16;
+        const uint32_t d_col = tmem + (uint32_t)g * kTcDStride;
+        const uint32_t e_col = tmem + kTcECol + (uint32_t)g * kTcEStride;
+        int j = 0, tend = recs[T0].tile_end;  // table of the current tile, and where it ends
+        uint32_t phase = 0;
+        bool bad = false;
+        TileRec r;
+        if (T0 + g < T1) r = load_record(recs + T0 + g);
+        for (int T = T0 + g; T < T1; T += 2) {
+            while (T >= tend) {  // this warpgroup's MMAs on table j have completed
+                if (lead) mbar_arrive(&b_empty[j & 1]);
+                ++j;
+                tend = __ldg(&recs[tend].tile_end);
+            }
+            __syncwarp();
+            const int i = r.i0 + lane;
+            const uint32_t v = (uint32_t)max(i - max(r.i0, r.s0), 0);
+            const unsigned long long fr = horner_fixed(r.r, v), fphi = horner_fixed(r.phi, v);
+            write_basis(e_col + quarter, fr, r.ks);
+            tc_wait_st();
+            tc_fence_before();
+            bad = wg_any(1 + g, bad);
+            if (bad) break;
+            if (lead) {
+                tc_fence_after();
+                if (mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1)) {
+                    const uint32_t b_hi = smem_u32(tcs + (j & 1) * kTcMaxTable);
+                    const uint32_t b_lo = b_hi + (uint32_t)tc_table_bytes(r.pairs, r.ks) / 2;
+                    const uint32_t idesc = (1u << 4) | ((uint32_t)(2 * r.pairs) << 17) |
+                                           ((uint32_t)(kTcTile >> 4) << 24);
+                    const uint32_t sbo = 256u * (uint32_t)r.ks;
+                    for (int a = 0; a < r.ks; ++a) {  // the small products first
+                        tc_mma_ta(d_col, e_col + kTcELo + 8 * a, smem_desc(b_hi + 256 * a, 128, sbo),
+                                  idesc, a != 0);
+                        tc_mma_ta(d_col, e_col + 8 * a, smem_desc(b_lo + 256 * a, 128, sbo), idesc, 1);
+                    }
+                    for (int a = 0; a < r.ks; ++a)
+                        tc_mma_ta(d_col, e_col + 8 * a, smem_desc(b_hi + 256 * a, 128, sbo), idesc, 1);
+                    tc_commit(&d_full[g]);
+                } else {
+                    s_abort = 1;
+                }
+            }
+            // while the MMAs run: this sample's factors, and the next tile's record
+            const TileRec cur = r;
+            if (T + 2 < T1) r = load_record(recs + T + 2);
+            const float u = fmaf((float)(i - cur.s0), cur.du, cur.u0);
+            const float inv = __ldg(cur.inv);
+            const long long nmid = (short)(cur.mids & 0xffff), mfin = (short)(cur.mids >> 16);
+            float zs, zc, ws, wc, gs, gc;
+            sincos_fixed((uint32_t)(fphi >> 32), zs, zc);
+            sincos_fixed((uint32_t)((2 * fphi) >> 32), ws, wc);
+            sincos_fixed((uint32_t)(((unsigned long long)mfin * fphi + (unsigned long long)nmid * fr) >> 32),
+                         gs, gc);
+            const float2 U = make_float2(u, u), U2 = make_float2(u * u, u * u);
+            const float2 WR = make_float2(wc, wc), WI = make_float2(-ws, -ws), NWI = make_float2(ws, ws);
+            float2 tr = make_float2(0.0f, 0.0f), ti = tr;  // rows 2 p and 2 p + 1: two chains in z_phi^2
+            if (!mbar_wait_bounded(&d_full[g], phase)) {
+                s_abort = 1;
+                bad = true;
+            }
+            phase ^= 1u;
+            tc_fence_after();
+            __syncwarp();
+            auto row_pair = [&](const float(&d)[16]) {
+                const float2 *c = reinterpret_cast<const float2 *>(d);
+                const float2 kr = fma2(fma2(c[3], U, c[2]), U2, fma2(c[1], U, c[0]));
+                const float2 ki = fma2(fma2(c[7], U, c[6]), U2, fma2(c[5], U, c[4]));
+                const float2 nr = fma2(ti, NWI, fma2(tr, WR, kr));
+                const float2 ni = fma2(ti, WR, fma2(tr, WI, ki));
+                tr = nr;
+                ti = ni;
+            };
+            const uint32_t d_lane = d_col + quarter;
+            float da[16], db[16];
+            tc_ld16(d_lane, da);
+            tc_wait_ld16(da);
+            for (int p = 0; p < cur.pairs; p += 2) {
+                const bool two = p + 1 < cur.pairs;
+                if (two) tc_ld16(d_lane + 16 * (p + 1), db);
+                row_pair(da);
+                if (!two) break;
+                tc_wait_ld16(db);
+                const bool more = p + 2 < cur.pairs;
+                if (more) tc_ld16(d_lane + 16 * (p + 2), da);
+                row_pair(db);
+                if (more) tc_wait_ld16(da);
+            }
+            tc_fence_before();
+            if (i >= cur.s0 && i < cur.s1) {
+                // h = (T_0 z_phi + T_1) z_phi^{m_fin} z_r^{n_mid}, z_phi = e^{-i Phi_phi}
+                const float hr = fmaf(tr.x, zc, fmaf(ti.x, zs, tr.y));
+                const float hi = fmaf(ti.x, zc, fmaf(-tr.x, zs, ti.y));
+                const float fc = gc * inv, fs = gs * inv;
+                const float yr = fmaf(hr, fc, hi * fs), yi = fmaf(hi, fc, -hr * fs);
+                if (cur.c64)
+                    reinterpret_cast<float2 *>(cur.out)[i] = make_float2(yr, yi);
+                else
+                    reinterpret_cast<double2 *>(cur.out)[i] = make_double2((double)yr, (double)yi);
+            }
+        }
+        if (lead) {  // tables that only the other warpgroup still needs
+            while (tend < T1) {
+                mbar_arrive(&b_empty[j & 1]);
+                ++j;
+                tend = recs[tend].tile_end;
+            }
+            if (bad) atomicOr(hp->err, ERRBIT_TIMEOUT);
+        }
+    }
+    __syncthreads();
+    if (tid == 0 && s_abort) atomicOr(hp->err, ERRBIT_TIMEOUT);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 8)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+}
+
+cudaError_t tc_configure()
+{
+    return cudaFuncSetAttribute(k_sum_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kTcMaxTable);
+}
+
+cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st)
+{
+    if (total_tiles <= 0) return cudaSuccess;
+    const int smem = kTcMaxN * staged_stride(kTcMaxKs) * (int)sizeof(float);
+    const int grid = total_segs + (total_tiles + kTcRecThreads - 1) / kTcRecThreads;
+    k_fold_tc<<<grid, kTcFoldThreads, smem, st>>>(hdr_dev);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sum_tc(const PlanHdr *hdr_dev, int grid, cudaStream_t st)
+{
+    if (grid <= 0) return cudaSuccess;
+    k_sum_tc<<<grid, kTcThreads, 2 * kTcMaxTable, st>>>(hdr_dev);
+    return cudaGetLastError();
+}
+
+}  // namespace fewsum

@@ -1,0 +1,149 @@
+"""Edges of the tensor-core summation (tcsum.cu): tile and segment remainders, row and basis
+limits on both sides of its dispatch, batches and budgets that mix it with the scalar chain.
+
+Tolerance: the basis and table splits (2^-24 and 2^-23 of a term), the reduced phases (2^-28 turn,
+a chain of at most four products), up to 12 accumulation steps (2^-23 each if truncated) and the
+11-step chain in z_phi^2 add up to at most 4e-6 of the terms of a sample.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2104_04582_gb300 import fewsum as F
+from paper_2104_04582_gb300 import runtime as RT
+from paper_2104_04582_gb300 import workloads as W
+from tests.gpu_common import MIXED_MISMATCH, oracle_threads, rel_l2, to_host
+
+pytestmark = pytest.mark.gpu
+REL = 4e-6
+
+
+def _modes(ms, ns, l=None):
+    return np.asarray([(l or max(2, m), m, n) for m in ms for n in ns], dtype=np.int32)
+
+
+SETS = {
+    "one_m0_mode": _modes([0], [3]),
+    "one_m2_mode": _modes([2], [-1]),
+    "n_range_15": _modes([0, 2], range(-7, 8)),            # one K step full
+    "n_range_17": _modes([0, 2], range(-8, 9)),            # one value into the second
+    "n_range_63": _modes([0, 1], range(-31, 32)),          # the whole basis
+    "n_range_64": _modes([0], range(-32, 32)),             # an even range: half-width 32, scalar
+    "n_shifted": _modes([0], range(40, 90)),               # m = 0 only: a centre far from zero
+    "rows_21": _modes(range(11), [-2, 0, 5], l=10),
+    "rows_22_empty": _modes([0, 10], [-30, 30], l=10),     # empty rows in between
+    "rows_23": _modes(range(12), [0, 1], l=11),            # too many rows: scalar
+}
+
+
+# just past the limits: these stay on the scalar chain, whose contract is the mixed path's gate
+PAST = ("n_range_64", "rows_23")
+
+
+@pytest.mark.parametrize("name", PAST)
+def test_mode_sets_past_the_limits(gpu_ctx, name):
+    import torch
+    w = W.make_inputs(4.0e5, 9, 100.0, SETS[name], 5, 4.0, 60.0)
+    tr = RT.from_inputs(gpu_ctx, w)
+    h = RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_MIXED)
+    torch.cuda.synchronize()
+    assert gpu_ctx.sync_status() == F.FEW_OK
+    o = oracle.waveform_inputs(w, nthreads=oracle_threads())
+    assert oracle.mismatch(to_host(h), o) <= MIXED_MISMATCH
+    tr.release()
+
+
+@pytest.mark.parametrize("name", [s for s in SETS if s not in PAST])
+@pytest.mark.parametrize("n_samples", [1, 128, 4001])
+def test_mode_set_edges(gpu_ctx, name, n_samples):
+    import torch
+    w = W.make_inputs(4.0e5, 9, 4.0e5 / max(n_samples, 200), SETS[name], 5, 4.0, 60.0,
+                      n_samples=n_samples)
+    tr = RT.from_inputs(gpu_ctx, w)
+    h = RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_MIXED)
+    torch.cuda.synchronize()
+    assert gpu_ctx.sync_status() == F.FEW_OK
+    assert rel_l2(to_host(h), oracle.waveform_inputs(w, nthreads=oracle_threads())) <= REL
+    tr.release()
+
+
+@pytest.mark.parametrize("K,n_samples,i0,count", [
+    (4, 127, 0, 127), (4, 129, 0, 129), (5, 1000, 1, 998), (300, 400, 0, 400),
+    (300, 5000, 77, 4097), (40, 152 * 128 + 1, 0, 152 * 128 + 1)])
+def test_sample_and_segment_edges(gpu_ctx, K, n_samples, i0, count):
+    """Segments shorter than a tile, empty segments, windows that start inside one, a run of tiles
+    that leaves CTAs with one tile and with two."""
+    import torch
+    w = W.make_inputs(3.0e5, K, 3.0e5 / n_samples, W.mode_grid(4, 9), 11, 3.0, 20.0,
+                      n_samples=n_samples)
+    tr = RT.from_inputs(gpu_ctx, w)
+    out = torch.full((count + 2,), complex(7.0, 7.0), dtype=torch.complex64, device="cuda")
+    h = RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_MIXED, i_begin=i0, count=count, out=out[1:-1])
+    torch.cuda.synchronize()
+    assert gpu_ctx.sync_status() == F.FEW_OK
+    g = to_host(out)
+    assert g[0] == g[-1] == complex(7.0, 7.0)
+    o = oracle.waveform_inputs(w, i0, count, nthreads=oracle_threads())
+    assert rel_l2(g[1:-1], o) <= REL
+    tr.release()
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-22, 1e25])
+def test_amplitude_range(gpu_ctx, scale):
+    """The table's power-of-two scaling: amplitudes far from one keep their relative accuracy."""
+    import torch
+    w = W.make_inputs(3.0e5, 12, 100.0, W.mode_grid(4, 9), 3, 3.0, 20.0)
+    tr = RT.from_inputs(gpu_ctx, w)
+    h = RT.waveform(gpu_ctx, tr, w.n_samples, w.t0, w.dt, w.theta, w.phi, F.FEW_MIXED, False, scale)
+    torch.cuda.synchronize()
+    o = oracle.waveform_inputs(w, nthreads=oracle_threads(), scale=scale)
+    assert rel_l2(to_host(h) / scale, o / scale) <= REL
+    tr.release()
+
+
+def test_batch_of_both_variants(gpu_ctx):
+    """A batch whose mode sets need both summation variants: each waveform as computed alone."""
+    import torch
+    sets = ["n_range_63", "rows_23", "n_range_15", "n_range_64"]
+    ws = [W.make_inputs(2.0e5, 7, 50.0, SETS[s], k, 4.0, 60.0) for k, s in enumerate(sets)]
+    trs = [RT.from_inputs(gpu_ctx, w) for w in ws]
+    outs = [RT.alloc_out(w.n_samples, True) for w in ws]
+    reqs = [RT.request(tr, o, w.n_samples, w.t0, w.dt, w.theta, w.phi, F.FEW_MIXED, w.scale)
+            for tr, o, w in zip(trs, outs, ws)]
+    for flags in (0, F.FEW_BATCH_NO_GRAPH):
+        b = F.few_batch_plan(gpu_ctx.handle, reqs, flags)
+        F.few_batch_run(gpu_ctx.handle, b, RT.current_stream())
+        torch.cuda.synchronize()
+        assert gpu_ctx.sync_status() == F.FEW_OK
+        for w, tr, o in zip(ws, trs, outs):
+            np.testing.assert_array_equal(to_host(o), to_host(RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_MIXED)))
+            o.zero_()
+        F.few_batch_release(gpu_ctx.handle, b)
+    for tr in trs:
+        tr.release()
+
+
+def test_budget_that_only_the_scalar_plan_fits():
+    """Two modes on 4096 knots: the operand tables (rows x basis) are far larger than the scalar
+    plan's two slots a segment; under a budget between the two the request still runs."""
+    import torch
+    w = W.make_inputs(3.0e6, 4096, 300.0, _modes([2], [-31, 31]), 3)
+    with RT.Context(0) as free:
+        tr = RT.from_inputs(free, w)
+        ref = to_host(RT.waveform_inputs(free, tr, w, F.FEW_MIXED))
+        held = free.memory()[0]
+        tr.release()
+    for extra, runs in ((16 << 20, True), (200 << 20, True), (1 << 10, False)):
+        with RT.Context(0, held + extra) as ctx:
+            tr = RT.from_inputs(ctx, w)
+            if not runs:
+                with pytest.raises(F.FewError) as e:
+                    RT.waveform_inputs(ctx, tr, w, F.FEW_MIXED)
+                assert e.value.status == F.FEW_ERR_BUDGET
+            else:
+                h = RT.waveform_inputs(ctx, tr, w, F.FEW_MIXED)
+                torch.cuda.synchronize()
+                assert ctx.sync_status() == F.FEW_OK
+                # under the small budget the scalar chain ran: the mixed path's gate
+                assert oracle.mismatch(to_host(h), ref) <= MIXED_MISMATCH
+            tr.release()
