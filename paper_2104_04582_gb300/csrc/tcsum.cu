@@ -38,7 +38,8 @@ namespace fewsum {
 
 namespace {
 
-constexpr int kTcThreads = 288;          // two warpgroups and the table producer's warp
+constexpr int kTcGroups = 4;                        // warpgroups
+constexpr int kTcThreads = 128 * kTcGroups + 32;    // and the table producer's warp
 constexpr int kTcMaxN = 8 * kTcMaxRows;  // accumulator columns
 constexpr int kTcMaxKs = (kTcMaxHalf + 8) / 8;
 constexpr int kTcMaxTable = 1024 * (kTcMaxRows / 2) * kTcMaxKs;
@@ -210,46 +211,43 @@ __global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *__res
 
 namespace {
 
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
+
 // cos and sin of 2 pi f 2^-32, f a 32-bit fixed-point turn: the quadrant is split off exactly, so
-// the reduced angle |x| <= pi/4 is rounded once (2^-28 turn at most); Taylor polynomials to x^10
-// and x^9 (truncation below 2e-9).
+// the rest, |t| <= 1/8 turn, is rounded once (2^-28 turn at most); Taylor polynomials in t to t^10
+// and t^9 (truncation below 2e-9), the linear coefficient 2 pi in two parts.
 __device__ __forceinline__ void sincos_fixed(uint32_t f, float &s, float &c)
 {
     const uint32_t q = f + 0x20000000u;
-    const int r = (int)(f - (q & 0xc0000000u));
-    const float x = (float)r * 1.4629180792671596e-9f;  // 2 pi 2^-32
-    const float x2 = x * x;
-    float ps = fmaf(x2, 2.7557319e-6f, -1.9841270e-4f);
-    ps = fmaf(ps, x2, 8.3333333e-3f);
-    ps = fmaf(ps, x2, -1.6666667e-1f);
-    ps = fmaf(ps * x2, x, x);
-    float pc = fmaf(x2, -2.7557319e-7f, 2.4801587e-5f);
-    pc = fmaf(pc, x2, -1.3888889e-3f);
-    pc = fmaf(pc, x2, 4.1666667e-2f);
-    pc = fmaf(pc, x2, -0.5f);
-    pc = fmaf(pc, x2, 1.0f);
+    const float t = (float)(int)(f - (q & 0xc0000000u)) * 2.3283064365386963e-10f;  // 2^-32
+    const float t2 = t * t;
+    float ps = fmaf(t2, 42.058693f, -76.70586f);
+    ps = fmaf(ps, t2, 81.60525f);
+    ps = fmaf(ps, t2, -41.3417f);
+    ps = fmaf(ps, t2, -1.7484556e-7f);
+    ps = fmaf(t, 6.2831855f, ps * t);
+    float pc = fmaf(t2, -26.426256f, 60.24464f);
+    pc = fmaf(pc, t2, -85.45682f);
+    pc = fmaf(pc, t2, 64.93939f);
+    pc = fmaf(pc, t2, -19.739208f);
+    pc = fmaf(pc, t2, 1.0f);
     const bool swap = (q & 0x40000000u) != 0;
     const float a = swap ? pc : ps, b = swap ? ps : pc;
     s = __uint_as_float(__float_as_uint(a) ^ (q & 0x80000000u));
     c = __uint_as_float(__float_as_uint(b) ^ ((q + 0x40000000u) & 0x80000000u));
 }
 
-__device__ __forceinline__ unsigned long long horner_fixed(const long long (&c)[4], uint32_t v)
+// c0 + c1 v + c2 v^2 + c3 v^3 in 64-bit wrap-around arithmetic (modulo one turn).
+__device__ __forceinline__ unsigned long long phase_fixed(const long long *c, uint32_t v)
 {
-    unsigned long long a = (unsigned long long)c[3];
-    a = a * v + (unsigned long long)c[2];
-    a = a * v + (unsigned long long)c[1];
-    return a * v + (unsigned long long)c[0];
-}
-
-__device__ __forceinline__ TileRec load_record(const TileRec *p)
-{
-    TileRec r;
-    const int4 *s = reinterpret_cast<const int4 *>(p);
-    int4 *d = reinterpret_cast<int4 *>(&r);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) d[k] = __ldg(s + k);
-    return r;
+    const longlong2 a = __ldg(reinterpret_cast<const longlong2 *>(c));
+    const longlong2 b = __ldg(reinterpret_cast<const longlong2 *>(c) + 1);
+    unsigned long long p = (unsigned long long)b.y;
+    p = p * v + (unsigned long long)b.x;
+    p = p * v + (unsigned long long)a.y;
+    return p * v + (unsigned long long)a.x;
 }
 
 // Barrier of one warpgroup that also tells every thread whether any of them failed.
@@ -267,73 +265,67 @@ __device__ __forceinline__ bool wg_any(int id, bool bad)
     return r != 0;
 }
 
-// Eight complex powers (c, s) as packed fp16 high and low parts into eight columns each.
-__device__ __forceinline__ void store_powers(uint32_t e_addr, const float (&c)[8], const float (&s)[8])
+// Eight powers (cos, sin), two to a float2, as packed fp16 high and low parts into eight columns
+// each: column k holds (cos, sin) of power k.
+__device__ __forceinline__ void store_powers(uint32_t e_addr, const float2 (&c)[4], const float2 (&s)[4])
 {
     uint32_t vh[8], vl[8];
+    const float2 neg = both(-1.0f);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const __half2 hi = __floats2half2_rn(c[k], s[k]);
-        const float2 hf = __half22float2(hi);
-        const __half2 lo = __floats2half2_rn(c[k] - hf.x, s[k] - hf.y);
-        vh[k] = *reinterpret_cast<const uint32_t *>(&hi);
-        vl[k] = *reinterpret_cast<const uint32_t *>(&lo);
+    for (int k = 0; k < 4; ++k) {
+        const __half2 h0 = __floats2half2_rn(c[k].x, s[k].x), h1 = __floats2half2_rn(c[k].y, s[k].y);
+        const float2 f0 = __half22float2(h0), f1 = __half22float2(h1);
+        const float2 lc = fma2(make_float2(f0.x, f1.x), neg, c[k]);
+        const float2 ls = fma2(make_float2(f0.y, f1.y), neg, s[k]);
+        const __half2 l0 = __floats2half2_rn(lc.x, ls.x), l1 = __floats2half2_rn(lc.y, ls.y);
+        vh[2 * k] = *reinterpret_cast<const uint32_t *>(&h0);
+        vh[2 * k + 1] = *reinterpret_cast<const uint32_t *>(&h1);
+        vl[2 * k] = *reinterpret_cast<const uint32_t *>(&l0);
+        vl[2 * k + 1] = *reinterpret_cast<const uint32_t *>(&l1);
     }
     tc_st8(e_addr, vh);
     tc_st8(e_addr + kTcELo, vl);
 }
 
-// The basis of one sample: powers z^0 .. z^(8 ks - 1) of z = e^{i theta}, eight at a time; z and
-// z^8 from the phase itself, z^2 .. z^7 and z^(8 a) by products.
-__device__ __forceinline__ void write_basis(uint32_t e_addr, unsigned long long fr, int ks)
+// (c, s) <- (ac, as) (bc, bs), two complex products at once.
+__device__ __forceinline__ void cmul2(float2 ac, float2 as, float2 bc, float2 bs, float2 &c, float2 &s)
 {
-    float c[8], s[8];
-    c[0] = 1.0f;
-    s[0] = 0.0f;
-    sincos_fixed((uint32_t)(fr >> 32), s[1], c[1]);
-    auto mul = [](float ac, float as, float bc, float bs, float &oc, float &os) {
-        oc = fmaf(ac, bc, -as * bs);
-        os = fmaf(ac, bs, as * bc);
-    };
-    mul(c[1], s[1], c[1], s[1], c[2], s[2]);
-    mul(c[2], s[2], c[1], s[1], c[3], s[3]);
-#pragma unroll
-    for (int k = 4; k < 8; ++k) mul(c[k / 2], s[k / 2], c[k - k / 2], s[k - k / 2], c[k], s[k]);
-    store_powers(e_addr, c, s);
-    if (ks > 1) {
-        float bc, bs;
-        sincos_fixed((uint32_t)((8 * fr) >> 32), bs, bc);
-        float gc = bc, gs = bs;
-        for (int a = 1; a < ks; ++a) {
-            float pc[8], ps[8];
-            pc[0] = gc;
-            ps[0] = gs;
-#pragma unroll
-            for (int k = 1; k < 8; ++k) mul(gc, gs, c[k], s[k], pc[k], ps[k]);
-            store_powers(e_addr + 8 * a, pc, ps);
-            float nc, ns;
-            mul(gc, gs, bc, bs, nc, ns);
-            gc = nc;
-            gs = ns;
-        }
-    }
+    const float2 nas = make_float2(-as.x, -as.y);
+    c = fma2(ac, bc, mul2(nas, bs));
+    s = fma2(ac, bs, mul2(as, bc));
 }
 
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// Powers 0 .. 7 of z = e^{2 pi i f}, f the top 32 bits of a fixed-point phase.
+__device__ __forceinline__ void first_powers(unsigned long long f, float2 (&c)[4], float2 (&s)[4])
+{
+    float s1, c1;
+    sincos_fixed((uint32_t)(f >> 32), s1, c1);
+    const float c2 = fmaf(c1, c1, -s1 * s1), s2 = 2.0f * (c1 * s1);
+    c[0] = make_float2(1.0f, c1);
+    s[0] = make_float2(0.0f, s1);
+    cmul2(c[0], s[0], both(c2), both(s2), c[1], s[1]);              // 2, 3
+    const float c4 = fmaf(c2, c2, -s2 * s2), s4 = 2.0f * (c2 * s2);
+    cmul2(c[0], s[0], both(c4), both(s4), c[2], s[2]);              // 4, 5
+    cmul2(c[1], s[1], both(c4), both(s4), c[3], s[3]);              // 6, 7
+}
 
 }  // namespace
 
+// Warpgroup k takes every fourth tile of the CTA's run, on slot k & 1 of tensor memory (operand and
+// accumulator columns).  A tile's operand columns are free when the slot's previous MMAs have
+// completed, its accumulator when the slot's previous tile has been drained, so a warpgroup
+// forms its basis while the slot's other warpgroup waits for its MMAs or drains them.
 __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restrict__ hp)
 {
     extern __shared__ __align__(128) unsigned char tcs[];  // two operand tables
-    __shared__ __align__(8) uint64_t b_full[2], b_empty[2], d_full[2];
+    __shared__ __align__(8) uint64_t b_full[2], b_empty[2], d_full[2], d_free[2];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
     const int tid = threadIdx.x, warp = tid >> 5;
     const TileRec *__restrict__ recs = hp->recs;
     const int T0 = hp->tile_cta[blockIdx.x], T1 = hp->tile_cta[blockIdx.x + 1];
     if (T0 >= T1) return;  // uniform across the CTA: no work
-    if (warp == 8) {
+    if (warp == 4 * kTcGroups) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&tmem_slot)),
                      "r"(512u)
@@ -343,8 +335,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
     if (tid == 0) {
         for (int b = 0; b < 2; ++b) {
             mbar_init(&b_full[b], 1);
-            mbar_init(&b_empty[b], 2);
+            mbar_init(&b_empty[b], kTcGroups);
             mbar_init(&d_full[b], 1);
+            mbar_init(&d_free[b], 4);
         }
         fence_mbar_init();
         s_abort = 0;
@@ -354,8 +347,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    if (warp == 8) {
-        if ((tid & 31) == 0) {  // operand tables of the slice's segments, in order
+    if (warp == 4 * kTcGroups) {
+        if ((tid & 31) == 0) {  // operand tables of the run's segments, in order
             int j = 0, landed = 0;
             for (int T = T0; T < T1 && !s_abort; ++j) {
                 const TileRec *r = recs + T;
@@ -366,7 +359,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
                     s_abort = 1;
                     break;
                 }
-                landed = max(landed, j - 1);  // both warpgroups have used table j - 2
+                landed = max(landed, j - 1);  // every warpgroup is past table j - 2
                 mbar_arrive_expect_tx(&b_full[b], bytes);
                 for (uint32_t o = 0; o < bytes; o += 16384u)
                     bulk_g2s(tcs + b * kTcMaxTable + o, src + o, min(16384u, bytes - o), &b_full[b]);
@@ -377,76 +370,108 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
         }
         __syncwarp();
     } else {
-        const int g = warp >> 2, lane = tid & 127;
+        const int group = warp >> 2, slot = group & 1, lane = tid & 127;
         const bool lead = lane == 0;
         const uint32_t quarter = (uint32_t)(32 * (warp & 3)) << 16;
-        const uint32_t d_col = tmem + (uint32_t)g * kTcDStride;
-        const uint32_t e_col = tmem + kTcECol + (uint32_t)g * kTcEStride;
-        int j = 0, tend = recs[T0].tile_end;  // table of the current tile, and where it ends
-        uint32_t phase = 0;
+        const uint32_t d_col = tmem + (uint32_t)slot * kTcDStride;
+        const uint32_t e_col = tmem + kTcECol + (uint32_t)slot * kTcEStride;
+        int j = 0, tend = __ldg(&recs[T0].tile_end);  // table of the current tile, and where it ends
         bool bad = false;
-        TileRec r;
-        if (T0 + g < T1) r = load_record(recs + T0 + g);
-        for (int T = T0 + g; T < T1; T += 2) {
-            while (T >= tend) {  // this warpgroup's MMAs on table j have completed
-                if (lead) mbar_arrive(&b_empty[j & 1]);
+        for (int T = T0 + group; T < T1; T += kTcGroups) {
+            // tables before this tile's: this warpgroup's MMAs on them have completed.  A table
+            // is released only once it has landed (also one that this warpgroup had no tile in):
+            // its buffer's previous table has then been released by every warpgroup, so an arrival
+            // or a parity wait cannot be taken for the previous table's.
+            while (T >= tend) {
+                if (lead && !bad) {
+                    if (mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1)) mbar_arrive(&b_empty[j & 1]);
+                    else bad = true;
+                }
                 ++j;
                 tend = __ldg(&recs[tend].tile_end);
             }
+            const TileRec *rp = recs + T;
+            const uint32_t use = (uint32_t)(T - T0) >> 1;  // of the slot
+            const int4 span = __ldg(reinterpret_cast<const int4 *>(&rp->i0));  // i0, s0, s1
+            const int i = span.x + lane;
+            const uint32_t v = (uint32_t)max(i - max(span.x, span.y), 0);
+            const unsigned long long fr = phase_fixed(rp->r, v), fphi = phase_fixed(rp->phi, v);
+            const int pairs = __ldg(&rp->pairs), ks = __ldg(&rp->ks);
+            // the basis: powers 0 .. 8 ks - 1, eight at a time, z and z^8 from the phase itself
+            float2 c[4], s[4];
+            first_powers(fr, c, s);
+            float gs = 0.0f, gc = 0.0f, bs = 0.0f, bc = 0.0f;
+            if (ks > 1) {
+                sincos_fixed((uint32_t)((8 * fr) >> 32), bs, bc);
+                gs = bs;
+                gc = bc;
+            }
+            if (use > 0 && !mbar_wait_bounded(&d_full[slot], (use - 1) & 1)) bad = true;
             __syncwarp();
-            const int i = r.i0 + lane;
-            const uint32_t v = (uint32_t)max(i - max(r.i0, r.s0), 0);
-            const unsigned long long fr = horner_fixed(r.r, v), fphi = horner_fixed(r.phi, v);
-            write_basis(e_col + quarter, fr, r.ks);
+            tc_fence_after();
+            store_powers(e_col + quarter, c, s);
+            for (int a = 1; a < ks; ++a) {
+                float2 pc[4], ps[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) cmul2(both(gc), both(gs), c[k], s[k], pc[k], ps[k]);
+                store_powers(e_col + quarter + 8 * a, pc, ps);
+                const float nc = fmaf(gc, bc, -gs * bs);
+                gs = fmaf(gc, bs, gs * bc);
+                gc = nc;
+            }
             tc_wait_st();
             tc_fence_before();
-            bad = wg_any(1 + g, bad);
+            bad = wg_any(1 + group, bad);
             if (bad) break;
             if (lead) {
                 tc_fence_after();
-                if (mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1)) {
+                if ((use == 0 || mbar_wait_bounded(&d_free[slot], (use - 1) & 1)) &&
+                    mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1)) {
+                    tc_fence_after();
                     const uint32_t b_hi = smem_u32(tcs + (j & 1) * kTcMaxTable);
-                    const uint32_t b_lo = b_hi + (uint32_t)tc_table_bytes(r.pairs, r.ks) / 2;
-                    const uint32_t idesc = (1u << 4) | ((uint32_t)(2 * r.pairs) << 17) |
+                    const uint32_t b_lo = b_hi + (uint32_t)tc_table_bytes(pairs, ks) / 2;
+                    const uint32_t idesc = (1u << 4) | ((uint32_t)(2 * pairs) << 17) |
                                            ((uint32_t)(kTcTile >> 4) << 24);
-                    const uint32_t sbo = 256u * (uint32_t)r.ks;
-                    for (int a = 0; a < r.ks; ++a) {  // the small products first
+                    const uint32_t sbo = 256u * (uint32_t)ks;
+                    for (int a = 0; a < ks; ++a) {  // the small products first
                         tc_mma_ta(d_col, e_col + kTcELo + 8 * a, smem_desc(b_hi + 256 * a, 128, sbo),
                                   idesc, a != 0);
                         tc_mma_ta(d_col, e_col + 8 * a, smem_desc(b_lo + 256 * a, 128, sbo), idesc, 1);
                     }
-                    for (int a = 0; a < r.ks; ++a)
+                    for (int a = 0; a < ks; ++a)
                         tc_mma_ta(d_col, e_col + 8 * a, smem_desc(b_hi + 256 * a, 128, sbo), idesc, 1);
-                    tc_commit(&d_full[g]);
+                    tc_commit(&d_full[slot]);
                 } else {
                     s_abort = 1;
                 }
             }
-            // while the MMAs run: this sample's factors, and the next tile's record
-            const TileRec cur = r;
-            if (T + 2 < T1) r = load_record(recs + T + 2);
-            const float u = fmaf((float)(i - cur.s0), cur.du, cur.u0);
-            const float inv = __ldg(cur.inv);
-            const long long nmid = (short)(cur.mids & 0xffff), mfin = (short)(cur.mids >> 16);
-            float zs, zc, ws, wc, gs, gc;
+            // while the MMAs run: this sample's factors
+            const float2 uu = __ldg(reinterpret_cast<const float2 *>(&rp->u0));
+            const float inv = __ldg(rp->inv);
+            const int mids = __ldg(&rp->mids), c64 = __ldg(&rp->c64);
+            void *out = reinterpret_cast<void *>(__ldg(reinterpret_cast<const unsigned long long *>(&rp->out)));
+            if (T + kTcGroups < T1)  // the next tile's record on its way to L1
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(rp + kTcGroups));
+            const float u = fmaf((float)(i - span.y), uu.y, uu.x);
+            const long long nmid = (short)(mids & 0xffff), mfin = (short)(mids >> 16);
+            float zs, zc, ws, wc, fs, fc;
             sincos_fixed((uint32_t)(fphi >> 32), zs, zc);
             sincos_fixed((uint32_t)((2 * fphi) >> 32), ws, wc);
             sincos_fixed((uint32_t)(((unsigned long long)mfin * fphi + (unsigned long long)nmid * fr) >> 32),
-                         gs, gc);
-            const float2 U = make_float2(u, u), U2 = make_float2(u * u, u * u);
-            const float2 WR = make_float2(wc, wc), WI = make_float2(-ws, -ws), NWI = make_float2(ws, ws);
-            float2 tr = make_float2(0.0f, 0.0f), ti = tr;  // rows 2 p and 2 p + 1: two chains in z_phi^2
-            if (!mbar_wait_bounded(&d_full[g], phase)) {
+                         fs, fc);
+            const float2 U = both(u), U2 = both(u * u);
+            const float2 WR = both(wc), WI = both(-ws), NWI = both(ws);
+            float2 tr = both(0.0f), ti = tr;  // rows 2 p and 2 p + 1: two chains in z_phi^2
+            if (!mbar_wait_bounded(&d_full[slot], use & 1)) {
                 s_abort = 1;
                 bad = true;
             }
-            phase ^= 1u;
-            tc_fence_after();
             __syncwarp();
+            tc_fence_after();
             auto row_pair = [&](const float(&d)[16]) {
-                const float2 *c = reinterpret_cast<const float2 *>(d);
-                const float2 kr = fma2(fma2(c[3], U, c[2]), U2, fma2(c[1], U, c[0]));
-                const float2 ki = fma2(fma2(c[7], U, c[6]), U2, fma2(c[5], U, c[4]));
+                const float2 *k = reinterpret_cast<const float2 *>(d);
+                const float2 kr = fma2(fma2(k[3], U, k[2]), U2, fma2(k[1], U, k[0]));
+                const float2 ki = fma2(fma2(k[7], U, k[6]), U2, fma2(k[5], U, k[4]));
                 const float2 nr = fma2(ti, NWI, fma2(tr, WR, kr));
                 const float2 ni = fma2(ti, WR, fma2(tr, WI, ki));
                 tr = nr;
@@ -456,37 +481,41 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
             float da[16], db[16];
             tc_ld16(d_lane, da);
             tc_wait_ld16(da);
-            for (int p = 0; p < cur.pairs; p += 2) {
-                const bool two = p + 1 < cur.pairs;
+            for (int p = 0; p < pairs; p += 2) {
+                const bool two = p + 1 < pairs;
                 if (two) tc_ld16(d_lane + 16 * (p + 1), db);
                 row_pair(da);
                 if (!two) break;
                 tc_wait_ld16(db);
-                const bool more = p + 2 < cur.pairs;
+                const bool more = p + 2 < pairs;
                 if (more) tc_ld16(d_lane + 16 * (p + 2), da);
                 row_pair(db);
                 if (more) tc_wait_ld16(da);
             }
             tc_fence_before();
-            if (i >= cur.s0 && i < cur.s1) {
+            __syncwarp();
+            if ((tid & 31) == 0) mbar_arrive(&d_free[slot]);
+            if (i >= span.y && i < span.z) {
                 // h = (T_0 z_phi + T_1) z_phi^{m_fin} z_r^{n_mid}, z_phi = e^{-i Phi_phi}
                 const float hr = fmaf(tr.x, zc, fmaf(ti.x, zs, tr.y));
                 const float hi = fmaf(ti.x, zc, fmaf(-tr.x, zs, ti.y));
-                const float fc = gc * inv, fs = gs * inv;
+                fc *= inv;
+                fs *= inv;
                 const float yr = fmaf(hr, fc, hi * fs), yi = fmaf(hi, fc, -hr * fs);
-                if (cur.c64)
-                    reinterpret_cast<float2 *>(cur.out)[i] = make_float2(yr, yi);
+                if (c64)
+                    reinterpret_cast<float2 *>(out)[i] = make_float2(yr, yi);
                 else
-                    reinterpret_cast<double2 *>(cur.out)[i] = make_double2((double)yr, (double)yi);
+                    reinterpret_cast<double2 *>(out)[i] = make_double2((double)yr, (double)yi);
             }
         }
-        if (lead) {  // tables that only the other warpgroup still needs
-            while (tend < T1) {
-                mbar_arrive(&b_empty[j & 1]);
+        if (lead) {  // tables that only other warpgroups still need
+            while (tend < T1 && !bad) {
+                if (mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1)) mbar_arrive(&b_empty[j & 1]);
+                else bad = true;
                 ++j;
-                tend = recs[tend].tile_end;
+                tend = __ldg(&recs[tend].tile_end);
             }
-            if (bad) atomicOr(hp->err, ERRBIT_TIMEOUT);
+            if (bad) s_abort = 1;
         }
     }
     __syncthreads();
@@ -494,7 +523,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 8)
+    if (warp == 4 * kTcGroups)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
