@@ -207,9 +207,9 @@ struct SlotPlan {
     std::vector<int2> contrib;
     std::vector<int2> rows;
     std::vector<int4> row_slot;  // (first slot, highest n, lowest n, 0) of each row
-    // tensor-core summation: row pairs, K steps, centre of the n range and signed m of the last
-    // pair's second row; pairs 0 where the mode set exceeds its accumulators or basis
-    int tc_pairs = 0, tc_ks = 0, n_mid = 0, m_fin = 0;
+    // tensor-core summation: pairs of rows m and -m, K steps, centre of the n range, largest m;
+    // pairs 0 where the mode set exceeds its accumulators or basis
+    int tc_pairs = 0, tc_ks = 0, n_mid = 0, m_top = 0;
 };
 
 few_status plan_slots(const int *l, const int *m, const int *n, int N, SlotPlan &P)
@@ -273,10 +273,10 @@ few_status plan_slots(const int *l, const int *m, const int *n, int N, SlotPlan 
     const int n_hi = *std::max_element(hi.begin(), hi.end());
     P.n_mid = n_lo + (n_hi - n_lo) / 2;
     const int half = n_hi - P.n_mid;
-    if (n_rows <= kTcMaxRows && half <= kTcMaxHalf) {
-        P.tc_pairs = (n_rows + 1) / 2;
+    P.m_top = mmax;
+    if (mmax < kTcMaxPairs && half <= kTcMaxHalf) {
+        P.tc_pairs = mmax + 1;
         P.tc_ks = half / 8 + 1;
-        P.m_fin = mmax - (2 * P.tc_pairs - 1);
     }
     P.n_slots = slot;
     P.m_last = m_last;
@@ -415,7 +415,7 @@ few_status validate_request(const few_request &r, bool need_device_out)
     return FEW_OK;
 }
 
-// Whether a request's mode set fits the tensor-core summation (kTcMaxRows, kTcMaxHalf).
+// Whether a request's mode set fits the tensor-core summation (kTcMaxPairs, kTcMaxHalf).
 bool tc_fits(const few_request &r) { return r.prec == FEW_MIXED && r.traj->plan.tc_pairs > 0; }
 
 // Build the host image of a plan for `n` requests of one precision; tc: by the tensor-core
@@ -952,7 +952,7 @@ few_status few_traj_create(few_ctx *ctx, const double *t_knots, int K, const int
     D.tc_pairs = P.tc_pairs;
     D.tc_ks = P.tc_ks;
     D.n_mid = P.n_mid;
-    D.m_fin = P.m_fin;
+    D.m_top = P.m_top;
     tr->job_dev = reinterpret_cast<BuildJob *>(d + o_job);
 
     cudaStream_t s = ctx->internal;

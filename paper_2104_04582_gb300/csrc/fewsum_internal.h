@@ -37,8 +37,8 @@ enum : int {
 // Tensor-core summation (tcsum.cu): tiles of kTcTile consecutive samples of one segment, starting
 // at multiples of kTcTile (so a sample's arithmetic does not depend on the request's slicing).
 constexpr int kTcTile = 128;    // the MMA's M: one sample per tensor-memory lane
-constexpr int kTcMaxRows = 22;  // rows (signed m): two accumulators of 8 columns per row, beside
-                                //   the operands, in the 512 tensor-memory columns
+constexpr int kTcMaxPairs = 11;  // rows m and -m, max m <= 10: two accumulators of 16 columns per
+                                 //   pair, beside the operands, in the 512 tensor-memory columns
 constexpr int kTcMaxHalf = 31;  // half-width of the n range: 64 basis values (K)
 constexpr int kTcFoldThreads = 704;
 constexpr int kTcRecThreads = 128;  // threads of a fold block that fill tile records
@@ -54,7 +54,7 @@ struct alignas(128) TileRec {
     const unsigned char *tab;  // the segment's operand table
     void *out;
     int pairs, ks;        // row pairs, K steps of 16 (8 powers of z_r each)
-    int mids;             // n_mid (low 16 bits, signed) and m_fin (high 16 bits, signed)
+    int n_mid;            // centre of the n range
     int c64;
 };
 static_assert(sizeof(TileRec) == 128, "one line");
@@ -109,7 +109,7 @@ struct TrajDev {
     const int2 *contrib;   // [n_contrib] (mode * 2 + kind, 2 * pair + kind); kind 0: A Y+,
                            //   1: conj(A) Y-
     int tc_pairs, tc_ks;   // tensor-core summation: row pairs, K steps (tc_pairs 0: not used)
-    int n_mid, m_fin;      //   centre of the n range; signed m of the last pair's second row
+    int n_mid, m_top;      //   centre of the n range; largest m
     const int4 *row_slot;  // [n_rows] (first slot, highest n, lowest n, 0); lowest > highest: empty
     const int2 *rows;      // [n_rows] (slots of the row, lowest n of the previous row minus
                            //   this row's lowest n); a row's slots run from its highest n down

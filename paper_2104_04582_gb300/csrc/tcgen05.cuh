@@ -53,6 +53,17 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32])
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// One lane of a converged warp.  MMAs are issued under this predicate in a branch that the compiler
+// can see to be uniform for the warp: their operands then stay in uniform registers.  Issued
+// under `lane == 0` they cost ~130 cycles each, whatever their size; elected, an M = 128, N = 176,
+// K = 16 MMA with A in tensor memory issues at its execution rate (97-104 cycles; 88 ideal).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // D[tmem] (+)= A[tmem] B[smem], kind::f16.  A: K-major rows on the tensor-memory lanes, two
 // consecutive K elements per 32-bit column (K = 16: eight columns from a_tmem on).
 __device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc,

@@ -18,15 +18,15 @@
 // lo.lo is below 2^-24 of the term.  Phases are 64-bit fixed-point turns: a cubic in the sample
 // number whose coefficients (the FP64 Taylor expansion of the phase splines at the tile's first
 // sample) are in units of 2^-64 turn, so that wrap-around arithmetic is the exact reduction modulo
-// one turn and z_r^8, z_phi^2 and the final factor come from exact integer multiples of the
+// one turn and z_r^8 and z_r^{n_mid} come from exact integer multiples of the
 // phases instead of powers of rounded exponentials.  Measured error against a 64-bit restatement
 // over the one-year 3843-mode waveform: see the table beside k_sum_tc.
 //
 // Work decomposition: tiles of 128 samples (one per tensor-memory lane) that start at multiples of
-// 128 within a segment; a persistent CTA per SM takes a contiguous run of tiles.  Two warpgroups
-// take its tiles in turn, each with its own accumulator and operand columns in tensor memory: one
-// generates its basis or drains its accumulator while the other's MMAs run.  A ninth warp keeps
-// the operand tables of this and the next segment in shared memory (bulk copies, two buffers).
+// 128 within a segment; a persistent CTA per SM takes a contiguous run of tiles.  Four warpgroups
+// take its tiles in turn on two slots of accumulator and operand columns in tensor memory.  The
+// operand tables of this and the next segment sit in shared memory (bulk copies, two buffers,
+// refilled by the last warpgroup to release one).
 #include <cuda_fp16.h>
 
 #include "fewsum_internal.h"
@@ -39,10 +39,10 @@ namespace fewsum {
 namespace {
 
 constexpr int kTcGroups = 4;                        // warpgroups
-constexpr int kTcThreads = 128 * kTcGroups + 32;    // and the table producer's warp
-constexpr int kTcMaxN = 8 * kTcMaxRows;  // accumulator columns
+constexpr int kTcThreads = 128 * kTcGroups;
+constexpr int kTcMaxN = 16 * kTcMaxPairs;  // accumulator columns
 constexpr int kTcMaxKs = (kTcMaxHalf + 8) / 8;
-constexpr int kTcMaxTable = 1024 * (kTcMaxRows / 2) * kTcMaxKs;
+constexpr int kTcMaxTable = 1024 * kTcMaxPairs * kTcMaxKs;
 constexpr uint32_t kTcDStride = 192, kTcECol = 384, kTcEStride = 64, kTcELo = 32;  // tmem columns
 
 __device__ __forceinline__ float pow2(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
@@ -107,7 +107,7 @@ __device__ void fill_record(const PlanHdr &h, int T)
     r.out = W.out;
     r.pairs = tr.tc_pairs;
     r.ks = tr.tc_ks;
-    r.mids = (tr.n_mid & 0xffff) | (int)((unsigned)tr.m_fin << 16);
+    r.n_mid = tr.n_mid;
     r.c64 = W.out_c64;
     h.recs[T] = r;
 }
@@ -122,8 +122,8 @@ __host__ __device__ constexpr int staged_stride(int ks) { return 16 * ks + 4; }
 // b) forming the cubics of the slots n_mid + b and n_mid - b and their X and Y; the block then
 // scales by the power of two that brings the table's largest entry into [2^14, 2^15) and packs
 // high and low fp16 parts as the MMA reads them (K-major without swizzle: 8 x 16 B core matrices,
-// 128 B apart along K).  Column 16 p + 2 x + e of the product is row 2 p + e (signed m descending),
-// x = 4 component + degree; basis value 2 b is cos(b theta), 2 b + 1 sin(b theta).  The blocks
+// 128 B apart along K).  Column 16 p + 2 x + e of the product is the row of signed m = m_top - p
+// (e = 0) or p - m_top (e = 1; zero for m = 0), x = 4 component + degree; basis value 2 b is cos(b theta), 2 b + 1 sin(b theta).  The blocks
 // after that fill the tile records (FP64 work beside the fold's gathers).
 __global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *__restrict__ hp)
 {
@@ -149,8 +149,9 @@ __global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *__res
         float X[8], Y[8];  // x = 4 component + degree
 #pragma unroll
         for (int x = 0; x < 8; ++x) X[x] = Y[x] = 0.0f;
-        if (row < tr.n_rows) {
-            const int4 rs = tr.row_slot[row];  // slots n = rs.y .. rs.z
+        const int m = (row & 1) ? (row >> 1) - tr.m_top : tr.m_top - (row >> 1), j = tr.m_top - m;
+        if (j < tr.n_rows && !((row & 1) && m == 0)) {
+            const int4 rs = tr.row_slot[j];  // slots n = rs.y .. rs.z
 #pragma unroll
             for (int sign = 0; sign < 2; ++sign) {
                 const int n = sign ? tr.n_mid - b : tr.n_mid + b;
@@ -265,11 +266,11 @@ __device__ __forceinline__ bool wg_any(int id, bool bad)
     return r != 0;
 }
 
-// Eight powers (cos, sin), two to a float2, as packed fp16 high and low parts into eight columns
-// each: column k holds (cos, sin) of power k.
-__device__ __forceinline__ void store_powers(uint32_t e_addr, const float2 (&c)[4], const float2 (&s)[4])
+// Eight powers (cos, sin), two to a float2, as packed fp16 high and low parts: word k holds
+// (cos, sin) of power k.
+__device__ __forceinline__ void split_powers(const float2 (&c)[4], const float2 (&s)[4],
+                                             uint32_t (&vh)[8], uint32_t (&vl)[8])
 {
-    uint32_t vh[8], vl[8];
     const float2 neg = both(-1.0f);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -283,8 +284,6 @@ __device__ __forceinline__ void store_powers(uint32_t e_addr, const float2 (&c)[
         vl[2 * k] = *reinterpret_cast<const uint32_t *>(&l0);
         vl[2 * k + 1] = *reinterpret_cast<const uint32_t *>(&l1);
     }
-    tc_st8(e_addr, vh);
-    tc_st8(e_addr + kTcELo, vl);
 }
 
 // (c, s) <- (ac, as) (bc, bs), two complex products at once.
@@ -311,219 +310,241 @@ __device__ __forceinline__ void first_powers(unsigned long long f, float2 (&c)[4
 
 }  // namespace
 
+// Starts the copy of table `n` of the CTA's run (first tile T) into its buffer (one thread).
+__device__ __forceinline__ void load_table(const TileRec *__restrict__ recs, int T, int n,
+                                           unsigned char *buf, uint64_t *full)
+{
+    const TileRec *r = recs + T;
+    const uint32_t bytes = (uint32_t)tc_table_bytes(__ldg(&r->pairs), __ldg(&r->ks));
+    const unsigned char *src = reinterpret_cast<const unsigned char *>(
+        __ldg(reinterpret_cast<const unsigned long long *>(&r->tab)));
+    mbar_arrive_expect_tx(&full[n & 1], bytes);
+    for (uint32_t o = 0; o < bytes; o += 16384u)
+        bulk_g2s(buf + (n & 1) * kTcMaxTable + o, src + o, min(16384u, bytes - o), &full[n & 1]);
+}
+
 // Warpgroup k takes every fourth tile of the CTA's run, on slot k & 1 of tensor memory (operand and
 // accumulator columns).  A tile's operand columns are free when the slot's previous MMAs have
-// completed, its accumulator when the slot's previous tile has been drained, so a warpgroup
-// forms its basis while the slot's other warpgroup waits for its MMAs or drains them.
+// completed, its accumulator when the slot's previous tile has been drained; a warpgroup forms
+// its basis in registers while the slot's other warpgroup waits for its MMAs, and stores it while
+// that one drains them.
 __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restrict__ hp)
 {
     extern __shared__ __align__(128) unsigned char tcs[];  // two operand tables
-    __shared__ __align__(8) uint64_t b_full[2], b_empty[2], d_full[2], d_free[2];
+    __shared__ __align__(8) uint64_t b_full[2], d_full[2], d_free[2];
+    __shared__ int b_left[2];  // warpgroups that still need the table in the buffer
+    __shared__ int s_loaded;   // tables whose copies have been started
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
     const TileRec *__restrict__ recs = hp->recs;
     const int T0 = hp->tile_cta[blockIdx.x], T1 = hp->tile_cta[blockIdx.x + 1];
     if (T0 >= T1) return;  // uniform across the CTA: no work
-    if (warp == 4 * kTcGroups) {
+    if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&tmem_slot)),
                      "r"(512u)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (tid == 0) {
+    if (tid == 32) {
         for (int b = 0; b < 2; ++b) {
             mbar_init(&b_full[b], 1);
-            mbar_init(&b_empty[b], kTcGroups);
             mbar_init(&d_full[b], 1);
             mbar_init(&d_free[b], 4);
+            b_left[b] = kTcGroups;
         }
         fence_mbar_init();
         s_abort = 0;
+        load_table(recs, T0, 0, tcs, b_full);
+        const int next = __ldg(&recs[T0].tile_end);
+        if (next < T1) load_table(recs, next, 1, tcs, b_full);
+        s_loaded = next < T1 ? 2 : 1;
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
-
-    if (warp == 4 * kTcGroups) {
-        if ((tid & 31) == 0) {  // operand tables of the run's segments, in order
-            int j = 0, landed = 0;
-            for (int T = T0; T < T1 && !s_abort; ++j) {
-                const TileRec *r = recs + T;
-                const uint32_t bytes = (uint32_t)tc_table_bytes(r->pairs, r->ks);
-                const unsigned char *src = r->tab;
-                const int b = j & 1;
-                if (!mbar_wait_bounded(&b_empty[b], ((j >> 1) & 1) ^ 1)) {
-                    s_abort = 1;
-                    break;
+    const int group = warp >> 2, slot = group & 1, lane = tid & 127;
+    const bool lead = lane == 0;
+    const uint32_t quarter = (uint32_t)(32 * (warp & 3)) << 16;
+    const uint32_t d_col = tmem + (uint32_t)slot * kTcDStride;
+    const uint32_t e_col = tmem + kTcECol + (uint32_t)slot * kTcEStride;
+    int j = 0, tend = __ldg(&recs[T0].tile_end);  // table of the current tile, and where it ends
+    bool bad = false;
+    // This warpgroup's MMAs on table j have completed: release it (lead), and let the last of the
+    // warpgroups refill its buffer.  A table is released only once it has landed (also one that the
+    // warpgroup had no tile in): its buffer's previous table has then been released by every
+    // warpgroup, so neither the count nor a parity wait can be taken for the previous table's.
+    auto release_table = [&]() {
+        const int next = __ldg(&recs[tend].tile_end);  // end of table j + 1, first tile of j + 2
+        if (lead && !bad) {
+            if (!mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1)) {
+                bad = true;
+            } else if (__threadfence_block(), atomicSub(&b_left[j & 1], 1) == 1) {
+                __threadfence_block();
+                b_left[j & 1] = kTcGroups;
+                if (next < T1) {
+                    s_loaded = j + 3;
+                    load_table(recs, next, j, tcs, b_full);  // table j + 2, the same buffer
                 }
-                landed = max(landed, j - 1);  // every warpgroup is past table j - 2
-                mbar_arrive_expect_tx(&b_full[b], bytes);
-                for (uint32_t o = 0; o < bytes; o += 16384u)
-                    bulk_g2s(tcs + b * kTcMaxTable + o, src + o, min(16384u, bytes - o), &b_full[b]);
-                T = r->tile_end;
             }
-            // no copy may land after the CTA's shared memory is gone
-            for (; landed < j; ++landed) mbar_wait_bounded(&b_full[landed & 1], (landed >> 1) & 1);
+        }
+        ++j;
+        tend = next;
+    };
+#pragma unroll 1
+    for (int T = T0 + group; T < T1; T += kTcGroups) {
+        while (T >= tend) release_table();
+        const TileRec *rp = recs + T;
+        const uint32_t use = (uint32_t)(T - T0) >> 1;  // of the slot
+        const int4 span = __ldg(reinterpret_cast<const int4 *>(&rp->i0));  // i0, s0, s1
+        const int4 shape = __ldg(reinterpret_cast<const int4 *>(&rp->pairs));  // pairs, ks, n_mid, c64
+        const int pairs = shape.x, ks = shape.y;
+        const int i = span.x + lane;
+        const uint32_t v = (uint32_t)max(i - max(span.x, span.y), 0);
+        const unsigned long long fr = phase_fixed(rp->r, v), fphi = phase_fixed(rp->phi, v);
+        // the basis: powers 0 .. 8 ks - 1, eight at a time, z and z^8 from the phase itself, held
+        // in registers until the slot's operand columns are free
+        uint32_t vh[kTcMaxKs][8], vl[kTcMaxKs][8];
+        float2 c[4], s[4];
+        first_powers(fr, c, s);
+        split_powers(c, s, vh[0], vl[0]);
+        float bs, bc, gs, gc;
+        sincos_fixed((uint32_t)((8 * fr) >> 32), bs, bc);
+        gs = bs;
+        gc = bc;
+        auto next_powers = [&](uint32_t(&h)[8], uint32_t(&l)[8]) {
+            float2 pc[4], ps[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) cmul2(both(gc), both(gs), c[k], s[k], pc[k], ps[k]);
+            split_powers(pc, ps, h, l);
+            const float nc = fmaf(gc, bc, -gs * bs);
+            gs = fmaf(gc, bs, gs * bc);
+            gc = nc;
+        };
+#pragma unroll
+        for (int a = 1; a < kTcMaxKs; ++a) {
+            if (a < ks) {
+                next_powers(vh[a], vl[a]);
+            } else {  // defined on every path: otherwise these registers stay live around the loop
+#pragma unroll
+                for (int k = 0; k < 8; ++k) vh[a][k] = vl[a][k] = 0;
+            }
+        }
+        if (use > 0 && !mbar_wait_bounded(&d_full[slot], (use - 1) & 1)) bad = true;
+        __syncwarp();
+        tc_fence_after();
+#pragma unroll
+        for (int a = 0; a < kTcMaxKs; ++a) {
+            if (a < ks) {
+                tc_st8(e_col + quarter + 8 * a, vh[a]);
+                tc_st8(e_col + quarter + kTcELo + 8 * a, vl[a]);
+            }
+        }
+        tc_wait_st();
+        tc_fence_before();
+        bad = wg_any(1 + group, bad);
+        if (bad) break;
+        if ((warp & 3) == 0) {  // the warpgroup's first warp issues the MMAs
+            const bool ok = (use == 0 || mbar_wait_bounded(&d_free[slot], (use - 1) & 1)) &&
+                            mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1);
+            if (__all_sync(0xffffffffu, ok)) {
+                tc_fence_after();
+                const int up = __shfl_sync(0xffffffffu, pairs, 0), uk = __shfl_sync(0xffffffffu, ks, 0);
+                const uint32_t b_hi = smem_u32(tcs) + (uint32_t)(j & 1) * kTcMaxTable;
+                const uint32_t b_lo = b_hi + (uint32_t)tc_table_bytes(up, uk) / 2;
+                const uint32_t idesc =
+                    (1u << 4) | ((uint32_t)(2 * up) << 17) | ((uint32_t)(kTcTile >> 4) << 24);
+                const uint64_t d_hi = smem_desc(b_hi, 128, 256u * (uint32_t)uk);
+                const uint64_t d_lo = smem_desc(b_lo, 128, 256u * (uint32_t)uk);
+                if (elect_one()) {
+                    for (int a = 0; a < uk; ++a) {  // the small products first; 256 B per K step
+                        tc_mma_ta(d_col, e_col + kTcELo + 8 * a, d_hi + 16 * a, idesc, a != 0);
+                        tc_mma_ta(d_col, e_col + 8 * a, d_lo + 16 * a, idesc, 1);
+                    }
+                    for (int a = 0; a < uk; ++a) tc_mma_ta(d_col, e_col + 8 * a, d_hi + 16 * a, idesc, 1);
+                    tc_commit(&d_full[slot]);
+                }
+                __syncwarp();
+            } else {
+                s_abort = 1;
+            }
+        }
+        // while the MMAs run: this sample's factors
+        const float2 uu = __ldg(reinterpret_cast<const float2 *>(&rp->u0));
+        const float inv = __ldg(rp->inv);
+        void *out = reinterpret_cast<void *>(__ldg(reinterpret_cast<const unsigned long long *>(&rp->out)));
+        if (T + kTcGroups < T1)  // the next tile's record on its way to L1
+            asm volatile("prefetch.global.L1 [%0];" ::"l"(rp + kTcGroups));
+        const float u = fmaf((float)(i - span.y), uu.y, uu.x);
+        float zs, zc;
+        sincos_fixed((uint32_t)(fphi >> 32), zs, zc);
+        float fs = 0.0f, fc = inv;  // z_r^{n_mid} over the table's scale
+        if (shape.z != 0) {
+            sincos_fixed((uint32_t)(((unsigned long long)(long long)shape.z * fr) >> 32), fs, fc);
+            fs *= inv;
+            fc *= inv;
+        }
+        const float2 U = both(u), U2 = both(u * u);
+        // rows m = m_top - p and p - m_top: Horner in z_phi and in its conjugate
+        const float2 WR = both(zc), WI = make_float2(-zs, zs), NWI = make_float2(zs, -zs);
+        float2 tr = both(0.0f), ti = tr;
+        if (!mbar_wait_bounded(&d_full[slot], use & 1)) {
+            s_abort = 1;
+            bad = true;
         }
         __syncwarp();
-    } else {
-        const int group = warp >> 2, slot = group & 1, lane = tid & 127;
-        const bool lead = lane == 0;
-        const uint32_t quarter = (uint32_t)(32 * (warp & 3)) << 16;
-        const uint32_t d_col = tmem + (uint32_t)slot * kTcDStride;
-        const uint32_t e_col = tmem + kTcECol + (uint32_t)slot * kTcEStride;
-        int j = 0, tend = __ldg(&recs[T0].tile_end);  // table of the current tile, and where it ends
-        bool bad = false;
-        for (int T = T0 + group; T < T1; T += kTcGroups) {
-            // tables before this tile's: this warpgroup's MMAs on them have completed.  A table
-            // is released only once it has landed (also one that this warpgroup had no tile in):
-            // its buffer's previous table has then been released by every warpgroup, so an arrival
-            // or a parity wait cannot be taken for the previous table's.
-            while (T >= tend) {
-                if (lead && !bad) {
-                    if (mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1)) mbar_arrive(&b_empty[j & 1]);
-                    else bad = true;
-                }
-                ++j;
-                tend = __ldg(&recs[tend].tile_end);
-            }
-            const TileRec *rp = recs + T;
-            const uint32_t use = (uint32_t)(T - T0) >> 1;  // of the slot
-            const int4 span = __ldg(reinterpret_cast<const int4 *>(&rp->i0));  // i0, s0, s1
-            const int i = span.x + lane;
-            const uint32_t v = (uint32_t)max(i - max(span.x, span.y), 0);
-            const unsigned long long fr = phase_fixed(rp->r, v), fphi = phase_fixed(rp->phi, v);
-            const int pairs = __ldg(&rp->pairs), ks = __ldg(&rp->ks);
-            // the basis: powers 0 .. 8 ks - 1, eight at a time, z and z^8 from the phase itself
-            float2 c[4], s[4];
-            first_powers(fr, c, s);
-            float gs = 0.0f, gc = 0.0f, bs = 0.0f, bc = 0.0f;
-            if (ks > 1) {
-                sincos_fixed((uint32_t)((8 * fr) >> 32), bs, bc);
-                gs = bs;
-                gc = bc;
-            }
-            if (use > 0 && !mbar_wait_bounded(&d_full[slot], (use - 1) & 1)) bad = true;
-            __syncwarp();
-            tc_fence_after();
-            store_powers(e_col + quarter, c, s);
-            for (int a = 1; a < ks; ++a) {
-                float2 pc[4], ps[4];
+        tc_fence_after();
+        auto row_pair = [&](const float(&d)[16]) {
+            const float2 *k = reinterpret_cast<const float2 *>(d);
+            const float2 kr = fma2(fma2(k[3], U, k[2]), U2, fma2(k[1], U, k[0]));
+            const float2 ki = fma2(fma2(k[7], U, k[6]), U2, fma2(k[5], U, k[4]));
+            const float2 nr = fma2(ti, NWI, fma2(tr, WR, kr));
+            const float2 ni = fma2(ti, WR, fma2(tr, WI, ki));
+            tr = nr;
+            ti = ni;
+        };
+        // four row pairs at a time: their loads in flight together
+        const uint32_t d_lane = d_col + quarter;
+#pragma unroll 1
+        for (int p = 0; p < pairs; p += 4) {
+            float d[4][16];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) cmul2(both(gc), both(gs), c[k], s[k], pc[k], ps[k]);
-                store_powers(e_col + quarter + 8 * a, pc, ps);
-                const float nc = fmaf(gc, bc, -gs * bs);
-                gs = fmaf(gc, bs, gs * bc);
-                gc = nc;
-            }
-            tc_wait_st();
-            tc_fence_before();
-            bad = wg_any(1 + group, bad);
-            if (bad) break;
-            if (lead) {
-                tc_fence_after();
-                if ((use == 0 || mbar_wait_bounded(&d_free[slot], (use - 1) & 1)) &&
-                    mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1)) {
-                    tc_fence_after();
-                    const uint32_t b_hi = smem_u32(tcs + (j & 1) * kTcMaxTable);
-                    const uint32_t b_lo = b_hi + (uint32_t)tc_table_bytes(pairs, ks) / 2;
-                    const uint32_t idesc = (1u << 4) | ((uint32_t)(2 * pairs) << 17) |
-                                           ((uint32_t)(kTcTile >> 4) << 24);
-                    const uint32_t sbo = 256u * (uint32_t)ks;
-                    for (int a = 0; a < ks; ++a) {  // the small products first
-                        tc_mma_ta(d_col, e_col + kTcELo + 8 * a, smem_desc(b_hi + 256 * a, 128, sbo),
-                                  idesc, a != 0);
-                        tc_mma_ta(d_col, e_col + 8 * a, smem_desc(b_lo + 256 * a, 128, sbo), idesc, 1);
-                    }
-                    for (int a = 0; a < ks; ++a)
-                        tc_mma_ta(d_col, e_col + 8 * a, smem_desc(b_hi + 256 * a, 128, sbo), idesc, 1);
-                    tc_commit(&d_full[slot]);
-                } else {
-                    s_abort = 1;
+            for (int q = 0; q < 4; ++q)  // past the last pair: columns of the slot that are not used
+                tc_ld16(d_lane + 16 * (p + q), d[q]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (p + q < pairs) {
+                    tc_wait_ld16(d[q]);
+                    row_pair(d[q]);
                 }
-            }
-            // while the MMAs run: this sample's factors
-            const float2 uu = __ldg(reinterpret_cast<const float2 *>(&rp->u0));
-            const float inv = __ldg(rp->inv);
-            const int mids = __ldg(&rp->mids), c64 = __ldg(&rp->c64);
-            void *out = reinterpret_cast<void *>(__ldg(reinterpret_cast<const unsigned long long *>(&rp->out)));
-            if (T + kTcGroups < T1)  // the next tile's record on its way to L1
-                asm volatile("prefetch.global.L1 [%0];" ::"l"(rp + kTcGroups));
-            const float u = fmaf((float)(i - span.y), uu.y, uu.x);
-            const long long nmid = (short)(mids & 0xffff), mfin = (short)(mids >> 16);
-            float zs, zc, ws, wc, fs, fc;
-            sincos_fixed((uint32_t)(fphi >> 32), zs, zc);
-            sincos_fixed((uint32_t)((2 * fphi) >> 32), ws, wc);
-            sincos_fixed((uint32_t)(((unsigned long long)mfin * fphi + (unsigned long long)nmid * fr) >> 32),
-                         fs, fc);
-            const float2 U = both(u), U2 = both(u * u);
-            const float2 WR = both(wc), WI = both(-ws), NWI = both(ws);
-            float2 tr = both(0.0f), ti = tr;  // rows 2 p and 2 p + 1: two chains in z_phi^2
-            if (!mbar_wait_bounded(&d_full[slot], use & 1)) {
-                s_abort = 1;
-                bad = true;
-            }
-            __syncwarp();
-            tc_fence_after();
-            auto row_pair = [&](const float(&d)[16]) {
-                const float2 *k = reinterpret_cast<const float2 *>(d);
-                const float2 kr = fma2(fma2(k[3], U, k[2]), U2, fma2(k[1], U, k[0]));
-                const float2 ki = fma2(fma2(k[7], U, k[6]), U2, fma2(k[5], U, k[4]));
-                const float2 nr = fma2(ti, NWI, fma2(tr, WR, kr));
-                const float2 ni = fma2(ti, WR, fma2(tr, WI, ki));
-                tr = nr;
-                ti = ni;
-            };
-            const uint32_t d_lane = d_col + quarter;
-            float da[16], db[16];
-            tc_ld16(d_lane, da);
-            tc_wait_ld16(da);
-            for (int p = 0; p < pairs; p += 2) {
-                const bool two = p + 1 < pairs;
-                if (two) tc_ld16(d_lane + 16 * (p + 1), db);
-                row_pair(da);
-                if (!two) break;
-                tc_wait_ld16(db);
-                const bool more = p + 2 < pairs;
-                if (more) tc_ld16(d_lane + 16 * (p + 2), da);
-                row_pair(db);
-                if (more) tc_wait_ld16(da);
-            }
-            tc_fence_before();
-            __syncwarp();
-            if ((tid & 31) == 0) mbar_arrive(&d_free[slot]);
-            if (i >= span.y && i < span.z) {
-                // h = (T_0 z_phi + T_1) z_phi^{m_fin} z_r^{n_mid}, z_phi = e^{-i Phi_phi}
-                const float hr = fmaf(tr.x, zc, fmaf(ti.x, zs, tr.y));
-                const float hi = fmaf(ti.x, zc, fmaf(-tr.x, zs, ti.y));
-                fc *= inv;
-                fs *= inv;
-                const float yr = fmaf(hr, fc, hi * fs), yi = fmaf(hi, fc, -hr * fs);
-                if (c64)
-                    reinterpret_cast<float2 *>(out)[i] = make_float2(yr, yi);
-                else
-                    reinterpret_cast<double2 *>(out)[i] = make_double2((double)yr, (double)yi);
             }
         }
-        if (lead) {  // tables that only other warpgroups still need
-            while (tend < T1 && !bad) {
-                if (mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1)) mbar_arrive(&b_empty[j & 1]);
-                else bad = true;
-                ++j;
-                tend = __ldg(&recs[tend].tile_end);
-            }
-            if (bad) s_abort = 1;
+        tc_fence_before();
+        __syncwarp();
+        if ((tid & 31) == 0) mbar_arrive(&d_free[slot]);
+        if (i >= span.y && i < span.z) {
+            const float hr = tr.x + tr.y, hi = ti.x + ti.y;
+            const float yr = fmaf(hr, fc, hi * fs), yi = fmaf(hi, fc, -hr * fs);
+            if (shape.w)
+                reinterpret_cast<float2 *>(out)[i] = make_float2(yr, yi);
+            else
+                reinterpret_cast<double2 *>(out)[i] = make_double2((double)yr, (double)yi);
         }
     }
+    while (tend < T1 && !bad) release_table();  // tables that only other warpgroups still need
+    if (lead && bad) s_abort = 1;
     __syncthreads();
-    if (tid == 0 && s_abort) atomicOr(hp->err, ERRBIT_TIMEOUT);
+    if (tid == 0 && s_abort) {
+        atomicOr(hp->err, ERRBIT_TIMEOUT);
+        // no copy may land after the CTA's shared memory is gone
+        for (int n = max(s_loaded - 2, 0); n < s_loaded; ++n) mbar_wait_bounded(&b_full[n & 1], (n >> 1) & 1);
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 4 * kTcGroups)
+    if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
