@@ -112,4 +112,13 @@ __device__ __forceinline__ void tc_wait_ld16(float (&v)[16])
                  : "memory");
 }
 
+// For further arrays whose loads the same wait covered.
+__device__ __forceinline__ void tc_landed16(float (&v)[16])
+{
+    asm volatile(""
+                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]),
+                   "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]),
+                   "+f"(v[13]), "+f"(v[14]), "+f"(v[15])::"memory");
+}
+
 }  // namespace fewsum

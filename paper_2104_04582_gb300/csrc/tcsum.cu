@@ -40,6 +40,7 @@ namespace {
 
 constexpr int kTcGroups = 4;                        // warpgroups
 constexpr int kTcThreads = 128 * kTcGroups;
+constexpr int kTcDrain = 6;                         // row pairs in registers while draining
 constexpr int kTcMaxN = 16 * kTcMaxPairs;  // accumulator columns
 constexpr int kTcMaxKs = (kTcMaxHalf + 8) / 8;
 constexpr int kTcMaxTable = 1024 * kTcMaxPairs * kTcMaxKs;
@@ -243,8 +244,8 @@ __device__ __forceinline__ void sincos_fixed(uint32_t f, float &s, float &c)
 // c0 + c1 v + c2 v^2 + c3 v^3 in 64-bit wrap-around arithmetic (modulo one turn).
 __device__ __forceinline__ unsigned long long phase_fixed(const long long *c, uint32_t v)
 {
-    const longlong2 a = __ldg(reinterpret_cast<const longlong2 *>(c));
-    const longlong2 b = __ldg(reinterpret_cast<const longlong2 *>(c) + 1);
+    const longlong2 a = reinterpret_cast<const longlong2 *>(c)[0];
+    const longlong2 b = reinterpret_cast<const longlong2 *>(c)[1];
     unsigned long long p = (unsigned long long)b.y;
     p = p * v + (unsigned long long)b.x;
     p = p * v + (unsigned long long)a.y;
@@ -334,6 +335,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
     __shared__ __align__(8) uint64_t b_full[2], d_full[2], d_free[2];
     __shared__ int b_left[2];  // warpgroups that still need the table in the buffer
     __shared__ int s_loaded;   // tables whose copies have been started
+    __shared__ __align__(16) uint32_t s_rec[4 * kTcGroups][32];  // each warp's tile record
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
@@ -393,13 +395,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
         ++j;
         tend = next;
     };
+    // a warp fetches the next tile's record a word a lane while its MMAs run, and reads it from its
+    // own line of shared memory
+    const TileRec *rp = reinterpret_cast<const TileRec *>(s_rec[warp]);
+    uint32_t next_word = 0;
+    if (T0 + group < T1) next_word = __ldg(reinterpret_cast<const uint32_t *>(recs + T0 + group) + (tid & 31));
 #pragma unroll 1
     for (int T = T0 + group; T < T1; T += kTcGroups) {
+        s_rec[warp][tid & 31] = next_word;
         while (T >= tend) release_table();
-        const TileRec *rp = recs + T;
+        __syncwarp();
         const uint32_t use = (uint32_t)(T - T0) >> 1;  // of the slot
-        const int4 span = __ldg(reinterpret_cast<const int4 *>(&rp->i0));  // i0, s0, s1
-        const int4 shape = __ldg(reinterpret_cast<const int4 *>(&rp->pairs));  // pairs, ks, n_mid, c64
+        const int4 span = *reinterpret_cast<const int4 *>(&rp->i0);      // i0, s0, s1
+        const int4 shape = *reinterpret_cast<const int4 *>(&rp->pairs);  // pairs, ks, n_mid, c64
         const int pairs = shape.x, ks = shape.y;
         const int i = span.x + lane;
         const uint32_t v = (uint32_t)max(i - max(span.x, span.y), 0);
@@ -472,11 +480,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
             }
         }
         // while the MMAs run: this sample's factors
-        const float2 uu = __ldg(reinterpret_cast<const float2 *>(&rp->u0));
+        const float2 uu = *reinterpret_cast<const float2 *>(&rp->u0);
         const float inv = __ldg(rp->inv);
-        void *out = reinterpret_cast<void *>(__ldg(reinterpret_cast<const unsigned long long *>(&rp->out)));
-        if (T + kTcGroups < T1)  // the next tile's record on its way to L1
-            asm volatile("prefetch.global.L1 [%0];" ::"l"(rp + kTcGroups));
+        void *out = rp->out;
+        if (T + kTcGroups < T1)
+            next_word = __ldg(reinterpret_cast<const uint32_t *>(recs + T + kTcGroups) + (tid & 31));
         const float u = fmaf((float)(i - span.y), uu.y, uu.x);
         float zs, zc;
         sincos_fixed((uint32_t)(fphi >> 32), zs, zc);
@@ -505,25 +513,30 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
             tr = nr;
             ti = ni;
         };
-        // four row pairs at a time: their loads in flight together
+        // six row pairs' loads in flight, then each pair's registers reloaded once it is used, so
+        // that the accumulator is free before the second half is computed (columns past the last
+        // pair belong to the slot and are not used)
         const uint32_t d_lane = d_col + quarter;
-#pragma unroll 1
-        for (int p = 0; p < pairs; p += 4) {
-            float d[4][16];
+        float d[kTcDrain][16];
 #pragma unroll
-            for (int q = 0; q < 4; ++q)  // past the last pair: columns of the slot that are not used
-                tc_ld16(d_lane + 16 * (p + q), d[q]);
+        for (int q = 0; q < kTcDrain; ++q) tc_ld16(d_lane + 16 * q, d[q]);
+        tc_wait_ld16(d[0]);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                if (p + q < pairs) {
-                    tc_wait_ld16(d[q]);
-                    row_pair(d[q]);
-                }
-            }
+        for (int q = 1; q < kTcDrain; ++q) tc_landed16(d[q]);
+#pragma unroll
+        for (int q = 0; q < kTcDrain; ++q) {
+            if (q < pairs) row_pair(d[q]);
+            if (q + kTcDrain < kTcMaxPairs) tc_ld16(d_lane + 16 * (q + kTcDrain), d[q]);
         }
+        tc_wait_ld16(d[0]);
+#pragma unroll
+        for (int q = 1; q < kTcMaxPairs - kTcDrain; ++q) tc_landed16(d[q]);
         tc_fence_before();
         __syncwarp();
         if ((tid & 31) == 0) mbar_arrive(&d_free[slot]);
+#pragma unroll
+        for (int q = kTcDrain; q < kTcMaxPairs; ++q)
+            if (q < pairs) row_pair(d[q - kTcDrain]);
         if (i >= span.y && i < span.z) {
             const float hr = tr.x + tr.y, hi = ti.x + ti.y;
             const float yr = fmaf(hr, fc, hi * fs), yi = fmaf(hi, fc, -hr * fs);
