@@ -337,7 +337,7 @@ struct LaunchPlan {
     int variant = kVariantFp64;
     int grid = 0, threads = 0, R = 0, smem = 0, total_pairs = 0, total_fold = 0;
     int total_anchor_segs = 0;
-    int total_segs = 0, total_tiles = 0;  // kVariantTc
+    int total_segs = 0, total_tiles = 0, ks = 0;  // kVariantTc
 };
 
 struct few_batch {
@@ -453,6 +453,7 @@ few_status build_image(few_ctx *c, const few_request *reqs, int n, bool tc, Plan
                 tiles += tiles_in_segment((int)P.seg[q][k], (int)P.seg[q][k + 1]);
         if (tiles > 0x7fffffff) return FEW_ERR_LIMIT;
         L.total_tiles = (int)tiles;
+        for (int q = 0; q < n; ++q) L.ks = std::max(L.ks, reqs[q].traj->plan.tc_ks);
         L.grid = (int)std::min<int64_t>(c->sm_count, tiles);
     }
 
@@ -691,7 +692,7 @@ cudaError_t launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, const LaunchPlan 
         if ((e = launch_fold_tc(hdr_dev, P.total_segs, P.total_tiles, st)) != cudaSuccess) return e;
         tm(2, true);
         tm(3, false);
-        if ((e = launch_sum_tc(hdr_dev, P.grid, st)) != cudaSuccess) return e;
+        if ((e = launch_sum_tc(hdr_dev, P.grid, P.ks, st)) != cudaSuccess) return e;
         tm(3, true);
         return cudaSuccess;
     }

@@ -223,7 +223,8 @@ inline int tiles_in_segment(int s_begin, int s_end)
 }
 cudaError_t tc_configure();
 cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st);
-cudaError_t launch_sum_tc(const PlanHdr *hdr_dev, int grid, cudaStream_t st);
+// ks: the most K steps of any wave of the plan.
+cudaError_t launch_sum_tc(const PlanHdr *hdr_dev, int grid, int ks, cudaStream_t st);
 // Bytes of one folded slot in the layout a variant reads.
 int sum_slot_bytes(int variant);
 cudaError_t launch_phases(const TrajDev &tr, const int *seg_start, double t0, double dt, int n,

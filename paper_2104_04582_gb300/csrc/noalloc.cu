@@ -238,7 +238,7 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     if (tc) {
         if (launch_ylm(hd, v.n_pairs, false, s) != cudaSuccess ||
             launch_fold_tc(hd, S, n_tiles, s) != cudaSuccess ||
-            launch_sum_tc(hd, grid_tc, s) != cudaSuccess) {
+            launch_sum_tc(hd, grid_tc, v.tc_ks, s) != cudaSuccess) {
             (void)cudaGetLastError();
             return FEW_ERR_CUDA;
         }

@@ -27,6 +27,8 @@
 // take its tiles in turn on two slots of accumulator and operand columns in tensor memory.  The
 // operand tables of this and the next segment sit in shared memory (bulk copies, two buffers,
 // refilled by the last warpgroup to release one).
+#include <type_traits>
+
 #include <cuda_fp16.h>
 
 #include "fewsum_internal.h"
@@ -290,8 +292,8 @@ __device__ __forceinline__ void split_powers(const float2 (&c)[4], const float2 
 // (c, s) <- (ac, as) (bc, bs), two complex products at once.
 __device__ __forceinline__ void cmul2(float2 ac, float2 as, float2 bc, float2 bs, float2 &c, float2 &s)
 {
-    const float2 nas = make_float2(-as.x, -as.y);
-    c = fma2(ac, bc, mul2(nas, bs));
+    const float2 nbs = make_float2(-bs.x, -bs.y);
+    c = fma2(ac, bc, mul2(as, nbs));
     s = fma2(ac, bs, mul2(as, bc));
 }
 
@@ -329,6 +331,8 @@ __device__ __forceinline__ void load_table(const TileRec *__restrict__ recs, int
 // completed, its accumulator when the slot's previous tile has been drained; a warpgroup forms
 // its basis in registers while the slot's other warpgroup waits for its MMAs, and stores it while
 // that one drains them.
+// KS: K steps of the plan's widest n range (a wave with fewer uses the first of them).
+template <int KS>
 __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restrict__ hp)
 {
     extern __shared__ __align__(128) unsigned char tcs[];  // two operand tables
@@ -414,41 +418,38 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
         const unsigned long long fr = phase_fixed(rp->r, v), fphi = phase_fixed(rp->phi, v);
         // the basis: powers 0 .. 8 ks - 1, eight at a time, z and z^8 from the phase itself, held
         // in registers until the slot's operand columns are free
-        uint32_t vh[kTcMaxKs][8], vl[kTcMaxKs][8];
-        float2 c[4], s[4];
-        first_powers(fr, c, s);
-        split_powers(c, s, vh[0], vl[0]);
-        float bs, bc, gs, gc;
-        sincos_fixed((uint32_t)((8 * fr) >> 32), bs, bc);
-        gs = bs;
-        gc = bc;
-        auto next_powers = [&](uint32_t(&h)[8], uint32_t(&l)[8]) {
-            float2 pc[4], ps[4];
+        uint32_t vh[KS][8], vl[KS][8];
+        {
+            float2 c[4], s[4];
+            first_powers(fr, c, s);
+            split_powers(c, s, vh[0], vl[0]);
+            if (KS > 1) {
+                float bs, bc;
+                sincos_fixed((uint32_t)((8 * fr) >> 32), bs, bc);
+                const float2 BC = both(bc), BS = both(bs);
+                float2 gc = BC, gs = BS;  // z^(8 a), in both halves
 #pragma unroll
-            for (int k = 0; k < 4; ++k) cmul2(both(gc), both(gs), c[k], s[k], pc[k], ps[k]);
-            split_powers(pc, ps, h, l);
-            const float nc = fmaf(gc, bc, -gs * bs);
-            gs = fmaf(gc, bs, gs * bc);
-            gc = nc;
-        };
+                for (int a = 1; a < KS; ++a) {
+                    float2 pc[4], ps[4];
 #pragma unroll
-        for (int a = 1; a < kTcMaxKs; ++a) {
-            if (a < ks) {
-                next_powers(vh[a], vl[a]);
-            } else {  // defined on every path: otherwise these registers stay live around the loop
-#pragma unroll
-                for (int k = 0; k < 8; ++k) vh[a][k] = vl[a][k] = 0;
+                    for (int k = 0; k < 4; ++k) cmul2(c[k], s[k], gc, gs, pc[k], ps[k]);
+                    split_powers(pc, ps, vh[a], vl[a]);
+                    if (a + 1 < KS) {
+                        float2 nc, ns;
+                        cmul2(gc, gs, BC, BS, nc, ns);
+                        gc = nc;
+                        gs = ns;
+                    }
+                }
             }
         }
         if (use > 0 && !mbar_wait_bounded(&d_full[slot], (use - 1) & 1)) bad = true;
         __syncwarp();
         tc_fence_after();
 #pragma unroll
-        for (int a = 0; a < kTcMaxKs; ++a) {
-            if (a < ks) {
-                tc_st8(e_col + quarter + 8 * a, vh[a]);
-                tc_st8(e_col + quarter + kTcELo + 8 * a, vl[a]);
-            }
+        for (int a = 0; a < KS; ++a) {
+            tc_st8(e_col + quarter + 8 * a, vh[a]);
+            tc_st8(e_col + quarter + kTcELo + 8 * a, vl[a]);
         }
         tc_wait_st();
         tc_fence_before();
@@ -517,26 +518,32 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
         // that the accumulator is free before the second half is computed (columns past the last
         // pair belong to the slot and are not used)
         const uint32_t d_lane = d_col + quarter;
-        float d[kTcDrain][16];
+        auto drain = [&](auto full) {  // full: every pair of the accumulator is in use
+            float d[kTcDrain][16];
 #pragma unroll
-        for (int q = 0; q < kTcDrain; ++q) tc_ld16(d_lane + 16 * q, d[q]);
-        tc_wait_ld16(d[0]);
+            for (int q = 0; q < kTcDrain; ++q) tc_ld16(d_lane + 16 * q, d[q]);
+            tc_wait_ld16(d[0]);
 #pragma unroll
-        for (int q = 1; q < kTcDrain; ++q) tc_landed16(d[q]);
+            for (int q = 1; q < kTcDrain; ++q) tc_landed16(d[q]);
 #pragma unroll
-        for (int q = 0; q < kTcDrain; ++q) {
-            if (q < pairs) row_pair(d[q]);
-            if (q + kTcDrain < kTcMaxPairs) tc_ld16(d_lane + 16 * (q + kTcDrain), d[q]);
-        }
-        tc_wait_ld16(d[0]);
+            for (int q = 0; q < kTcDrain; ++q) {
+                if (decltype(full)::value || q < pairs) row_pair(d[q]);
+                if (q + kTcDrain < kTcMaxPairs) tc_ld16(d_lane + 16 * (q + kTcDrain), d[q]);
+            }
+            tc_wait_ld16(d[0]);
 #pragma unroll
-        for (int q = 1; q < kTcMaxPairs - kTcDrain; ++q) tc_landed16(d[q]);
-        tc_fence_before();
-        __syncwarp();
-        if ((tid & 31) == 0) mbar_arrive(&d_free[slot]);
+            for (int q = 1; q < kTcMaxPairs - kTcDrain; ++q) tc_landed16(d[q]);
+            tc_fence_before();
+            __syncwarp();
+            if ((tid & 31) == 0) mbar_arrive(&d_free[slot]);
 #pragma unroll
-        for (int q = kTcDrain; q < kTcMaxPairs; ++q)
-            if (q < pairs) row_pair(d[q - kTcDrain]);
+            for (int q = kTcDrain; q < kTcMaxPairs; ++q)
+                if (decltype(full)::value || q < pairs) row_pair(d[q - kTcDrain]);
+        };
+        if (pairs == kTcMaxPairs)
+            drain(std::true_type());
+        else
+            drain(std::false_type());
         if (i >= span.y && i < span.z) {
             const float hr = tr.x + tr.y, hi = ti.x + ti.y;
             const float yr = fmaf(hr, fc, hi * fs), yi = fmaf(hi, fc, -hr * fs);
@@ -561,9 +568,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
 }
 
+namespace {
+using TcKernel = void (*)(const PlanHdr *);
+const TcKernel kTcKernels[kTcMaxKs] = {k_sum_tc<1>, k_sum_tc<2>, k_sum_tc<3>, k_sum_tc<4>};
+}  // namespace
+
 cudaError_t tc_configure()
 {
-    return cudaFuncSetAttribute(k_sum_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kTcMaxTable);
+    for (TcKernel k : kTcKernels) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kTcMaxTable);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st)
@@ -575,10 +592,11 @@ cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, int total_segs, int total_til
     return cudaGetLastError();
 }
 
-cudaError_t launch_sum_tc(const PlanHdr *hdr_dev, int grid, cudaStream_t st)
+cudaError_t launch_sum_tc(const PlanHdr *hdr_dev, int grid, int ks, cudaStream_t st)
 {
     if (grid <= 0) return cudaSuccess;
-    k_sum_tc<<<grid, kTcThreads, 2 * kTcMaxTable, st>>>(hdr_dev);
+    if (ks < 1 || ks > kTcMaxKs) return cudaErrorInvalidValue;
+    kTcKernels[ks - 1]<<<grid, kTcThreads, 2 * kTcMaxTable, st>>>(hdr_dev);
     return cudaGetLastError();
 }
 
