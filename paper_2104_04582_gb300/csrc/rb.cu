@@ -177,27 +177,25 @@ __global__ void k_rb_pack_b(const double *__restrict__ bre, const double *__rest
 // ---- per call -----------------------------------------------------------------------------
 
 // Quadratic form q_k = ||alpha_k B||^2 = sum_j Re(alpha_j t_j), t_j = sum_l G_jl conj(alpha_l), in
-// the arithmetic type T of the path, as a small register-blocked product: a block takes 32 knots
+// FP32, as a small register-blocked product: a block takes 32 knots
 // and 64 values of j, l advancing in chunks of 64 staged in (dynamic) shared memory; a thread owns
 // 4 knots x 2 values of j (j and j + 32), so 6 shared-memory reads feed 16 complex multiply-adds.
 // Partial sums over j are reduced per warp and added to q (FP64, zeroed beforehand); k_rb_norm
-// then forms s_k.  Used by the FP64 path and, in FP32, for bases of more than 128 vectors.
+// then forms s_k.  Used for bases of more than 128 vectors.
 constexpr int kQRows = 32, kQJ = 64, kQL = 64, kQThreads = 256, kQPer = 4;
 
-template <typename C>
-constexpr int rb_quad_smem() { return (kQL * kQJ + kQRows * kQL) * (int)sizeof(C); }
+constexpr int kQSmem = (kQL * kQJ + kQRows * kQL) * (int)sizeof(float2);
 
-template <typename T, typename C>
 __global__ void __launch_bounds__(kQThreads)
 k_rb_quad(const double *__restrict__ are, const double *__restrict__ aim, int M, int Nb,
-          const C *__restrict__ gt, double *__restrict__ q)
+          const float2 *__restrict__ gt, double *__restrict__ q)
 {
     extern __shared__ __align__(16) unsigned char rb_quad_smem_raw[];
-    C(*sg)[kQJ] = reinterpret_cast<C(*)[kQJ]>(rb_quad_smem_raw);                       // G_jl [l][j]
-    C(*sa)[kQL] = reinterpret_cast<C(*)[kQL]>(rb_quad_smem_raw + kQL * kQJ * sizeof(C));  // alpha
+    float2(*sg)[kQJ] = reinterpret_cast<float2(*)[kQJ]>(rb_quad_smem_raw);                       // G_jl [l][j]
+    float2(*sa)[kQL] = reinterpret_cast<float2(*)[kQL]>(rb_quad_smem_raw + kQL * kQJ * sizeof(float2));  // alpha
     const int tid = threadIdx.x, jl = tid & 31, rg = tid >> 5;  // rg: knots 4 rg .. 4 rg + 3
     const int j0 = blockIdx.x * kQJ + jl, k0 = blockIdx.y * kQRows;
-    T tr[kQPer][2], ti[kQPer][2];
+    float tr[kQPer][2], ti[kQPer][2];
 #pragma unroll
     for (int i = 0; i < kQPer; ++i) tr[i][0] = tr[i][1] = ti[i][0] = ti[i][1] = 0;
     for (int l0 = 0; l0 < Nb; l0 += kQL) {
@@ -205,24 +203,24 @@ k_rb_quad(const double *__restrict__ are, const double *__restrict__ aim, int M,
         __syncthreads();
         for (int e = tid; e < lc * kQJ; e += kQThreads) {
             const int l = l0 + e / kQJ, jx = blockIdx.x * kQJ + e % kQJ;
-            sg[e / kQJ][e % kQJ] = jx < Nb ? gt[(size_t)l * Nb + jx] : C{};
+            sg[e / kQJ][e % kQJ] = jx < Nb ? gt[(size_t)l * Nb + jx] : float2{};
         }
         for (int e = tid; e < kQRows * lc; e += kQThreads) {
             const int r = e / lc, l = l0 + e % lc, k = k0 + r;
-            C v{};
+            float2 v{};
             if (k < M) {
-                v.x = (T)are[(size_t)k * Nb + l];
-                v.y = (T)aim[(size_t)k * Nb + l];
+                v.x = (float)are[(size_t)k * Nb + l];
+                v.y = (float)aim[(size_t)k * Nb + l];
             }
             sa[r][e % lc] = v;
         }
         __syncthreads();
 #pragma unroll 2
         for (int l = 0; l < lc; ++l) {
-            const C g0 = sg[l][jl], g1 = sg[l][jl + 32];
+            const float2 g0 = sg[l][jl], g1 = sg[l][jl + 32];
 #pragma unroll
             for (int i = 0; i < kQPer; ++i) {
-                const C x = sa[rg * kQPer + i][l];
+                const float2 x = sa[rg * kQPer + i][l];
                 tr[i][0] += g0.x * x.x + g0.y * x.y;  // G_jl conj(alpha_l)
                 ti[i][0] += g0.y * x.x - g0.x * x.y;
                 tr[i][1] += g1.x * x.x + g1.y * x.y;
@@ -233,12 +231,12 @@ k_rb_quad(const double *__restrict__ are, const double *__restrict__ aim, int M,
 #pragma unroll
     for (int i = 0; i < kQPer; ++i) {
         const int k = k0 + rg * kQPer + i;
-        T c = 0;
+        float c = 0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int j = j0 + 32 * h;
             if (k < M && j < Nb)
-                c += (T)are[(size_t)k * Nb + j] * tr[i][h] - (T)aim[(size_t)k * Nb + j] * ti[i][h];
+                c += (float)are[(size_t)k * Nb + j] * tr[i][h] - (float)aim[(size_t)k * Nb + j] * ti[i][h];
         }
         for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(0xffffffffu, c, o);
         if (jl == 0 && k < M) atomicAdd(q + k, (double)c);
@@ -584,61 +582,98 @@ __global__ void __launch_bounds__(kRbMmaThreads, 1) k_rb_mma(RbMmaArgs a)
 
 // ---- FP64 GEMM ----------------------------------------------------------------------------
 
-constexpr int kRb64Rows = 32, kRb64Modes = 64, kRb64J = 16;
+// The FP64 pipe is the bound (two FMA a cycle and SM), so all that matters is that every SM gets the
+// same share of the multiply-adds and none is spent on padding: a warp takes at most 8 knots (the
+// knots spread evenly over the groups) x 32 modes, one mode a lane, straight from L1 (coalesced
+// basis loads, broadcast coefficients), one warp to a block.  The tiled form
+// before it (32 knots x 64 modes a block) left 100 knots x 3843 modes in 1.6 waves with 28 % of its
+// rows padding.
+constexpr int kRb64Max = 8, kRb64Threads = 32;
 
-// 32 knots x 64 modes per block of 256 threads; thread (ty, tx) owns knots ty, ty + 16 and
-// modes tx + 16 q, q < 4; coefficient and basis tiles staged in shared memory.
-__global__ void __launch_bounds__(256) k_rb_fp64(const double *__restrict__ are,
-                                                 const double *__restrict__ aim,
-                                                 const double *__restrict__ bre,
-                                                 const double *__restrict__ bim, int M, int Nb, int N,
-                                                 const double *__restrict__ scale,
-                                                 double *__restrict__ ore, double *__restrict__ oim)
+template <int R>
+__device__ __forceinline__ void rb64_rows(const double *__restrict__ are, const double *__restrict__ aim,
+                                          const double *__restrict__ bre, const double *__restrict__ bim,
+                                          int k0, int i, int Nb, int N, const double *__restrict__ scale,
+                                          double *__restrict__ ore, double *__restrict__ oim)
 {
-    __shared__ double2 sa[kRb64Rows][kRb64J];
-    __shared__ double2 sb[kRb64J][kRb64Modes];
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int k0 = blockIdx.y * kRb64Rows, i0 = blockIdx.x * kRb64Modes;
-    double accr[2][4] = {}, acci[2][4] = {};
-    for (int j0 = 0; j0 < Nb; j0 += kRb64J) {
-        for (int e = threadIdx.x; e < kRb64Rows * kRb64J; e += 256) {
-            const int r = e / kRb64J, j = e % kRb64J, k = k0 + r, jj = j0 + j;
-            sa[r][j] = (k < M && jj < Nb) ? make_double2(are[(size_t)k * Nb + jj], aim[(size_t)k * Nb + jj])
-                                          : make_double2(0.0, 0.0);
-        }
-        for (int e = threadIdx.x; e < kRb64J * kRb64Modes; e += 256) {
-            const int j = e / kRb64Modes, c = e % kRb64Modes, jj = j0 + j, i = i0 + c;
-            sb[j][c] = (jj < Nb && i < N) ? make_double2(bre[(size_t)jj * N + i], bim[(size_t)jj * N + i])
-                                          : make_double2(0.0, 0.0);
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int j = 0; j < kRb64J; ++j) {
-            const double2 x0 = sa[ty][j], x1 = sa[ty + 16][j];
+    double ar[R], ai[R];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const double2 b = sb[j][tx + 16 * q];
-                accr[0][q] = fma(x0.x, b.x, fma(-x0.y, b.y, accr[0][q]));
-                acci[0][q] = fma(x0.x, b.y, fma(x0.y, b.x, acci[0][q]));
-                accr[1][q] = fma(x1.x, b.x, fma(-x1.y, b.y, accr[1][q]));
-                acci[1][q] = fma(x1.x, b.y, fma(x1.y, b.x, acci[1][q]));
-            }
+    for (int r = 0; r < R; ++r) ar[r] = ai[r] = 0.0;
+    const int col = min(i, N - 1);  // a lane past the end computes the last column and stores nothing
+    const double *xr = are + (size_t)k0 * Nb, *xi = aim + (size_t)k0 * Nb;
+#pragma unroll 2
+    for (int j = 0; j < Nb; ++j) {
+        const double br = __ldg(bre + (size_t)j * N + col), bi = __ldg(bim + (size_t)j * N + col);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const double cr = __ldg(xr + (size_t)r * Nb + j), ci = __ldg(xi + (size_t)r * Nb + j);
+            ar[r] = fma(cr, br, fma(-ci, bi, ar[r]));
+            ai[r] = fma(cr, bi, fma(ci, br, ai[r]));
         }
-        __syncthreads();
     }
+    if (i >= N) return;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int k = k0 + ty + 16 * h;
-        if (k >= M) continue;
-        const double s = scale ? scale[k] : 1.0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int i = i0 + tx + 16 * q;
-            if (i < N) {
-                ore[(size_t)k * N + i] = s * accr[h][q];
-                oim[(size_t)k * N + i] = s * acci[h][q];
-            }
-        }
+    for (int r = 0; r < R; ++r) {
+        const double s = scale ? scale[k0 + r] : 1.0;
+        ore[(size_t)(k0 + r) * N + i] = s * ar[r];
+        oim[(size_t)(k0 + r) * N + i] = s * ai[r];
+    }
+}
+
+__global__ void __launch_bounds__(kRb64Threads)
+k_rb_fp64(const double *__restrict__ are, const double *__restrict__ aim, const double *__restrict__ bre,
+          const double *__restrict__ bim, int M, int Nb, int N, const double *__restrict__ scale,
+          double *__restrict__ ore, double *__restrict__ oim)
+{
+    const int cols = (N + kRb64Threads - 1) / kRb64Threads, groups = (M + kRb64Max - 1) / kRb64Max;
+    const int g = blockIdx.x / cols, i = (blockIdx.x % cols) * kRb64Threads + threadIdx.x;
+    if ((i & ~31) >= N) return;  // a whole warp past the last mode
+    const int k0 = (int)((long long)M * g / groups), rows = (int)((long long)M * (g + 1) / groups) - k0;
+    switch (rows) {
+    case 1: rb64_rows<1>(are, aim, bre, bim, k0, i, Nb, N, scale, ore, oim); break;
+    case 2: rb64_rows<2>(are, aim, bre, bim, k0, i, Nb, N, scale, ore, oim); break;
+    case 3: rb64_rows<3>(are, aim, bre, bim, k0, i, Nb, N, scale, ore, oim); break;
+    case 4: rb64_rows<4>(are, aim, bre, bim, k0, i, Nb, N, scale, ore, oim); break;
+    case 5: rb64_rows<5>(are, aim, bre, bim, k0, i, Nb, N, scale, ore, oim); break;
+    case 6: rb64_rows<6>(are, aim, bre, bim, k0, i, Nb, N, scale, ore, oim); break;
+    case 7: rb64_rows<7>(are, aim, bre, bim, k0, i, Nb, N, scale, ore, oim); break;
+    case 8: rb64_rows<8>(are, aim, bre, bim, k0, i, Nb, N, scale, ore, oim); break;
+    default: break;
+    }
+}
+
+// The renormalisation of the FP64 path, one block per knot: warp w forms q_k's terms of j = 32 w +
+// lane, t_j = sum_l G_jl conj(alpha_l) with coalesced rows of the transposed Gram matrix, and the
+// warps' sums are added in order: s_k = nu_k / sqrt(q_k).  (k_rb_quad leaves 100 knots to 8 blocks:
+// most of the chip's FP64 pipes idle, and two more launches.)
+__global__ void __launch_bounds__(FEW_MAX_BASIS)
+k_rb_scale64(const double *__restrict__ are, const double *__restrict__ aim, int Nb,
+             const double2 *__restrict__ gt, const double *__restrict__ nu,
+             double *__restrict__ scale, unsigned *__restrict__ err)
+{
+    __shared__ double2 a[FEW_MAX_BASIS];
+    __shared__ double part[FEW_MAX_BASIS / 32];
+    const int k = blockIdx.x, j = threadIdx.x;
+    if (j < Nb) a[j] = make_double2(are[(size_t)k * Nb + j], aim[(size_t)k * Nb + j]);
+    __syncthreads();
+    double tr[2] = {0.0, 0.0}, ti[2] = {0.0, 0.0};
+    const int jj = min(j, Nb - 1);
+#pragma unroll 4
+    for (int l = 0; l < Nb; ++l) {
+        const double2 g = __ldg(gt + (size_t)l * Nb + jj), x = a[l];
+        tr[l & 1] = fma(g.x, x.x, fma(g.y, x.y, tr[l & 1]));
+        ti[l & 1] = fma(g.y, x.x, fma(-g.x, x.y, ti[l & 1]));
+    }
+    double q = j < Nb ? a[j].x * (tr[0] + tr[1]) - a[j].y * (ti[0] + ti[1]) : 0.0;
+    for (int o = 16; o > 0; o >>= 1) q += __shfl_down_sync(0xffffffffu, q, o);
+    if ((j & 31) == 0) part[j >> 5] = q;
+    __syncthreads();
+    if (j == 0) {
+        q = 0.0;
+        for (int w = 0; w < (int)blockDim.x / 32; ++w) q += part[w];
+        const double v = nu[k];
+        if (!(v >= 0.0) || !isfinite(v)) atomicOr(err, ERRBIT_NONFINITE);
+        scale[k] = q > 0.0 ? v / sqrt(q) : 0.0;
     }
 }
 
@@ -699,29 +734,25 @@ cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N
         k_rb_scale_tile<<<(M + kTRows - 1) / kTRows, kTThreads, smem, ss>>>(are, aim, M, Nb, gt32, nu,
                                                                              scale, err);
         sc = scale;
+    } else if (nu && fp64) {
+        k_rb_scale64<<<M, (Nb + 31) / 32 * 32, 0, ss>>>(are, aim, Nb, gt64, nu, scale, err);
+        sc = scale;
     } else if (nu) {
         double *q = scale + M;  // the caller's scratch holds scale [M] then q [M]
         e = cudaMemsetAsync(q, 0, sizeof(double) * (size_t)M, ss);
         if (e != cudaSuccess) return fail(e);
         const dim3 grid((Nb + kQJ - 1) / kQJ, (M + kQRows - 1) / kQRows);
-        if (fp64) {
-            e = cudaFuncSetAttribute(k_rb_quad<double, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     rb_quad_smem<double2>());
-            if (e != cudaSuccess) return fail(e);
-            k_rb_quad<double, double2><<<grid, kQThreads, rb_quad_smem<double2>(), ss>>>(are, aim, M, Nb, gt64, q);
-        } else {
-            e = cudaFuncSetAttribute(k_rb_quad<float, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     rb_quad_smem<float2>());
-            if (e != cudaSuccess) return fail(e);
-            k_rb_quad<float, float2><<<grid, kQThreads, rb_quad_smem<float2>(), ss>>>(are, aim, M, Nb, gt32, q);
-        }
+        e = cudaFuncSetAttribute(k_rb_quad, cudaFuncAttributeMaxDynamicSharedMemorySize, kQSmem);
+        if (e != cudaSuccess) return fail(e);
+        k_rb_quad<<<grid, kQThreads, kQSmem, ss>>>(are, aim, M, Nb, gt32, q);
         k_rb_norm<<<(M + 255) / 256, 256, 0, ss>>>(q, nu, M, scale, err);
         sc = scale;
     }
     if (fork && (e = cudaEventRecord(join_ev, side)) != cudaSuccess) return fail(e);
     if (fp64) {
-        dim3 grid((N + kRb64Modes - 1) / kRb64Modes, (M + kRb64Rows - 1) / kRb64Rows);
-        k_rb_fp64<<<grid, 256, 0, st>>>(are, aim, bre, bim, M, Nb, N, sc, ore, oim);
+        const unsigned grid = (unsigned)((N + kRb64Threads - 1) / kRb64Threads) *
+                              (unsigned)((M + kRb64Max - 1) / kRb64Max);
+        k_rb_fp64<<<grid, kRb64Threads, 0, st>>>(are, aim, bre, bim, M, Nb, N, sc, ore, oim);
         return cudaGetLastError();
     }
     const int rows = L.m_tiles * kRbTileN;

@@ -160,3 +160,15 @@ def test_rb_basis_limit(gpu_ctx):
     with pytest.raises(F.FewError) as e:
         F.few_basis_create(gpu_ctx.handle, b, b)
     assert e.value.status == F.FEW_ERR_LIMIT
+
+
+@pytest.mark.parametrize("M", [1, 2, 7, 8, 9, 15, 17])
+def test_rb_fp64_knot_groups(gpu_ctx, M):
+    """Every size of a knot group of the FP64 product, with a last mode warp that is partly past N."""
+    rng = np.random.default_rng(M)
+    alpha = rng.standard_normal((M, 33)) + 1j * rng.standard_normal((M, 33))
+    basis = rng.standard_normal((33, 161)) + 1j * rng.standard_normal((33, 161))
+    nu = rng.uniform(0.5, 2.0, M)
+    g = _gpu_rb(gpu_ctx, alpha, basis, nu, F.FEW_FP64)
+    assert np.all(np.isfinite(g))
+    _check_rows(g, oracle.rb_amplitudes(alpha, basis, nu), alpha, basis, nu, F.FEW_FP64)
