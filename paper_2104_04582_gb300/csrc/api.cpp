@@ -212,88 +212,108 @@ struct SlotPlan {
     int tc_pairs = 0, tc_ks = 0, n_mid = 0, m_top = 0;
 };
 
-few_status plan_slots(const int *l, const int *m, const int *n, int N, SlotPlan &P)
+// Rows of a mode list, dense by signed m (from the largest m down), and the check of the list.
+// The list is looked at in a few flat passes (no trees or hash sets): it is planned on the path of
+// every new trajectory and checked on that of every direct sum.
+struct RowRange {
+    int m_top = 0, m_last = 0, n_rows = 0;
+    int n_min = 0, n_max = 0;        // of the listed modes
+    std::vector<int> lo, hi, first;  // [n_rows] n range (lo > hi: empty), first slot
+    int slots = 0;
+    int slot(int ms, int ns) const { return first[m_top - ms] + hi[m_top - ms] - ns; }
+};
+
+few_status check_modes(const int *l, const int *m, const int *n, int N, RowRange &R)
 {
     if (!l || !m || !n || N < 1) return FEW_ERR_MODES;
-    std::set<std::tuple<int, int, int>> seen;
-    int mmax = 0;
+    int m_top = 0;
     for (int i = 0; i < N; ++i) {
         if (l[i] < 2 || l[i] > kMaxL || m[i] < 0 || m[i] > l[i] || n[i] < -kMaxAbsN ||
             n[i] > kMaxAbsN)
             return FEW_ERR_MODES;
-        if (!seen.insert(std::make_tuple(l[i], m[i], n[i])).second) return FEW_ERR_MODES;
-        mmax = std::max(mmax, m[i]);
+        m_top = std::max(m_top, m[i]);
+        R.n_min = std::min(i ? R.n_min : n[0], n[i]);
+        R.n_max = std::max(i ? R.n_max : n[0], n[i]);
     }
-    // (l, m) pairs
-    std::map<std::pair<int, int>, int> pairs;
+    R.m_top = m_top;
+    R.m_last = -m_top;  // 0 when every mode has m = 0
+    R.n_rows = 2 * m_top + 1;
+    R.lo.assign(R.n_rows, kMaxAbsN + 1);
+    R.hi.assign(R.n_rows, -kMaxAbsN - 1);
+    for (int i = 0; i < N; ++i) {  // the modes and, for m > 0, their (-m, -n) partners
+        int j = m_top - m[i];
+        R.lo[j] = std::min(R.lo[j], n[i]);
+        R.hi[j] = std::max(R.hi[j], n[i]);
+        if (m[i] > 0) {
+            j = m_top + m[i];
+            R.lo[j] = std::min(R.lo[j], -n[i]);
+            R.hi[j] = std::max(R.hi[j], -n[i]);
+        }
+    }
+    R.first.assign(R.n_rows, 0);
+    for (int j = 0; j < R.n_rows; ++j) {
+        R.first[j] = R.slots;
+        if (R.hi[j] >= R.lo[j]) R.slots += R.hi[j] - R.lo[j] + 1;
+    }
+    std::vector<uint64_t> seen(R.slots, 0);  // bit l of each (m, n)
+    for (int i = 0; i < N; ++i) {
+        uint64_t &s = seen[R.slot(m[i], n[i])];
+        if (s >> l[i] & 1) return FEW_ERR_MODES;  // duplicate (l, m, n)
+        s |= (uint64_t)1 << l[i];
+    }
+    return FEW_OK;
+}
+
+few_status plan_slots(const int *l, const int *m, const int *n, int N, SlotPlan &P)
+{
+    RowRange R;
+    const few_status st = check_modes(l, m, n, N, R);
+    if (st) return st;
+    // (l, m) pairs, numbered as they appear
+    std::vector<int> pair_id((kMaxL + 1) * (kMaxL + 1), -1);
     P.mode_pair.resize(N);
     for (int i = 0; i < N; ++i) {
-        auto key = std::make_pair(l[i], m[i]);
-        auto it = pairs.find(key);
-        if (it == pairs.end()) {
-            const int id = (int)P.pair_lm.size();
-            pairs.emplace(key, id);
+        int &id = pair_id[l[i] * (kMaxL + 1) + m[i]];
+        if (id < 0) {
+            id = (int)P.pair_lm.size();
             P.pair_lm.push_back(make_int2(l[i], m[i]));
-            P.mode_pair[i] = id;
-        } else {
-            P.mode_pair[i] = it->second;
         }
+        P.mode_pair[i] = id;
     }
-    // n range of every signed m: the modes and, for m > 0, their (-m, -n) partners
-    bool any_neg = false;
-    for (int i = 0; i < N; ++i) any_neg |= (m[i] > 0);
-    const int m_last = any_neg ? -mmax : 0;
-    const int n_rows = mmax - m_last + 1;
-    std::vector<int> lo(n_rows, kMaxAbsN + 1), hi(n_rows, -kMaxAbsN - 1);
-    auto touch = [&](int ms, int ns) {
-        const int j = mmax - ms;
-        lo[j] = std::min(lo[j], ns);
-        hi[j] = std::max(hi[j], ns);
-    };
-    for (int i = 0; i < N; ++i) {
-        touch(m[i], n[i]);
-        if (m[i] > 0) touch(-m[i], -n[i]);
-    }
-    // rows m = mmax..m_last, slots n = hi..lo in each
-    std::map<std::pair<int, int>, int> slot_of;  // (signed m, n) -> slot
-    int slot = 0, prev_lo = 0;
-    for (int j = 0; j < n_rows; ++j) {
-        const int ms = mmax - j;
-        int L = 0, cur_lo = prev_lo;
-        if (hi[j] >= lo[j]) {
-            L = hi[j] - lo[j] + 1;
-            cur_lo = lo[j];
-            for (int q = hi[j]; q >= lo[j]; --q) slot_of[std::make_pair(ms, q)] = slot++;
-        }
+    // rows m = m_top..m_last, slots n = hi..lo in each
+    int prev_lo = 0;
+    for (int j = 0; j < R.n_rows; ++j) {
+        const bool any = R.hi[j] >= R.lo[j];
+        const int L = any ? R.hi[j] - R.lo[j] + 1 : 0, cur_lo = any ? R.lo[j] : prev_lo;
         P.rows.push_back(make_int2(L, j == 0 ? 0 : prev_lo - cur_lo));
-        P.row_slot.push_back(make_int4(slot - L, L ? hi[j] : -1, L ? lo[j] : 0, 0));
+        P.row_slot.push_back(make_int4(R.first[j], L ? R.hi[j] : -1, L ? R.lo[j] : 0, 0));
         prev_lo = cur_lo;
     }
-    const int n_lo = *std::min_element(lo.begin(), lo.end());
-    const int n_hi = *std::max_element(hi.begin(), hi.end());
+    const int n_lo = *std::min_element(R.lo.begin(), R.lo.end());
+    const int n_hi = *std::max_element(R.hi.begin(), R.hi.end());
     P.n_mid = n_lo + (n_hi - n_lo) / 2;
     const int half = n_hi - P.n_mid;
-    P.m_top = mmax;
-    if (mmax < kTcMaxPairs && half <= kTcMaxHalf) {
-        P.tc_pairs = mmax + 1;
+    P.m_top = R.m_top;
+    if (R.m_top < kTcMaxPairs && half <= kTcMaxHalf) {
+        P.tc_pairs = R.m_top + 1;
         P.tc_ks = half / 8 + 1;
     }
-    P.n_slots = slot;
-    P.m_last = m_last;
+    P.n_slots = R.slots;
+    P.m_last = R.m_last;
     P.lo_last = prev_lo;
-    // contributions CSR
-    std::vector<std::vector<int>> lists(slot);
+    // contributions CSR, each slot's in list order
+    P.slot_ptr.assign(R.slots + 1, 0);
     for (int i = 0; i < N; ++i) {
-        lists[slot_of[std::make_pair(m[i], n[i])]].push_back(2 * i);
-        if (m[i] > 0) lists[slot_of[std::make_pair(-m[i], -n[i])]].push_back(2 * i + 1);
+        ++P.slot_ptr[R.slot(m[i], n[i]) + 1];
+        if (m[i] > 0) ++P.slot_ptr[R.slot(-m[i], -n[i]) + 1];
     }
-    P.slot_ptr.assign(slot + 1, 0);
-    for (int s = 0; s < slot; ++s) P.slot_ptr[s + 1] = P.slot_ptr[s] + (int)lists[s].size();
-    P.contrib.clear();
-    P.contrib.reserve(P.slot_ptr[slot]);
-    for (int s = 0; s < slot; ++s)
-        for (int code : lists[s])
-            P.contrib.push_back(make_int2(code, 2 * P.mode_pair[code >> 1] + (code & 1)));
+    for (int s = 0; s < R.slots; ++s) P.slot_ptr[s + 1] += P.slot_ptr[s];
+    P.contrib.resize(P.slot_ptr[R.slots]);
+    std::vector<int> at(P.slot_ptr.begin(), P.slot_ptr.end() - 1);
+    for (int i = 0; i < N; ++i) {
+        P.contrib[at[R.slot(m[i], n[i])]++] = make_int2(2 * i, 2 * P.mode_pair[i]);
+        if (m[i] > 0) P.contrib[at[R.slot(-m[i], -n[i])]++] = make_int2(2 * i + 1, 2 * P.mode_pair[i] + 1);
+    }
     return FEW_OK;
 }
 
@@ -1226,8 +1246,8 @@ few_status few_direct_sum(few_ctx *ctx, const double *pphi, const double *pr, co
     if (!ctx || !pphi || !pr || !are || !aim || !out) return FEW_ERR_INVALID_ARG;
     if (prec != FEW_FP64 && prec != FEW_MIXED) return FEW_ERR_INVALID_ARG;
     if (!is_fin(theta) || !is_fin(phi) || !is_fin(scale) || ns < 0) return FEW_ERR_INVALID_ARG;
-    SlotPlan P;
-    few_status st = plan_slots(l, m, n, N, P);  // validates the modes
+    RowRange modes;
+    few_status st = check_modes(l, m, n, N, modes);
     if (st) return st;
     if (ns == 0) return FEW_OK;
     std::lock_guard<std::recursive_mutex> lk(ctx->mu);
@@ -1249,7 +1269,8 @@ few_status few_direct_sum(few_ctx *ctx, const double *pphi, const double *pr, co
         const int *dl = reinterpret_cast<const int *>(b + mc_bytes);
         cudaError_t e = launch_direct(pphi, pr, are, aim, (long long)ns, dl, dl + stride,
                                       dl + 2 * stride, N, theta, phi, scale, prec == FEW_FP64, out,
-                                      out_c64 ? 1 : 0, b, ctx->sm_count, s);
+                                      out_c64 ? 1 : 0, b, modes.m_top, modes.n_min, modes.n_max,
+                                      ctx->sm_count, s);
         if (e != cudaSuccess) {
             (void)cudaGetLastError();
             st = FEW_ERR_CUDA;

@@ -127,11 +127,104 @@ k_direct(const double *__restrict__ pphi, const double *__restrict__ pr,
     }
 }
 
+// FP64 with exponential tables.  The plain path is bound by the FP64 pipe, and sincospi per mode
+// and sample was most of it (~60 of ~75 FP64 operations).  A mode list has few distinct m and n
+// (11 + 31 against 1953 modes on the |n| <= 15 grid), so each warp first fills a table of
+// e^{i m Phi_phi} (m = 0 .. m_top) and e^{i n Phi_r} (n_lo .. n_hi) for its sample in shared
+// memory, and a mode costs 12 FP64 operations: e^{i Phi} = the product of two entries, w = A
+// e^{-i Phi}, and
+//     h += w Y+ + conj(w) Y- = [a Re w - b Im w] + i [g Re w + d Im w]   (a, b, g, d as above).
+// Small blocks (4 samples), so that the last wave is spread evenly.  4001 samples x 1953 modes:
+// see launch_direct for both sides.
+constexpr int kTabThreads = 128;
+constexpr int kTabMaxEntries = 512;  // (m_top + 1) + (n_hi - n_lo + 1): 8 KB a warp
+
+struct alignas(16) ModeConstTab {
+    double a, b, g, d;
+    int m, n, pad[2];  // table entries of m and n
+};
+
+__global__ void k_mode_consts_tab(const int *__restrict__ l, const int *__restrict__ m,
+                                  const int *__restrict__ n, int N, double theta, double phi,
+                                  int m_top, int n_lo, ModeConstTab *__restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    const double2 yp = swsh_m2(l[i], m[i], theta, phi);
+    double2 ym = make_double2(0.0, 0.0);
+    if (m[i] > 0) {
+        ym = swsh_m2(l[i], -m[i], theta, phi);
+        if (l[i] & 1) ym = make_double2(-ym.x, -ym.y);
+    }
+    out[i] = ModeConstTab{yp.x + ym.x, yp.y - ym.y, yp.y + ym.y, yp.x - ym.x,
+                          m[i], m_top + 1 + n[i] - n_lo, {0, 0}};
+}
+
+__global__ void __launch_bounds__(kTabThreads)
+k_direct_tab(const double *__restrict__ pphi, const double *__restrict__ pr,
+             const double *__restrict__ are, const double *__restrict__ aim, long long ns, int N,
+             const ModeConstTab *__restrict__ mc, int m_top, int n_lo, int entries, double scale,
+             void *__restrict__ out, int out_c64)
+{
+    extern __shared__ __align__(16) double2 dir_tab[];
+    const double kInv2Pi = 0.15915494309189533577;
+    const int lane = threadIdx.x & 31;
+    const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // sample
+    if (i >= ns) return;  // a whole warp
+    double2 *tab = dir_tab + (threadIdx.x >> 5) * entries;
+    const double xp = reduce_2pi(pphi[i]) * kInv2Pi, xr = reduce_2pi(pr[i]) * kInv2Pi;
+    const double fphi = xp - rint(xp), fr = xr - rint(xr);
+    for (int e = lane; e < entries; e += 32) {
+        const double x = e <= m_top ? e * fphi : (double)(n_lo + e - m_top - 1) * fr;
+        double s, c;
+        sincospi(2.0 * (x - rint(x)), &s, &c);
+        tab[e] = make_double2(c, s);
+    }
+    __syncwarp();
+    const double *ar = are + (size_t)i * N, *ai = aim + (size_t)i * N;
+    double hr = 0.0, hi = 0.0;
+#pragma unroll 4
+    for (int j = lane; j < N; j += 32) {
+        const double vr = __ldcs(ar + j), vi = __ldcs(ai + j);
+        const double2 y0 = *reinterpret_cast<const double2 *>(&mc[j].a);
+        const double2 y1 = *reinterpret_cast<const double2 *>(&mc[j].g);
+        const int2 mn = *reinterpret_cast<const int2 *>(&mc[j].m);
+        const double2 p = tab[mn.x], q = tab[mn.y];
+        const double co = fma(p.x, q.x, -p.y * q.y), s = fma(p.y, q.x, p.x * q.y);
+        const double wr = fma(vr, co, vi * s), wi = fma(vi, co, -vr * s);
+        hr = fma(wr, y0.x, fma(-wi, y0.y, hr));
+        hi = fma(wr, y1.x, fma(wi, y1.y, hi));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        hr += __shfl_down_sync(0xffffffffu, hr, o);
+        hi += __shfl_down_sync(0xffffffffu, hi, o);
+    }
+    if (lane == 0) {
+        if (out_c64)
+            reinterpret_cast<float2 *>(out)[i] = make_float2((float)(hr * scale), (float)(hi * scale));
+        else
+            reinterpret_cast<double2 *>(out)[i] = make_double2(hr * scale, hi * scale);
+    }
+}
+
 cudaError_t launch_direct(const double *pphi, const double *pr, const double *are,
                           const double *aim, long long ns, const int *l, const int *m, const int *n,
                           int N, double theta, double phi, double scale, bool fp64, void *out,
-                          int out_c64, void *mode_consts, int sm_count, cudaStream_t st)
+                          int out_c64, void *mode_consts, int m_top, int n_lo, int n_hi, int sm_count,
+                          cudaStream_t st)
 {
+    // the tables pay wherever they hold fewer exponentials than there are modes
+    const int entries = m_top + 1 + n_hi - n_lo + 1;
+    if (fp64 && entries <= kTabMaxEntries && entries < N && ns > 0) {
+        auto *mc = static_cast<ModeConstTab *>(mode_consts);
+        k_mode_consts_tab<<<(N + 63) / 64, 64, 0, st>>>(l, m, n, N, theta, phi, m_top, n_lo, mc);
+        const int per = kTabThreads / 32;
+        const int smem = per * entries * (int)sizeof(double2);
+        k_direct_tab<<<(unsigned)((ns + per - 1) / per), kTabThreads, smem, st>>>(
+            pphi, pr, are, aim, ns, N, mc, m_top, n_lo, entries, scale, out, out_c64);
+        return cudaGetLastError();
+    }
     // one wave of resident blocks (8 warps, i.e. 8 samples, per block per round)
     static int resident[2] = {0, 0};
     int &rb = resident[fp64 ? 1 : 0];
@@ -159,6 +252,7 @@ cudaError_t launch_direct(const double *pphi, const double *pr, const double *ar
     return cudaGetLastError();
 }
 
+static_assert(sizeof(ModeConstTab) == sizeof(ModeConst<double>), "one scratch size for both");
 size_t direct_mode_const_bytes(int N) { return sizeof(ModeConst<double>) * (size_t)N; }
 
 }  // namespace fewsum

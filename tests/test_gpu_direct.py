@@ -114,3 +114,23 @@ def test_direct_mixed_unaligned_amplitudes(gpu_ctx):
     assert gpu_ctx.sync_status() == F.FEW_OK
     o = oracle.direct_dense(pphi, pr, w.modes, are, aim, w.theta, w.phi, 1.0, oracle_threads())
     assert oracle.mismatch(to_host(out), o) <= MIXED_MISMATCH
+
+
+@pytest.mark.parametrize("ms,ns_range,ns", [
+    ([0], range(0, 3), 1),            # as many table entries as modes: the per-mode exponentials
+    ([0, 1, 2], range(-2, 3), 5),     # tables, one warp past a block of four samples
+    ([3], range(-200, 309), 4),       # gaps below m_top, 4 + 509 entries: past the tables' limit
+    ([2], range(-200, 309), 4),       # 3 + 509 entries: the largest table
+])
+def test_direct_fp64_table_edges(gpu_ctx, ms, ns_range, ns):
+    """Both sides of the FP64 path's choice between exponential tables and per-mode exponentials."""
+    rng = np.random.default_rng(7)
+    modes = np.asarray([(4, m, n) for m in ms for n in ns_range] + [(5, m, n) for m in ms for n in ns_range][:-1]
+                       if len(ms) * len(ns_range) > 3 else [(4, m, n) for m in ms for n in ns_range],
+                       dtype=np.int32)
+    N = len(modes)
+    pphi, pr = rng.uniform(-1e5, 1e5, (2, ns))
+    are, aim = rng.standard_normal((2, ns, N))
+    g = _gpu_direct(gpu_ctx, pphi, pr, are, aim, modes, 0.9, 2.1, F.FEW_FP64)
+    o = oracle.direct_dense(pphi, pr, modes, are, aim, 0.9, 2.1)
+    assert rel_l2(g, o) <= FP64_REL_L2
