@@ -357,12 +357,12 @@ struct LaunchPlan {
     int variant = kVariantFp64;
     int grid = 0, threads = 0, R = 0, smem = 0, total_pairs = 0, total_fold = 0;
     int total_anchor_segs = 0;
-    int total_segs = 0, total_tiles = 0, ks = 0;  // kVariantTc
+    int total_segs = 0, total_tiles = 0, ks = 0;  // tensor-core variants
 };
 
 struct few_batch {
-    // The waves of one summation variant: a mixed batch may need both (kVariantTc and
-    // kVariantScalar), which then run one after the other.
+    // The waves of one summation variant: a batch may need both the tensor-core and the scalar
+    // one of its precision, which then run one after the other.
     struct Part {
         void *blob_dev = nullptr;
         void *scratch_dev = nullptr;
@@ -385,7 +385,7 @@ struct PlanImage {
     size_t off_waves = 0, off_cta = 0, off_seg = 0, off_anc = 0;
     size_t scratch_bytes = 0;
     std::vector<size_t> fcoef_off, ylm_off, anchor_off;
-    size_t recs_off = 0;  // kVariantTc: tile records of all waves
+    size_t recs_off = 0;  // tensor-core variants: tile records of all waves
     std::vector<std::vector<int64_t>> seg;  // per wave: segment sample ranges [K]
     bool fp64 = false;
     LaunchPlan launch;
@@ -436,7 +436,7 @@ few_status validate_request(const few_request &r, bool need_device_out)
 }
 
 // Whether a request's mode set fits the tensor-core summation (kTcMaxPairs, kTcMaxHalf).
-bool tc_fits(const few_request &r) { return r.prec == FEW_MIXED && r.traj->plan.tc_pairs > 0; }
+bool tc_fits(const few_request &r) { return r.traj->plan.tc_pairs > 0; }
 
 // Build the host image of a plan for `n` requests of one precision; tc: by the tensor-core
 // summation (every request fits it).
@@ -466,7 +466,7 @@ few_status build_image(few_ctx *c, const few_request *reqs, int n, bool tc, Plan
         segments(r.traj->t_host.data(), r.traj->K, r.t0, r.dt, r.n_samples, P.seg[q].data());
     }
     if (tc) {
-        L.variant = kVariantTc;
+        L.variant = P.fp64 ? kVariantTc64 : kVariantTc;
         int64_t tiles = 0;
         for (int q = 0; q < n; ++q)
             for (int k = 0; k + 1 < reqs[q].traj->K; ++k)
@@ -481,14 +481,14 @@ few_status build_image(few_ctx *c, const few_request *reqs, int n, bool tc, Plan
     size_t off = align_up(sizeof(PlanHdr), 64);
     P.off_waves = off;
     off = align_up(off + sizeof(WaveDev) * n, 64);
-    P.off_cta = off;  // kVariantTc: int first tiles instead
+    P.off_cta = off;  // tensor-core variants: int first tiles instead
     off = align_up(off + sizeof(CtaStart) * (L.grid + 1), 64);
     P.off_seg = off;
     size_t seg_ints = 0;
     for (int q = 0; q < n; ++q) seg_ints += reqs[q].traj->K;
     off = align_up(off + sizeof(int) * seg_ints, 64);
     P.off_anc = off;  // per wave: first anchor (or tile) of each segment, then the wave's total
-    if (!P.fp64) off += sizeof(int) * seg_ints;
+    if (!P.fp64 || tc) off += sizeof(int) * seg_ints;
     off = align_up(off, 256);
     P.blob.assign(off, 0);
 
@@ -502,8 +502,7 @@ few_status build_image(few_ctx *c, const few_request *reqs, int n, bool tc, Plan
         const few_traj *tr = reqs[q].traj;
         P.fcoef_off[q] = s_off;
         if (tc)
-            s_off = align_up(s_off + (size_t)tr->S * (tc_table_bytes(tr->plan.tc_pairs, tr->plan.tc_ks) +
-                                                      sizeof(float)), 256);
+            s_off = align_up(s_off + tr->S * tc_segment_bytes(P.fp64, tr->plan.tc_pairs, tr->plan.tc_ks), 256);
         else
             s_off = align_up(s_off + (size_t)tr->S * tr->plan.n_slots * slot_bytes, 256);
         P.ylm_off[q] = s_off;
@@ -596,7 +595,7 @@ void fill_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P, unsign
     int *seg = reinterpret_cast<int *>(P.blob.data() + P.off_seg);
     int *anc = reinterpret_cast<int *>(P.blob.data() + P.off_anc);
     LaunchPlan &L = P.launch;
-    const bool tc = L.variant == kVariantTc;
+    const bool tc = is_tc(L.variant);
     size_t seg_pos = 0;
     int pair_begin = 0, fold_begin = 0, anchor_seg_begin = 0, seg_begin = 0;
     std::vector<int> tile_begin(1, 0);
@@ -633,14 +632,18 @@ void fill_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P, unsign
             }
             anc[seg_pos + tr->K - 1] = a;
             W.tab = scratch_dev + P.fcoef_off[q];
-            W.tab_inv = reinterpret_cast<float *>(
-                W.tab + (size_t)tr->S * tc_table_bytes(tr->plan.tc_pairs, tr->plan.tc_ks));
+            if (P.fp64)
+                W.seg64 = reinterpret_cast<TcSeg64 *>(
+                    W.tab + (size_t)tr->S * tc64_table_bytes(tr->plan.tc_pairs, tr->plan.tc_ks));
+            else
+                W.tab_inv = reinterpret_cast<float *>(
+                    W.tab + (size_t)tr->S * tc_table_bytes(tr->plan.tc_pairs, tr->plan.tc_ks));
             W.tile_off = reinterpret_cast<const int *>(blob_dev + P.off_anc) + seg_pos;
             W.tile_begin = tile_begin[q];
             W.seg_begin = seg_begin;
             seg_begin += tr->S;
             tile_begin.push_back(tile_begin[q] + a);
-            tile_cost.push_back(tc_tile_cost(tr->plan.tc_pairs, tr->plan.tc_ks));
+            tile_cost.push_back(tc_tile_cost(P.fp64, tr->plan.tc_pairs, tr->plan.tc_ks));
         } else if (!P.fp64) {
             int a = 0;
             for (int k = 0; k + 1 < tr->K; ++k) {
@@ -702,17 +705,20 @@ cudaError_t launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, const LaunchPlan 
     auto tm = [&](int slot, bool end) {
         if (mark) tmark(c, slot, end, st);
     };
-    const bool fp64 = P.variant == kVariantFp64;
+    const bool fp64 = P.variant == kVariantFp64 || P.variant == kVariantTc64;
     cudaError_t e;
-    if (P.variant == kVariantTc) {
+    if (is_tc(P.variant)) {
         tm(1, false);
-        if ((e = launch_ylm(hdr_dev, P.total_pairs, false, st)) != cudaSuccess) return e;
+        if ((e = launch_ylm(hdr_dev, P.total_pairs, fp64, st)) != cudaSuccess) return e;
         tm(1, true);
         tm(2, false);
-        if ((e = launch_fold_tc(hdr_dev, P.total_segs, P.total_tiles, st)) != cudaSuccess) return e;
+        e = fp64 ? launch_fold_tc64(hdr_dev, P.total_segs, P.total_tiles, st)
+                 : launch_fold_tc(hdr_dev, P.total_segs, P.total_tiles, st);
+        if (e != cudaSuccess) return e;
         tm(2, true);
         tm(3, false);
-        if ((e = launch_sum_tc(hdr_dev, P.grid, P.ks, st)) != cudaSuccess) return e;
+        e = fp64 ? launch_sum_tc64(hdr_dev, P.grid, P.ks, st) : launch_sum_tc(hdr_dev, P.grid, P.ks, st);
+        if (e != cudaSuccess) return e;
         tm(3, true);
         return cudaSuccess;
     }
@@ -823,7 +829,9 @@ few_status few_ctx_create(few_ctx **out, int device, size_t hbm_budget_bytes)
             return fail(FEW_ERR_CUDA);
     if (cudaMalloc(&c->d_err, sizeof(unsigned)) != cudaSuccess) return fail(FEW_ERR_NOMEM);
     if (cudaMemset(c->d_err, 0, sizeof(unsigned)) != cudaSuccess) return fail(FEW_ERR_CUDA);
-    if (sum_configure() != cudaSuccess || tc_configure() != cudaSuccess) return fail(FEW_ERR_CUDA);
+    if (sum_configure() != cudaSuccess || tc_configure() != cudaSuccess ||
+        tc64_configure() != cudaSuccess)
+        return fail(FEW_ERR_CUDA);
     for (auto &e : c->tev)
         if (cudaEventCreate(&e) != cudaSuccess) return fail(FEW_ERR_CUDA);
     *out = c;

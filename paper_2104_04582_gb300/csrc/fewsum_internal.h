@@ -31,8 +31,10 @@ constexpr int kMinStageSlots = 16, kMaxStageSlots = 4096;
 enum : int {
     kVariantFp64 = 0,   // FP64 throughout; slot = 8 doubles
     kVariantScalar = 1,  // mixed: FP64 phases at anchors, FP32 everything else; slot = 8 floats
-    kVariantTc = 2       // mixed: the sum over n on the tensor cores (tcsum.cu)
+    kVariantTc = 2,      // mixed: the sum over n on the tensor cores (tcsum.cu)
+    kVariantTc64 = 3     // FP64: the same in exact integer slices (tcsum64.cu)
 };
+inline bool is_tc(int variant) { return variant == kVariantTc || variant == kVariantTc64; }
 
 // Tensor-core summation (tcsum.cu): tiles of kTcTile consecutive samples of one segment, starting
 // at multiples of kTcTile (so a sample's arithmetic does not depend on the request's slicing).
@@ -49,8 +51,9 @@ struct alignas(128) TileRec {
     long long phi[4], r[4];
     int i0, s0, s1;       // first sample of lane 0; the segment's samples [s0, s1)
     int tile_end;         // first tile after the segment
-    float u0, du;         // u of sample i: u0 + (i - s0) du
-    const float *inv;     // inverse of the segment table's power-of-two scale
+    float u0, du;         // mixed: u of sample i is u0 + (i - s0) du; FP64: the next 32 bits (units of
+                          //   2^-96 turn) of the phases' c3, as int bits
+    const void *seg;      // mixed: float, inverse of the table's power-of-two scale; FP64: TcSeg64
     const unsigned char *tab;  // the segment's operand table
     void *out;
     int pairs, ks;        // row pairs, K steps of 16 (8 powers of z_r each)
@@ -58,6 +61,14 @@ struct alignas(128) TileRec {
     int c64;
 };
 static_assert(sizeof(TileRec) == 128, "one line");
+// FP64 tensor-core summation (tcsum64.cu): what a segment's tiles read beside its table.
+constexpr int kTc64Slices = 7;  // 8-bit digits per operand
+struct TcSeg64 {
+    double inv1, inv2;        // output factors: table scale and fixed-point unit
+    double tk, ih, t0, dt;    // u = (t0 + i dt - tk) ih
+    int shift;                // fixed-point sums are shifted left by this (right if negative)
+    int pad[3];
+};
 
 // Phase anchors of the mixed path: the FP64 phase splines are evaluated and reduced modulo one
 // turn at every kAnchorGroup-th sample (absolute sample index a = kAnchorGroup * q), together
@@ -153,7 +164,8 @@ struct WaveDev {
     const int *anchor_off;  // mixed plans: [K] first anchor of each segment, then the total
     int anchor_seg_begin; // first global segment index of this wave (anchor kernel grid)
     unsigned char *tab;   // tensor-core plans: [S] operand tables of tc_table_bytes
-    float *tab_inv;       //   [S] inverse table scales
+    float *tab_inv;       //   [S] inverse table scales (mixed)
+    TcSeg64 *seg64;       //   [S] segment constants (FP64)
     const int *tile_off;  //   [K] first tile of each segment, then the total
     int tile_begin;       //   first tile of this wave in the plan
     int seg_begin;        //   first segment of this wave in the plan
@@ -215,13 +227,27 @@ cudaError_t launch_sum(const PlanHdr *hdr_dev, int grid, int threads, int sample
 // Bytes of one segment's tensor-core operand table: fp16 high and low parts, N = 16 pairs rows of
 // 16 ks columns each.
 __host__ __device__ inline int tc_table_bytes(int pairs, int ks) { return 1024 * pairs * ks; }
-// Relative cost of one tile: the MMAs' cycles plus the per-sample work around them.
-inline double tc_tile_cost(int pairs, int ks) { return 24.0 * pairs * ks + 300.0; }
+// FP64: 7 digit slices, each row pair's 16 rows of 16 ks fp16 columns together.
+__host__ __device__ inline int tc64_table_bytes(int pairs, int ks) { return 512 * kTc64Slices * pairs * ks; }
+// Bytes of a segment's table and constants.
+inline size_t tc_segment_bytes(bool fp64, int pairs, int ks)
+{
+    return fp64 ? tc64_table_bytes(pairs, ks) + sizeof(TcSeg64) : tc_table_bytes(pairs, ks) + sizeof(float);
+}
+// Relative cost of one tile (cycles): the MMAs, or the per-sample work around them.
+inline double tc_tile_cost(bool fp64, int pairs, int ks)
+{
+    if (fp64) return pairs * (364.0 * ks > 1000.0 ? 364.0 * ks : 1000.0) + 1200.0 * ks + 1600.0;
+    return 24.0 * pairs * ks + 300.0;
+}
 inline int tiles_in_segment(int s_begin, int s_end)
 {
     return s_end > s_begin ? (s_end - 1) / kTcTile - s_begin / kTcTile + 1 : 0;
 }
 cudaError_t tc_configure();
+cudaError_t tc64_configure();
+cudaError_t launch_fold_tc64(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st);
+cudaError_t launch_sum_tc64(const PlanHdr *hdr_dev, int grid, int ks, cudaStream_t st);
 cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st);
 // ks: the most K steps of any wave of the plan.
 cudaError_t launch_sum_tc(const PlanHdr *hdr_dev, int grid, int ks, cudaStream_t st);

@@ -111,11 +111,12 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     const size_t off_cta = up(off_waves + sizeof(WaveDev), 64);
     const size_t off_seg = up(off_cta + sizeof(CtaStart) * (grid + 1), 64);
     const size_t off_anc = up(off_seg + sizeof(int) * K, 64);
-    const size_t blob_bytes = up(off_anc + (fp64 ? 0 : sizeof(int) * K), 256);
-    if (blob_bytes > kBlobMax) return FEW_ERR_LIMIT;
+    const size_t blob_all = up(off_anc + sizeof(int) * K, 256);  // with anchors or tiles
+    const size_t blob_plain = fp64 ? up(off_anc, 256) : blob_all;
+    if (blob_plain > kBlobMax) return FEW_ERR_LIMIT;
 
     std::lock_guard<std::mutex> blk(g_blob_mu);
-    std::memset(g_blob, 0, blob_bytes);
+    std::memset(g_blob, 0, blob_all <= kBlobMax ? blob_all : blob_plain);
     PlanHdr *hdr = reinterpret_cast<PlanHdr *>(g_blob);
     WaveDev *W = reinterpret_cast<WaveDev *>(g_blob + off_waves);
     CtaStart *cta = reinterpret_cast<CtaStart *>(g_blob + off_cta);
@@ -146,15 +147,17 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     const size_t anc_bytes = up(sizeof(Anchor) * (size_t)n_anchors, 256);
     // what fits is decided by the plain layout; the tensor-core plan (tile records, operand tables
     // and their scales instead of anchors and folded coefficients) is taken where it fits too
-    if (blob_bytes + fcoef_bytes + ylm_bytes + anc_bytes > kScratchBytes) return FEW_ERR_LIMIT;
+    if (blob_plain + fcoef_bytes + ylm_bytes + anc_bytes > kScratchBytes) return FEW_ERR_LIMIT;
     int n_tiles = 0;
-    if (!fp64 && v.tc_pairs > 0)
+    if (v.tc_pairs > 0)
         for (int k = 0; k + 1 < K; ++k) n_tiles += tiles_in_segment(seg[k], seg[k + 1]);
-    const size_t tab_bytes = up((size_t)S * tc_table_bytes(v.tc_pairs, v.tc_ks), 256);
-    const size_t inv_bytes = up((size_t)S * sizeof(float), 256);
+    const size_t tab_bytes =
+        up((size_t)S * (fp64 ? tc64_table_bytes(v.tc_pairs, v.tc_ks) : tc_table_bytes(v.tc_pairs, v.tc_ks)), 256);
+    const size_t inv_bytes = up((size_t)S * (fp64 ? sizeof(TcSeg64) : sizeof(float)), 256);
     const size_t rec_bytes = sizeof(TileRec) * (size_t)n_tiles;
-    const bool tc = n_tiles > 0 &&
-                    blob_bytes + rec_bytes + tab_bytes + inv_bytes + ylm_bytes <= kScratchBytes;
+    const bool tc = n_tiles > 0 && blob_all <= kBlobMax &&
+                    blob_all + rec_bytes + tab_bytes + inv_bytes + ylm_bytes <= kScratchBytes;
+    const size_t blob_bytes = tc ? blob_all : blob_plain;
     const int grid_tc = n_tiles < v.sm_count ? n_tiles : v.sm_count;
     unsigned char *d_fcoef = base + blob_bytes;
     unsigned char *d_ylm = tc ? base + blob_bytes + rec_bytes + tab_bytes + inv_bytes : d_fcoef + fcoef_bytes;
@@ -188,7 +191,10 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
         }
         anc[K - 1] = a;
         W->tab = base + blob_bytes + rec_bytes;
-        W->tab_inv = reinterpret_cast<float *>(W->tab + tab_bytes);
+        if (fp64)
+            W->seg64 = reinterpret_cast<TcSeg64 *>(W->tab + tab_bytes);
+        else
+            W->tab_inv = reinterpret_cast<float *>(W->tab + tab_bytes);
         W->tile_off = reinterpret_cast<const int *>(base + off_anc);
         W->tile_begin = 0;
         W->seg_begin = 0;
@@ -221,7 +227,7 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     hdr->buf_bytes = buf_bytes;
     hdr->stage_slots = stage_slots;
     hdr->ring = kDefaultRing;
-    hdr->variant = tc ? kVariantTc : variant;
+    hdr->variant = tc ? (fp64 ? kVariantTc64 : kVariantTc) : variant;
     hdr->waves = reinterpret_cast<const WaveDev *>(base + off_waves);
     hdr->cta = reinterpret_cast<const CtaStart *>(base + off_cta);
     hdr->err = v.d_err;
@@ -236,9 +242,10 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     if (cudaGetLastError() != cudaSuccess) return FEW_ERR_CUDA;
     const PlanHdr *hd = reinterpret_cast<const PlanHdr *>(base);
     if (tc) {
-        if (launch_ylm(hd, v.n_pairs, false, s) != cudaSuccess ||
-            launch_fold_tc(hd, S, n_tiles, s) != cudaSuccess ||
-            launch_sum_tc(hd, grid_tc, v.tc_ks, s) != cudaSuccess) {
+        if (launch_ylm(hd, v.n_pairs, fp64, s) != cudaSuccess ||
+            (fp64 ? launch_fold_tc64(hd, S, n_tiles, s) : launch_fold_tc(hd, S, n_tiles, s)) != cudaSuccess ||
+            (fp64 ? launch_sum_tc64(hd, grid_tc, v.tc_ks, s) : launch_sum_tc(hd, grid_tc, v.tc_ks, s)) !=
+                cudaSuccess) {
             (void)cudaGetLastError();
             return FEW_ERR_CUDA;
         }

@@ -33,8 +33,7 @@
 
 #include "fewsum_internal.h"
 #include "fold_slot.cuh"
-#include "phase_eval.cuh"
-#include "tcgen05.cuh"
+#include "tctile.cuh"
 
 namespace fewsum {
 
@@ -49,71 +48,6 @@ constexpr int kTcMaxTable = 1024 * kTcMaxPairs * kTcMaxKs;
 constexpr uint32_t kTcDStride = 192, kTcECol = 384, kTcEStride = 64, kTcELo = 32;  // tmem columns
 
 __device__ __forceinline__ float pow2(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
-
-// A value in turns as 2^-64 turn units modulo one turn.
-__device__ __forceinline__ long long turns_fixed(double y)
-{
-    return __double2ll_rn((y - rint(y)) * 18446744073709551616.0);
-}
-
-__device__ int wave_of_seg(const PlanHdr &h, int g)
-{
-    int lo = 0, hi = h.n_waves - 1;
-    while (lo < hi) {  // largest w with seg_begin <= g
-        const int mid = (lo + hi + 1) >> 1;
-        if (h.waves[mid].seg_begin <= g) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// Record of tile T: its segment, the FP64 phases at its first sample and their Taylor expansion.
-__device__ void fill_record(const PlanHdr &h, int T)
-{
-    int lo = 0, hi = h.n_waves - 1;
-    while (lo < hi) {  // largest w with tile_begin <= T
-        const int mid = (lo + hi + 1) >> 1;
-        if (h.waves[mid].tile_begin <= T) lo = mid; else hi = mid - 1;
-    }
-    const WaveDev &W = h.waves[lo];
-    const TrajDev &tr = W.tr;
-    const int t = T - W.tile_begin;
-    int s = 0, e = tr.S - 1;
-    while (s < e) {  // largest s with tile_off[s] <= t: the segment that holds tile t
-        const int mid = (s + e + 1) >> 1;
-        if (W.tile_off[mid] <= t) s = mid; else e = mid - 1;
-    }
-    TileRec r;
-    r.s0 = W.seg_start[s];
-    r.s1 = W.seg_start[s + 1];
-    r.i0 = (r.s0 / kTcTile + (t - W.tile_off[s])) * kTcTile;
-    r.tile_end = W.tile_begin + W.tile_off[s + 1];
-    const SegPhase sp = seg_phase(tr, s, W.dphi_phi, W.dphi_r);
-    const double kInv2Pi = 0.15915494309189533577;
-    const double u = (fma((double)max(r.i0, r.s0), W.dt, W.t0) - sp.tk) * sp.ih, du = W.dt * sp.ih;
-    double all = 0.0;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const double *p = k ? sp.pr : sp.pphi;
-        long long *c = k ? r.r : r.phi;
-        const double f0 = fma(fma(fma(p[2], u, p[1]), u, p[0]), u, k ? sp.c0r : sp.c0phi) * kInv2Pi;
-        c[0] = turns_fixed(f0);
-        c[1] = turns_fixed(fma(fma(3.0 * p[2], u, 2.0 * p[1]), u, p[0]) * du * kInv2Pi);
-        c[2] = turns_fixed(fma(3.0 * p[2], u, p[1]) * du * du * kInv2Pi);
-        c[3] = turns_fixed(p[2] * du * du * du * kInv2Pi);
-        all += f0;
-    }
-    // integers cannot carry a NaN: non-finite phases (latched by the build) reach the output here
-    r.u0 = (float)((fma((double)r.s0, W.dt, W.t0) - sp.tk) * sp.ih) + (float)(all - all);
-    r.du = (float)du;
-    r.inv = W.tab_inv + s;
-    r.tab = W.tab + (size_t)s * tc_table_bytes(tr.tc_pairs, tr.tc_ks);
-    r.out = W.out;
-    r.pairs = tr.tc_pairs;
-    r.ks = tr.tc_ks;
-    r.n_mid = tr.n_mid;
-    r.c64 = W.out_c64;
-    h.recs[T] = r;
-}
 
 // Row stride (floats) of the staged table: 16-byte aligned, and 8 consecutive rows start 4 banks
 // apart, so the packing reads of a quarter-warp do not collide.
@@ -136,10 +70,10 @@ __global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *__res
     const int tid = threadIdx.x;
     if ((int)blockIdx.x >= h.total_segs) {
         const int T = ((int)blockIdx.x - h.total_segs) * kTcRecThreads + tid;
-        if (tid < kTcRecThreads && T < h.total_tiles) fill_record(h, T);
+        if (tid < kTcRecThreads && T < h.total_tiles) tc_fill_record(h, T, false);
         return;
     }
-    const WaveDev &W = h.waves[wave_of_seg(h, blockIdx.x)];
+    const WaveDev &W = h.waves[tc_wave_of_seg(h, blockIdx.x)];
     const TrajDev &tr = W.tr;
     const int s = (int)blockIdx.x - W.seg_begin;
     if (s >= tr.S || W.tile_off[s] == W.tile_off[s + 1]) return;  // no sample in this segment
@@ -241,32 +175,6 @@ __device__ __forceinline__ void sincos_fixed(uint32_t f, float &s, float &c)
     const float a = swap ? pc : ps, b = swap ? ps : pc;
     s = __uint_as_float(__float_as_uint(a) ^ (q & 0x80000000u));
     c = __uint_as_float(__float_as_uint(b) ^ ((q + 0x40000000u) & 0x80000000u));
-}
-
-// c0 + c1 v + c2 v^2 + c3 v^3 in 64-bit wrap-around arithmetic (modulo one turn).
-__device__ __forceinline__ unsigned long long phase_fixed(const long long *c, uint32_t v)
-{
-    const longlong2 a = reinterpret_cast<const longlong2 *>(c)[0];
-    const longlong2 b = reinterpret_cast<const longlong2 *>(c)[1];
-    unsigned long long p = (unsigned long long)b.y;
-    p = p * v + (unsigned long long)b.x;
-    p = p * v + (unsigned long long)a.y;
-    return p * v + (unsigned long long)a.x;
-}
-
-// Barrier of one warpgroup that also tells every thread whether any of them failed.
-__device__ __forceinline__ bool wg_any(int id, bool bad)
-{
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 p, %1, 0;\n\t"
-        "barrier.cta.red.or.pred q, %2, 128, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(r)
-        : "r"((uint32_t)bad), "r"(id)
-        : "memory");
-    return r != 0;
 }
 
 // Eight powers (cos, sin), two to a float2, as packed fp16 high and low parts: word k holds
@@ -482,7 +390,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
         }
         // while the MMAs run: this sample's factors
         const float2 uu = *reinterpret_cast<const float2 *>(&rp->u0);
-        const float inv = __ldg(rp->inv);
+        const float inv = __ldg(static_cast<const float *>(rp->seg));
         void *out = rp->out;
         if (T + kTcGroups < T1)
             next_word = __ldg(reinterpret_cast<const uint32_t *>(recs + T + kTcGroups) + (tid & 31));

@@ -1,7 +1,11 @@
-"""Edges of the tensor-core summation (tcsum.cu): tile and segment remainders, row and basis
-limits on both sides of its dispatch, batches and budgets that mix it with the scalar chain.
+"""Edges of the tensor-core summations (tcsum.cu, tcsum64.cu): tile and segment remainders, row and
+basis limits on both sides of their dispatch, batches and budgets that mix them with the scalar chain.
 
-Tolerance: the basis and table splits (2^-24 and 2^-23 of a term), the reduced phases (2^-28 turn,
+FP64 tolerance: the operands' digits and the products left out (2^-50 of the table's largest entry,
+which is at most a few times a sample's size in these sets) and the phases (FP64 rounding of ~1e3 rad,
+1e-13, times |m| + |n| <= 70) add up to at most 1e-11.
+
+Mixed tolerance: the basis and table splits (2^-24 and 2^-23 of a term), the reduced phases (2^-28 turn,
 a chain of at most four products), up to 12 accumulation steps (2^-23 each if truncated) and the
 11-step chain in z_phi^2 add up to at most 4e-6 of the terms of a sample.
 """
@@ -15,7 +19,8 @@ from paper_2104_04582_gb300 import workloads as W
 from tests.gpu_common import MIXED_MISMATCH, oracle_threads, rel_l2, to_host
 
 pytestmark = pytest.mark.gpu
-REL = 4e-6
+REL = {F.FEW_MIXED: 4e-6, F.FEW_FP64: 1e-11}
+PRECS = [F.FEW_MIXED, F.FEW_FP64]
 
 
 def _modes(ms, ns, l=None):
@@ -55,60 +60,65 @@ def test_mode_sets_past_the_limits(gpu_ctx, name):
 
 @pytest.mark.parametrize("name", [s for s in SETS if s not in PAST])
 @pytest.mark.parametrize("n_samples", [1, 128, 4001])
-def test_mode_set_edges(gpu_ctx, name, n_samples):
+@pytest.mark.parametrize("prec", PRECS)
+def test_mode_set_edges(gpu_ctx, prec, name, n_samples):
     import torch
     w = W.make_inputs(4.0e5, 9, 4.0e5 / max(n_samples, 200), SETS[name], 5, 4.0, 60.0,
                       n_samples=n_samples)
     tr = RT.from_inputs(gpu_ctx, w)
-    h = RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_MIXED)
+    h = RT.waveform_inputs(gpu_ctx, tr, w, prec)
     torch.cuda.synchronize()
     assert gpu_ctx.sync_status() == F.FEW_OK
-    assert rel_l2(to_host(h), oracle.waveform_inputs(w, nthreads=oracle_threads())) <= REL
+    assert rel_l2(to_host(h), oracle.waveform_inputs(w, nthreads=oracle_threads())) <= REL[prec]
     tr.release()
 
 
 @pytest.mark.parametrize("K,n_samples,i0,count", [
     (4, 127, 0, 127), (4, 129, 0, 129), (5, 1000, 1, 998), (300, 400, 0, 400),
     (300, 5000, 77, 4097), (40, 152 * 128 + 1, 0, 152 * 128 + 1)])
-def test_sample_and_segment_edges(gpu_ctx, K, n_samples, i0, count):
+@pytest.mark.parametrize("prec", PRECS)
+def test_sample_and_segment_edges(gpu_ctx, prec, K, n_samples, i0, count):
     """Segments shorter than a tile, empty segments, windows that start inside one, a run of tiles
     that leaves CTAs with one tile and with two."""
     import torch
     w = W.make_inputs(3.0e5, K, 3.0e5 / n_samples, W.mode_grid(4, 9), 11, 3.0, 20.0,
                       n_samples=n_samples)
     tr = RT.from_inputs(gpu_ctx, w)
-    out = torch.full((count + 2,), complex(7.0, 7.0), dtype=torch.complex64, device="cuda")
-    h = RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_MIXED, i_begin=i0, count=count, out=out[1:-1])
+    out = torch.full((count + 2,), complex(7.0, 7.0), device="cuda",
+                     dtype=torch.complex64 if prec == F.FEW_MIXED else torch.complex128)
+    h = RT.waveform_inputs(gpu_ctx, tr, w, prec, i_begin=i0, count=count, out=out[1:-1])
     torch.cuda.synchronize()
     assert gpu_ctx.sync_status() == F.FEW_OK
     g = to_host(out)
     assert g[0] == g[-1] == complex(7.0, 7.0)
     o = oracle.waveform_inputs(w, i0, count, nthreads=oracle_threads())
-    assert rel_l2(g[1:-1], o) <= REL
+    assert rel_l2(g[1:-1], o) <= REL[prec]
     tr.release()
 
 
-@pytest.mark.parametrize("scale", [1e-30, 1e-22, 1e25])
-def test_amplitude_range(gpu_ctx, scale):
+@pytest.mark.parametrize("prec,scale", [(F.FEW_MIXED, 1e-30), (F.FEW_MIXED, 1e-22), (F.FEW_MIXED, 1e25),
+                                        (F.FEW_FP64, 1e-290), (F.FEW_FP64, 1e-22), (F.FEW_FP64, 1e290)])
+def test_amplitude_range(gpu_ctx, prec, scale):
     """The table's power-of-two scaling: amplitudes far from one keep their relative accuracy."""
     import torch
     w = W.make_inputs(3.0e5, 12, 100.0, W.mode_grid(4, 9), 3, 3.0, 20.0)
     tr = RT.from_inputs(gpu_ctx, w)
-    h = RT.waveform(gpu_ctx, tr, w.n_samples, w.t0, w.dt, w.theta, w.phi, F.FEW_MIXED, False, scale)
+    h = RT.waveform(gpu_ctx, tr, w.n_samples, w.t0, w.dt, w.theta, w.phi, prec, False, scale)
     torch.cuda.synchronize()
     o = oracle.waveform_inputs(w, nthreads=oracle_threads(), scale=scale)
-    assert rel_l2(to_host(h) / scale, o / scale) <= REL
+    assert rel_l2(to_host(h) / scale, o / scale) <= REL[prec]
     tr.release()
 
 
-def test_batch_of_both_variants(gpu_ctx):
+@pytest.mark.parametrize("prec", PRECS)
+def test_batch_of_both_variants(gpu_ctx, prec):
     """A batch whose mode sets need both summation variants: each waveform as computed alone."""
     import torch
     sets = ["n_range_63", "rows_23", "n_range_15", "n_range_64"]
     ws = [W.make_inputs(2.0e5, 7, 50.0, SETS[s], k, 4.0, 60.0) for k, s in enumerate(sets)]
     trs = [RT.from_inputs(gpu_ctx, w) for w in ws]
-    outs = [RT.alloc_out(w.n_samples, True) for w in ws]
-    reqs = [RT.request(tr, o, w.n_samples, w.t0, w.dt, w.theta, w.phi, F.FEW_MIXED, w.scale)
+    outs = [RT.alloc_out(w.n_samples, prec == F.FEW_MIXED) for w in ws]
+    reqs = [RT.request(tr, o, w.n_samples, w.t0, w.dt, w.theta, w.phi, prec, w.scale)
             for tr, o, w in zip(trs, outs, ws)]
     for flags in (0, F.FEW_BATCH_NO_GRAPH):
         b = F.few_batch_plan(gpu_ctx.handle, reqs, flags)
@@ -116,7 +126,7 @@ def test_batch_of_both_variants(gpu_ctx):
         torch.cuda.synchronize()
         assert gpu_ctx.sync_status() == F.FEW_OK
         for w, tr, o in zip(ws, trs, outs):
-            np.testing.assert_array_equal(to_host(o), to_host(RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_MIXED)))
+            np.testing.assert_array_equal(to_host(o), to_host(RT.waveform_inputs(gpu_ctx, tr, w, prec)))
             o.zero_()
         F.few_batch_release(gpu_ctx.handle, b)
     for tr in trs:
