@@ -66,7 +66,7 @@ constexpr int kTc64Slices = 7;  // 8-bit digits per operand
 struct TcSeg64 {
     double inv1, inv2;        // output factors: table scale and fixed-point unit
     double tk, ih, t0, dt;    // u = (t0 + i dt - tk) ih
-    int shift;                // fixed-point sums are shifted left by this (right if negative)
+    int shift;                // the rows' fixed-point sums are shifted right by this
     int pad[3];
 };
 

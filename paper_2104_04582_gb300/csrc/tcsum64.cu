@@ -12,8 +12,8 @@
 // < 2^23, so the FP32 accumulators are exact integers.  What is left out (o >= 7) and the operands'
 // rounding are below 2^-50 of the table's largest entry, as is FP64's own rounding of such a sum.
 // The accumulators are put together as 64-bit integers, and the cubic in u and Horner's rules in
-// z_phi and its conjugate run in 64-bit fixed point too (a 64 x 64-bit product costs ~28 issue
-// cycles of a scheduler, an FP64 operation 64).  Powers of z_r and sincos are 62-bit fixed point
+// z_phi and its conjugate run in 64-bit fixed point too (a product costs ~6 instructions; an FP64
+// operation holds a scheduler's share of the pipe for 64 cycles).  Powers of z_r and sincos are 62-bit fixed point
 // (Taylor series); phases as in tcsum.cu.
 //
 // Work decomposition: as tcsum.cu, tiles of 128 samples, a persistent CTA per SM.  The segment's
@@ -135,13 +135,15 @@ __global__ void __launch_bounds__(kT64FoldThreads) k_fold_tc64(const PlanHdr *__
     const double f1 = pow2d(e / 2), f2 = pow2d(e - e / 2);
     if (tid == 0) {
         TcSeg64 g;
-        // the digit sums come out in units of 2^-52 of the scaled table; every partial sum is at
-        // most l1, and is kept below 2^61: left shifts are guard bits, right shifts headroom
+        // the digit sums come out in units of 2^-52 of the scaled table; every partial sum of a
+        // sample is at most l1
         const double l1 = sum * f1 * f2 * 1048576.0;
         int up = 14;  // l1 < 2^up (sums too small to be added up: as many entries as there are)
         if (l1 >= 0.5) up = (int)((unsigned)__double2hiint(l1) >> 20) - 1022;
-        g.shift = max(-30, min(3, 9 - up));
-        const int x = -e - 52 - g.shift;  // 2^x: one unit of the shifted sums
+        // (sums of one row have two guard bits, 2^-54, and stay below 2^62; the rows' total is kept
+        // below 2^61)
+        g.shift = max(0, min(32, up - 7));
+        const int x = -e - 54 + g.shift;  // 2^x: one unit of the shifted sums
         g.inv1 = pow2d(x / 2);
         // non-finite data (latched by the build) reach the output
         double all = sum - sum;
@@ -180,21 +182,47 @@ __global__ void __launch_bounds__(kT64FoldThreads) k_fold_tc64(const PlanHdr *__
 
 namespace {
 
-// a b 2^-62, 62-bit fixed point.
-__device__ __forceinline__ long long mul62(long long a, long long b)
+// 62-bit fixed point in balanced halves: value = h 2^32 + l, l signed.  A product then takes three
+// 32 x 32 -> 64-bit multiply-adds (the low halves' product, below half a unit of 2^-60, is left
+// out), against ~25 instructions for a 128-bit product.
+struct Q62 {
+    int h, l;
+};
+__device__ __forceinline__ Q62 q62(long long v)
 {
-    return (long long)(((__int128)a * b) >> 62);
+    const int l = (int)v;
+    return Q62{(int)(v >> 32) - (l >> 31), l};
+}
+__device__ __forceinline__ long long value(const Q62 &a) { return ((long long)a.h << 32) + a.l; }
+// a b + c, one instruction (written out: from C++ the products came out unsigned with corrections)
+__device__ __forceinline__ long long wide(int a, int b, long long c)
+{
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
 }
 
-struct Cq {  // complex, 62-bit fixed point
-    long long c, s;
+// a b 2^-64, rounded; |a|, |b| <= 2^62.
+__device__ __forceinline__ long long mul_hi(const Q62 &a, const Q62 &b)
+{
+    const long long t = wide(a.h, b.l, wide(a.l, b.h, 0x80000000ll));
+    return wide(a.h, b.h, t >> 32);
+}
+__device__ __forceinline__ long long mul62(const Q62 &a, const Q62 &b) { return mul_hi(a, b) << 2; }
+
+struct Cq {  // complex
+    Q62 c, s;
 };
 
+// (c, s) of a b in 62-bit fixed point, |a| = |b| = 1.
 __device__ __forceinline__ Cq cmul(const Cq &a, const Cq &b)
 {
-    // three products: (ac + as) bc, as (bc + bs), ac (bs - bc); sums of two below 2 fit
-    const long long k = mul62(a.c + a.s, b.c);
-    return Cq{k - mul62(a.s, b.c + b.s), k + mul62(a.c, b.s - b.c)};
+    const long long t = wide(a.c.h, b.c.l, wide(a.c.l, b.c.h, 0x80000000ll));
+    const long long v = wide(a.s.h, b.s.l, wide(a.s.l, b.s.h, 0));
+    const long long re = wide(a.c.h, b.c.h, (t - v) >> 32) - wide(a.s.h, b.s.h, 0);
+    const long long w = wide(a.c.h, b.s.l, wide(a.c.l, b.s.h, wide(a.s.h, b.c.l, wide(a.s.l, b.c.h, 0x80000000ll))));
+    const long long im = wide(a.c.h, b.s.h, wide(a.s.h, b.c.h, w >> 32));
+    return Cq{q62(re << 2), q62(im << 2)};
 }
 
 // cos and sin of 2 pi f 2^-64 in 62-bit fixed point: quadrant split off exactly, Taylor series to
@@ -204,36 +232,37 @@ __device__ __forceinline__ Cq sincos62(unsigned long long f)
     const unsigned long long q = f + 0x2000000000000000ull;
     const long long r = (long long)(f - (q & 0xc000000000000000ull));
     const long long one = 1ll << 62;
-    const long long x = mul62(r, 7244019458077122842ll);  // pi/2 2^62: r 2 pi 2^-64 in units of 2^-62
-    const long long x2 = mul62(x, x);
+    const Q62 x = q62(mul62(q62(r), q62(7244019458077122842ll)));  // pi/2 2^62: r 2 pi 2^-64 in 2^-62
+    const Q62 x2 = q62(mul62(x, x));
+    auto step = [&](long long p, long long k) { return mul62(x2, q62(p)) + k; };
     // 2^62 / n!, rounded
-    long long p = mul62(x2, 12966ll) - 3526632ll;     // 17!, 15!
-    p = mul62(x2, p) + 740592679ll;                   // 13!
-    p = mul62(x2, p) - 115532457973ll;                // 11!
-    p = mul62(x2, p) + 12708570377060ll;              // 9!
-    p = mul62(x2, p) - 915017067148291ll;             // 7!
-    p = mul62(x2, p) + 38430716820228233ll;           // 5!
-    p = mul62(x2, p) - 768614336404564651ll;          // 3!
-    const long long sn = x + mul62(x, mul62(x2, p));
-    long long c = mul62(x2, 220414ll) - 52899477ll;   // 16!, 14!
-    c = mul62(x2, c) + 9627704831ll;                  // 12!
-    c = mul62(x2, c) - 1270857037706ll;               // 10!
-    c = mul62(x2, c) + 114377133393536ll;             // 8!
-    c = mul62(x2, c) - 6405119470038039ll;            // 6!
-    c = mul62(x2, c) + 192153584101141163ll;          // 4!
-    c = mul62(x2, c) - (one >> 1);                    // 2!
-    const long long cs = one + mul62(x2, c);
+    long long p = step(12966ll, -3526632ll);     // 17!, 15!
+    p = step(p, 740592679ll);                    // 13!
+    p = step(p, -115532457973ll);                // 11!
+    p = step(p, 12708570377060ll);               // 9!
+    p = step(p, -915017067148291ll);             // 7!
+    p = step(p, 38430716820228233ll);            // 5!
+    p = step(p, -768614336404564651ll);          // 3!
+    const long long sn = value(x) + mul62(x, q62(mul62(x2, q62(p))));
+    long long c = step(220414ll, -52899477ll);   // 16!, 14!
+    c = step(c, 9627704831ll);                   // 12!
+    c = step(c, -1270857037706ll);               // 10!
+    c = step(c, 114377133393536ll);              // 8!
+    c = step(c, -6405119470038039ll);            // 6!
+    c = step(c, 192153584101141163ll);           // 4!
+    c = step(c, -(one >> 1));                    // 2!
+    const long long cs = one + mul62(x2, q62(c));
     const bool swap = (q >> 62) & 1;
     const long long a = swap ? cs : sn, b = swap ? sn : cs;
     const bool ns = (q >> 63) & 1, nc = ((q + 0x4000000000000000ull) >> 63) & 1;
-    return Cq{nc ? -b : b, ns ? -a : a};
+    return Cq{q62(nc ? -b : b), q62(ns ? -a : a)};
 }
 
 // The digits of one power into column `col` of every slice (this thread's lane).
 __device__ __forceinline__ void digit_words(const Cq &z, uint32_t (&w)[kTc64Slices])
 {
     // 62-bit -> multiples of 2^-54, rounded
-    const unsigned long long c = digit_bytes((z.c + 128) >> 8), s = digit_bytes((z.s + 128) >> 8);
+    const unsigned long long c = digit_bytes((value(z.c) + 128) >> 8), s = digit_bytes((value(z.s) + 128) >> 8);
     const uint32_t cl = (uint32_t)c, ch = (uint32_t)(c >> 32), sl = (uint32_t)s, sh = (uint32_t)(s >> 32);
     const uint32_t a = __byte_perm(cl, sl, 0x5140), b = __byte_perm(cl, sl, 0x7362);  // bytes 0 1, 2 3
     const uint32_t d = __byte_perm(ch, sh, 0x5140), g = __byte_perm(ch, sh, 0x7362);  // bytes 4 5, 6
@@ -260,25 +289,36 @@ __device__ __forceinline__ void store_digits(uint32_t e_addr, const Cq (&z)[8])
     for (int q = 0; q < kTc64Slices; ++q) tc_st8(e_addr + kT64EStride * q, w[q]);
 }
 
-// The sums of one column, orders 0 .. 6, as a 64-bit integer: sum_o S_o 2^(40 - 8 o), orders 0 .. 4
-// exact (|S_o| < 2^22: the 1.5 2^23 addition leaves the integer in the low mantissa bits), orders
-// 5 and 6 to a unit.
-__device__ __forceinline__ long long join_orders(float s0, float s1, float s2, float s3, float s4, float s5,
-                                                 float s6)
+// The sums of one column pair (even, odd row), orders 0 .. 6, as 64-bit integers 4 sum_o S_o
+// 2^(40 - 8 o) (two guard bits): orders 0 .. 4 exact (|S_o| < 2^22: the 1.5 2^23 addition leaves the
+// integer in the low mantissa bits), orders 5 and 6 to a unit.  S: orders 16 columns apart.
+__device__ __forceinline__ void join_orders(const float2 (&S)[kTc64Slices], long long (&v)[2])
 {
-    const float kM = 12582912.0f;
-    const int kMi = 0x4b400000;
-    const float t = fmaf(s6, 0.00390625f, s5);
-    const float cm = fmaf(t, 0.00390625f, kM), rest = fmaf(cm - kM, -256.0f, t);
-    const int n0 = __float_as_int(s0 + kM) - kMi, n1 = __float_as_int(s1 + kM) - kMi;
-    const int n2 = __float_as_int(s2 + kM) - kMi, n3 = __float_as_int(s3 + kM) - kMi;
-    const int n4 = __float_as_int(s4 + kM) - kMi + (__float_as_int(cm) - kMi);
-    const int n5 = __float_as_int(rest + kM) - kMi;
-    const int p1 = n0 * 256 + n1, p2 = n2 * 256 + n3, p3 = n4 * 256 + n5;
-    return ((long long)p1 << 32) + (long long)p2 * 65536ll + p3;
+    const float2 kM = make_float2(12582912.0f, 12582912.0f), kNM = make_float2(-12582912.0f, -12582912.0f);
+    const float2 k256 = make_float2(0.00390625f, 0.00390625f), kN256 = make_float2(-256.0f, -256.0f);
+    const uint32_t kMi = 0x4b400000u;
+    // (an opaque copy: from __float_as_uint of the packed sums nvcc 13.0 drops the shift of n4c below
+    // for the even column)
+    auto bits = [](float x) {
+        uint32_t u;
+        asm("mov.b32 %0, %1;" : "=r"(u) : "f"(x));
+        return u;
+    };
+    const float2 t = __ffma2_rn(S[6], k256, S[5]);
+    const float2 cm = __ffma2_rn(t, k256, kM);
+    const float2 rest = __fadd2_rn(__ffma2_rn(__fadd2_rn(cm, kNM), kN256, t), kM);
+    const float2 n0 = __fadd2_rn(S[0], kM), n1 = __fadd2_rn(S[1], kM), n2 = __fadd2_rn(S[2], kM);
+    const float2 n3 = __fadd2_rn(S[3], kM), n4 = __fadd2_rn(S[4], kM);
+    auto join = [&](float a0, float a1, float a2, float a3, float a4, float c, float a5) {
+        const uint32_t p1 = (bits(a0) << 8) + (bits(a1) - (kMi << 8) - kMi);
+        const uint32_t p2 = (bits(a2) << 8) + (bits(a3) - (kMi << 8) - kMi);
+        const uint32_t n4c = bits(a4) - kMi + (bits(c) - kMi);
+        const uint32_t p3 = (n4c << 8) + (bits(a5) - kMi);
+        return wide((int)p2, 1 << 18, wide((int)p3, 4, (long long)((unsigned long long)p1 << 34)));
+    };
+    v[0] = join(n0.x, n1.x, n2.x, n3.x, n4.x, cm.x, rest.x);
+    v[1] = join(n0.y, n1.y, n2.y, n3.y, n4.y, cm.y, rest.y);
 }
-
-__device__ __forceinline__ long long shift_by(long long v, int sh) { return sh >= 0 ? v << sh : v >> -sh; }
 
 __device__ __forceinline__ bool warp_ok(bool ok) { return __all_sync(0xffffffffu, ok); }
 
@@ -423,10 +463,10 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
                 reinterpret_cast<const void *>(__ldg(reinterpret_cast<const unsigned long long *>(&rp->seg))));
             // (lanes outside the segment take its first or last sample's u: sums stay in range)
             const double u = (fma((double)min(max(i, span.y), span.z - 1), sg->dt, sg->t0) - sg->tk) * sg->ih;
-            const long long U = __double2ll_rn(u * 4611686018427387904.0);
+            const Q62 U = q62(__double2ll_rn(u * 4611686018427387904.0));
             const Cq zphi = sincos62(fphi);
             Cq z[8];  // e^{i k theta}
-            z[0] = Cq{1ll << 62, 0};
+            z[0] = Cq{q62(1ll << 62), q62(0)};
             z[1] = sincos62(fr);
             z[2] = cmul(z[1], z[1]);
             z[3] = cmul(z[2], z[1]);
@@ -467,7 +507,8 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
             }
             if ((tid & 31) == 0) mbar_arrive(&e_full[group]);
             const int shift = sg->shift;
-            long long t0r = 0, t0i = 0, t1r = 0, t1i = 0;  // rows m >= 0 in z_phi^-1, rows m < 0 in z_phi
+            const long long round = (1ll << shift) >> 1;
+            Q62 t0r{0, 0}, t0i{0, 0}, t1r{0, 0}, t1i{0, 0};  // rows m >= 0 in z_phi^-1, rows m < 0 in z_phi
 #pragma unroll 1
             for (int p = 0; p < pairs; ++p) {
                 const uint32_t ch = chunk + (uint32_t)p, b = ch & 1u;
@@ -491,40 +532,41 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
                 // rows m = m_top - p (even columns) and p - m_top (odd): the cubics, then Horner's step
                 long long a[2][2];
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
+                for (int c = 0; c < 2; ++c) {
+                    long long acc[2];
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        long long acc = 0;
+                    for (int dg = 3; dg >= 0; --dg) {
+                        float2 w[kTc64Slices];
+                        long long k[2];
 #pragma unroll
-                        for (int dg = 3; dg >= 0; --dg) {
-                            const int col = 2 * (4 * c + dg) + e;
-                            const long long k =
-                                shift_by(join_orders(S[0][col], S[1][col], S[2][col], S[3][col], S[4][col],
-                                                     S[5][col], S[6][col]), shift);
-                            acc = dg == 3 ? k : mul62(acc, U) + k;
-                        }
-                        a[e][c] = acc;
+                        for (int o = 0; o < kTc64Slices; ++o)
+                            w[o] = reinterpret_cast<const float2 *>(S[o])[4 * c + dg];
+                        join_orders(w, k);
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) acc[e] = dg == 3 ? k[e] : mul62(q62(acc[e]), U) + k[e];
                     }
+                    a[0][c] = (acc[0] + round) >> shift;
+                    a[1][c] = (acc[1] + round) >> shift;
                 }
                 // z_phi = e^{-i Phi_phi} = (c, -s)
                 const long long n0r = mul62(t0r, zphi.c) + mul62(t0i, zphi.s) + a[0][0];
                 const long long n0i = mul62(t0i, zphi.c) - mul62(t0r, zphi.s) + a[0][1];
                 const long long n1r = mul62(t1r, zphi.c) - mul62(t1i, zphi.s) + a[1][0];
                 const long long n1i = mul62(t1i, zphi.c) + mul62(t1r, zphi.s) + a[1][1];
-                t0r = n0r;
-                t0i = n0i;
-                t1r = n1r;
-                t1i = n1i;
+                t0r = q62(n0r);
+                t0i = q62(n0i);
+                t1r = q62(n1r);
+                t1i = q62(n1i);
             }
             if (bad) break;
             if (i >= span.y && i < span.z) {
-                const double hr = (double)(t0r + t1r), hi = (double)(t0i + t1i);
+                const double hr = (double)(value(t0r) + value(t1r)), hi = (double)(value(t0i) + value(t1i));
                 const double inv = sg->inv1;
                 double fc = inv, fs = 0.0;
                 if (shape.z != 0) {  // z_r^{n_mid}
                     const Cq w = sincos62((unsigned long long)(long long)shape.z * fr);
-                    fc = (double)w.c * 2.168404344971008868e-19 * inv;  // 2^-62
-                    fs = (double)w.s * 2.168404344971008868e-19 * inv;
+                    fc = (double)value(w.c) * 2.168404344971008868e-19 * inv;  // 2^-62
+                    fs = (double)value(w.s) * 2.168404344971008868e-19 * inv;
                 }
                 const double yr = fma(hr, fc, hi * fs) * sg->inv2, yi = fma(hi, fc, -hr * fs) * sg->inv2;
                 void *out = reinterpret_cast<void *>(__ldg(reinterpret_cast<const unsigned long long *>(&rp->out)));
