@@ -32,7 +32,8 @@ namespace fewsum {
 namespace {
 
 constexpr int kT64FoldThreads = 352;  // FP64 fold: registers for a thread's two cubics
-constexpr int kT64Groups = 2, kT64Threads = 128 * kT64Groups + 32;  // and the MMAs' warp
+constexpr int kT64Groups = 2, kT64Issuers = 2;
+constexpr int kT64Threads = 128 * kT64Groups + 32 * kT64Issuers;  // and the MMAs' warps
 constexpr int kT64MaxKs = (kTcMaxHalf + 8) / 8;
 constexpr int kT64MaxTable = 512 * kTc64Slices * kTcMaxPairs * kT64MaxKs;
 constexpr uint32_t kT64EStride = 32;                    // tensor-memory columns of a digit slice
@@ -322,16 +323,19 @@ __device__ __forceinline__ void join_orders(const float2 (&S)[kTc64Slices], long
 
 __device__ __forceinline__ bool warp_ok(bool ok) { return __all_sync(0xffffffffu, ok); }
 
-// The MMAs of one row pair (one elected thread): accumulator o sums the products of digits e of the
-// basis and o - e of the table.  Everything but three bases is a compile-time offset: with run-time
-// loops the uniform datapath's address arithmetic took ~50 cycles an MMA, four times its execution.
-template <int KS>
-__device__ __forceinline__ void issue_pair(uint32_t d, uint32_t e, uint64_t desc)
+// Half of the MMAs of one row pair (one elected thread): accumulator o sums the products of digits q
+// of the basis and o - q of the table.  Issuer 0 takes orders 1 .. 4, issuer 1 orders 0, 5 and 6 (14
+// products each): one warp issues an N = 16 MMA every ~13 cycles, two together one every 10.6.
+// Everything but three bases is a compile-time offset: with run-time loops the uniform datapath's
+// address arithmetic took ~50 cycles an MMA.
+template <int KS, int ISSUER>
+__device__ __forceinline__ void issue_half(uint32_t d, uint32_t e, uint64_t desc)
 {
     constexpr uint32_t idesc = (1u << 4) | (2u << 17) | ((uint32_t)(kTcTile >> 4) << 24);
     constexpr uint32_t slice = 512u * KS;
 #pragma unroll
     for (int o = 0; o < kTc64Slices; ++o) {
+        if ((o >= 1 && o <= 4) != (ISSUER == 0)) continue;
 #pragma unroll
         for (int q = 0; q <= o; ++q) {
 #pragma unroll
@@ -341,11 +345,19 @@ __device__ __forceinline__ void issue_pair(uint32_t d, uint32_t e, uint64_t desc
         }
     }
 }
+template <int KS>
+__device__ __forceinline__ void issue_pair(int issuer, uint32_t d, uint32_t e, uint64_t desc)
+{
+    if (issuer == 0)
+        issue_half<KS, 0>(d, e, desc);
+    else
+        issue_half<KS, 1>(d, e, desc);
+}
 
 }  // namespace
 
-// Warps 0 - 7: two warpgroups, every other tile of the CTA's run each.  Warp 8 loads the tables and
-// issues the MMAs, tile by tile and row pair by row pair.  Barriers (chunk = row pair, counted over
+// Warps 0 - 7: two warpgroups, every other tile of the CTA's run each.  Warps 8 and 9 issue the MMAs,
+// tile by tile and row pair by row pair (half of each), warp 8 loads the tables.  Barriers (chunk = row pair, counted over
 // the run): e_full[g] the basis of group g's tile is stored; done[g] its MMAs have completed (the
 // operand columns are free); d_full[b], d_empty[b] accumulator set b = chunk & 1.
 template <int KS>
@@ -369,12 +381,12 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
     if (tid == 32) {
         mbar_init(&b_full, 1);
         for (int b = 0; b < 2; ++b) {
-            mbar_init(&d_full[b], 1);
+            mbar_init(&d_full[b], kT64Issuers);
             mbar_init(&d_empty[b], 4);
         }
         for (int g = 0; g < kT64Groups; ++g) {
             mbar_init(&e_full[g], 4);
-            mbar_init(&done[g], 1);
+            mbar_init(&done[g], kT64Issuers);
         }
         fence_mbar_init();
         s_abort = 0;
@@ -384,7 +396,8 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    if (warp == 4 * kT64Groups) {
+    if (warp >= 4 * kT64Groups) {
+        const int issuer = warp - 4 * kT64Groups;
         int tend = T0, table = -1;
         uint32_t chunk = 0;
         bool ok = true;
@@ -396,7 +409,7 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
                 tend = __ldg(&recs[T].tile_end);
                 ++table;
                 if (T > T0) ok = warp_ok(mbar_wait_bounded(&done[g ^ 1], (uint32_t)(T - 1 - T0) >> 1 & 1u));
-                if (ok && (tid & 31) == 0) {
+                if (ok && issuer == 0 && (tid & 31) == 0) {
                     const uint32_t bytes = (uint32_t)tc64_table_bytes(pairs, ks);
                     const unsigned char *src = reinterpret_cast<const unsigned char *>(
                         __ldg(reinterpret_cast<const unsigned long long *>(&recs[T].tab)));
@@ -418,11 +431,11 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
                     smem_u32(tcs64) + (uint32_t)(p * kTc64Slices * ks) * 512u, 128, 256u * (uint32_t)ks);
                 if (elect_one()) {
                     if (ks == KS) {
-                        issue_pair<KS>(d, tmem, desc);
+                        issue_pair<KS>(issuer, d, tmem, desc);
                     } else {  // a wave with fewer K steps than the plan's widest
-                        if (KS > 1 && ks == 1) issue_pair<1>(d, tmem, desc);
-                        if (KS > 2 && ks == 2) issue_pair<2>(d, tmem, desc);
-                        if (KS > 3 && ks == 3) issue_pair<3>(d, tmem, desc);
+                        if (KS > 1 && ks == 1) issue_pair<1>(issuer, d, tmem, desc);
+                        if (KS > 2 && ks == 2) issue_pair<2>(issuer, d, tmem, desc);
+                        if (KS > 3 && ks == 3) issue_pair<3>(issuer, d, tmem, desc);
                     }
                     tc_commit(&d_full[b]);
                     if (p + 1 == pairs) tc_commit(&done[g]);
