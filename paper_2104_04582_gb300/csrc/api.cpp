@@ -11,6 +11,7 @@
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <set>
@@ -345,7 +346,6 @@ struct few_traj {
     SlotPlan plan;
     void *dmem = nullptr;
     double *ybuf = nullptr;  // device staging for host-provided knot data (lazy)
-    BuildJob *job_dev = nullptr;
     TrajDev dev{};
     bool has_data = false;
     // device pointers of the current knot data (for batched rebuilds)
@@ -606,14 +606,10 @@ void fill_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P, unsign
         WaveDev &W = wv[q];
         std::memset(&W, 0, sizeof(W));
         W.tr = tr->dev;
-        W.theta = r.theta;
-        W.phi = r.phi;
+        set_wave_angles(r, W);
         W.scale = r.scale;
         W.dphi_phi = r.dphi_phi0;
         W.dphi_r = r.dphi_r0;
-        W.frame = r.frame;
-        W.theta_K = r.theta_K;
-        W.phi_K = r.phi_K;
         W.t0 = r.t0;
         W.dt = r.dt;
         W.n_samples = (int)r.n_samples;
@@ -693,14 +689,16 @@ void fill_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P, unsign
     hdr->stage_slots = P.stage_slots;
     hdr->ring = P.ring;
     hdr->variant = L.variant;
+    hdr->self = blob_dev;
     hdr->waves = reinterpret_cast<const WaveDev *>(blob_dev + P.off_waves);
     hdr->cta = reinterpret_cast<const CtaStart *>(blob_dev + P.off_cta);
     hdr->err = c->d_err;
 }
 
 // Queue a plan's kernels on `st`.  Errors are returned after everything queued has been joined.
-cudaError_t launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, const LaunchPlan &P, cudaStream_t st,
-                           bool mark)
+// plan: a tensor-core plan that travels in the fold's parameters instead of being at hdr_dev already.
+cudaError_t launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, const PlanParam *plan, const LaunchPlan &P,
+                           cudaStream_t st, bool mark)
 {
     auto tm = [&](int slot, bool end) {
         if (mark) tmark(c, slot, end, st);
@@ -709,11 +707,12 @@ cudaError_t launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, const LaunchPlan 
     cudaError_t e;
     if (is_tc(P.variant)) {
         tm(1, false);
-        if ((e = launch_ylm(hdr_dev, P.total_pairs, fp64, st)) != cudaSuccess) return e;
+        // the first kernel takes the plan: the harmonics, or the mixed fold, which forms its own
+        if (fp64 && (e = launch_ylm(hdr_dev, plan, P.total_pairs, fp64, st)) != cudaSuccess) return e;
         tm(1, true);
         tm(2, false);
         e = fp64 ? launch_fold_tc64(hdr_dev, P.total_segs, P.total_tiles, st)
-                 : launch_fold_tc(hdr_dev, P.total_segs, P.total_tiles, st);
+                 : launch_fold_tc(hdr_dev, plan, P.total_segs, P.total_tiles, st);
         if (e != cudaSuccess) return e;
         tm(2, true);
         tm(3, false);
@@ -747,7 +746,7 @@ cudaError_t launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, const LaunchPlan 
         return err;
     };
     tm(1, false);
-    if ((e = joined(launch_ylm(hdr_dev, P.total_pairs, fp64, st))) != cudaSuccess) return e;
+    if ((e = joined(launch_ylm(hdr_dev, nullptr, P.total_pairs, fp64, st))) != cudaSuccess) return e;
     tm(1, true);
     tm(2, false);
     if ((e = joined(launch_fold(hdr_dev, P.total_fold, fp64, st))) != cudaSuccess) return e;
@@ -928,7 +927,7 @@ few_status few_traj_create(few_ctx *ctx, const double *t_knots, int K, const int
                  o_sp = take(sizeof(int) * P.slot_ptr.size()),
                  o_ct = take(sizeof(int2) * std::max<size_t>(1, P.contrib.size())),
                  o_rows = take(sizeof(int2) * P.rows.size()),
-                 o_rslot = take(sizeof(int4) * P.row_slot.size()), o_job = take(sizeof(BuildJob));
+                 o_rslot = take(sizeof(int4) * P.row_slot.size());
     if ((st = dev_alloc(ctx, off, ctx->internal, &tr->dmem))) {
         delete tr;
         return st;
@@ -982,7 +981,6 @@ few_status few_traj_create(few_ctx *ctx, const double *t_knots, int K, const int
     D.tc_ks = P.tc_ks;
     D.n_mid = P.n_mid;
     D.m_top = P.m_top;
-    tr->job_dev = reinterpret_cast<BuildJob *>(d + o_job);
 
     cudaStream_t s = ctx->internal;
     few_status us = upload(ctx, d, img.data(), o_h, s);  // knot times
@@ -1064,16 +1062,14 @@ few_status few_traj_set_data(few_ctx *ctx, few_traj *tr, const double *phi_phi, 
         job.amp_im = amp_im;
     }
     job.block_begin = 0;
-    few_status s = upload(ctx, tr->job_dev, &job, sizeof(job), st);
+    few_status s = FEW_OK;
     const int blocks = (tr->J + kBuildSplines - 1) / kBuildSplines;
-    if (!s) {
-        tmark(ctx, 0, false, st);
-        if (launch_build(tr->job_dev, 1, blocks, tr->K, ctx->d_err, st) != cudaSuccess) {
-            (void)cudaGetLastError();
-            s = FEW_ERR_CUDA;
-        }
-        tmark(ctx, 0, true, st);
+    tmark(ctx, 0, false, st);
+    if (launch_build_one(job, blocks, ctx->d_err, st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        s = FEW_ERR_CUDA;
     }
+    tmark(ctx, 0, true, st);
     if (copied) {
         lk.unlock();  // the copies' completion concerns this call only
         if (cudaEventSynchronize(copied) != cudaSuccess && !s) {
@@ -1129,14 +1125,11 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream)
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     PlanImage P;
     const size_t out_bytes = (size_t)req->n_samples * (req->out_c64 ? 8 : 16);
-    void *blob = nullptr, *scratch = nullptr, *dout = nullptr;
+    void *blob = nullptr, *dout = nullptr;  // the plan, its scratch behind it
     auto plan = [&](bool tc) {
         P = PlanImage();
-        few_status e = build_image(ctx, req, 1, tc, P);
-        if (e) return e;
-        if ((e = dev_alloc(ctx, P.blob.size(), s, &blob))) return e;
-        if ((e = dev_alloc(ctx, P.scratch_bytes, s, &scratch))) dev_free(ctx, blob, s);
-        return e;
+        const few_status e = build_image(ctx, req, 1, tc, P);
+        return e ? e : dev_alloc(ctx, P.blob.size() + P.scratch_bytes, s, &blob);
     };
     const bool tc = tc_fits(*req);
     st = plan(tc);
@@ -1155,17 +1148,26 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream)
         } else {
             (void)cudaGetLastError();
             if ((st = dev_alloc(ctx, out_bytes, s, &dout))) {
-                dev_free(ctx, scratch, s);
                 dev_free(ctx, blob, s);
                 return st;
             }
             out_dev = dout;
         }
     }
-    fill_image(ctx, req, 1, P, static_cast<unsigned char *>(blob),
-               static_cast<unsigned char *>(scratch), &out_dev);
-    st = upload(ctx, blob, P.blob.data(), P.blob.size(), s);
-    if (!st && launch_kernels(ctx, static_cast<const PlanHdr *>(blob), P.launch, s, true) != cudaSuccess) {
+    unsigned char *blob_dev = static_cast<unsigned char *>(blob);
+    fill_image(ctx, req, 1, P, blob_dev, blob_dev + P.blob.size(), &out_dev);
+    // a small tensor-core plan travels in the fold's parameters: no copy stands between the kernels
+    std::unique_ptr<PlanParam> param;
+    if (is_tc(P.launch.variant) && P.blob.size() <= (size_t)kPlanParamBytes) param.reset(new (std::nothrow) PlanParam);
+    if (param) {
+        std::memcpy(param->bytes, P.blob.data(), P.blob.size());
+        param->dev = blob_dev;
+        param->n = (int)P.blob.size();
+    } else {
+        st = upload(ctx, blob, P.blob.data(), P.blob.size(), s);
+    }
+    if (!st && launch_kernels(ctx, static_cast<const PlanHdr *>(blob), param.get(), P.launch, s, true) !=
+                   cudaSuccess) {
         (void)cudaGetLastError();
         st = FEW_ERR_CUDA;
     }
@@ -1177,7 +1179,6 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream)
         }
     }
     dev_free(ctx, dout, s);
-    dev_free(ctx, scratch, s);
     dev_free(ctx, blob, s);
     if (!st && req->out_where == FEW_MEM_HOST) {
         // everything is queued: wait for the result without holding the context, so calls from
@@ -1507,7 +1508,7 @@ few_status few_batch_plan(few_ctx *ctx, const few_request *reqs, int n, unsigned
                              b->max_knots, ctx->d_err, cap);
             // the same forks and joins as a direct run, recorded into the graph
             for (const auto &p : b->parts)
-                launch_kernels(ctx, static_cast<const PlanHdr *>(p.blob_dev), p.launch, cap, false);
+                launch_kernels(ctx, static_cast<const PlanHdr *>(p.blob_dev), nullptr, p.launch, cap, false);
             e = cudaStreamEndCapture(cap, &b->graph);
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
@@ -1538,7 +1539,7 @@ few_status few_batch_run(few_ctx *ctx, few_batch *b, void *stream)
         tmark(ctx, 0, true, s);
     }
     for (const auto &p : b->parts)
-        FEW_CUDA_TRY(launch_kernels(ctx, static_cast<const PlanHdr *>(p.blob_dev), p.launch, s, true));
+        FEW_CUDA_TRY(launch_kernels(ctx, static_cast<const PlanHdr *>(p.blob_dev), nullptr, p.launch, s, true));
     return FEW_OK;
 }
 
@@ -1725,6 +1726,44 @@ std::recursive_mutex &ctx_mutex(few_ctx *ctx) { return ctx->mu; }
 few_status check_request(const few_request &r, bool need_device_out)
 {
     return validate_request(r, need_device_out);
+}
+
+// Frame transformation (Sec. 2.A): from the sky position (tS, pS) and the spin direction
+// (tK, pK) in the barycentre frame, the source-frame viewing angles of the propagation direction
+// -R in the basis x = R x S/|R x S|, y = (R - (R.S) S)/|R x S|, z = S, and the polarization
+// angle psi with tan psi = (cos tS sin tK cos(pS - pK) - sin tS cos tK)/(sin tK sin(pS - pK)).
+// The detector-frame waveform is -e^{-2 i psi} times the source-frame one (a pi phase shift for
+// the pi/2 basis rotation, then the 2 psi rotation), a constant folded into the harmonics.  All of it
+// is per request: formed once here instead of by every harmonic's thread (a dozen FP64 functions).
+void set_wave_angles(const few_request &r, WaveDev &W)
+{
+    W.theta = r.theta;
+    W.phi = r.phi;
+    W.rotate = 0;
+    W.rot_r = 1.0;
+    W.rot_i = 0.0;
+    if (r.frame != FEW_FRAME_SSB) return;
+    const double stS = std::sin(r.theta), ctS = std::cos(r.theta), spS = std::sin(r.phi),
+                 cpS = std::cos(r.phi), stK = std::sin(r.theta_K), ctK = std::cos(r.theta_K),
+                 spK = std::sin(r.phi_K), cpK = std::cos(r.phi_K);
+    const double R[3] = {stS * cpS, stS * spS, ctS};
+    const double S[3] = {stK * cpK, stK * spK, ctK};
+    const double X[3] = {R[1] * S[2] - R[2] * S[1], R[2] * S[0] - R[0] * S[2],
+                         R[0] * S[1] - R[1] * S[0]};
+    const double nx = std::sqrt(X[0] * X[0] + X[1] * X[1] + X[2] * X[2]);
+    const double rs = R[0] * S[0] + R[1] * S[1] + R[2] * S[2];
+    // components of -R: along x (R x S is orthogonal to R), along y, along z = S
+    const double vx = 0.0;
+    const double vy = -((R[0] - rs * S[0]) * R[0] + (R[1] - rs * S[1]) * R[1] +
+                        (R[2] - rs * S[2]) * R[2]) / nx;
+    const double vz = -rs;
+    W.theta = std::acos(std::max(-1.0, std::min(1.0, vz)));
+    W.phi = std::atan2(vy, vx);
+    const double psi = std::atan2(ctS * stK * std::cos(r.phi - r.phi_K) - stS * ctK,
+                                  stK * std::sin(r.phi - r.phi_K));
+    W.rotate = 1;
+    W.rot_r = -std::cos(2.0 * psi);  // -e^{-2 i psi}
+    W.rot_i = std::sin(2.0 * psi);
 }
 
 }  // namespace fewsum

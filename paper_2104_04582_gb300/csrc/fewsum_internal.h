@@ -153,7 +153,7 @@ struct BuildJob {
 // One waveform of a plan (a request).
 struct WaveDev {
     TrajDev tr;
-    double theta, phi, scale;
+    double theta, phi, scale;   // source-frame viewing angles
     double dphi_phi, dphi_r;    // phase offsets (rad)
     double t0, dt;
     int n_samples;
@@ -174,8 +174,8 @@ struct WaveDev {
     int pair_begin;       // first global pair index of this wave (ylm kernel)
     int fold_begin;       // first fold block of this wave
     int fold_blocks_per_seg;
-    int frame;            // few_frame: (theta, phi) source-frame angles, or sky position
-    double theta_K, phi_K;  // spin direction (frame == FEW_FRAME_SSB)
+    int rotate;           // detector frame: the harmonics are multiplied by (rot_r, rot_i)
+    double rot_r, rot_i;
 };
 
 // Start of one CTA's slice of the summation work: (wave, sample).
@@ -198,11 +198,20 @@ struct PlanHdr {
     int total_segs, total_tiles;  // tensor-core plans
     const int *tile_cta;  //   [grid + 1] first tile of each CTA
     TileRec *recs;        //   [total_tiles]
+    const unsigned char *self;    // the plan's device address
     const WaveDev *waves;
     const CtaStart *cta;
     unsigned *err;
 };
 
+// A plan small enough to travel as a kernel parameter (no upload): its bytes, to be read at
+// `bytes` and copied to device address `dev`, for which its pointers into itself are made.
+constexpr int kPlanParamBytes = 6144;
+struct alignas(16) PlanParam {
+    unsigned char bytes[kPlanParamBytes];
+    unsigned char *dev;
+    int n;
+};
 // Kernel launchers (defined in the .cu files; every launcher returns the launch error).
 // Output arrays of k_factor (the trajectory's TrajDev fields of the same names).
 struct FactorArrays {
@@ -212,7 +221,10 @@ struct FactorArrays {
 cudaError_t launch_factor(const double *t, int K, const FactorArrays &f, cudaStream_t st);
 cudaError_t launch_build(const BuildJob *jobs_dev, int n_jobs, int total_blocks,
                          int max_knots, unsigned *err, cudaStream_t st);
-cudaError_t launch_ylm(const PlanHdr *hdr_dev, int total_pairs, bool fp64, cudaStream_t st);
+// One trajectory's build, the job as a kernel parameter.
+cudaError_t launch_build_one(const BuildJob &job, int blocks, unsigned *err, cudaStream_t st);
+cudaError_t launch_ylm(const PlanHdr *hdr_dev, const PlanParam *plan, int total_pairs, bool fp64,
+                       cudaStream_t st);
 cudaError_t launch_fold(const PlanHdr *hdr_dev, int total_fold_blocks, bool fp64, cudaStream_t st);
 cudaError_t launch_anchor(const PlanHdr *hdr_dev, int total_anchor_segs, cudaStream_t st);
 // Anchors of one segment's samples [s_begin, s_end): groups floor(s_begin / G) ..
@@ -248,7 +260,10 @@ cudaError_t tc_configure();
 cudaError_t tc64_configure();
 cudaError_t launch_fold_tc64(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st);
 cudaError_t launch_sum_tc64(const PlanHdr *hdr_dev, int grid, int ks, cudaStream_t st);
-cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st);
+// plan: the plan itself (the kernel then writes it to hdr_dev for those that follow), or null when it
+// is at hdr_dev already.
+cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, const PlanParam *plan, int total_segs, int total_tiles,
+                           cudaStream_t st);
 // ks: the most K steps of any wave of the plan.
 cudaError_t launch_sum_tc(const PlanHdr *hdr_dev, int grid, int ks, cudaStream_t st);
 // Bytes of one folded slot in the layout a variant reads.
@@ -316,6 +331,8 @@ struct DeviceScope {
 // Host validation of one request (few_waveform's checks; need_device_out additionally requires
 // out_where == FEW_MEM_DEVICE).
 few_status check_request(const few_request &r, bool need_device_out);
+// Viewing direction and frame constant of a request.
+void set_wave_angles(const few_request &r, WaveDev &W);
 
 // Read-only snapshot of a context and one of its trajectories (filled by api.cpp).
 struct CtxTrajView {

@@ -21,7 +21,7 @@
 #include "fewsum_internal.h"
 #include "harmonics.cuh"
 #include "convert.cuh"
-#include "fold_slot.cuh"
+#include "tctile.cuh"
 
 namespace fewsum {
 
@@ -36,86 +36,63 @@ __device__ __forceinline__ int wave_of(const WaveDev *waves, int n, int g, bool 
     return lo;
 }
 
-// Frame transformation (Sec. 2.A): from the sky position (tS, pS) and the spin direction
-// (tK, pK) in the barycentre frame, the source-frame viewing angles of the propagation direction
-// -R in the basis x = R x S/|R x S|, y = (R - (R.S) S)/|R x S|, z = S, and the polarization
-// angle psi with tan psi = (cos tS sin tK cos(pS - pK) - sin tS cos tK)/(sin tK sin(pS - pK)).
-// The detector-frame waveform is -e^{-2 i psi} times the source-frame one (a pi phase shift for
-// the pi/2 basis rotation, then the 2 psi rotation), a constant folded into the harmonics.
-__device__ void frame_angles(double tS, double pS, double tK, double pK, double &theta,
-                             double &phi, double &psi)
-{
-    double stS, ctS, spS, cpS, stK, ctK, spK, cpK;
-    sincos(tS, &stS, &ctS);
-    sincos(pS, &spS, &cpS);
-    sincos(tK, &stK, &ctK);
-    sincos(pK, &spK, &cpK);
-    const double R[3] = {stS * cpS, stS * spS, ctS};
-    const double S[3] = {stK * cpK, stK * spK, ctK};
-    const double X[3] = {R[1] * S[2] - R[2] * S[1], R[2] * S[0] - R[0] * S[2],
-                         R[0] * S[1] - R[1] * S[0]};
-    const double nx = sqrt(X[0] * X[0] + X[1] * X[1] + X[2] * X[2]);
-    const double rs = R[0] * S[0] + R[1] * S[1] + R[2] * S[2];
-    // components of -R: along x (R x S is orthogonal to R), along y, along z = S
-    const double vx = 0.0;
-    const double vy = -((R[0] - rs * S[0]) * R[0] + (R[1] - rs * S[1]) * R[1] +
-                        (R[2] - rs * S[2]) * R[2]) / nx;
-    const double vz = -rs;
-    theta = acos(fmax(-1.0, fmin(1.0, vz)));
-    phi = atan2(vy, vx);
-    double sd, cd;
-    sincos(pS - pK, &sd, &cd);
-    psi = atan2(ctS * stK * cd - stS * ctK, stK * sd);
-}
-
 // Two threads per (wave, (l, m) pair): one computes Y+, the other Y- (halves the dependency
 // chain each thread waits on).  FP64 plans evaluate the harmonics in FP64; mixed plans, whose
 // folded coefficients are FP32, evaluate them in FP32 (relative error near 1e-7, far below the
-// path's 1e-6 mismatch budget) and stay off GB300's narrow FP64 pipe.  The frame angles are FP64.
+// path's 1e-6 mismatch budget) and stay off GB300's narrow FP64 pipe.
 // One instantiation per arithmetic type keeps each kernel's code small (it runs cold, once).
+template <bool FP64>
+__device__ __forceinline__ void ylm_thread(const PlanHdr &h, bool wait)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int g = t >> 1, which = t & 1;
+    double2 y = make_double2(0.0, 0.0);
+    double2 *dst = nullptr;
+    if (g < h.total_pairs) {
+        const WaveDev *waves = tc_local(h, h.waves);
+        const WaveDev &W = waves[wave_of(waves, h.n_waves, g, true)];
+        const int p = g - W.pair_begin;
+        if (p < W.tr.n_pairs) {
+            const int2 lm = W.tr.pair_lm[p];
+            y = FP64 ? wave_harmonic<double>(W, lm, which) : wave_harmonic<float>(W, lm, which);
+            dst = W.ylm + 2 * p + which;
+        } else {
+            atomicOr(h.err, ERRBIT_INTERNAL);
+        }
+    }
+    if (wait) pdl_wait();
+    if (dst) *dst = y;
+}
+
 template <bool FP64>
 __global__ void __launch_bounds__(kYlmThreads) k_ylm(const PlanHdr *__restrict__ hp)
 {
-    const PlanHdr h = *hp;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int g = t >> 1, which = t & 1;
-    if (g >= h.total_pairs) return;
-    const int w = wave_of(h.waves, h.n_waves, g, true);
-    const WaveDev &W = h.waves[w];
-    const int p = g - W.pair_begin;
-    if (p >= W.tr.n_pairs) {
-        atomicOr(h.err, ERRBIT_INTERNAL);
-        return;
-    }
-    const int2 lm = W.tr.pair_lm[p];
-    double theta = W.theta, phi = W.phi, psi = 0.0;
-    if (W.frame == FEW_FRAME_SSB) frame_angles(W.theta, W.phi, W.theta_K, W.phi_K, theta, phi, psi);
-    double2 y = make_double2(0.0, 0.0);
-    const int mm = which == 0 ? lm.y : -lm.y;
-    if (which == 0 || lm.y > 0) {
-        y = FP64 ? swsh_m2_t<double>(lm.x, mm, theta, phi)
-                 : swsh_m2_t<float>(lm.x, mm, (float)theta, (float)phi);
-        if (which == 1 && (lm.x & 1)) y = make_double2(-y.x, -y.y);
-    }
-    if (W.frame == FEW_FRAME_SSB) {
-        double s2, c2;
-        sincos(2.0 * psi, &s2, &c2);
-        const double fr = -c2, fi = s2;  // -e^{-2 i psi}
-        y = make_double2(y.x * fr - y.y * fi, y.x * fi + y.y * fr);
-    }
-    W.ylm[2 * p + which] = y;
+    pdl_wait();
+    pdl_launch_dependents();
+    ylm_thread<FP64>(*hp, false);
 }
 
-cudaError_t launch_ylm(const PlanHdr *hdr_dev, int total_pairs, bool fp64, cudaStream_t st)
+// The plan in the parameters: the harmonics need nothing of an earlier kernel, only their store waits;
+// the last block copies the plan to the device for the kernels that follow.
+template <bool FP64>
+__global__ void __launch_bounds__(kYlmThreads) k_ylm_param(const __grid_constant__ PlanParam plan)
+{
+    pdl_launch_dependents();
+    ylm_thread<FP64>(*reinterpret_cast<const PlanHdr *>(plan.bytes), true);
+    tc_store_plan(plan);
+}
+
+cudaError_t launch_ylm(const PlanHdr *hdr_dev, const PlanParam *plan, int total_pairs, bool fp64,
+                       cudaStream_t st)
 {
     if (total_pairs <= 0) return cudaSuccess;
     const int threads = 2 * total_pairs, grid = (threads + kYlmThreads - 1) / kYlmThreads;
-    if (fp64)
-        k_ylm<true><<<grid, kYlmThreads, 0, st>>>(hdr_dev);
-    else
-        k_ylm<false><<<grid, kYlmThreads, 0, st>>>(hdr_dev);
-    return cudaGetLastError();
+    if (plan) return launch_pdl(fp64 ? k_ylm_param<true> : k_ylm_param<false>, grid, kYlmThreads, 0, st, *plan);
+    return launch_pdl(fp64 ? k_ylm<true> : k_ylm<false>, grid, kYlmThreads, 0, st, hdr_dev);
 }
+
+__device__ __forceinline__ double cvt(double v, double) { return v; }
+__device__ __forceinline__ float cvt(double v, float) { return f64_to_f32_fast(v); }
 
 template <typename T> struct Slot8;
 template <> struct Slot8<double> {
@@ -137,8 +114,11 @@ template <> struct Slot8<float> {
     }
 };
 
-// One thread per (wave, segment, slot).  T is the arithmetic and storage type of the folded
-// coefficients (double for FEW_FP64, float for FEW_MIXED, whose amplitudes are FP32 by design).
+// One thread per (wave, segment, slot): K_slot = scale * sum of its contributions, summed on the
+// splines' Hermite data (values and slopes at the segment's two knots) and turned into power
+// coefficients in u once.
+// T is the arithmetic and storage type of the folded coefficients (double for FEW_FP64,
+// float for FEW_MIXED, whose amplitudes are FP32 by design).
 template <typename T>
 __global__ void __launch_bounds__(kFoldThreads) k_fold(const PlanHdr *__restrict__ hp)
 {
@@ -151,8 +131,39 @@ __global__ void __launch_bounds__(kFoldThreads) k_fold(const PlanHdr *__restrict
     const int slot = (local % W.fold_blocks_per_seg) * kFoldThreads + threadIdx.x;
     const TrajDev &tr = W.tr;
     if (s >= tr.S || slot >= tr.n_slots) return;
+    T re[4] = {0, 0, 0, 0}, im[4] = {0, 0, 0, 0};
+    const int c0 = tr.slot_ptr[slot], c1 = tr.slot_ptr[slot + 1];
+    const double *__restrict__ cs = tr.coef + (size_t)s * tr.J * 4;
+    for (int c = c0; c < c1; ++c) {
+        const int2 code = tr.contrib[c];  // (mode * 2 + kind, harmonic-table index)
+        const int i = code.x >> 1, kind = code.x & 1;
+        const double2 Yd = W.ylm[code.y];
+        const T yr = cvt(Yd.x, T()), yi = cvt(Yd.y, T());
+        const double2 *ca = reinterpret_cast<const double2 *>(cs + (size_t)(2 + 2 * i) * 4);
+        const double2 r01 = ca[0], r23 = ca[1], i01 = ca[2], i23 = ca[3];
+        const T ar[4] = {cvt(r01.x, T()), cvt(r01.y, T()), cvt(r23.x, T()), cvt(r23.y, T())};
+        T ai[4] = {cvt(i01.x, T()), cvt(i01.y, T()), cvt(i23.x, T()), cvt(i23.y, T())};
+        if (kind) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) ai[q] = -ai[q];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            re[q] += ar[q] * yr - ai[q] * yi;
+            im[q] += ar[q] * yi + ai[q] * yr;
+        }
+    }
+    // the folded values are Hermite data (the fold is linear in them): power coefficients in u
+    // once per (segment, slot)
+    const T hk = cvt(tr.h[s], T()), sc = cvt(W.scale, T());
     T pre[4], pim[4];
-    fold_slot<T>(tr, W.ylm, tr.coef + (size_t)s * tr.J * 4, slot, tr.h[s], W.scale, pre, pim);
+    hermite_to_power(re[0], re[1], re[2], re[3], hk, pre);
+    hermite_to_power(im[0], im[1], im[2], im[3], hk, pim);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        pre[q] *= sc;
+        pim[q] *= sc;
+    }
     T *dst = reinterpret_cast<T *>(W.fcoef) + ((size_t)s * tr.n_slots + slot) * 8;
     Slot8<T>::store(dst, pre, pim);
 }

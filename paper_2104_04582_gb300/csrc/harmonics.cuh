@@ -9,6 +9,8 @@
 // and the Jacobi polynomial by its three-term recurrence in the degree.
 #pragma once
 
+#include "fewsum_internal.h"
+
 namespace fewsum {
 
 // Arithmetic-type overloads (double for the FP64 path, float for the mixed path).
@@ -108,6 +110,20 @@ __device__ inline double2 swsh_m2_t(int l, int m, T theta, T phi)
 __device__ inline double2 swsh_m2(int l, int m, double theta, double phi)
 {
     return swsh_m2_t<double>(l, m, theta, phi);
+}
+
+// Harmonic `which` (0: Y+ = -2Y_{l,m}, 1: Y- = (-1)^l -2Y_{l,-m}, zero for m = 0) of one (l, m) pair
+// for a wave's viewing direction, in the arithmetic type T, times the frame's constant.
+template <typename T>
+__device__ inline double2 wave_harmonic(const WaveDev &W, int2 lm, int which)
+{
+    double2 y = make_double2(0.0, 0.0);
+    if (which == 0 || lm.y > 0) {
+        y = swsh_m2_t<T>(lm.x, which == 0 ? lm.y : -lm.y, (T)W.theta, (T)W.phi);
+        if (which == 1 && (lm.x & 1)) y = make_double2(-y.x, -y.y);
+    }
+    if (W.rotate) y = make_double2(y.x * W.rot_r - y.y * W.rot_i, y.x * W.rot_i + y.y * W.rot_r);
+    return y;
 }
 
 }  // namespace fewsum

@@ -1,0 +1,35 @@
+// launch.cuh -- programmatic dependent launch: a call's kernels (spline build, fold, summation) follow one
+// another on a stream, and each may be put on the chip while the one before it still runs; it does
+// what needs none of that one's results (barriers, tensor memory, harmonics), then waits for its
+// completion.  Every kernel launched by launch_pdl executes pdl_wait() before it reads or writes
+// anything that an earlier kernel may use, in every block.
+#pragma once
+
+#include <cuda_runtime.h>
+
+namespace fewsum {
+
+// Waits until the kernels this one depends on have completed and their writes are visible.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Lets the next kernel's blocks be scheduled once every block of this one has got here.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem,
+                              cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
+}  // namespace fewsum

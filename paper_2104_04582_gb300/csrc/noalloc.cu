@@ -164,8 +164,7 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     unsigned char *d_anc = d_ylm + ylm_bytes;
 
     W->tr = v.dev;
-    W->theta = r.theta;
-    W->phi = r.phi;
+    set_wave_angles(r, *W);
     W->scale = r.scale;
     W->dphi_phi = r.dphi_phi0;
     W->dphi_r = r.dphi_r0;
@@ -174,9 +173,6 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     W->n_samples = (int)ns;
     W->out_c64 = r.out_c64 ? 1 : 0;
     W->out = r.out;
-    W->frame = r.frame;
-    W->theta_K = r.theta_K;
-    W->phi_K = r.phi_K;
     W->fcoef = d_fcoef;
     W->ylm = reinterpret_cast<double2 *>(d_ylm);
     W->seg_start = reinterpret_cast<const int *>(base + off_seg);
@@ -227,6 +223,7 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     hdr->buf_bytes = buf_bytes;
     hdr->stage_slots = stage_slots;
     hdr->ring = kDefaultRing;
+    hdr->self = base;
     hdr->variant = tc ? (fp64 ? kVariantTc64 : kVariantTc) : variant;
     hdr->waves = reinterpret_cast<const WaveDev *>(base + off_waves);
     hdr->cta = reinterpret_cast<const CtaStart *>(base + off_cta);
@@ -242,8 +239,9 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     if (cudaGetLastError() != cudaSuccess) return FEW_ERR_CUDA;
     const PlanHdr *hd = reinterpret_cast<const PlanHdr *>(base);
     if (tc) {
-        if (launch_ylm(hd, v.n_pairs, fp64, s) != cudaSuccess ||
-            (fp64 ? launch_fold_tc64(hd, S, n_tiles, s) : launch_fold_tc(hd, S, n_tiles, s)) != cudaSuccess ||
+        if ((fp64 && launch_ylm(hd, nullptr, v.n_pairs, true, s) != cudaSuccess) ||
+            (fp64 ? launch_fold_tc64(hd, S, n_tiles, s)
+                  : launch_fold_tc(hd, nullptr, S, n_tiles, s)) != cudaSuccess ||
             (fp64 ? launch_sum_tc64(hd, grid_tc, v.tc_ks, s) : launch_sum_tc(hd, grid_tc, v.tc_ks, s)) !=
                 cudaSuccess) {
             (void)cudaGetLastError();
@@ -251,7 +249,7 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
         }
         return FEW_OK;
     }
-    if (launch_ylm(hd, v.n_pairs, fp64, s) != cudaSuccess ||
+    if (launch_ylm(hd, nullptr, v.n_pairs, fp64, s) != cudaSuccess ||
         launch_fold(hd, hdr->total_fold_blocks, fp64, s) != cudaSuccess ||
         launch_anchor(hd, fp64 ? 0 : S, s) != cudaSuccess ||
         launch_sum(hd, grid, T, R, smem, variant, s) != cudaSuccess) {

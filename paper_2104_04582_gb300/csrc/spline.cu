@@ -25,6 +25,7 @@
 // two phase arrays are fitted in radians as given (their reduction modulo 2 pi happens per
 // segment and per sample in the summation kernel).
 #include "fewsum_internal.h"
+#include "launch.cuh"
 
 namespace fewsum {
 
@@ -224,19 +225,11 @@ constexpr int kBuildSharedKnots = 180;  // largest K parked in shared memory (< 
 constexpr int kSepN = kBuildParts - 1;  // separators of a spline at most
 
 template <bool kShared>
-__global__ void __launch_bounds__(kBuildThreads)
-k_build(const BuildJob *__restrict__ jobs, int n_jobs, unsigned *err)
+__device__ __forceinline__ void build_block(const BuildJob &jb, int blk, unsigned *err)
 {
     extern __shared__ double sk[];  // [kBuildStaged][K], then (kShared) values, slopes [K][8]
     __shared__ double s_sinv[kSepN * kSepN];
     __shared__ int s_parts[kBuildParts + 2];
-    int lo = 0, hi = n_jobs - 1;
-    const int blk = blockIdx.x;
-    while (lo < hi) {  // job of this block: largest q with jobs[q].block_begin <= blk
-        int mid = (lo + hi + 1) >> 1;
-        if (jobs[mid].block_begin <= blk) lo = mid; else hi = mid - 1;
-    }
-    const BuildJob &jb = jobs[lo];
     const TrajDev &tr = jb.tr;
     const int K = tr.K, J = tr.J;
     double *ra = sk, *rb = sk + K, *fl = sk + 2 * K, *fu = sk + 3 * K, *fv = sk + 4 * K,
@@ -251,6 +244,7 @@ k_build(const BuildJob *__restrict__ jobs, int n_jobs, unsigned *err)
     }
     for (int i = threadIdx.x; i < kSepN * kSepN; i += blockDim.x) s_sinv[i] = tr.fac_sinv[i];
     if (threadIdx.x < kBuildParts + 2) s_parts[threadIdx.x] = tr.parts[threadIdx.x];
+    pdl_wait();  // the factors above are the trajectory's own; the knot data may be an earlier kernel's
     __syncthreads();
     const int P = s_parts[0];
     const int b = threadIdx.x & (kBuildParts - 1);
@@ -419,12 +413,40 @@ k_build(const BuildJob *__restrict__ jobs, int n_jobs, unsigned *err)
     if ((bad & 0x80000000u) && live) atomicOr(err, ERRBIT_NONFINITE);
 }
 
+// A batch's jobs: block -> job by its first block.
+template <bool kShared>
+__global__ void __launch_bounds__(kBuildThreads)
+k_build(const BuildJob *__restrict__ jobs, int n_jobs, unsigned *err)
+{
+    pdl_launch_dependents();
+    int lo = 0, hi = n_jobs - 1;
+    const int blk = blockIdx.x;
+    while (lo < hi) {  // job of this block: largest q with jobs[q].block_begin <= blk
+        int mid = (lo + hi + 1) >> 1;
+        if (jobs[mid].block_begin <= blk) lo = mid; else hi = mid - 1;
+    }
+    build_block<kShared>(jobs[lo], blk, err);
+}
+
+// One trajectory, its job in the parameters (no upload before the launch).
+template <bool kShared>
+__global__ void __launch_bounds__(kBuildThreads)
+k_build_one(const __grid_constant__ BuildJob job, unsigned *err)
+{
+    pdl_launch_dependents();
+    build_block<kShared>(job, blockIdx.x, err);
+}
+
+static int build_smem(bool shared, int knots)
+{
+    return (kBuildStaged + (shared ? 2 * kBuildSplines : 0)) * knots * (int)sizeof(double);
+}
+
 cudaError_t launch_build(const BuildJob *jobs_dev, int n_jobs, int total_blocks, int max_knots,
                          unsigned *err, cudaStream_t st)
 {
     const bool shared = max_knots <= kBuildSharedKnots;
-    const int per_knot = kBuildStaged + (shared ? 2 * kBuildSplines : 0);
-    const int smem_bytes = per_knot * max_knots * (int)sizeof(double);
+    const int smem_bytes = build_smem(shared, max_knots);
     auto kern = shared ? k_build<true> : k_build<false>;
     if (smem_bytes > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -432,8 +454,20 @@ cudaError_t launch_build(const BuildJob *jobs_dev, int n_jobs, int total_blocks,
         if (e != cudaSuccess) return e;
     }
     if (total_blocks <= 0) return cudaSuccess;
-    kern<<<total_blocks, kBuildThreads, smem_bytes, st>>>(jobs_dev, n_jobs, err);
-    return cudaGetLastError();
+    return launch_pdl(kern, total_blocks, kBuildThreads, smem_bytes, st, jobs_dev, n_jobs, err);
+}
+
+cudaError_t launch_build_one(const BuildJob &job, int blocks, unsigned *err, cudaStream_t st)
+{
+    const bool shared = job.tr.K <= kBuildSharedKnots;
+    const int smem_bytes = build_smem(shared, job.tr.K);
+    auto kern = shared ? k_build_one<true> : k_build_one<false>;
+    if (smem_bytes > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             smem_bytes);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_pdl(kern, blocks, kBuildThreads, smem_bytes, st, job, err);
 }
 
 }  // namespace fewsum

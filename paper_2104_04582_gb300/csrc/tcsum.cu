@@ -32,7 +32,9 @@
 #include <cuda_fp16.h>
 
 #include "fewsum_internal.h"
-#include "fold_slot.cuh"
+#include "convert.cuh"
+#include "fold_tc.cuh"
+#include "harmonics.cuh"
 #include "tctile.cuh"
 
 namespace fewsum {
@@ -42,76 +44,57 @@ namespace {
 constexpr int kTcGroups = 4;                        // warpgroups
 constexpr int kTcThreads = 128 * kTcGroups;
 constexpr int kTcDrain = 6;                         // row pairs in registers while draining
-constexpr int kTcMaxN = 16 * kTcMaxPairs;  // accumulator columns
 constexpr int kTcMaxKs = (kTcMaxHalf + 8) / 8;
+constexpr int kTcMaxLm = 31 * kTcMaxPairs;  // (l, m) pairs: 2 <= l <= 32, m <= 10
 constexpr int kTcMaxTable = 1024 * kTcMaxPairs * kTcMaxKs;
 constexpr uint32_t kTcDStride = 192, kTcECol = 384, kTcEStride = 64, kTcELo = 32;  // tmem columns
 
 __device__ __forceinline__ float pow2(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
 
-// Row stride (floats) of the staged table: 16-byte aligned, and 8 consecutive rows start 4 banks
-// apart, so the packing reads of a quarter-warp do not collide.
-__host__ __device__ constexpr int staged_stride(int ks) { return 16 * ks + 4; }
-
 }  // namespace
 
-// Operand tables and tile records.  Block g < total_segs: segment g's table, one thread per (row,
-// b) forming the cubics of the slots n_mid + b and n_mid - b and their X and Y; the block then
-// scales by the power of two that brings the table's largest entry into [2^14, 2^15) and packs
+// Operand tables and tile records.  Block g < total_segs: segment g's table.  The block computes the
+// harmonics (252 of them for l <= 10; they need nothing of the spline build before it), forms the
+// cubics, scales by the power of two that brings the table's largest entry into [2^14, 2^15) and packs
 // high and low fp16 parts as the MMA reads them (K-major without swizzle: 8 x 16 B core matrices,
-// 128 B apart along K).  Column 16 p + 2 x + e of the product is the row of signed m = m_top - p
-// (e = 0) or p - m_top (e = 1; zero for m = 0), x = 4 component + degree; basis value 2 b is cos(b theta), 2 b + 1 sin(b theta).  The blocks
-// after that fill the tile records (FP64 work beside the fold's gathers).
-__global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *__restrict__ hp)
+// 128 B apart along K; column 16 p + 2 x + e of the product is row 16 p + 2 x + e of the cubics, basis
+// value 2 b is cos(b theta), 2 b + 1 sin(b theta)).  The blocks after that fill the tile records (FP64
+// work beside the fold's gathers).
+// wait: the plan is in the parameters (at a device address it is read after pdl_wait).
+__device__ __forceinline__ void fold_tc_block(const PlanHdr &h, bool wait)
 {
-    extern __shared__ __align__(16) float tcf[];
+    extern __shared__ __align__(16) float tcf[];  // cubics, then harmonics
     __shared__ float s_max[kTcFoldThreads / 32];
-    const PlanHdr &h = *hp;
     const int tid = threadIdx.x;
     if ((int)blockIdx.x >= h.total_segs) {
+        if (wait) pdl_wait();
         const int T = ((int)blockIdx.x - h.total_segs) * kTcRecThreads + tid;
         if (tid < kTcRecThreads && T < h.total_tiles) tc_fill_record(h, T, false);
         return;
     }
-    const WaveDev &W = h.waves[tc_wave_of_seg(h, blockIdx.x)];
+    const WaveDev &W = tc_wave(h, tc_wave_of_seg(h, blockIdx.x));
     const TrajDev &tr = W.tr;
     const int s = (int)blockIdx.x - W.seg_begin;
-    if (s >= tr.S || W.tile_off[s] == W.tile_off[s + 1]) return;  // no sample in this segment
-    const int P = tr.tc_pairs, ks = tr.tc_ks, nb = 8 * ks, ld = staged_stride(ks);
-    const double *cs = tr.coef + (size_t)s * tr.J * 4;
-    const double hk = tr.h[s];
+    const int *tile_off = tc_local(h, W.tile_off);
+    const bool any = s < tr.S && tile_off[s] < tile_off[s + 1];  // samples in this segment
+    const int P = tr.tc_pairs, ks = tr.tc_ks, ld = fold_stride(ks, sizeof(float));
+    float2 *Y = reinterpret_cast<float2 *>(tcf + 16 * P * ld);
+    if (any) {
+        for (int t = tid; t < 2 * tr.n_pairs; t += blockDim.x) {
+            const double2 y = wave_harmonic<float>(W, tr.pair_lm[t >> 1], t & 1);
+            Y[t] = make_float2(f64_to_f32_fast(y.x), f64_to_f32_fast(y.y));
+        }
+    }
+    if (wait) pdl_wait();
+    if (!any) return;
+    __syncthreads();
+    fold_rows<float>(tr, s, W.scale, Y, tcf);
+    __syncthreads();
     float mx = 0.0f;
-    for (int it = tid; it < 2 * P * nb; it += blockDim.x) {
-        const int row = it / nb, b = it - row * nb;
-        float X[8], Y[8];  // x = 4 component + degree
-#pragma unroll
-        for (int x = 0; x < 8; ++x) X[x] = Y[x] = 0.0f;
-        const int m = (row & 1) ? (row >> 1) - tr.m_top : tr.m_top - (row >> 1), j = tr.m_top - m;
-        if (j < tr.n_rows && !((row & 1) && m == 0)) {
-            const int4 rs = tr.row_slot[j];  // slots n = rs.y .. rs.z
-#pragma unroll
-            for (int sign = 0; sign < 2; ++sign) {
-                const int n = sign ? tr.n_mid - b : tr.n_mid + b;
-                if ((sign && b == 0) || n > rs.y || n < rs.z) continue;
-                float pr[4], pi[4];
-                fold_slot<float>(tr, W.ylm, cs, rs.x + rs.y - n, hk, W.scale, pr, pi);
-#pragma unroll
-                for (int d = 0; d < 4; ++d) {
-                    X[d] += pr[d];
-                    X[4 + d] += pi[d];
-                    if (b > 0) {  // Y = -i (c_+ - c_-)
-                        Y[d] += sign ? -pi[d] : pi[d];
-                        Y[4 + d] += sign ? pr[d] : -pr[d];
-                    }
-                }
-            }
-        }
-        float *dst = tcf + (16 * (row >> 1) + (row & 1)) * ld + 2 * b;
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            *reinterpret_cast<float2 *>(dst + 2 * x * ld) = make_float2(X[x], Y[x]);
-            mx = fmaxf(mx, fmaxf(fabsf(X[x]), fabsf(Y[x])));
-        }
+    for (int it = tid; it < 16 * P * 8 * ks; it += blockDim.x) {
+        float X, Z;
+        fold_basis(tcf, ks, it / (8 * ks), it % (8 * ks), X, Z);
+        mx = fmaxf(mx, fmaxf(fabsf(X), fabsf(Z)));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -129,13 +112,13 @@ __global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *__res
     const int c8n = 2 * ks;
     for (int id = tid; id < 16 * P * c8n; id += blockDim.x) {  // 16-byte chunks in memory order
         const int r8 = id & 7, g = id >> 3, c8 = g % c8n, r = (g / c8n) * 8 + r8;
-        const float4 *src = reinterpret_cast<const float4 *>(tcf + r * ld + 8 * c8);
-        const float4 p = src[0], q = src[1];
-        const float v[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
         uint32_t wh[4], wl[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const float x0 = v[2 * k] * f, x1 = v[2 * k + 1] * f;
+            float x0, x1;
+            fold_basis(tcf, ks, r, 4 * c8 + k, x0, x1);
+            x0 *= f;
+            x1 *= f;
             const __half2 hi = __floats2half2_rn(x0, x1);
             const float2 hf = __half22float2(hi);
             const __half2 lo = __floats2half2_rn(x0 - hf.x, x1 - hf.y);
@@ -145,6 +128,21 @@ __global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *__res
         reinterpret_cast<uint4 *>(hi_dst)[id] = make_uint4(wh[0], wh[1], wh[2], wh[3]);
         reinterpret_cast<uint4 *>(lo_dst)[id] = make_uint4(wl[0], wl[1], wl[2], wl[3]);
     }
+}
+
+__global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *__restrict__ hp)
+{
+    pdl_wait();
+    pdl_launch_dependents();
+    fold_tc_block(*hp, false);
+}
+
+// The plan in the parameters; the last block copies it to the device for the summation.
+__global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc_param(const __grid_constant__ PlanParam plan)
+{
+    pdl_launch_dependents();
+    fold_tc_block(*reinterpret_cast<const PlanHdr *>(plan.bytes), true);
+    tc_store_plan(plan);
 }
 
 namespace {
@@ -250,6 +248,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
     __shared__ __align__(16) uint32_t s_rec[4 * kTcGroups][32];  // each warp's tile record
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
+    pdl_wait();
+    pdl_launch_dependents();
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
     const TileRec *__restrict__ recs = hp->recs;
     const int T0 = hp->tile_cta[blockIdx.x], T1 = hp->tile_cta[blockIdx.x + 1];
@@ -478,6 +478,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
 
 namespace {
 using TcKernel = void (*)(const PlanHdr *);
+// cubics and harmonics of a fold block
+constexpr int kFoldSmem =
+    (16 * kTcMaxPairs * fold_stride(kTcMaxKs, sizeof(float)) + 4 * kTcMaxLm) * (int)sizeof(float);
 const TcKernel kTcKernels[kTcMaxKs] = {k_sum_tc<1>, k_sum_tc<2>, k_sum_tc<3>, k_sum_tc<4>};
 }  // namespace
 
@@ -488,24 +491,26 @@ cudaError_t tc_configure()
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kTcMaxTable);
         if (e != cudaSuccess) return e;
     }
-    return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(k_fold_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_fold_tc_param, cudaFuncAttributeMaxDynamicSharedMemorySize, kFoldSmem);
+    return e;
 }
 
-cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st)
+cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, const PlanParam *plan, int total_segs, int total_tiles,
+                           cudaStream_t st)
 {
     if (total_tiles <= 0) return cudaSuccess;
-    const int smem = kTcMaxN * staged_stride(kTcMaxKs) * (int)sizeof(float);
-    const int grid = total_segs + (total_tiles + kTcRecThreads - 1) / kTcRecThreads;
-    k_fold_tc<<<grid, kTcFoldThreads, smem, st>>>(hdr_dev);
-    return cudaGetLastError();
+    const unsigned grid = total_segs + (total_tiles + kTcRecThreads - 1) / kTcRecThreads;
+    if (plan) return launch_pdl(k_fold_tc_param, grid, kTcFoldThreads, kFoldSmem, st, *plan);
+    return launch_pdl(k_fold_tc, grid, kTcFoldThreads, kFoldSmem, st, hdr_dev);
 }
 
 cudaError_t launch_sum_tc(const PlanHdr *hdr_dev, int grid, int ks, cudaStream_t st)
 {
     if (grid <= 0) return cudaSuccess;
     if (ks < 1 || ks > kTcMaxKs) return cudaErrorInvalidValue;
-    kTcKernels[ks - 1]<<<grid, kTcThreads, 2 * kTcMaxTable, st>>>(hdr_dev);
-    return cudaGetLastError();
+    return launch_pdl(kTcKernels[ks - 1], grid, kTcThreads, 2 * kTcMaxTable, st, hdr_dev);
 }
 
 }  // namespace fewsum

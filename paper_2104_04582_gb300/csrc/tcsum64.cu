@@ -24,7 +24,7 @@
 #include <cuda_fp16.h>
 
 #include "fewsum_internal.h"
-#include "fold_slot.cuh"
+#include "fold_tc.cuh"
 #include "tctile.cuh"
 
 namespace fewsum {
@@ -41,8 +41,6 @@ constexpr uint32_t kT64DCol = kTc64Slices * kT64EStride;  // two accumulator set
 constexpr uint32_t kT64DStride = 16 * kTc64Slices;
 
 __device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }
-
-__host__ __device__ constexpr int staged64_stride(int ks) { return 16 * ks + 2; }
 
 // The 7 digits of x (a multiple of 2^-54, |x| <= 1) as unsigned bytes digit + 128, least
 // significant first.
@@ -61,59 +59,37 @@ __device__ __forceinline__ uint32_t digit_pair(uint32_t word, uint32_t sel)
 
 }  // namespace
 
-// Operand tables (block per segment) and tile records, as k_fold_tc, in FP64.  Chunk p of a table is
-// row pair p: 7 digit slices (most significant first) of 16 rows each.
-__global__ void __launch_bounds__(kT64FoldThreads) k_fold_tc64(const PlanHdr *__restrict__ hp)
+// Operand tables (block per segment) and tile records, as fold_tc_block, in FP64 (the harmonics by
+// k_ylm: in FP64 their latency is too long to be repeated in every block).  Chunk p of a table is row
+// pair p: 7 digit slices (most significant first) of 16 rows each.
+__device__ __forceinline__ void fold_tc64_block(const PlanHdr &h)
 {
     extern __shared__ __align__(16) double tcf64[];
     __shared__ double s_max[kT64FoldThreads / 32], s_sum[kT64FoldThreads / 32];
-    const PlanHdr &h = *hp;
     const int tid = threadIdx.x;
+    pdl_wait();
     if ((int)blockIdx.x >= h.total_segs) {
         const int T = ((int)blockIdx.x - h.total_segs) * kTcRecThreads + tid;
         if (tid < kTcRecThreads && T < h.total_tiles) tc_fill_record(h, T, true);
         return;
     }
-    const WaveDev &W = h.waves[tc_wave_of_seg(h, blockIdx.x)];
+    const WaveDev &W = tc_wave(h, tc_wave_of_seg(h, blockIdx.x));
     const TrajDev &tr = W.tr;
     const int s = (int)blockIdx.x - W.seg_begin;
-    if (s >= tr.S || W.tile_off[s] == W.tile_off[s + 1]) return;  // no sample in this segment
-    const int P = tr.tc_pairs, ks = tr.tc_ks, nb = 8 * ks, ld = staged64_stride(ks);
+    const int *tile_off = tc_local(h, W.tile_off);
+    if (s >= tr.S || tile_off[s] == tile_off[s + 1]) return;  // no sample in this segment
+    const int P = tr.tc_pairs, ks = tr.tc_ks;
     const double *cs = tr.coef + (size_t)s * tr.J * 4;
-    const double hk = tr.h[s];
+    fold_rows<double>(tr, s, W.scale, W.ylm, tcf64);
+    __syncthreads();
     double mx = 0.0, sum = 0.0;
-    for (int it = tid; it < 2 * P * nb; it += blockDim.x) {
-        const int row = it / nb, b = it - row * nb;
-        double X[8], Y[8];  // x = 4 component + degree
-#pragma unroll
-        for (int x = 0; x < 8; ++x) X[x] = Y[x] = 0.0;
-        const int m = (row & 1) ? (row >> 1) - tr.m_top : tr.m_top - (row >> 1), j = tr.m_top - m;
-        if (j < tr.n_rows && !((row & 1) && m == 0)) {
-            const int4 rs = tr.row_slot[j];  // slots n = rs.y .. rs.z
-#pragma unroll 1
-            for (int sign = 0; sign < 2; ++sign) {
-                const int n = sign ? tr.n_mid - b : tr.n_mid + b;
-                if ((sign && b == 0) || n > rs.y || n < rs.z) continue;
-                double pr[4], pi[4];
-                fold_slot<double>(tr, W.ylm, cs, rs.x + rs.y - n, hk, W.scale, pr, pi);
-#pragma unroll
-                for (int d = 0; d < 4; ++d) {
-                    X[d] += pr[d];
-                    X[4 + d] += pi[d];
-                    if (b > 0) {  // Y = -i (c_+ - c_-)
-                        Y[d] += sign ? -pi[d] : pi[d];
-                        Y[4 + d] += sign ? pr[d] : -pr[d];
-                    }
-                }
-            }
-        }
-        double *dst = tcf64 + (16 * (row >> 1) + (row & 1)) * ld + 2 * b;
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            *reinterpret_cast<double2 *>(dst + 2 * x * ld) = make_double2(X[x], Y[x]);
-            mx = fmax(mx, fmax(fabs(X[x]), fabs(Y[x])));
-            sum += 9.5367431640625e-7 * (fabs(X[x]) + fabs(Y[x]));  // 2^-20: no overflow
-        }
+    for (int it = tid; it < 16 * P * 8 * ks; it += blockDim.x) {
+        double X, Z;
+        fold_basis(tcf64, ks, it / (8 * ks), it % (8 * ks), X, Z);
+        X = fabs(X);
+        Z = fabs(Z);
+        mx = fmax(mx, fmax(X, Z));
+        sum += 9.5367431640625e-7 * (X + Z);  // 2^-20: no overflow
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -161,10 +137,14 @@ __global__ void __launch_bounds__(kT64FoldThreads) k_fold_tc64(const PlanHdr *__
     const int c8n = 2 * ks, slice = 512 * ks;  // bytes of one slice of one pair
     for (int id = tid; id < 16 * P * c8n; id += blockDim.x) {  // 16-byte chunks in memory order
         const int r8 = id & 7, g = id >> 3, c8 = g % c8n, r = (g / c8n) * 8 + r8;  // row 0 .. 16 P - 1
-        const double *src = tcf64 + r * ld + 8 * c8;
         unsigned long long v[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = digit_bytes(__double2ll_rn(src[k] * f1 * f2 * 18014398509481984.0));
+        for (int k = 0; k < 4; ++k) {
+            double X, Z;
+            fold_basis(tcf64, ks, r, 4 * c8 + k, X, Z);
+            v[2 * k] = digit_bytes(__double2ll_rn(X * f1 * f2 * 18014398509481984.0));
+            v[2 * k + 1] = digit_bytes(__double2ll_rn(Z * f1 * f2 * 18014398509481984.0));
+        }
         unsigned char *dst = tab + (size_t)(r >> 4) * kTc64Slices * slice + ((r >> 3) & 1) * 256 * ks +
                              c8 * 128 + r8 * 16;
 #pragma unroll
@@ -179,6 +159,12 @@ __global__ void __launch_bounds__(kT64FoldThreads) k_fold_tc64(const PlanHdr *__
             *reinterpret_cast<uint4 *>(dst + (size_t)q * slice) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
+}
+
+__global__ void __launch_bounds__(kT64FoldThreads) k_fold_tc64(const PlanHdr *__restrict__ hp)
+{
+    pdl_launch_dependents();
+    fold_tc64_block(*hp);
 }
 
 namespace {
@@ -367,6 +353,8 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
     __shared__ __align__(8) uint64_t b_full, d_full[2], d_empty[2], e_full[kT64Groups], done[kT64Groups];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
+    pdl_wait();
+    pdl_launch_dependents();
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
     const TileRec *__restrict__ recs = hp->recs;
     const int T0 = hp->tile_cta[blockIdx.x], T1 = hp->tile_cta[blockIdx.x + 1];
@@ -603,7 +591,7 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
 namespace {
 using Tc64Kernel = void (*)(const PlanHdr *);
 const Tc64Kernel kTc64Kernels[kT64MaxKs] = {k_sum_tc64<1>, k_sum_tc64<2>, k_sum_tc64<3>, k_sum_tc64<4>};
-constexpr int kFold64Smem = 16 * kTcMaxPairs * staged64_stride(kT64MaxKs) * (int)sizeof(double);
+constexpr int kFold64Smem = 16 * kTcMaxPairs * fold_stride(kT64MaxKs, sizeof(double)) * (int)sizeof(double);
 }  // namespace
 
 cudaError_t tc64_configure()
@@ -619,17 +607,15 @@ cudaError_t tc64_configure()
 cudaError_t launch_fold_tc64(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st)
 {
     if (total_tiles <= 0) return cudaSuccess;
-    const int grid = total_segs + (total_tiles + kTcRecThreads - 1) / kTcRecThreads;
-    k_fold_tc64<<<grid, kT64FoldThreads, kFold64Smem, st>>>(hdr_dev);
-    return cudaGetLastError();
+    const unsigned grid = total_segs + (total_tiles + kTcRecThreads - 1) / kTcRecThreads;
+    return launch_pdl(k_fold_tc64, grid, kT64FoldThreads, kFold64Smem, st, hdr_dev);
 }
 
 cudaError_t launch_sum_tc64(const PlanHdr *hdr_dev, int grid, int ks, cudaStream_t st)
 {
     if (grid <= 0) return cudaSuccess;
     if (ks < 1 || ks > kT64MaxKs) return cudaErrorInvalidValue;
-    kTc64Kernels[ks - 1]<<<grid, kT64Threads, kT64MaxTable, st>>>(hdr_dev);
-    return cudaGetLastError();
+    return launch_pdl(kTc64Kernels[ks - 1], grid, kT64Threads, kT64MaxTable, st, hdr_dev);
 }
 
 }  // namespace fewsum

@@ -3,10 +3,30 @@
 #pragma once
 
 #include "fewsum_internal.h"
+#include "launch.cuh"
 #include "phase_eval.cuh"
 #include "tcgen05.cuh"
 
 namespace fewsum {
+
+// A pointer into the plan, for a plan that may be read elsewhere than at its device address (from the
+// kernel parameters).
+template <typename T>
+__device__ __forceinline__ const T *tc_local(const PlanHdr &h, const T *p)
+{
+    return reinterpret_cast<const T *>(reinterpret_cast<const unsigned char *>(&h) +
+                                       (reinterpret_cast<const unsigned char *>(p) - h.self));
+}
+__device__ __forceinline__ const WaveDev &tc_wave(const PlanHdr &h, int w) { return tc_local(h, h.waves)[w]; }
+
+// The last block writes a plan that came in the parameters to its device address (after pdl_wait).
+__device__ __forceinline__ void tc_store_plan(const PlanParam &plan)
+{
+    if (blockIdx.x + 1 != gridDim.x) return;
+    const uint4 *src = reinterpret_cast<const uint4 *>(plan.bytes);
+    for (int i = threadIdx.x; i < (plan.n + 15) / 16; i += blockDim.x)
+        reinterpret_cast<uint4 *>(plan.dev)[i] = src[i];
+}
 
 // A value in turns as 2^-64 turn units modulo one turn.
 __device__ __forceinline__ long long turns_fixed(double y)
@@ -81,7 +101,7 @@ __device__ __forceinline__ int tc_wave_of_seg(const PlanHdr &h, int g)
     int lo = 0, hi = h.n_waves - 1;
     while (lo < hi) {  // largest w with seg_begin <= g
         const int mid = (lo + hi + 1) >> 1;
-        if (h.waves[mid].seg_begin <= g) lo = mid; else hi = mid - 1;
+        if (tc_wave(h, mid).seg_begin <= g) lo = mid; else hi = mid - 1;
     }
     return lo;
 }
@@ -93,21 +113,22 @@ __device__ inline void tc_fill_record(const PlanHdr &h, int T, bool fp64)
     int lo = 0, hi = h.n_waves - 1;
     while (lo < hi) {  // largest w with tile_begin <= T
         const int mid = (lo + hi + 1) >> 1;
-        if (h.waves[mid].tile_begin <= T) lo = mid; else hi = mid - 1;
+        if (tc_wave(h, mid).tile_begin <= T) lo = mid; else hi = mid - 1;
     }
-    const WaveDev &W = h.waves[lo];
+    const WaveDev &W = tc_wave(h, lo);
     const TrajDev &tr = W.tr;
+    const int *tile_off = tc_local(h, W.tile_off), *seg_start = tc_local(h, W.seg_start);
     const int t = T - W.tile_begin;
     int s = 0, e = tr.S - 1;
     while (s < e) {  // largest s with tile_off[s] <= t: the segment that holds tile t
         const int mid = (s + e + 1) >> 1;
-        if (W.tile_off[mid] <= t) s = mid; else e = mid - 1;
+        if (tile_off[mid] <= t) s = mid; else e = mid - 1;
     }
     TileRec r;
-    r.s0 = W.seg_start[s];
-    r.s1 = W.seg_start[s + 1];
-    r.i0 = (r.s0 / kTcTile + (t - W.tile_off[s])) * kTcTile;
-    r.tile_end = W.tile_begin + W.tile_off[s + 1];
+    r.s0 = seg_start[s];
+    r.s1 = seg_start[s + 1];
+    r.i0 = (r.s0 / kTcTile + (t - tile_off[s])) * kTcTile;
+    r.tile_end = W.tile_begin + tile_off[s + 1];
     const SegPhase sp = seg_phase(tr, s, W.dphi_phi, W.dphi_r);
     const double kInv2Pi = 0.15915494309189533577;
     const double u = (fma((double)max(r.i0, r.s0), W.dt, W.t0) - sp.tk) * sp.ih, du = W.dt * sp.ih;
