@@ -639,7 +639,7 @@ void fill_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P, unsign
             W.seg_begin = seg_begin;
             seg_begin += tr->S;
             tile_begin.push_back(tile_begin[q] + a);
-            tile_cost.push_back(tc_tile_cost(P.fp64, tr->plan.tc_pairs, tr->plan.tc_ks));
+            tile_cost.push_back(tc_tile_cost(P.fp64, tr->plan.tc_pairs, L.ks));
         } else if (!P.fp64) {
             int a = 0;
             for (int k = 0; k + 1 < tr->K; ++k) {

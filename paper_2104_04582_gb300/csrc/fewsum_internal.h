@@ -246,11 +246,11 @@ inline size_t tc_segment_bytes(bool fp64, int pairs, int ks)
 {
     return fp64 ? tc64_table_bytes(pairs, ks) + sizeof(TcSeg64) : tc_table_bytes(pairs, ks) + sizeof(float);
 }
-// Relative cost of one tile (cycles): the MMAs, or the per-sample work around them.
+// Relative cost of one tile, as measured (mixed: ns; its per-sample work around the MMAs is
+// nearly the same for every mode set): pairs of the wave, K steps of the plan's widest.
 inline double tc_tile_cost(bool fp64, int pairs, int ks)
 {
-    if (fp64) return pairs * (364.0 * ks > 1000.0 ? 364.0 * ks : 1000.0) + 1200.0 * ks + 1600.0;
-    return 24.0 * pairs * ks + 300.0;
+    return fp64 ? 1900.0 + 690.0 * pairs + 650.0 * ks : 390.0 + 9.0 * pairs + 43.0 * ks;
 }
 inline int tiles_in_segment(int s_begin, int s_end)
 {
