@@ -711,8 +711,8 @@ cudaError_t launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, const PlanParam *
         if (fp64 && (e = launch_ylm(hdr_dev, plan, P.total_pairs, fp64, st)) != cudaSuccess) return e;
         tm(1, true);
         tm(2, false);
-        e = fp64 ? launch_fold_tc64(hdr_dev, P.total_segs, P.total_tiles, st)
-                 : launch_fold_tc(hdr_dev, plan, P.total_segs, P.total_tiles, st);
+        e = fp64 ? launch_fold_tc64(hdr_dev, P.total_segs, P.total_tiles, c->sm_count, st)
+                 : launch_fold_tc(hdr_dev, plan, P.total_segs, P.total_tiles, c->sm_count, st);
         if (e != cudaSuccess) return e;
         tm(2, true);
         tm(3, false);

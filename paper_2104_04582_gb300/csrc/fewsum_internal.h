@@ -43,7 +43,13 @@ constexpr int kTcMaxPairs = 11;  // rows m and -m, max m <= 10: two accumulators
                                  //   pair, beside the operands, in the 512 tensor-memory columns
 constexpr int kTcMaxHalf = 31;  // half-width of the n range: 64 basis values (K)
 constexpr int kTcFoldThreads = 704;
-constexpr int kTcRecThreads = 128;  // threads of a fold block that fill tile records
+// Fold blocks that fill tile records: 128 tiles each, until there are four a multiprocessor.
+constexpr int kTcRecTiles = 128;
+inline int tc_record_blocks(int total_tiles, int sm_count)
+{
+    const int n = (total_tiles + kTcRecTiles - 1) / kTcRecTiles, most = 4 * sm_count;
+    return n < most ? n : most;
+}
 // Everything the summation reads for one tile, one 128-byte line.  Phases of sample a + v, a =
 // max(i0, s0): c0 + c1 v + c2 v^2 + c3 v^3 turns modulo 1, each coefficient in units of 2^-64 turn
 // (64-bit wrap-around arithmetic is then the exact reduction modulo one turn).
@@ -258,12 +264,12 @@ inline int tiles_in_segment(int s_begin, int s_end)
 }
 cudaError_t tc_configure();
 cudaError_t tc64_configure();
-cudaError_t launch_fold_tc64(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st);
+cudaError_t launch_fold_tc64(const PlanHdr *hdr_dev, int total_segs, int total_tiles, int sm_count, cudaStream_t st);
 cudaError_t launch_sum_tc64(const PlanHdr *hdr_dev, int grid, int ks, cudaStream_t st);
 // plan: the plan itself (the kernel then writes it to hdr_dev for those that follow), or null when it
 // is at hdr_dev already.
 cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, const PlanParam *plan, int total_segs, int total_tiles,
-                           cudaStream_t st);
+                           int sm_count, cudaStream_t st);
 // ks: the most K steps of any wave of the plan.
 cudaError_t launch_sum_tc(const PlanHdr *hdr_dev, int grid, int ks, cudaStream_t st);
 // Bytes of one folded slot in the layout a variant reads.

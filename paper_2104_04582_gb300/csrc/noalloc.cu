@@ -240,8 +240,8 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     const PlanHdr *hd = reinterpret_cast<const PlanHdr *>(base);
     if (tc) {
         if ((fp64 && launch_ylm(hd, nullptr, v.n_pairs, true, s) != cudaSuccess) ||
-            (fp64 ? launch_fold_tc64(hd, S, n_tiles, s)
-                  : launch_fold_tc(hd, nullptr, S, n_tiles, s)) != cudaSuccess ||
+            (fp64 ? launch_fold_tc64(hd, S, n_tiles, v.sm_count, s)
+                  : launch_fold_tc(hd, nullptr, S, n_tiles, v.sm_count, s)) != cudaSuccess ||
             (fp64 ? launch_sum_tc64(hd, grid_tc, v.tc_ks, s) : launch_sum_tc(hd, grid_tc, v.tc_ks, s)) !=
                 cudaSuccess) {
             (void)cudaGetLastError();

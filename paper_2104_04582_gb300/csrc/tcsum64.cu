@@ -69,8 +69,7 @@ __device__ __forceinline__ void fold_tc64_block(const PlanHdr &h)
     const int tid = threadIdx.x;
     pdl_wait();
     if ((int)blockIdx.x >= h.total_segs) {
-        const int T = ((int)blockIdx.x - h.total_segs) * kTcRecThreads + tid;
-        if (tid < kTcRecThreads && T < h.total_tiles) tc_fill_record(h, T, true);
+        tc_fill_records<true>(h, reinterpret_cast<SegFill<true> *>(tcf64));
         return;
     }
     const WaveDev &W = tc_wave(h, tc_wave_of_seg(h, blockIdx.x));
@@ -604,10 +603,11 @@ cudaError_t tc64_configure()
     return cudaFuncSetAttribute(k_fold_tc64, cudaFuncAttributeMaxDynamicSharedMemorySize, kFold64Smem);
 }
 
-cudaError_t launch_fold_tc64(const PlanHdr *hdr_dev, int total_segs, int total_tiles, cudaStream_t st)
+cudaError_t launch_fold_tc64(const PlanHdr *hdr_dev, int total_segs, int total_tiles, int sm_count,
+                             cudaStream_t st)
 {
     if (total_tiles <= 0) return cudaSuccess;
-    const unsigned grid = total_segs + (total_tiles + kTcRecThreads - 1) / kTcRecThreads;
+    const unsigned grid = total_segs + tc_record_blocks(total_tiles, sm_count);
     return launch_pdl(k_fold_tc64, grid, kT64FoldThreads, kFold64Smem, st, hdr_dev);
 }
 

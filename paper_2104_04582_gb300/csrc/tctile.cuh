@@ -2,6 +2,8 @@
 // fixed-point phases and the warpgroup barrier.
 #pragma once
 
+#include <type_traits>
+
 #include "fewsum_internal.h"
 #include "launch.cuh"
 #include "phase_eval.cuh"
@@ -28,10 +30,20 @@ __device__ __forceinline__ void tc_store_plan(const PlanParam &plan)
         reinterpret_cast<uint4 *>(plan.dev)[i] = src[i];
 }
 
-// A value in turns as 2^-64 turn units modulo one turn.
+// A value in turns as 2^-64 turn units modulo one turn (0 if not finite): the significand shifted into
+// place.  (Four FP64 instructions would do it too, of 64 cycles each for a scheduler's warp.)
 __device__ __forceinline__ long long turns_fixed(double y)
 {
-    return __double2ll_rn((y - rint(y)) * 18446744073709551616.0);
+    const unsigned long long b = (unsigned long long)__double_as_longlong(y);
+    const int e = (int)(b >> 52) & 2047, sh = e - 1011;  // significand 2^(e - 1075) = units 2^sh
+    const unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    unsigned long long v = 0;
+    if (sh >= 0) {
+        if (sh < 64) v = m << sh;
+    } else if (sh > -55) {
+        v = ((m >> (-sh - 1)) + 1) >> 1;
+    }
+    return (long long)((long long)b < 0 ? 0ull - v : v);
 }
 
 // Pairs hi + lo of doubles (106 bits) for the FP64 plans' records: one anchor stands for 128 samples,
@@ -67,33 +79,7 @@ __device__ __forceinline__ Dd dd_div(const Dd &a, double b)
 }
 __device__ __forceinline__ long long dd_turns_fixed(const Dd &a)
 {
-    return (long long)((unsigned long long)__double2ll_rn((a.h - rint(a.h)) * 18446744073709551616.0) +
-                       (unsigned long long)__double2ll_rn(a.l * 18446744073709551616.0));
-}
-
-// The Taylor coefficients (turns per sample^k, fixed point) of one phase spline about time x after the
-// segment's first knot, from its Hermite data (values y0, y1, slopes s0, s1, width h) in pairs; offset
-// added to the phase.  v^3 reaches 2^21, so the cubic coefficient also gets its next 32 bits (lo3, units
-// of 2^-96 turn).
-__device__ inline void dd_phase_taylor(const double *c, double h, const Dd &x, double dt, double offset,
-                                       long long (&out)[4], int &lo3)
-{
-    const Dd inv2pi{0.15915494309189535, -9.8393400450386e-18};  // 1/(2 pi)
-    const Dd a = dd_prod(h, c[2]), b = dd_prod(h, c[3]), D = dd_sum(c[1], -c[0]);
-    const Dd p1 = dd_add(dd_scale(D, 3.0), dd_add(dd_scale(a, -2.0), Dd{-b.h, -b.l}));
-    const Dd p2 = dd_add(dd_add(a, b), dd_scale(D, -2.0));
-    const Dd u = dd_div(x, h), du = dd_mul(dd_div(Dd{dt, 0.0}, h), inv2pi), w = dd_div(Dd{dt, 0.0}, h);
-    const Dd v0 = dd_mul(dd_add(dd_mul(dd_add(dd_mul(p2, u), p1), u), a), u);
-    out[0] = dd_turns_fixed(dd_mul(dd_add(v0, dd_sum(c[0], offset)), inv2pi));
-    const Dd q = dd_add(dd_scale(dd_mul(p2, u), 3.0), p1);                                // Phi''/2
-    const Dd d1 = dd_add(dd_mul(dd_add(dd_scale(dd_mul(p2, u), 3.0), dd_scale(p1, 2.0)), u), a);  // Phi'
-    out[1] = dd_turns_fixed(dd_mul(d1, du));
-    out[2] = dd_turns_fixed(dd_mul(dd_mul(q, w), du));
-    const Dd c3 = dd_mul(dd_mul(dd_mul(p2, w), w), du);
-    const double x3 = (c3.h - rint(c3.h)) * 18446744073709551616.0;
-    out[3] = __double2ll_rn(x3);
-    const double rest = (x3 - (double)out[3]) + c3.l * 18446744073709551616.0;
-    lo3 = __double2int_rn(rest * 4294967296.0);
+    return (long long)((unsigned long long)turns_fixed(a.h) + (unsigned long long)turns_fixed(a.l));
 }
 
 __device__ __forceinline__ int tc_wave_of_seg(const PlanHdr &h, int g)
@@ -106,9 +92,158 @@ __device__ __forceinline__ int tc_wave_of_seg(const PlanHdr &h, int g)
     return lo;
 }
 
-// Record of tile T: its segment, the phases at its first sample and their Taylor expansion (FP64;
-// pairs of FP64 for the FP64 plans).
-__device__ inline void tc_fill_record(const PlanHdr &h, int T, bool fp64)
+// Tile records.  A record holds the Taylor expansion of its segment's phases about the tile's first
+// sample: polynomials in u = (t - t_k)/h of the phase and of its derivatives per sample, in turns, whose
+// coefficients are the segment's.  A lane a segment forms those for 32 segments at a time in shared
+// memory, and a thread a tile only evaluates them: FP64 arithmetic bounds the fill (16 cycles a warp
+// instruction and SM), and every tile forming its own coefficients took four times as many.
+struct PhaseFill {  // the phase c, its derivative per sample d, half the second one q, a sixth of the third
+    double c[4], d[3], q[2];
+    long long c3;
+};
+struct PhaseFill64 {  // the same in pairs; v^3 reaches 2^21, so c3 also has its next 32 bits (2^-96 turn)
+    Dd c[4], d[3], q[2];
+    long long c3;
+    int lo3;
+};
+template <bool FP64>
+struct SegFill {
+    std::conditional_t<FP64, PhaseFill64, PhaseFill> p[2];
+    double tk, t0, dt;
+    Dd ih;
+    const void *seg, *tab;
+    void *out;
+    float u0, du;
+    int first, end;  // tiles
+    int s0, s1;
+    int pairs, ks, n_mid, c64;
+};
+constexpr int kTcFillSegs = 32;
+
+// x modulo 2 pi (2 pi in two parts; see reduce_2pi).
+__device__ __forceinline__ double tc_reduce(double x)
+{
+    const double k = rint(x * 0.15915494309189533577);
+    return fma(-k, 2.4492935982947064e-16, fma(-k, 6.283185307179586232, x));
+}
+
+// Every product that is added to something is an explicit fma or an explicit product, so that the two
+// places this is inlined in round alike.
+__device__ inline void tc_phase_fill(const double *y, double h, Dd ih, double dt, double offset,
+                                     PhaseFill &o)
+{
+    const double kInv2Pi = 0.15915494309189533577;
+    const double D = y[1] - y[0], a = __dmul_rn(h, y[2]), b = __dmul_rn(h, y[3]);  // (hermite_to_power)
+    const double c2 = fma(-2.0, a, fma(3.0, D, -b)), c3 = fma(-2.0, D, a + b);
+    const double w = dt * ih.h, w2 = w * w, t = 3.0 * c3 * kInv2Pi;
+    o.c[0] = (tc_reduce(y[0]) + tc_reduce(offset)) * kInv2Pi;
+    o.c[1] = a * kInv2Pi;
+    o.c[2] = c2 * kInv2Pi;
+    o.c[3] = c3 * kInv2Pi;
+    o.d[0] = o.c[1] * w;
+    o.d[1] = __dmul_rn(o.c[2], 2.0 * w);
+    o.d[2] = t * w;
+    o.q[0] = o.c[2] * w2;
+    o.q[1] = t * w2;
+    o.c3 = turns_fixed(o.c[3] * w * w2);
+}
+
+__device__ inline void tc_phase_fill(const double *y, double h, Dd ih, double dt, double offset,
+                                     PhaseFill64 &o)
+{
+    const Dd inv2pi{0.15915494309189535, -9.8393400450386e-18};  // 1/(2 pi)
+    const Dd a = dd_prod(h, y[2]), b = dd_prod(h, y[3]), D = dd_sum(y[1], -y[0]);
+    const Dd p1 = dd_add(dd_scale(D, 3.0), dd_add(dd_scale(a, -2.0), Dd{-b.h, -b.l}));
+    const Dd p2 = dd_add(dd_add(a, b), dd_scale(D, -2.0));
+    const Dd w = dd_scale(ih, dt);
+    o.c[0] = dd_mul(dd_sum(y[0], offset), inv2pi);
+    o.c[1] = dd_mul(a, inv2pi);
+    o.c[2] = dd_mul(p1, inv2pi);
+    o.c[3] = dd_mul(p2, inv2pi);
+    o.d[0] = dd_mul(o.c[1], w);
+    o.q[0] = dd_mul(o.c[2], w);
+    const Dd c3 = dd_mul(o.c[3], w);
+    o.d[1] = Dd{2.0 * o.q[0].h, 2.0 * o.q[0].l};
+    o.d[2] = dd_scale(c3, 3.0);
+    o.q[0] = dd_mul(o.q[0], w);
+    o.q[1] = dd_mul(o.d[2], w);
+    const Dd f = dd_mul(dd_mul(c3, w), w);
+    const double x3 = (f.h - rint(f.h)) * 18446744073709551616.0;
+    o.c3 = __double2ll_rn(x3);
+    o.lo3 = __double2int_rn(((x3 - (double)o.c3) + f.l * 18446744073709551616.0) * 4294967296.0);
+}
+
+__device__ __forceinline__ double tc_u(const SegFill<false> &S, int i)
+{
+    return (fma((double)i, S.dt, S.t0) - S.tk) * S.ih.h;
+}
+__device__ __forceinline__ Dd tc_u(const SegFill<true> &S, int i)
+{
+    return dd_mul(dd_add(dd_prod((double)i, S.dt), dd_sum(S.t0, -S.tk)), S.ih);
+}
+// The expansion about u; returns whether the phase is finite.
+__device__ __forceinline__ bool tc_phase_at(const PhaseFill &p, double u, long long (&o)[4])
+{
+    const double f = fma(fma(fma(p.c[3], u, p.c[2]), u, p.c[1]), u, p.c[0]);
+    o[0] = turns_fixed(f);
+    o[1] = turns_fixed(fma(fma(p.d[2], u, p.d[1]), u, p.d[0]));
+    o[2] = turns_fixed(fma(p.q[1], u, p.q[0]));
+    o[3] = p.c3;
+    return (__double2hiint(f) & 0x7ff00000) != 0x7ff00000;
+}
+__device__ __forceinline__ bool tc_phase_at(const PhaseFill64 &p, const Dd &u, long long (&o)[4])
+{
+    o[0] = dd_turns_fixed(
+        dd_add(dd_mul(dd_add(dd_mul(dd_add(dd_mul(p.c[3], u), p.c[2]), u), p.c[1]), u), p.c[0]));
+    o[1] = dd_turns_fixed(dd_add(dd_mul(dd_add(dd_mul(p.d[2], u), p.d[1]), u), p.d[0]));
+    o[2] = dd_turns_fixed(dd_add(dd_mul(p.q[1], u), p.q[0]));
+    o[3] = p.c3;
+    return true;
+}
+
+template <bool FP64>
+__device__ inline void tc_seg_fill(const PlanHdr &h, const WaveDev &W, int s, SegFill<FP64> &o)
+{
+    const TrajDev &tr = W.tr;
+    const int *tile_off = tc_local(h, W.tile_off), *seg_start = tc_local(h, W.seg_start);
+    o.first = W.tile_begin + tile_off[s];
+    o.end = W.tile_begin + tile_off[s + 1];
+    o.s0 = seg_start[s];
+    o.s1 = seg_start[s + 1];
+    o.tk = tr.t[s];
+    o.t0 = W.t0;
+    o.dt = W.dt;
+    const double ih = tr.inv_h[s], hk = tr.h[s];
+    o.ih = FP64 ? dd_div(Dd{1.0, 0.0}, hk) : Dd{ih, 0.0};
+    const double *c = tr.coef + (size_t)s * tr.J * 4;
+    tc_phase_fill(c, hk, o.ih, W.dt, W.dphi_phi, o.p[0]);
+    tc_phase_fill(c + 4, hk, o.ih, W.dt, W.dphi_r, o.p[1]);
+    o.u0 = (float)((fma((double)o.s0, W.dt, W.t0) - o.tk) * ih);
+    o.du = (float)(W.dt * ih);
+    o.seg = FP64 ? (const void *)(W.seg64 + s) : (const void *)(W.tab_inv + s);
+    o.tab = W.tab + (size_t)s * (FP64 ? tc64_table_bytes(tr.tc_pairs, tr.tc_ks)
+                                      : tc_table_bytes(tr.tc_pairs, tr.tc_ks));
+    o.out = W.out;
+    o.pairs = tr.tc_pairs;
+    o.ks = tr.tc_ks;
+    o.n_mid = tr.n_mid;
+    o.c64 = W.out_c64;
+}
+
+// Segment g of the plan for a block's cache; past the last one: no tiles.
+template <bool FP64>
+__device__ inline void tc_cache_seg(const PlanHdr &h, int g, SegFill<FP64> &o)
+{
+    if (g >= h.total_segs) {
+        o.first = o.end = h.total_tiles;
+        return;
+    }
+    const WaveDev &W = tc_wave(h, tc_wave_of_seg(h, g));
+    tc_seg_fill<FP64>(h, W, g - W.seg_begin, o);
+}
+
+// The segment s of wave W that holds tile T.
+__device__ inline const WaveDev &tc_find_tile(const PlanHdr &h, int T, int &s)
 {
     int lo = 0, hi = h.n_waves - 1;
     while (lo < hi) {  // largest w with tile_begin <= T
@@ -116,56 +251,81 @@ __device__ inline void tc_fill_record(const PlanHdr &h, int T, bool fp64)
         if (tc_wave(h, mid).tile_begin <= T) lo = mid; else hi = mid - 1;
     }
     const WaveDev &W = tc_wave(h, lo);
-    const TrajDev &tr = W.tr;
-    const int *tile_off = tc_local(h, W.tile_off), *seg_start = tc_local(h, W.seg_start);
-    const int t = T - W.tile_begin;
-    int s = 0, e = tr.S - 1;
-    while (s < e) {  // largest s with tile_off[s] <= t: the segment that holds tile t
+    const int *tile_off = tc_local(h, W.tile_off);
+    int e = W.tr.S - 1;
+    s = 0;
+    while (s < e) {  // largest s with tile_off[s] <= t: the segment that holds tile T
         const int mid = (s + e + 1) >> 1;
-        if (tile_off[mid] <= t) s = mid; else e = mid - 1;
+        if (tile_off[mid] <= T - W.tile_begin) s = mid; else e = mid - 1;
     }
+    return W;
+}
+
+template <bool FP64>
+__device__ __forceinline__ void tc_store_record(const PlanHdr &h, const SegFill<FP64> &S, int t)
+{
     TileRec r;
-    r.s0 = seg_start[s];
-    r.s1 = seg_start[s + 1];
-    r.i0 = (r.s0 / kTcTile + (t - tile_off[s])) * kTcTile;
-    r.tile_end = W.tile_begin + tile_off[s + 1];
-    const SegPhase sp = seg_phase(tr, s, W.dphi_phi, W.dphi_r);
-    const double kInv2Pi = 0.15915494309189533577;
-    const double u = (fma((double)max(r.i0, r.s0), W.dt, W.t0) - sp.tk) * sp.ih, du = W.dt * sp.ih;
-    double all = 0.0;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const double *p = k ? sp.pr : sp.pphi;
-        long long *c = k ? r.r : r.phi;
-        const double f0 = fma(fma(fma(p[2], u, p[1]), u, p[0]), u, k ? sp.c0r : sp.c0phi) * kInv2Pi;
-        c[0] = turns_fixed(f0);
-        c[1] = turns_fixed(fma(fma(3.0 * p[2], u, 2.0 * p[1]), u, p[0]) * du * kInv2Pi);
-        c[2] = turns_fixed(fma(3.0 * p[2], u, p[1]) * du * du * kInv2Pi);
-        c[3] = turns_fixed(p[2] * du * du * du * kInv2Pi);
-        all += f0;
+    r.i0 = (S.s0 / kTcTile + (t - S.first)) * kTcTile;
+    r.s0 = S.s0;
+    r.s1 = S.s1;
+    r.tile_end = S.end;
+    const auto u = tc_u(S, max(r.i0, r.s0));
+    bool fin = tc_phase_at(S.p[0], u, r.phi);
+    fin = tc_phase_at(S.p[1], u, r.r) && fin;
+    if constexpr (FP64) {  // non-finite data reach the output through the segment's factor
+        r.u0 = __int_as_float(S.p[0].lo3);
+        r.du = __int_as_float(S.p[1].lo3);
+    } else {  // integers cannot carry a NaN: non-finite phases (latched by the build) go here
+        r.u0 = fin ? S.u0 : __int_as_float(0x7fffffff);
+        r.du = S.du;
     }
-    // integers cannot carry a NaN: non-finite phases (latched by the build) reach the output here
-    // (FP64: in the segment's factor)
-    r.u0 = (float)((fma((double)r.s0, W.dt, W.t0) - sp.tk) * sp.ih) + (float)(all - all);
-    r.du = (float)du;
-    if (fp64) {
-        const double *c = tr.coef + (size_t)s * tr.J * 4;
-        const Dd x = dd_add(dd_prod((double)max(r.i0, r.s0), W.dt), dd_sum(W.t0, -sp.tk));
-        int lo_phi, lo_r;
-        dd_phase_taylor(c, tr.h[s], x, W.dt, W.dphi_phi, r.phi, lo_phi);
-        dd_phase_taylor(c + 4, tr.h[s], x, W.dt, W.dphi_r, r.r, lo_r);
-        r.u0 = __int_as_float(lo_phi);
-        r.du = __int_as_float(lo_r);
+    r.seg = S.seg;
+    r.tab = static_cast<const unsigned char *>(S.tab);
+    r.out = S.out;
+    r.pairs = S.pairs;
+    r.ks = S.ks;
+    r.n_mid = S.n_mid;
+    r.c64 = S.c64;
+    h.recs[t] = r;
+}
+
+// The records of a block after the segments' (an even share of the tiles; seg: kTcFillSegs entries in
+// shared memory).  Shares of one tile a thread form their segments' coefficients themselves (mixed): one
+// chain of latencies instead of two, 1.5 us of a one-week waveform's 25; with more tiles the cache wins:
+// records and fold of a four-year one 190 -> 74 us.
+template <bool FP64>
+__device__ inline void tc_fill_records(const PlanHdr &h, SegFill<FP64> *seg)
+{
+    const int blocks = (int)gridDim.x - h.total_segs, share = (h.total_tiles + blocks - 1) / blocks;
+    int T = ((int)blockIdx.x - h.total_segs) * share;
+    const int T1 = min(h.total_tiles, T + share);
+    if (!FP64 && share <= kTcRecTiles) {
+        T += threadIdx.x;
+        if (T >= T1) return;
+        int s;
+        const WaveDev &W = tc_find_tile(h, T, s);
+        SegFill<FP64> S;
+        tc_seg_fill<FP64>(h, W, s, S);
+        tc_store_record<FP64>(h, S, T);
+        return;
     }
-    r.seg = fp64 ? (const void *)(W.seg64 + s) : (const void *)(W.tab_inv + s);
-    r.tab = W.tab + (size_t)s * (fp64 ? tc64_table_bytes(tr.tc_pairs, tr.tc_ks)
-                                      : tc_table_bytes(tr.tc_pairs, tr.tc_ks));
-    r.out = W.out;
-    r.pairs = tr.tc_pairs;
-    r.ks = tr.tc_ks;
-    r.n_mid = tr.n_mid;
-    r.c64 = W.out_c64;
-    h.recs[T] = r;
+    while (T < T1) {  // uniform
+        int s;
+        const WaveDev &W = tc_find_tile(h, T, s);
+        if (threadIdx.x < kTcFillSegs) tc_cache_seg<FP64>(h, W.seg_begin + s + threadIdx.x, seg[threadIdx.x]);
+        __syncthreads();
+        const int Te = min(T1, seg[kTcFillSegs - 1].end);
+        for (int t = T + threadIdx.x; t < Te; t += blockDim.x) {
+            int k = 0, ke = kTcFillSegs - 1;
+            while (k < ke) {  // largest k with first <= t
+                const int mid = (k + ke + 1) >> 1;
+                if (seg[mid].first <= t) k = mid; else ke = mid - 1;
+            }
+            tc_store_record<FP64>(h, seg[k], t);
+        }
+        __syncthreads();
+        T = Te;
+    }
 }
 
 // c0 + c1 v + c2 v^2 + c3 v^3 in 64-bit wrap-around arithmetic (modulo one turn).

@@ -96,6 +96,25 @@ def test_sample_and_segment_edges(gpu_ctx, prec, K, n_samples, i0, count):
     tr.release()
 
 
+def test_long_request_equals_its_windows(gpu_ctx):
+    """More tiles than one a thread of the blocks that fill their records: the same samples as short
+    requests (whose records are formed one by one), to the bit where the first sample's time is the
+    same number (t0 + i_begin dt is rounded)."""
+    import torch
+    n = 128 * (152 * 4 * 128 + 1000) + 5
+    w = W.make_inputs(3.0e7, 300, 3.0e7 / n, SETS["n_range_15"], 5, 4.0, 60.0, n_samples=n)
+    tr = RT.from_inputs(gpu_ctx, w)
+    h = RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_MIXED)
+    torch.cuda.synchronize()
+    for i0 in (0, n // 3, n // 2 + 77, n - 5000):
+        g = to_host(RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_MIXED, i_begin=i0, count=5000))
+        if i0 == 0:
+            np.testing.assert_array_equal(to_host(h[:5000]), g)
+        assert rel_l2(to_host(h[i0:i0 + 5000]), g) <= 4e-6
+        assert rel_l2(g, oracle.waveform_inputs(w, i0, 5000, nthreads=oracle_threads())) <= 4e-6
+    tr.release()
+
+
 @pytest.mark.parametrize("prec,scale", [(F.FEW_MIXED, 1e-30), (F.FEW_MIXED, 1e-22), (F.FEW_MIXED, 1e25),
                                         (F.FEW_FP64, 1e-290), (F.FEW_FP64, 1e-22), (F.FEW_FP64, 1e290)])
 def test_amplitude_range(gpu_ctx, prec, scale):
