@@ -11,24 +11,30 @@
 // left-to-right FP64 sums over the sorted powers, c_j = fl(c_{j-1} + p_j), with the total equal
 // to the last of them.  Any other summation order can round differently and move the cut.
 //
-// One CTA per knot, P = max(128, next power of two >= N) sort slots, P/4 threads holding four
-// consecutive slots each in registers.  Each warp sorts its 128 slots of (power, index) pairs by
-// a bitonic network (exchanges at distances 1 and 2 inside a thread, 4..64 by warp shuffles),
-// then the sorted runs are merged pairwise in shared memory by merge path (a binary search per
-// thread for where its four outputs split between the two runs), log2(P / 128) levels.  The
-// sorted powers then go to shared memory.  The cumulative sums are exact integer prefix sums
-// inside each binade of the running sum (see the comment at the scan), so the whole block
-// computes them in a few rounds of a block-wide scan instead of one thread running N dependent
-// FP64 additions.  The first rank whose sum reaches the target is found by all threads with an
-// atomic minimum, and the kept modes are marked with plain byte stores of 1 into a mask zeroed
-// beforehand (every writer stores the same value, so the union needs no atomics).
+// One CTA per knot, P = max(128, next power of two >= N) slots, P/4 threads.  The sums need the modes in
+// order only down to p_0 2^-54 or so (what is smaller changes no sum and is never kept), and in a range
+// of 54 binades a mode's place is nearly known from its leading bits: P/16 buckets a binade, a
+// histogram, a prefix sum and the few modes of a bucket compared with one another sort them in five
+// barriers.  The cumulative sums are exact integer prefix sums inside each binade of the running sum
+// (see select_q).  The first 128 ranks, where the sum leaves a binade every few steps, are summed by
+// one warp alone, the rest block-wide.  The kept modes are marked with plain byte stores of 1 into a
+// mask zeroed beforehand (every writer stores the same value, so the union needs no atomics).
+// What that cannot take (non-finite powers, sums that overflow, subnormal sums, more than 64 modes in
+// a bucket, a sum of very many rounding ties) goes to select_general: bitonic sorts by warp, merge
+// path, and a sequential chain as the last resort.
+// Bound by the latency of one knot, and in it by instruction issue: 100 knots are 100 CTAs of 32 warps,
+// one a multiprocessor.  100 knots of 3843 modes: 59 us a call with select_general for all (13 us warp
+// sorts, 14 merges, 17 in eight block-wide rounds of sums, 5.5 the powers), 27 us with the buckets
+// (powers 4, buckets 6, sums 5 to 9).
 #include "fewsum_internal.h"
+#include "launch.cuh"
 
 namespace fewsum {
 
 constexpr int kSelectMaxThreads = 1024;
 constexpr int kSelectPerThread = 4;  // consecutive sort slots per thread
 constexpr int kSelectWarpSlots = 32 * kSelectPerThread;
+constexpr int kSelectChain = 32;     // ranks summed one by one before the scans
 constexpr int kSelectMaxRounds = 64;  // scan rounds before the sequential chain takes over
 
 // Non-negative doubles order exactly like their IEEE bit patterns read as unsigned integers, so
@@ -70,18 +76,23 @@ __device__ __forceinline__ void cx_keep(unsigned long long &k, int &i, unsigned 
     if (sorts_before(ko, io, k, i) == keep_first) { k = ko; i = io; }
 }
 
-__global__ void __launch_bounds__(kSelectMaxThreads)
-k_mode_select(const double *__restrict__ amp_re, const double *__restrict__ amp_im, int N,
-              const __grid_constant__ ModeDoubling dbl, double eps, int P,
-              unsigned char *__restrict__ mask)
+// Power of mode i and its bits (doubled for m > 0).
+__device__ __forceinline__ double mode_power(double re, double im, bool twice)
 {
-    extern __shared__ __align__(16) unsigned long long sel_key[];  // [P] keys, then [P] indices
+    const double p = __dadd_rn(__dmul_rn(re, re), __dmul_rn(im, im));
+    return twice ? p * 2.0 : p;
+}
+
+__device__ __noinline__ void select_general(const double *__restrict__ amp_re, const double *__restrict__ amp_im,
+                                            int N, const ModeDoubling &dbl, double eps, int P,
+                                            unsigned char *__restrict__ mask, unsigned long long *sel_key)
+{
     int *sel_ix = reinterpret_cast<int *>(sel_key + P);
     __shared__ double s_total;
     __shared__ unsigned long long s_cbits;  // bits of the running sum where a round starts
     __shared__ unsigned long long s_wsum[kSelectMaxThreads / 32];
     __shared__ int s_a, s_exit, s_fallback, s_cut;
-    const int k = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+    const int k = blockIdx.x, tid = threadIdx.x;
     const int lane = tid & 31, wid = tid >> 5;
     const int p0 = kSelectPerThread * tid;  // first slot of this thread
 
@@ -91,10 +102,8 @@ k_mode_select(const double *__restrict__ amp_re, const double *__restrict__ amp_
     for (int r = 0; r < kSelectPerThread; ++r) {
         const int i = p0 + r;
         if (i < N) {
-            const double re = amp_re[(size_t)k * N + i], im = amp_im[(size_t)k * N + i];
-            double p = __dadd_rn(__dmul_rn(re, re), __dmul_rn(im, im));
-            if ((dbl.w[i >> 5] >> (i & 31)) & 1u) p *= 2.0;  // m > 0
-            key[r] = power_key(p);
+            key[r] = power_key(mode_power(amp_re[(size_t)k * N + i], amp_im[(size_t)k * N + i],
+                                          (dbl.w[i >> 5] >> (i & 31)) & 1u));  // m > 0
             ix[r] = i;
         } else {
             key[r] = ~0ull;  // padding: power +0, sorts after every real mode
@@ -309,21 +318,326 @@ k_mode_select(const double *__restrict__ amp_re, const double *__restrict__ amp_
         if (p0 + r < N && p0 + r <= cut) mask[ix[r]] = 1;
 }
 
+// What a step adds to the running sum c, in units of c's last place U: fl(c + p) = c + U q while c stays
+// in its binade (exponent E), q the integer nearest p/U, unless p/U lies exactly halfway between two
+// (tie: the parity of the sum decides).  pm, pe: significand and exponent of p, pe <= E.
+__device__ __forceinline__ unsigned long long select_q(unsigned long long pm, int d, bool &tie)
+{
+    if (d > 53) return 0ull;  // p < U/2
+    const unsigned long long one = 1ull << d, half = one >> 1;
+    tie = d > 0 && (pm & (one - 1ull)) == half;
+    return (pm + half) >> d;
+}
+
+__global__ void __launch_bounds__(kSelectMaxThreads)
+k_mode_select(const double *__restrict__ amp_re, const double *__restrict__ amp_im, int N,
+              const __grid_constant__ ModeDoubling dbl, double eps, int P, int sub,
+              unsigned char *__restrict__ mask)
+{
+    using u64 = unsigned long long;
+    constexpr int R = kSelectPerThread;
+    constexpr u64 kTop = 1ull << 53, kFrac = (1ull << 52) - 1ull;
+    extern __shared__ __align__(16) u64 sel[];
+    u64 *s_key = sel;                                   // [P] bits of the powers in their order
+    u64 *s_raw = sel + P;                               // [P] the same by bucket, in any order
+    unsigned short *s_ix = reinterpret_cast<unsigned short *>(sel + 2 * P);  // [P] modes of s_key
+    unsigned short *s_rix = s_ix + P;                                        // [P] modes of s_raw
+    uint4 *s_cnt = reinterpret_cast<uint4 *>(s_key);    // [P/4] 4 P buckets' sizes, a byte each
+    int *s_off = reinterpret_cast<int *>(s_key) + P;    // [P/4] first place of each 16 buckets
+    __shared__ unsigned s_wmax[kSelectMaxThreads / 32], s_wcnt[kSelectMaxThreads / 32];
+    __shared__ u64 s_wsum[kSelectMaxThreads / 32], s_c, s_total;
+    __shared__ int s_a, s_exit, s_cut;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+    const int p0 = R * tid;
+
+    // the powers (mode r nt + tid) and the largest one's exponent
+    u64 pb[R];
+    unsigned top = 0u;
+    {
+        const double *re = amp_re + (size_t)blockIdx.x * N, *im = amp_im + (size_t)blockIdx.x * N;
+        double x[R], y[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = r * nt + tid;
+            x[r] = i < N ? re[i] : 0.0;
+            y[r] = i < N ? im[i] : 0.0;
+        }
+        s_cnt[tid] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = r * nt + tid;
+            // doubled for m > 0 in the exponent (what is not a normal number then goes to select_general)
+            const bool twice = i < N && ((dbl.w[i >> 5] >> (i & 31)) & 1u);
+            pb[r] = (u64)__double_as_longlong(mode_power(x[r], y[r], false));
+            top = max(top, (unsigned)(pb[r] >> 32));
+            if (twice) pb[r] += 1ull << 52;
+            top = max(top, (unsigned)(pb[r] >> 32));
+        }
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (lane == 0) s_wmax[wid] = top;
+    if (tid == 0) s_cut = 0x7fffffff;
+    __syncthreads();
+    top = __reduce_max_sync(0xffffffffu, lane < nw ? s_wmax[lane] : 0u);
+    const int e0 = (int)(top >> 20);
+    bool general = e0 < 60 || e0 > 2030;  // (uniform)
+
+    // the buckets, in descending order: `sub` leading bits of the significand and the exponent; powers
+    // below 2^(e0 - 53) are less than half a unit in the last place of any sum
+    if (!general) {
+        const int vtop = (int)(((unsigned)e0 << sub) | ((1u << sub) - 1u));
+        int bucket[R], place[R];
+        bool crowded = false;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int e = (int)(pb[r] >> 52);
+            bucket[r] = e0 - e <= 53 ? vtop - (int)(pb[r] >> (52 - sub)) : -1;
+            if (bucket[r] < 0) continue;
+            const int sh = 8 * (bucket[r] & 3);
+            place[r] = (int)(atomicAdd(reinterpret_cast<unsigned *>(s_cnt) + (bucket[r] >> 2), 1u << sh) >> sh & 255u);
+            crowded |= place[r] >= 64;  // (seen before a byte can overflow)
+        }
+        __syncthreads();
+        const uint4 c = s_cnt[tid];
+        const unsigned own = __dp4a(c.x, 0x01010101u, __dp4a(c.y, 0x01010101u, __dp4a(c.z, 0x01010101u,
+                             __dp4a(c.w, 0x01010101u, 0u))));
+        unsigned incl = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += v;
+        }
+        if (lane == 31) s_wcnt[wid] = incl;
+        general = __syncthreads_or(crowded);
+        if (!general) {
+            const unsigned cnt = lane < nw ? s_wcnt[lane] : 0u;
+            const int n = (int)__reduce_add_sync(0xffffffffu, cnt);  // modes that count
+            const int first = (int)(__reduce_add_sync(0xffffffffu, lane < wid ? cnt : 0u) + incl - own);
+            s_off[tid] = first;
+            __syncthreads();
+            int size[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (bucket[r] < 0) continue;
+                // the bucket's first place: its group's and the sizes of the buckets before it
+                const uint4 g = s_cnt[bucket[r] >> 4];
+                const int w = (bucket[r] >> 2) & 3, sh = 8 * (bucket[r] & 3);
+                const unsigned mine = w == 0 ? g.x : w == 1 ? g.y : w == 2 ? g.z : g.w;
+                unsigned at = __dp4a(mine & ((1u << sh) - 1u), 0x01010101u, (unsigned)s_off[bucket[r] >> 4]);
+                at = __dp4a(w > 0 ? g.x : 0u, 0x01010101u, at);
+                at = __dp4a(w > 1 ? g.y : 0u, 0x01010101u, at);
+                at = __dp4a(w > 2 ? g.z : 0u, 0x01010101u, at);
+                size[r] = (int)(mine >> sh & 255u);
+                place[r] += (int)at;
+                size[r] |= (int)at << 8;
+                s_raw[place[r]] = pb[r];
+                s_rix[place[r]] = (unsigned short)(r * nt + tid);
+            }
+            __syncthreads();
+            // a mode's place: the modes of its bucket that come before it (larger, or as large and of
+            // lower index)
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (bucket[r] < 0) continue;
+                const int b0 = size[r] >> 8, b1 = b0 + (size[r] & 255), self = place[r];
+                if (b1 - b0 == 1) continue;
+                place[r] = b0;
+                for (int q = b0; q < b1; ++q) {
+                    const u64 o = s_raw[q];
+                    if (o > pb[r])
+                        ++place[r];
+                    else if (o == pb[r] && q != self && (int)s_rix[q] < r * nt + tid)
+                        ++place[r];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                if (bucket[r] < 0) continue;
+                s_key[place[r]] = pb[r];
+                s_ix[place[r]] = (unsigned short)(r * nt + tid);
+            }
+            __syncthreads();
+
+            // the cumulative sums c_j = fl(c_{j-1} + p_j) of the ranks p0 .. p0 + 3
+            u64 pm[R], cj[R];
+            int pe[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const u64 b = p0 + r < n ? s_key[p0 + r] : 0ull;
+                pb[r] = b;
+                pm[r] = (b & kFrac) | (kFrac + 1ull);
+                pe[r] = (int)(b >> 52);
+                cj[r] = b;  // (rank 0)
+            }
+            // One round over the ranks a .. lim - 1 from the sum with bits c: integer prefix sums up to
+            // the first step that leaves the binade (the integer reaches 2^53) or ties.
+            u64 q[R], m[R], run;
+            bool tie[R];
+            auto add_up = [&](int a, int lim, int E) {  // -> the warp's inclusive prefix of the threads' sums
+                run = 0ull;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int j = p0 + r;
+                    tie[r] = false;
+                    q[r] = j >= a && j < lim ? select_q(pm[r], E - pe[r], tie[r]) : 0ull;
+                    run += q[r];
+                }
+                u64 incl = run;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const u64 v = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += v;
+                }
+                return incl;
+            };
+            auto first_exit = [&](int a, int lim, u64 base) {
+                int jx = 0x7fffffff;
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    base += q[r];
+                    m[r] = base;
+                    const int j = p0 + r;
+                    if (j >= a && j < lim && (base >= kTop || tie[r])) jx = min(jx, j);
+                }
+                return (int)__reduce_min_sync(0xffffffffu, (unsigned)jx);
+            };
+            // the sums of the ranks before the exit; the FP64 adder takes the exit's step
+            auto settle = [&](int a, int lim, int jx, int E, u64 c) {
+                const u64 ebase = (u64)(E - 1) << 52;  // bits of a sum: exponent field E, M - 2^52
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int j = p0 + r;
+                    if (j >= a && j < lim && j < jx) cj[r] = ebase + m[r];
+                    if (j == jx) {
+                        const u64 prev = j == a ? c : ebase + (m[r] - q[r]);
+                        cj[r] = (u64)__double_as_longlong(
+                            __dadd_rn(__longlong_as_double((long long)prev), __longlong_as_double((long long)pb[r])));
+                    }
+                }
+            };
+            const int lim0 = min(n, 32 * R);
+            if (wid == 0) {  // the first 128 ranks
+                int a = 1;
+                u64 c = s_key[0];
+                double sum = __longlong_as_double((long long)c);
+#pragma unroll
+                for (int j = 1; j < kSelectChain; ++j) {  // the first few one by one
+                    if (j >= lim0) break;
+                    sum = __dadd_rn(sum, __longlong_as_double((long long)s_key[j]));
+                    if (lane == j / R) cj[j % R] = (u64)__double_as_longlong(sum);
+                    a = j + 1;
+                }
+                c = (u64)__double_as_longlong(sum);
+                for (int round = 0; a < lim0 && round < kSelectMaxRounds; ++round) {
+                    const int E = (int)(c >> 52);
+                    const u64 incl = add_up(a, lim0, E);
+                    const int jx = first_exit(a, lim0, ((c & kFrac) | (kFrac + 1ull)) + (incl - run));
+                    settle(a, lim0, jx, E, c);
+                    const int last = min(jx, lim0 - 1);
+                    u64 mine = cj[0];
+#pragma unroll
+                    for (int r = 1; r < R; ++r)
+                        if ((last & (R - 1)) == r) mine = cj[r];
+                    c = __shfl_sync(0xffffffffu, mine, last / R);
+                    a = last + 1;
+                }
+                if (lane == 0) {
+                    s_c = c;
+                    s_a = a;
+                }
+            }
+            for (int round = 0;; ++round) {
+                __syncthreads();
+                const int a = s_a;
+                if (a >= n) break;
+                if (a < lim0 || round >= kSelectMaxRounds) {  // very many ties
+                    general = true;
+                    break;
+                }
+                const u64 c = s_c;
+                const int E = (int)(c >> 52);
+                const bool any = R * (32 * wid + 32) > a;  // a rank of this warp is summed
+                u64 incl = 0ull;
+                run = 0ull;
+                if (any) incl = add_up(a, n, E);
+                if (lane == 31) s_wsum[wid] = incl;
+                if (tid == 0) s_exit = 0x7fffffff;
+                __syncthreads();
+                if (any) {
+                    u64 before = lane < wid ? s_wsum[lane] : 0ull;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+                    const int jx =
+                        first_exit(a, n, ((c & kFrac) | (kFrac + 1ull)) + before + (incl - run));
+                    if (lane == 0 && jx != 0x7fffffff) atomicMin(&s_exit, jx);
+                }
+                __syncthreads();
+                const int jx = s_exit;
+                if (any) {
+                    settle(a, n, jx, E, c);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        if (p0 + r != jx) continue;
+                        s_c = cj[r];
+                        s_a = jx + 1;
+                    }
+                }
+                if (jx == 0x7fffffff) break;
+            }
+            if (!general) {
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (p0 + r == n - 1) s_total = cj[r];
+                __syncthreads();
+                const double total = __longlong_as_double((long long)s_total);
+                const long long target = __double_as_longlong((1.0 - eps) * total);
+                // (non-negative doubles compare as integers, and any as not less than a negative one)
+                unsigned cut = 0x7fffffffu;
+#pragma unroll
+                for (int r = R - 1; r >= 0; --r)
+                    if (p0 + r < n && (long long)cj[r] >= target) cut = (unsigned)(p0 + r);
+                cut = __reduce_min_sync(0xffffffffu, cut);
+                if (lane == 0 && cut != 0x7fffffffu) atomicMin(&s_cut, (int)cut);
+                pdl_wait();  // the mask has been zeroed
+                __syncthreads();
+                const int last = s_cut;  // total >= target: some rank reaches it
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+                    if (p0 + r < n && p0 + r <= last) mask[s_ix[p0 + r]] = 1;
+                return;
+            }
+        }
+    }
+    pdl_wait();
+    __syncthreads();
+    select_general(amp_re, amp_im, N, dbl, eps, P, mask, sel);
+}
+
+// Zeroes the mask, while the selection's blocks sort.
+__global__ void k_mask_zero(unsigned char *__restrict__ mask, int N)
+{
+    pdl_launch_dependents();
+    for (int i = threadIdx.x; i < N; i += blockDim.x) mask[i] = 0;
+}
+
 cudaError_t launch_mode_select(const double *amp_re, const double *amp_im, int K, int N,
                                const ModeDoubling &dbl, double eps, unsigned char *mask,
                                cudaStream_t st)
 {
-    int P = kSelectWarpSlots;
-    while (P < N) P <<= 1;
+    int P = kSelectWarpSlots, sub = 3;  // 2^sub = P/16 buckets a binade: 54 binades fit in 4 P
+    while (P < N) P <<= 1, ++sub;
     const int threads = P / kSelectPerThread;
-    const int smem = P * (int)(sizeof(unsigned long long) + sizeof(int));
+    constexpr int kSlotBytes = 2 * sizeof(unsigned long long) + 2 * sizeof(unsigned short);
+    const int smem = P * kSlotBytes;
     cudaError_t e = cudaFuncSetAttribute(k_mode_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         smem);
+                                         kSelectMaxModes * kSlotBytes);
     if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(mask, 0, (size_t)N, st);
+    k_mask_zero<<<1, 1024, 0, st>>>(mask, N);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_mode_select<<<K, threads, smem, st>>>(amp_re, amp_im, N, dbl, eps, P, mask);
-    return cudaGetLastError();
+    return launch_pdl(k_mode_select, (unsigned)K, (unsigned)threads, (size_t)smem, st, amp_re, amp_im, N, dbl, eps,
+                      P, sub, mask);
 }
 
 int mode_select_max_modes() { return kSelectMaxModes; }

@@ -144,3 +144,22 @@ def test_mode_select_subnormal_and_infinite_powers(gpu_ctx):
         g = _gpu_select(gpu_ctx, re, im, modes, eps)
         o = oracle.mode_select(re, im, modes, eps)
         np.testing.assert_array_equal(g, o, err_msg=f"eps={eps}")
+
+
+@pytest.mark.parametrize("top,N", [(0, 1), (0, 129), (0, 3843), (-962, 700), (-964, 700), (1006, 700), (1008, 700)])
+def test_mode_select_bucket_edges(gpu_ctx, top, N):
+    """Powers 2^top and down to 2^(top - 55) with few and with many (64, 65 and 1000) modes of one size:
+    both sides of the range, of the bucket size and of the exponents that the bucket sort takes."""
+    rng = np.random.default_rng(N)
+    modes = np.stack([np.full(N, 2), rng.integers(0, 2, N), np.zeros(N, int)], axis=1)
+    p = 2.0 ** -rng.uniform(0.0, 55.0, (6, N))
+    for k, (at, count) in enumerate([(1, 0), (1, 64), (1, 65), (0, 1000), (53, 30), (54, 30)]):
+        p[k, rng.permutation(N)[:count]] = 2.0 ** -at
+    p[5, 1:] = np.minimum(p[5, 1:], 2.0 ** -49)  # hundreds of steps of a few units in the last place
+    p[:, 0] = 1.0
+    re = np.sqrt(p) * 2.0 ** (top // 2)  # (top even: exact scaling)
+    im = np.zeros_like(re)
+    for eps in (1e-3, 1e-15, 0.0):
+        g = _gpu_select(gpu_ctx, re, im, modes, eps)
+        o = oracle.mode_select(re, im, modes, eps)
+        np.testing.assert_array_equal(g, o, err_msg=f"eps={eps}")
