@@ -53,4 +53,15 @@ __device__ __forceinline__ double f32_to_f64(float x)
     return __hiloint2double(static_cast<int>(hi), static_cast<int>(lo));
 }
 
+// The same for a normal x in four instructions, and whether it is one.
+__device__ __forceinline__ double f32_normal_to_f64(float x)
+{
+    const int u = __float_as_int(x);
+    return __hiloint2double(((u >> 3) & (int)0x8fffffff) + 0x38000000, u << 29);
+}
+__device__ __forceinline__ bool f32_is_normal(float x)
+{
+    return 2u * __float_as_uint(x) - 0x01000000u < 0xfe000000u;
+}
+
 }  // namespace fewsum

@@ -296,6 +296,7 @@ size_t direct_mode_const_bytes(int N);
 // Reduced-basis amplitudes (rb.cu): tile counts of the packed tensor-core operands.
 struct RbLayout {
     int n_kb = 0, n_tiles = 0, m_tiles = 0, modes_padded = 0, rows_padded = 0;
+    int groups = 0, step = 0;  // groups of 32 modes, and modes between their first ones
     size_t bpack_bytes = 0, apack_bytes = 0;
 };
 RbLayout rb_layout(int Nb, int N, int M);

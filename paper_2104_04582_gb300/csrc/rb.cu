@@ -23,26 +23,32 @@
 // an absolute error near 2^-24 of that maximum.
 //
 // The product is computed transposed, A^T = Bhat^T a^T: the MMA's M side (tensor-memory lanes)
-// is 128 real output columns of 64 modes (rows 0-63 the real parts, 64-127 the imaginary parts)
+// is 128 real output columns of two groups of 32 modes (rows 0-63 the real parts, 64-127 the
+// imaginary parts)
 // and its N side (tensor-memory columns) 256 knots.  A lane of the accumulator then holds one
 // output column for consecutive knots, so for each knot a warp stores 32 consecutive modes (256
-// contiguous bytes) straight from registers.  Operands are packed once into the canonical K-major
+// contiguous bytes) straight from registers.  With N not a multiple of four the rows start at any of
+// four places in a 32-byte sector; groups then overlap by four modes, and a warp stores the 28 of
+// its 32 that fill whole sectors (written in parts by two warps, the sectors held the stores to
+// 4.8 TB/s, whole they reach 6.1: see k_rb_mma).  Operands are packed once into the canonical K-major
 // layout without swizzle that the tensor core's shared-memory descriptors read: 8 x 8 fp16 "core
 // matrices" of 16-byte rows, core matrices adjacent in K 128 bytes apart, 8-row groups 1024
 // bytes apart.  A k-block of 64 columns of a 128-row basis tile or a 256-row coefficient tile is
 // one contiguous 16 / 32 KB block in global memory, so each pipeline stage is filled by two bulk
 // asynchronous copies.
+#include <type_traits>
+
 #include <cuda_fp16.h>
 
 #include "async.cuh"
 #include "convert.cuh"
 #include "fewsum_internal.h"
+#include "launch.cuh"
 #include "tcgen05.cuh"
 
 namespace fewsum {
 
 constexpr int kRbTileM = 128;   // MMA M, tensor-memory lanes: real output columns of 64 modes
-constexpr int kRbModes = kRbTileM / 2;  // modes per basis tile
 constexpr int kRbTileN = 256;   // MMA N, tensor-memory columns: knots per coefficient tile
 constexpr int kRbTileK = 64;    // fp16 columns per k-block: 128 bytes per row
 constexpr int kRbStages = 4;    // shared-memory pipeline depth
@@ -133,11 +139,12 @@ __global__ void k_rb_bexp(const double *__restrict__ bre, const double *__restri
 }
 
 // Basis operand (the MMA's A side), scaled, split and packed: row r of basis tile b is the real
-// (r < 64) or imaginary (r >= 64) output column of mode 64 b + (r mod 64); column c = g 2Nb + q
+// (r < 64) or imaginary (r >= 64) output column of mode r mod 32 of group 2 b + (r mod 64) / 32, whose
+// first mode is `step` times its number; column c = g 2Nb + q
 // holds part part_b(g) of 2^bexp[mode] Bhat for that column.  Modes past N and columns past
 // 3 x 2Nb are zero.
 __global__ void k_rb_pack_b(const double *__restrict__ bre, const double *__restrict__ bim, int Nb,
-                            int N, int n_kb, int n_tiles, const int *__restrict__ bexp,
+                            int N, int n_kb, int n_tiles, int step, const int *__restrict__ bexp,
                             unsigned char *__restrict__ bpack)
 {
     const long long chunks = (long long)n_tiles * kRbTileM * n_kb * (kRbTileK / 8);
@@ -147,8 +154,8 @@ __global__ void k_rb_pack_b(const double *__restrict__ bre, const double *__rest
         const int q8 = (int)(t % (n_kb * (kRbTileK / 8)));
         const int row = (int)(t / (n_kb * (kRbTileK / 8)));
         const int c0 = q8 * 8;
-        const int rr = row % kRbTileM, i = (row / kRbTileM) * kRbModes + (rr % kRbModes);
-        const bool imag_out = rr >= kRbModes;
+        const int rr = row % kRbTileM, i = ((row / kRbTileM) * 2 + (rr / 32) % 2) * step + rr % 32;
+        const bool imag_out = rr >= kRbTileM / 2;
         uint32_t w[4];
         for (int e = 0; e < 8; e += 2) {
             __half v[2];
@@ -246,20 +253,23 @@ k_rb_quad(const double *__restrict__ are, const double *__restrict__ aim, int M,
 // Mixed path, Nb <= 128: the renormalisation scale in one kernel, one wave.  A block takes
 // kTRows knots; their FP32 coefficients and the whole FP32 Gram matrix (j padded to 128) sit in
 // shared memory.  The sum over l is split among kTParts thread groups (l = part mod kTParts);
-// within a group thread (rg, jg) owns knots 4 rg .. 4 rg + 3 and j = jg + 16 t, t < 8, so 12
-// shared-memory reads (half of them broadcasts) feed 128 multiply-adds per l.  The 16 threads of
+// within a group thread (rg, jg) owns knots 4 rg .. 4 rg + 3 and j = jg + 16 t, t < T = ceil(Nb / 16),
+// so 12 shared-memory reads (half of them broadcasts) feed 128 multiply-adds per l (T = 8).  The 16 threads of
 // a knot group share a half-warp and reduce their partial q_k by shuffles; the groups' partials
 // are added in group order and s_k = nu_k / sqrt(q_k) written directly (0 for q_k = 0; a
 // non-finite or negative nu_k latches ERRBIT_NONFINITE).
-constexpr int kTRows = 48, kTJ = 128, kTGroup = (kTRows / 4) * 16, kTParts = 3;
+constexpr int kTRows = 44, kTGroup = (kTRows / 4) * 16, kTParts = 3;
 constexpr int kTThreads = kTGroup * kTParts;
-constexpr int kTMaxBasis = kTJ;
+constexpr int kTMaxBasis = 128;
 
+template <int T>
 __global__ void __launch_bounds__(kTThreads)
 k_rb_scale_tile(const double *__restrict__ are, const double *__restrict__ aim, int M, int Nb,
                 const float2 *__restrict__ gt, const double *__restrict__ nu,
                 double *__restrict__ scale, unsigned *__restrict__ err)
 {
+    constexpr int kTJ = 16 * T;
+    pdl_launch_dependents();  // the pack
     extern __shared__ __align__(16) float2 rb_tile_smem[];
     float2 *as = rb_tile_smem;                 // [kTRows][Nb] alpha
     float2 *gs = rb_tile_smem + kTRows * Nb;   // [Nb][kTJ] G_jl stored [l][j], zero for j >= Nb
@@ -267,16 +277,30 @@ k_rb_scale_tile(const double *__restrict__ are, const double *__restrict__ aim, 
     const int tid = threadIdx.x, part = tid / kTGroup, local = tid - part * kTGroup;
     const int jg = local & 15, rg = local >> 4;
     const int k0 = blockIdx.x * kTRows;
-    // staging: 8 independent loads in flight per thread per round trip
-    constexpr int kU = 8;
+    // staging: the Gram matrix by asynchronous copies, all in flight, while the coefficients (9 loads of
+    // each array in flight a thread) pass through registers
+    for (int l = tid / 16; l < Nb; l += kTThreads / 16) {
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            const int j = (tid & 15) + 16 * t;
+            if (j < Nb)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(gs + l * kTJ + j)),
+                             "l"(gt + (size_t)l * Nb + j)
+                             : "memory");
+            else
+                gs[l * kTJ + j] = make_float2(0.f, 0.f);
+        }
+    }
+    constexpr int kU = 9;
+    const int live = min(kTRows, M - k0) * Nb;
+    const double *pr = are + (size_t)k0 * Nb, *pi = aim + (size_t)k0 * Nb;  // rows k0 .. are contiguous
     for (int e0 = tid; e0 < kTRows * Nb; e0 += kTThreads * kU) {
         double vr[kU], vi[kU];
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
-            const int e = e0 + u * kTThreads, k = k0 + e / (Nb > 0 ? Nb : 1);
-            const bool ok = e < kTRows * Nb && k < M;
-            vr[u] = ok ? are[(size_t)k0 * Nb + e] : 0.0;  // rows k0.. are contiguous: index k0*Nb + e
-            vi[u] = ok ? aim[(size_t)k0 * Nb + e] : 0.0;
+            const int e = e0 + u * kTThreads;
+            vr[u] = e < live ? pr[e] : 0.0;
+            vi[u] = e < live ? pi[e] : 0.0;
         }
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
@@ -284,35 +308,23 @@ k_rb_scale_tile(const double *__restrict__ are, const double *__restrict__ aim, 
             if (e < kTRows * Nb) as[e] = make_float2(f64_to_f32(vr[u]), f64_to_f32(vi[u]));
         }
     }
-    for (int e0 = tid; e0 < Nb * kTJ; e0 += kTThreads * kU) {
-        float2 v[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int e = e0 + u * kTThreads, l = e / kTJ, j = e % kTJ;
-            v[u] = (e < Nb * kTJ && j < Nb) ? gt[(size_t)l * Nb + j] : make_float2(0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int e = e0 + u * kTThreads;
-            if (e < Nb * kTJ) gs[e] = v[u];
-        }
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    float tr[4][8], ti[4][8];
+    float tr[4][T], ti[4][T];
 #pragma unroll
     for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int t = 0; t < 8; ++t) tr[r][t] = ti[r][t] = 0.f;
+        for (int t = 0; t < T; ++t) tr[r][t] = ti[r][t] = 0.f;
     for (int l = part; l < Nb; l += kTParts) {
-        float2 x[4], g[8];
+        float2 x[4], g[T];
 #pragma unroll
         for (int r = 0; r < 4; ++r) x[r] = as[(rg * 4 + r) * Nb + l];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) g[t] = gs[l * kTJ + jg + 16 * t];
+        for (int t = 0; t < T; ++t) g[t] = gs[l * kTJ + jg + 16 * t];
 #pragma unroll
         for (int r = 0; r < 4; ++r)
 #pragma unroll
-            for (int t = 0; t < 8; ++t) {
+            for (int t = 0; t < T; ++t) {
                 tr[r][t] += g[t].x * x[r].x + g[t].y * x[r].y;  // G_jl conj(alpha_l)
                 ti[r][t] += g[t].y * x[r].x - g[t].x * x[r].y;
             }
@@ -322,14 +334,15 @@ k_rb_scale_tile(const double *__restrict__ are, const double *__restrict__ aim, 
         const int row = rg * 4 + r;
         float q = 0.f;
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
+        for (int t = 0; t < T; ++t) {
             const int j = jg + 16 * t;
             if (j < Nb) {
                 const float2 a = as[row * Nb + j];
                 q += a.x * tr[r][t] - a.y * ti[r][t];  // Re(alpha_j t_j)
             }
         }
-        for (int o = 8; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        const unsigned half = 0xffffu << (tid & 16);  // (the block's last warp is a half one)
+        for (int o = 8; o > 0; o >>= 1) q += __shfl_xor_sync(half, q, o);
         if (jg == 0) q_part[part][row] = q;
     }
     __syncthreads();
@@ -368,6 +381,7 @@ __global__ void __launch_bounds__(kRbPackWarps * 32)
 k_rb_pack_a(const double *__restrict__ are, const double *__restrict__ aim, int M, int Nb, int n_kb,
             int m_tiles, unsigned char *__restrict__ apack, int *__restrict__ aexp)
 {
+    pdl_launch_dependents();  // the product
     __shared__ float xs[kRbPackWarps][2 * FEW_MAX_BASIS];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, Kr = 2 * Nb;
     float *x = xs[w];
@@ -406,13 +420,14 @@ k_rb_pack_a(const double *__restrict__ are, const double *__restrict__ aim, int 
         }
         __syncwarp();
     }
+    pdl_wait();  // the scale's kernel: the product waits for this one alone
 }
 
 // ---- tensor-core GEMM ---------------------------------------------------------------------
 
 // Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), fp16 A and B (bits 7-9
-// and 10-12 = 0), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22, M >> 4 at bits 24-28.
-constexpr uint32_t kRbIdesc = (1u << 4) | ((uint32_t)(kRbTileN >> 3) << 17) | ((uint32_t)(kRbTileM >> 4) << 24);
+// and 10-12 = 0), both K-major (bits 15, 16 = 0), M >> 4 at bits 24-28 (N >> 3 goes to bits 17-22).
+constexpr uint32_t kRbIdesc = (1u << 4) | ((uint32_t)(kRbTileM >> 4) << 24);
 
 struct RbMmaArgs {
     const unsigned char *apack;  // coefficients: [m_tiles][n_kb] blocks of kRbBBytes (B operand)
@@ -420,7 +435,7 @@ struct RbMmaArgs {
     double *out_re, *out_im;     // [M][N]
     const int *aexp, *bexp;      // scaling exponents of the coefficient rows and basis columns
     const double *scale;         // [M] renormalisation s_k, applied in the epilogue (or null)
-    int M, N, n_kb, m_tiles, n_tiles;
+    int M, N, n_kb, m_tiles, n_tiles, groups, step;
     int k16_last;                // K = 16 steps of the last k-block holding real columns
     unsigned *err;
 };
@@ -435,14 +450,22 @@ __device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity)
     return __all_sync(0xffffffffu, mbar_wait_bounded(bar, parity));
 }
 
-// Persistent: CTA b takes tiles b, b + grid, ... (tile t = knot tile t / n_tiles, basis tile
-// t % n_tiles).  Warp 0 (one lane) streams each tile's k-blocks through a kRbStages ring of
+// Persistent: CTA b takes items of an equal share (see `item`; tile t = knot tile t / n_tiles, basis tile
+// t % n_tiles: neighbours write neighbouring parts of the same rows at about the same time; with each
+// CTA on one basis tile the stores alone took 76 us instead of 65).  Warp 0 (one lane) streams each tile's k-blocks through a kRbStages ring of
 // shared-memory stages with bulk copies; warp 1 (one lane) issues the MMAs of a tile into one of
 // two tensor-memory accumulators of 256 columns and commits; warps 2.. drain the other
 // accumulator meanwhile: warp w reads lanes 32 (w % 4) .. + 31 (32 output columns: real parts
 // for w % 4 < 2, imaginary parts otherwise) and one in kRbEpiPerQuarter chunks of 32 knots, and
-// for each knot stores the 32 columns' FP64 values, 256 contiguous bytes, from registers.  Every wait is bounded; a timeout latches ERRBIT_TIMEOUT and the CTA waits
-// for its copies and MMAs in flight before it frees tensor memory.
+// for each knot stores its columns' FP64 values, 28 modes in seven whole sectors (or 32, see rb_layout),
+// from registers.  Bound by the stores and, nearly as much, by shared memory (an MMA reads 12 KB, and as
+// much is filled for it: 190 cycles for the tensor core's 128).  6400 knots of 3843 modes and 99 basis
+// vectors, the stores alone: 81 us with 256 bytes a warp across nine sectors, 65 as whole sectors;
+// the whole call 130 -> 121 us (28 of 32 columns used cost 13 % more tiles, so the conversion to FP64
+// takes four instructions instead of ~15, the factors come from shared memory instead of by shuffles,
+// and CTAs get equal shares: 12 tiles for each had been 11.4 on average).
+// Every wait is bounded; a timeout latches ERRBIT_TIMEOUT and the CTA waits for its copies and MMAs in
+// flight before it frees tensor memory.
 __global__ void __launch_bounds__(kRbMmaThreads, 1) k_rb_mma(RbMmaArgs a)
 {
     extern __shared__ unsigned char rb_mma_smem[];
@@ -450,8 +473,28 @@ __global__ void __launch_bounds__(kRbMmaThreads, 1) k_rb_mma(RbMmaArgs a)
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_abort;
     __shared__ uint32_t s_issued, s_consumed;
+    __shared__ __align__(16) float s_fa[kRbEpiWarps][32];  // a warp's 32 knots' factors
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int total = a.m_tiles * a.n_tiles;
+    // Item u of this CTA: rows k0 .. k0 + nn - 1 (nn a multiple of 16) of basis tile nt.  What is left
+    // over of the tiles after as many for every CTA is cut in up to eight parts that come first: the
+    // stores start after a small product, and no CTA has a whole tile more than another.
+    const int grid = gridDim.x, whole = a.m_tiles * a.n_tiles / grid, left = a.m_tiles * a.n_tiles - whole * grid;
+    int cut = 8;
+    while (cut > 1 && left * cut > grid) cut >>= 1;
+    const int parts = (left * cut + grid - 1) / grid;  // (0 or 1)
+    auto item = [&](int u, int &nt, int &k0, int &nn) {
+        int t = (u - parts) * grid + (int)blockIdx.x, n = kRbTileN, n0 = 0;
+        if (u < parts) {
+            const bool mine = (int)blockIdx.x < left * cut;
+            n = mine ? kRbTileN / cut : 0;
+            n0 = ((int)blockIdx.x % cut) * n;
+            t = mine ? whole * grid + (int)blockIdx.x / cut : 0;
+        }
+        nt = t % a.n_tiles;
+        k0 = (t / a.n_tiles) * kRbTileN + n0;
+        nn = min(n, (a.M - k0 + 15) & ~15);
+    };
+    const int items = parts + whole;
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(rb_mma_smem) + 127) & ~(uintptr_t)127);
     unsigned char *sA = base, *sB = base + kRbStages * kRbABytes;
@@ -481,20 +524,26 @@ __global__ void __launch_bounds__(kRbMmaThreads, 1) k_rb_mma(RbMmaArgs a)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
+    pdl_wait();
 
     if (warp == 0) {
         if (lane == 0) {  // producer
             const uint64_t keep = l2_evict_last_policy();  // operands are re-read by other CTAs
             uint32_t g = 0;
-            for (int t = blockIdx.x; t < total && !s_abort; t += gridDim.x) {
-                const unsigned char *ga = a.bpack + (size_t)(t % a.n_tiles) * a.n_kb * kRbABytes;  // basis
-                const unsigned char *gb = a.apack + (size_t)(t / a.n_tiles) * a.n_kb * kRbBBytes;  // coefficients
+            for (int w = 0; w < items && !s_abort; ++w) {
+                int nt, k0, nn;
+                item(w, nt, k0, nn);
+                if (nn <= 0) continue;
+                const unsigned char *ga = a.bpack + (size_t)nt * a.n_kb * kRbABytes;  // basis
+                const unsigned char *gb = a.apack + (size_t)(k0 / kRbTileN) * a.n_kb * kRbBBytes +
+                                          (size_t)(k0 % kRbTileN) * (kRbTileK * 2);  // coefficients
+                const uint32_t b_bytes = (uint32_t)nn * (kRbTileK * 2);
                 for (int kb = 0; kb < a.n_kb; ++kb, ++g) {
                     const int s = g % kRbStages;
                     if (!mbar_wait_bounded(&empty[s], ((g / kRbStages) & 1) ^ 1)) { s_abort = 1; break; }
-                    mbar_arrive_expect_tx(&full[s], kRbStageBytes);
+                    mbar_arrive_expect_tx(&full[s], kRbABytes + b_bytes);
                     bulk_g2s_hint(sA + s * kRbABytes, ga + (size_t)kb * kRbABytes, kRbABytes, &full[s], keep);
-                    bulk_g2s_hint(sB + s * kRbBBytes, gb + (size_t)kb * kRbBBytes, kRbBBytes, &full[s], keep);
+                    bulk_g2s_hint(sB + s * kRbBBytes, gb + (size_t)kb * kRbBBytes, b_bytes, &full[s], keep);
                 }
             }
             s_issued = g;
@@ -504,7 +553,11 @@ __global__ void __launch_bounds__(kRbMmaThreads, 1) k_rb_mma(RbMmaArgs a)
         if (lane == 0) {  // MMA issuer
             uint32_t g = 0;
             int u = 0;
-            for (int t = blockIdx.x; t < total && !s_abort; t += gridDim.x, ++u) {
+            for (int w = 0; w < items && !s_abort; ++w) {
+                int nt, k0, nn;
+                item(w, nt, k0, nn);
+                if (nn <= 0) continue;
+                const uint32_t idesc = kRbIdesc | ((uint32_t)(nn >> 3) << 17);
                 const int b = u & 1;
                 if (!mbar_wait_bounded(&tempty[b], ((u >> 1) & 1) ^ 1)) { s_abort = 1; break; }
                 tc_fence_after();
@@ -521,12 +574,13 @@ __global__ void __launch_bounds__(kRbMmaThreads, 1) k_rb_mma(RbMmaArgs a)
                     for (int k = 0; k < kRbTileK / 16; ++k)  // K = 16 per MMA: two core matrices
                         if (k < nk)
                             tc_mma(d, smem_desc(a0 + k * 256, 128, 1024),
-                                   smem_desc(b0 + k * 256, 128, 1024), kRbIdesc,
+                                   smem_desc(b0 + k * 256, 128, 1024), idesc,
                                    (uint32_t)((kb | k) != 0));
                     tc_commit(&empty[s]);
                 }
                 if (!ok) break;
                 tc_commit(&tfull[b]);
+                ++u;
             }
             s_consumed = g;
             tc_commit(&drain);  // arrives once every MMA issued above has completed
@@ -536,31 +590,73 @@ __global__ void __launch_bounds__(kRbMmaThreads, 1) k_rb_mma(RbMmaArgs a)
         const int e = warp - 2, qd = warp & 3;  // a warp reads tensor-memory lanes 32 (warp % 4) ..
         const int c_first = e / 4;              // and chunks c_first + kRbEpiPerQuarter i
         int u = 0;
-        for (int t = blockIdx.x; t < total && !__any_sync(0xffffffffu, s_abort != 0); t += gridDim.x, ++u) {
+        for (int w = 0; w < items && !__any_sync(0xffffffffu, s_abort != 0); ++w) {
+            int nt, k0, nn;
+            item(w, nt, k0, nn);
+            if (nn <= 0) continue;
             const int b = u & 1;
             if (!warp_wait(&tfull[b], (u >> 1) & 1)) { s_abort = 1; break; }
             tc_fence_after();
-            const int mode = (t % a.n_tiles) * kRbModes + (qd & 1) * 32 + lane;  // this lane's column
+            const int group = nt * 2 + (qd & 1), m0 = group * a.step, mode = m0 + lane;
             double *dst = qd < 2 ? a.out_re : a.out_im;
+            // the lanes whose modes fill whole 32-byte sectors of the row, and the row's two ends
+            const bool overlap = a.step < 32, first = group == 0, last = group >= a.groups - 1;
+            const bool live = group < a.groups && mode < a.N;
+            const int at0 = (int)(reinterpret_cast<uintptr_t>(dst) >> 3) + m0;
             const float fb = pow2f(-a.bexp[mode]);  // undo the column scaling (exact)
-            const int k0 = (t / a.n_tiles) * kRbTileN;
-            for (int c = c_first; c < kRbTileN / 32; c += kRbEpiPerQuarter) {
-                uint32_t v[32];
-                tc_ld32(tmem + (uint32_t)(b * kRbTileN) + ((uint32_t)(32 * qd) << 16) + (uint32_t)(32 * c), v);
+            for (int c = c_first; c < (nn + 31) / 32; c += kRbEpiPerQuarter) {
+                float v[32];
+                tc_ld32(tmem + (uint32_t)(b * kRbTileN) + ((uint32_t)(32 * qd) << 16) + (uint32_t)(32 * c),
+                        reinterpret_cast<uint32_t(&)[32]>(v));
                 const int kc = k0 + 32 * c;
-                // knot kc + lane's row scaling (exact) times its renormalisation s_k
+                // knot kc + lane's row scaling (exact) times its renormalisation s_k, for the other lanes
                 float fa_lane = pow2f(-a.aexp[kc + lane]);
                 if (a.scale && kc + lane < a.M) fa_lane *= (float)a.scale[kc + lane];
+                s_fa[e][lane] = fa_lane;
+                __syncwarp();
+                bool on[4];  // of knots kc + j, by j mod 4
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float fa = __shfl_sync(0xffffffffu, fa_lane, j);
-                    if (kc + j < a.M && mode < a.N)  // streamed once: evict-first
-                        __stcs(dst + (size_t)(kc + j) * a.N + mode, f32_to_f64(__uint_as_float(v[j]) * fb * fa));
+                for (int j = 0; j < 4; ++j) {
+                    const int off = overlap ? -(at0 + (kc + j) * a.N) & 3 : 0;
+                    on[j] = live && (first || lane >= off) && (last || lane < off + a.step);
                 }
+                double *row = dst + (size_t)kc * a.N + mode;
+                auto store = [&](auto whole) {  // every knot of the chunk is one of the call's
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4) {
+                        const float4 fa = *reinterpret_cast<const float4 *>(&s_fa[e][j]);
+                        const float2 fb2 = make_float2(fb, fb);
+                        const float2 y0 = __fmul2_rn(__fmul2_rn(make_float2(v[j], v[j + 1]), fb2), make_float2(fa.x, fa.y));
+                        const float2 y1 = __fmul2_rn(__fmul2_rn(make_float2(v[j + 2], v[j + 3]), fb2), make_float2(fa.z, fa.w));
+                        const float y[4] = {y0.x, y0.y, y1.x, y1.y};
+                        double w[4];
+                        bool odd = false;  // not a normal number
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            w[i] = f32_normal_to_f64(y[i]);
+                            odd |= !f32_is_normal(y[i]);
+                        }
+                        if (odd) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) w[i] = f32_to_f64(y[i]);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {  // streamed once: evict-first
+                            if (on[i] && (decltype(whole)::value || kc + j + i < a.M)) __stcs(row, w[i]);
+                            row += a.N;
+                        }
+                    }
+                };
+                if (kc + 32 <= a.M)
+                    store(std::true_type());
+                else
+                    store(std::false_type());
+                __syncwarp();  // s_fa is rewritten
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tempty[b]);
+            ++u;
         }
     }
 
@@ -683,9 +779,12 @@ RbLayout rb_layout(int Nb, int N, int M)
 {
     RbLayout L;
     L.n_kb = (kRbParts * 2 * Nb + kRbTileK - 1) / kRbTileK;
-    L.n_tiles = (N + kRbModes - 1) / kRbModes;
+    // whole sectors: 28 modes of each group (N a multiple of four: every row is aligned alike, all 32)
+    L.step = N % 4 ? 28 : 32;
+    L.groups = N <= 32 ? 1 : (N - (32 - L.step) + L.step - 1) / L.step;
+    L.n_tiles = (L.groups + 1) / 2;
     L.m_tiles = (M + kRbTileN - 1) / kRbTileN;
-    L.modes_padded = L.n_tiles * kRbModes;
+    L.modes_padded = (2 * L.n_tiles - 1) * L.step + 32;
     L.rows_padded = L.m_tiles * kRbTileN;
     L.bpack_bytes = (size_t)L.n_tiles * L.n_kb * kRbABytes;
     L.apack_bytes = (size_t)L.m_tiles * L.n_kb * kRbBBytes;
@@ -698,7 +797,7 @@ cudaError_t launch_rb_basis(const double *bre, const double *bim, int Nb, int N,
     const RbLayout L = rb_layout(Nb, N, 0);
     k_rb_gram<<<Nb * Nb, 128, 0, st>>>(bre, bim, Nb, N, gt64, gt32);
     k_rb_bexp<<<(L.modes_padded + 127) / 128, 128, 0, st>>>(bre, bim, Nb, N, L.modes_padded, bexp);
-    k_rb_pack_b<<<sm_count * 8, 256, 0, st>>>(bre, bim, Nb, N, L.n_kb, L.n_tiles, bexp, bpack);
+    k_rb_pack_b<<<sm_count * 8, 256, 0, st>>>(bre, bim, Nb, N, L.n_kb, L.n_tiles, L.step, bexp, bpack);
     return cudaGetLastError();
 }
 
@@ -713,9 +812,12 @@ cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N
     const RbLayout L = rb_layout(Nb, N, M);
     cudaError_t e;
     const double *sc = nullptr;
-    // mixed path: the scale is applied in the product's epilogue, so its kernels run on the side
-    // stream beside the coefficient pack and are joined before the product
-    const bool fork = nu && !fp64 && side;
+    // mixed path: the scale is applied in the product's epilogue, so its kernels run beside the
+    // coefficient pack: the one-kernel form (Nb <= 128) lets the pack start with it and the product
+    // with the pack's end (dependent launches; 1,486 knots of 60 vectors and 279 modes 37.6 -> 21.5 us
+    // without the side stream's two events), the longer one runs on a side stream
+    const bool tile = nu && !fp64 && Nb <= kTMaxBasis;
+    const bool fork = nu && !fp64 && !tile && side;
     cudaStream_t ss = fork ? side : st;
     if (fork) {
         if ((e = cudaEventRecord(fork_ev, st)) != cudaSuccess) return e;
@@ -727,12 +829,19 @@ cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N
         if (fork) cudaStreamSynchronize(side);
         return err;
     };
-    if (nu && !fp64 && Nb <= kTMaxBasis) {
-        const int smem = (kTRows * Nb + Nb * kTJ) * (int)sizeof(float2);
-        e = cudaFuncSetAttribute(k_rb_scale_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return fail(e);
-        k_rb_scale_tile<<<(M + kTRows - 1) / kTRows, kTThreads, smem, ss>>>(are, aim, M, Nb, gt32, nu,
-                                                                             scale, err);
+    if (tile) {
+        using Kernel = void (*)(const double *, const double *, int, int, const float2 *, const double *, double *,
+                                unsigned *);
+        static const Kernel kernels[8] = {k_rb_scale_tile<1>, k_rb_scale_tile<2>, k_rb_scale_tile<3>,
+                                          k_rb_scale_tile<4>, k_rb_scale_tile<5>, k_rb_scale_tile<6>,
+                                          k_rb_scale_tile<7>, k_rb_scale_tile<8>};
+        const int T = (Nb + 15) / 16, smem = (kTRows * Nb + Nb * 16 * T) * (int)sizeof(float2);
+        const Kernel k = kernels[T - 1];
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (kTRows + kTMaxBasis) * kTMaxBasis * (int)sizeof(float2));
+        if (e != cudaSuccess) return e;
+        k<<<(M + kTRows - 1) / kTRows, kTThreads, smem, st>>>(are, aim, M, Nb, gt32, nu, scale, err);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
         sc = scale;
     } else if (nu && fp64) {
         k_rb_scale64<<<M, (Nb + 31) / 32 * 32, 0, ss>>>(are, aim, Nb, gt64, nu, scale, err);
@@ -757,18 +866,27 @@ cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N
     }
     const int rows = L.m_tiles * kRbTileN;
     const int pgrid = (rows + kRbPackWarps - 1) / kRbPackWarps;
-    k_rb_pack_a<<<pgrid < sm_count * 8 ? pgrid : sm_count * 8, kRbPackWarps * 32, 0, st>>>(
-        are, aim, M, Nb, L.n_kb, L.m_tiles, apack, aexp);
-    if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
+    const unsigned pblocks = pgrid < sm_count * 8 ? pgrid : sm_count * 8;
+    if (tile) {  // beside the scale's kernel
+        e = launch_pdl(k_rb_pack_a, pblocks, kRbPackWarps * 32, 0, st, are, aim, M, Nb, L.n_kb, L.m_tiles, apack,
+                       aexp);
+    } else {
+        k_rb_pack_a<<<pblocks, kRbPackWarps * 32, 0, st>>>(are, aim, M, Nb, L.n_kb, L.m_tiles, apack, aexp);
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess) return fail(e);
     if (fork && (e = cudaStreamWaitEvent(st, join_ev, 0)) != cudaSuccess) return fail(e);
     const int smem = kRbStages * (int)kRbStageBytes + 128;
     e = cudaFuncSetAttribute(k_rb_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const int tiles = L.m_tiles * L.n_tiles;
     const int k_last = kRbParts * 2 * Nb - (L.n_kb - 1) * kRbTileK;  // real columns, last block
-    RbMmaArgs args{apack, bpack, ore, oim, aexp, bexp, sc, M, N, L.n_kb, L.m_tiles, L.n_tiles,
+    RbMmaArgs args{apack, bpack, ore, oim, aexp, bexp, sc, M, N, L.n_kb, L.m_tiles, L.n_tiles, L.groups, L.step,
                    (k_last + 15) / 16, err};
-    k_rb_mma<<<tiles < sm_count ? tiles : sm_count, kRbMmaThreads, smem, st>>>(args);
+    // (small calls: a CTA for each part of a tile)
+    const int blocks = tiles * 8 < sm_count ? tiles * 8 : sm_count;
+    if (!fork) return launch_pdl(k_rb_mma, blocks, kRbMmaThreads, smem, st, args);
+    k_rb_mma<<<blocks, kRbMmaThreads, smem, st>>>(args);
     return cudaGetLastError();
 }
 

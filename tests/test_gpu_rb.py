@@ -172,3 +172,32 @@ def test_rb_fp64_knot_groups(gpu_ctx, M):
     g = _gpu_rb(gpu_ctx, alpha, basis, nu, F.FEW_FP64)
     assert np.all(np.isfinite(g))
     _check_rows(g, oracle.rb_amplitudes(alpha, basis, nu), alpha, basis, nu, F.FEW_FP64)
+
+
+@pytest.mark.parametrize("M,N,shift", [(1, 28, 0), (16, 32, 1), (17, 33, 0), (33, 60, 1), (255, 61, 3), (257, 63, 2),
+                                       (300, 3843, 1), (520, 3841, 0)])
+@pytest.mark.parametrize("Nb", [3, 99, 128])
+def test_rb_mixed_store_edges(gpu_ctx, M, N, Nb, shift):
+    """Every way the output rows can start in a sector, groups of modes that just fit, parts of tiles; the
+    output is written whole and nothing around it."""
+    import torch
+    rng = np.random.default_rng(M + 7 * N + Nb)
+    alpha = rng.standard_normal((M, Nb)) + 1j * rng.standard_normal((M, Nb))
+    basis = rng.standard_normal((Nb, N)) + 1j * rng.standard_normal((Nb, N))
+    nu = rng.uniform(0.5, 2.0, M)
+    h = F.few_basis_create(gpu_ctx.handle, basis.real, basis.imag, RT.current_stream())
+    try:
+        out = [torch.full((M * N + 8,), 7.0, dtype=torch.float64, device="cuda") for _ in range(2)]
+        re, im = (o[2 + shift:2 + shift + M * N].view(M, N) for o in out)
+        F.few_rb_amplitudes(gpu_ctx.handle, h, _dev(alpha.real), _dev(alpha.imag), re, im, _dev(nu),
+                            F.FEW_MIXED, RT.current_stream())
+        torch.cuda.synchronize()
+        assert gpu_ctx.sync_status() == F.FEW_OK
+        plain = alpha @ basis
+        s = (nu / np.linalg.norm(plain, axis=1))[:, None]
+        err = np.linalg.norm(to_host(re) + 1j * to_host(im) - s * plain, axis=1)
+        assert np.all(err <= MIXED_GAMMA * np.linalg.norm(s * (np.abs(alpha) @ np.abs(basis)), axis=1))
+        for o in out:
+            assert torch.all(o[:2 + shift] == 7.0) and torch.all(o[2 + shift + M * N:] == 7.0)
+    finally:
+        F.few_basis_release(gpu_ctx.handle, h)
