@@ -218,7 +218,7 @@ struct SlotPlan {
 // every new trajectory and checked on that of every direct sum.
 struct RowRange {
     int m_top = 0, m_last = 0, n_rows = 0;
-    int n_min = 0, n_max = 0;        // of the listed modes
+    int l_top = 0, n_min = 0, n_max = 0;  // of the listed modes
     std::vector<int> lo, hi, first;  // [n_rows] n range (lo > hi: empty), first slot
     int slots = 0;
     int slot(int ms, int ns) const { return first[m_top - ms] + hi[m_top - ms] - ns; }
@@ -233,6 +233,7 @@ few_status check_modes(const int *l, const int *m, const int *n, int N, RowRange
             n[i] > kMaxAbsN)
             return FEW_ERR_MODES;
         m_top = std::max(m_top, m[i]);
+        R.l_top = std::max(R.l_top, l[i]);
         R.n_min = std::min(i ? R.n_min : n[0], n[i]);
         R.n_max = std::max(i ? R.n_max : n[0], n[i]);
     }
@@ -829,7 +830,7 @@ few_status few_ctx_create(few_ctx **out, int device, size_t hbm_budget_bytes)
     if (cudaMalloc(&c->d_err, sizeof(unsigned)) != cudaSuccess) return fail(FEW_ERR_NOMEM);
     if (cudaMemset(c->d_err, 0, sizeof(unsigned)) != cudaSuccess) return fail(FEW_ERR_CUDA);
     if (sum_configure() != cudaSuccess || tc_configure() != cudaSuccess ||
-        tc64_configure() != cudaSuccess)
+        tc64_configure() != cudaSuccess || direct_configure() != cudaSuccess)
         return fail(FEW_ERR_CUDA);
     for (auto &e : c->tev)
         if (cudaEventCreate(&e) != cudaSuccess) return fail(FEW_ERR_CUDA);
@@ -1278,8 +1279,8 @@ few_status few_direct_sum(few_ctx *ctx, const double *pphi, const double *pr, co
         const int *dl = reinterpret_cast<const int *>(b + mc_bytes);
         cudaError_t e = launch_direct(pphi, pr, are, aim, (long long)ns, dl, dl + stride,
                                       dl + 2 * stride, N, theta, phi, scale, prec == FEW_FP64, out,
-                                      out_c64 ? 1 : 0, b, modes.m_top, modes.n_min, modes.n_max,
-                                      ctx->sm_count, s);
+                                      out_c64 ? 1 : 0, b, modes.l_top, modes.m_top, modes.n_min, modes.n_max,
+                                      ctx->sm_count, ctx->d_err, s);
         if (e != cudaSuccess) {
             (void)cudaGetLastError();
             st = FEW_ERR_CUDA;

@@ -58,6 +58,14 @@ __device__ __forceinline__ uint64_t l2_evict_last_policy()
     return pol;
 }
 
+// L2 policy for data that is read once.
+__device__ __forceinline__ uint64_t l2_evict_first_policy()
+{
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+
 // Bulk copy global -> shared with an L2 cache policy for the source lines.
 __device__ __forceinline__ void bulk_g2s_hint(void *dst, const void *src, uint32_t bytes, uint64_t *bar,
                                               uint64_t policy)

@@ -41,6 +41,19 @@ __device__ __forceinline__ float f64_to_f32_fast(double d)
     return __uint_as_float(f);
 }
 
+// The same in four instructions for an x that is a normal FP32 number unrounded, and whether it is one.
+__device__ __forceinline__ float f64_normal_to_f32(double x)
+{
+    const unsigned long long raw = static_cast<unsigned long long>(__double_as_longlong(x));
+    const unsigned long long b = raw + (0x10000000ull - (896ull << 52));  // rounded, the exponent rebiased
+    return __uint_as_float(__funnelshift_l(static_cast<unsigned>(b), static_cast<unsigned>(b >> 32), 3) |
+                           (static_cast<unsigned>(raw >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ bool f64_is_f32_normal(double x)
+{
+    return 2u * static_cast<unsigned>(__double2hiint(x)) - 0x70200000u < 0x1fc00000u;
+}
+
 // FP32 -> FP64 on the integer pipe: exact for normal floats (rebias the exponent 127 -> 1023,
 // widen the significand); zero and subnormal inputs give a signed zero, inf and nan stay so.
 __device__ __forceinline__ double f32_to_f64(float x)

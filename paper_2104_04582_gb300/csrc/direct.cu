@@ -12,7 +12,13 @@
 // exponentials from the sample's reduced phases (FP64 reduction of Phi_phi and Phi_r modulo 2 pi,
 // then the sine and cosine of the reduced integer combination), and the warp reduces its partial
 // sums with shuffles.
+#include <type_traits>
+
+#include <cuda_fp16.h>
+
+#include "async.cuh"
 #include "fewsum_internal.h"
+#include "launch.cuh"
 #include "harmonics.cuh"
 #include "phase_eval.cuh"
 #include "convert.cuh"
@@ -208,12 +214,265 @@ k_direct_tab(const double *__restrict__ pphi, const double *__restrict__ pr,
     }
 }
 
+// Mixed precision with the amplitudes streamed through shared memory.  The kernel is bound by HBM, and a
+// warp of k_direct that holds its loads in registers has none in flight while it computes.  Here every
+// warp keeps a ring of three chunks (256 modes of one sample, 4 KB) filled by bulk copies, two of them on
+// the way while it works on the third: 130 KB in flight on each multiprocessor, no barrier between
+// warps.  The ring leaves L1 too small for 32 bytes of constants per mode (four times the amplitudes'
+// bytes), but Y+ and Y- belong to (l, m), not to n: a word per mode (its (l, m), n) and a record per
+// (l, m), which a warp's 32 modes mostly share, fit in shared memory beside the ring.
+// A copy starts and ends on 16-byte boundaries, so it may take a neighbouring element with it; a chunk
+// for which that would lie outside the arrays is read directly.  At four warps a scheduler instruction
+// issue comes next: amplitudes that are normal FP32 numbers take a four-instruction conversion, a mode
+// 36 instructions, and a lane forms the phases of one of the next 32 samples (FP64 work that every lane
+// did for every sample: half the time of 132-mode calls).
+// 100,000 samples x 3843 modes: see launch_direct for both sides.
+constexpr int kRingWarps = 16, kRingStages = 3, kRingModes = 256;
+constexpr int kRingRow = (kRingModes + 2) * (int)sizeof(double);  // one component of a chunk
+constexpr int kRingBytes = kRingWarps * kRingStages * 2 * kRingRow;
+constexpr int kRingTables = 32 * 1024;  // words and records beside the ring
+
+struct alignas(16) PairConst {
+    float a, b, g, d;  // as ModeConst
+    float m, pad[3];
+};
+
+__host__ __device__ inline int ring_table_bytes(int N, int pairs)
+{
+    return ((N * (int)sizeof(unsigned) + 15) & ~15) + pairs * (int)sizeof(PairConst);
+}
+
+// The tables: (l, m) is record (l - 2) (m_top + 1) + m; a word is the record's place in bytes (later its address) and n in fp16
+// (exact: |n| <= 1024).
+__global__ void k_mode_words(const int *__restrict__ l, const int *__restrict__ m, const int *__restrict__ n, int N,
+                             double theta, double phi, int l_top, int m_top, unsigned *__restrict__ words,
+                             PairConst *__restrict__ pairs)
+{
+    pdl_launch_dependents();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N)
+        words[i] = (unsigned)(((l[i] - 2) * (m_top + 1) + m[i]) * (int)sizeof(PairConst)) |
+                   (unsigned)__half_as_ushort(__int2half_rn(n[i])) << 16;
+    if (i >= (l_top - 1) * (m_top + 1)) return;
+    const int li = 2 + i / (m_top + 1), mi = i % (m_top + 1);
+    if (mi > li) return;  // no such mode
+    const double2 yp = swsh_m2(li, mi, theta, phi);
+    double2 ym = make_double2(0.0, 0.0);
+    if (mi > 0) {
+        ym = swsh_m2(li, -mi, theta, phi);
+        if (li & 1) ym = make_double2(-ym.x, -ym.y);
+    }
+    pairs[i] = PairConst{(float)(yp.x + ym.x), (float)(yp.y - ym.y), (float)(yp.y + ym.y), (float)(yp.x - ym.x),
+                         (float)mi, {}};
+}
+
+__global__ void __launch_bounds__(32 * kRingWarps, 1)
+k_direct_ring(const double *__restrict__ pphi, const double *__restrict__ pr, const double *__restrict__ are,
+              const double *__restrict__ aim, long long ns, int N, const uint4 *__restrict__ tables, int table_bytes,
+              double scale, void *__restrict__ out, int out_c64, unsigned *__restrict__ err)
+{
+    extern __shared__ __align__(16) unsigned char ring_smem[];
+    __shared__ __align__(8) uint64_t full[kRingWarps][kRingStages];
+    const double kInv2Pi = 0.15915494309189533577;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the tables (a word's record as its address in shared memory), then the warps' rings
+    const int word_uints = (N + 3) & ~3;
+    const unsigned recs = smem_u32(ring_smem) + 4u * word_uints;
+    unsigned char *ring = ring_smem + table_bytes + warp * kRingStages * 2 * kRingRow;
+    uint64_t *bar = full[warp];
+    if (lane == 0) {
+        for (int s = 0; s < kRingStages; ++s) mbar_init(&bar[s], 1);
+        fence_mbar_init();
+    }
+    // this warp's samples, spread over the multiprocessors first
+    const long long first = (long long)warp * gridDim.x + blockIdx.x, step = (long long)kRingWarps * gridDim.x;
+    const int chunks = (N + kRingModes - 1) / kRingModes, tail = N - (chunks - 1) * kRingModes;
+    const long long items = first < ns ? ((ns - 1 - first) / step + 1) * chunks : 0;
+    // an item is copied unless its 16-byte units reach before the arrays' start or past their end
+    const uintptr_t end = sizeof(double) * (uintptr_t)ns * (uintptr_t)N;
+    const bool skip0 = first == 0 && ((reinterpret_cast<uintptr_t>(are) | reinterpret_cast<uintptr_t>(aim)) & 8);
+    const bool skip1 = (ns - 1 - first) % step == 0 &&
+                       (((reinterpret_cast<uintptr_t>(are) + end) | (reinterpret_cast<uintptr_t>(aim) + end)) & 8);
+    auto copied = [&](long long it) { return !(it == 0 && skip0) && !(it + 1 == items && skip1); };
+    const uint64_t once = l2_evict_first_policy();
+    // the next item to fill (one lane): address of its first elements and its chunk
+    const long long row0 = sizeof(double) * first * N;
+    uintptr_t fa = reinterpret_cast<uintptr_t>(are) + row0;
+    const intptr_t other = reinterpret_cast<intptr_t>(aim) - reinterpret_cast<intptr_t>(are);
+    const long long next_row = (long long)sizeof(double) * (step * N - (long long)(chunks - 1) * kRingModes);
+    long long filled = 0;
+    int fc = 0;
+    auto fill = [&](int s) {
+        if (filled == items) return;
+        const bool last = ++fc == chunks;
+        if (copied(filled)) {
+            const uint32_t len = (uint32_t)(last ? tail : kRingModes) * 8u;
+            const uintptr_t sa = fa & ~(uintptr_t)15, sb = (fa + other) & ~(uintptr_t)15;
+            const uint32_t la = (uint32_t)(fa & 8) + len + 15 & ~15u, lb = (uint32_t)((fa + other) & 8) + len + 15 & ~15u;
+            mbar_arrive_expect_tx(&bar[s], la + lb);
+            bulk_g2s_hint(ring + 2 * s * kRingRow, reinterpret_cast<const void *>(sa), la, &bar[s], once);
+            bulk_g2s_hint(ring + (2 * s + 1) * kRingRow, reinterpret_cast<const void *>(sb), lb, &bar[s], once);
+        } else {
+            mbar_arrive(&bar[s]);
+        }
+        fa += last ? next_row : (long long)(8 * kRingModes);
+        if (last) fc = 0;
+        ++filled;
+    };
+    if (lane == 0)
+        for (int s = 0; s < kRingStages; ++s) fill(s);
+    pdl_wait();  // the tables (the amplitudes were there before their kernel)
+    for (int i = threadIdx.x; i < table_bytes / 16; i += blockDim.x) {
+        uint4 v = tables[i];
+        if (4 * i < word_uints) {
+            v.x += recs;
+            v.y += recs;
+            v.z += recs;
+            v.w += recs;
+        }
+        reinterpret_cast<uint4 *>(ring_smem)[i] = v;
+    }
+    __syncthreads();
+    if (items == 0) return;
+    long long i = first;
+    int c = 0, s = 0;
+    uint32_t parity = 0;
+    float fphi = 0.0f, fr = 0.0f, hr = 0.0f, hi = 0.0f;
+    float vphi = 0.0f, vr = 0.0f;  // phases of 32 samples, one a lane
+    int ahead = 0;                 // of them, used
+    bool ok = true;
+    for (long long it = 0; it < items; ++it) {
+        if (c == 0) {
+            if (ahead == 0) {
+                const long long mine = i + lane * step;
+                const double xp = reduce_2pi(pphi[mine < ns ? mine : i]) * kInv2Pi;
+                const double xr = reduce_2pi(pr[mine < ns ? mine : i]) * kInv2Pi;
+                vphi = (float)(xp - rint(xp));
+                vr = (float)(xr - rint(xr));
+            }
+            fphi = __shfl_sync(0xffffffffu, vphi, ahead);
+            fr = __shfl_sync(0xffffffffu, vr, ahead);
+            ahead = (ahead + 1) & 31;
+            hr = hi = 0.0f;
+        }
+        ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar[s], parity));
+        if (!ok) break;
+        const size_t at = (size_t)i * N + (size_t)c * kRingModes;
+        const int left = N - c * kRingModes - lane;  // modes of the chunk from this lane's first on
+        const unsigned *wp = reinterpret_cast<const unsigned *>(ring_smem) + c * kRingModes + lane;
+        constexpr int U = kRingModes / 32;
+        auto sum = [&](auto whole, const double *ra, const double *rb) {
+            constexpr bool kWhole = decltype(whole)::value;  // every lane has all its modes
+            double va[U], vb[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                va[u] = kWhole || 32 * u < left ? ra[32 * u] : 1.0;
+                vb[u] = kWhole || 32 * u < left ? rb[32 * u] : 1.0;
+            }
+            float xa[U], xb[U];
+            bool odd = false;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                xa[u] = f64_normal_to_f32(va[u]);
+                xb[u] = f64_normal_to_f32(vb[u]);
+                odd |= !f64_is_f32_normal(va[u]);
+                odd |= !f64_is_f32_normal(vb[u]);
+            }
+            if (odd) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    xa[u] = f64_to_f32_fast(va[u]);
+                    xb[u] = f64_to_f32_fast(vb[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (!kWhole && 32 * u >= left) break;
+                const unsigned w = wp[32 * u];
+                float ka, kb, kg, kd, km;  // the record
+                asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(ka), "=f"(kb), "=f"(kg), "=f"(kd) : "r"(w & 0xffffu));
+                asm("ld.shared.f32 %0, [%1 + 16];" : "=f"(km) : "r"(w & 0xffffu));
+                const float n = __half2float(__ushort_as_half((unsigned short)(w >> 16)));
+                float ph = fmaf(n, fr, km * fphi);
+                ph -= round_near(ph);
+                float sn, co;
+                expi_turns(ph, &sn, &co);
+                // A e^{-i Phi}
+                const float wr = fmaf(xb[u], sn, xa[u] * co), wi = fmaf(xb[u], co, -xa[u] * sn);
+                hr += fmaf(ka, wr, -(kb * wi));  // (one rounding at the sum's size)
+                hi += fmaf(kg, wr, kd * wi);
+            }
+        };
+        if (copied(it)) {
+            const uintptr_t pa = reinterpret_cast<uintptr_t>(are) + 8 * at, pb = reinterpret_cast<uintptr_t>(aim) + 8 * at;
+            const double *ra = reinterpret_cast<const double *>(ring + 2 * s * kRingRow + (pa & 8)) + lane;
+            const double *rb = reinterpret_cast<const double *>(ring + (2 * s + 1) * kRingRow + (pb & 8)) + lane;
+            if (c + 1 < chunks || tail == kRingModes)
+                sum(std::true_type(), ra, rb);
+            else
+                sum(std::false_type(), ra, rb);
+        } else {
+            sum(std::false_type(), are + at + lane, aim + at + lane);
+        }
+        __syncwarp();  // the chunk has been read
+        if (lane == 0) fill(s);
+        __syncwarp();
+        if (++s == kRingStages) {
+            s = 0;
+            parity ^= 1u;
+        }
+        if (++c < chunks) continue;
+        c = 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            hr += __shfl_down_sync(0xffffffffu, hr, o);
+            hi += __shfl_down_sync(0xffffffffu, hi, o);
+        }
+        if (lane == 0) {
+            const double vr0 = (double)hr * scale, vi0 = (double)hi * scale;
+            if (out_c64)
+                reinterpret_cast<float2 *>(out)[i] = make_float2((float)vr0, (float)vi0);
+            else
+                reinterpret_cast<double2 *>(out)[i] = make_double2(vr0, vi0);
+        }
+        i += step;
+    }
+    if (!ok && lane == 0) {
+        atomicOr(err, ERRBIT_TIMEOUT);
+        // no copy may land after the block's shared memory is gone: this round's stages from s on, the
+        // next one's before it (those that were filled)
+        for (int q = s; q < s + kRingStages; ++q)
+            mbar_wait_bounded(&bar[q % kRingStages], q < kRingStages ? parity : parity ^ 1u);
+    }
+}
+
+cudaError_t direct_configure()
+{
+    return cudaFuncSetAttribute(k_direct_ring, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kRingBytes + kRingTables);
+}
+
 cudaError_t launch_direct(const double *pphi, const double *pr, const double *are,
                           const double *aim, long long ns, const int *l, const int *m, const int *n,
                           int N, double theta, double phi, double scale, bool fp64, void *out,
-                          int out_c64, void *mode_consts, int m_top, int n_lo, int n_hi, int sm_count,
-                          cudaStream_t st)
+                          int out_c64, void *mode_consts, int l_top, int m_top, int n_lo, int n_hi, int sm_count,
+                          unsigned *err, cudaStream_t st)
 {
+    // mixed precision: through the ring while the mode tables fit beside it and in the caller's scratch
+    // (100,000 samples: 3843 modes 1,095 -> 875 us, reading them alone takes 835; 78,314 samples of 132
+    // modes 163 -> 87 us a call), else a warp a sample from registers
+    const int pairs = (l_top - 1) * (m_top + 1), table = ring_table_bytes(N, pairs);
+    if (!fp64 && ns > 0 && table <= kRingTables && (size_t)table <= direct_mode_const_bytes(N)) {
+        auto *words = static_cast<unsigned *>(mode_consts);
+        auto *recs = reinterpret_cast<PairConst *>(static_cast<unsigned char *>(mode_consts) + table) - pairs;
+        const int n_thr = N > pairs ? N : pairs;
+        k_mode_words<<<(n_thr + 63) / 64, 64, 0, st>>>(l, m, n, N, theta, phi, l_top, m_top, words, recs);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        return launch_pdl(k_direct_ring, (unsigned)(ns < sm_count ? ns : sm_count), 32 * kRingWarps,
+                          (size_t)(kRingBytes + table), st, pphi, pr, are, aim, ns, N,
+                          static_cast<const uint4 *>(mode_consts), table, scale, out, out_c64, err);
+    }
     // the tables pay wherever they hold fewer exponentials than there are modes
     const int entries = m_top + 1 + n_hi - n_lo + 1;
     if (fp64 && entries <= kTabMaxEntries && entries < N && ns > 0) {
@@ -252,6 +511,7 @@ cudaError_t launch_direct(const double *pphi, const double *pr, const double *ar
     return cudaGetLastError();
 }
 
+static_assert(kMaxAbsN <= 2048 && kRingTables + 4096 <= 65536, "a word: n in fp16, a record's address");
 static_assert(sizeof(ModeConstTab) == sizeof(ModeConst<double>), "one scratch size for both");
 size_t direct_mode_const_bytes(int N) { return sizeof(ModeConst<double>) * (size_t)N; }
 

@@ -290,9 +290,10 @@ int mode_select_max_modes();
 cudaError_t launch_direct(const double *pphi, const double *pr, const double *are,
                           const double *aim, long long ns, const int *l, const int *m, const int *n,
                           int N, double theta, double phi, double scale, bool fp64, void *out,
-                          int out_c64, void *mode_consts, int m_top, int n_lo, int n_hi, int sm_count,
-                          cudaStream_t st);
+                          int out_c64, void *mode_consts, int l_top, int m_top, int n_lo, int n_hi, int sm_count,
+                          unsigned *err, cudaStream_t st);
 size_t direct_mode_const_bytes(int N);
+cudaError_t direct_configure();
 // Reduced-basis amplitudes (rb.cu): tile counts of the packed tensor-core operands.
 struct RbLayout {
     int n_kb = 0, n_tiles = 0, m_tiles = 0, modes_padded = 0, rows_padded = 0;

@@ -134,3 +134,31 @@ def test_direct_fp64_table_edges(gpu_ctx, ms, ns_range, ns):
     g = _gpu_direct(gpu_ctx, pphi, pr, are, aim, modes, 0.9, 2.1, F.FEW_FP64)
     o = oracle.direct_dense(pphi, pr, modes, are, aim, 0.9, 2.1)
     assert rel_l2(g, o) <= FP64_REL_L2
+
+
+@pytest.mark.parametrize("ms,ns_range,ns", [
+    ([2], range(255), 3), ([2], range(-128, 128), 153), ([2], range(-128, 129), 4867),  # a chunk less one, one, one more
+    (range(11), range(-30, 31), 17), (range(11), range(-330, 331), 5)])  # the last: tables too large for the ring
+@pytest.mark.parametrize("shift", [0, 1])
+def test_direct_mixed_ring_edges(gpu_ctx, ms, ns_range, ns, shift):
+    """Both sides of the mixed path's choice between amplitudes streamed through shared memory and read
+    directly; odd and even rows, and arrays that start and end between 16-byte boundaries."""
+    import torch
+    rng = np.random.default_rng(ns)
+    modes = np.asarray([(10, m, n) for m in ms for n in ns_range], dtype=np.int32)
+    N = len(modes)
+    pphi, pr = rng.uniform(-1e5, 1e5, (2, ns))
+    are, aim = rng.standard_normal((2, ns, N))
+    views = []
+    for a in (are, aim):
+        buf = torch.full((ns * N + 2,), float("nan"), dtype=torch.float64, device="cuda")
+        v = buf[shift:shift + ns * N].view(ns, N)
+        v.copy_(torch.as_tensor(a))
+        views.append(v)
+    out = torch.empty(ns, dtype=torch.complex64, device="cuda")
+    F.few_direct_sum(gpu_ctx.handle, torch.as_tensor(pphi).cuda(), torch.as_tensor(pr).cuda(), *views, modes,
+                     0.9, 2.1, out, 1.0, F.FEW_MIXED, RT.current_stream())
+    torch.cuda.synchronize()
+    assert gpu_ctx.sync_status() == F.FEW_OK
+    o = oracle.direct_dense(pphi, pr, modes, are, aim, 0.9, 2.1)
+    assert oracle.mismatch(to_host(out), o) <= MIXED_MISMATCH
