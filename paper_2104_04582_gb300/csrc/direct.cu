@@ -140,14 +140,22 @@ k_direct(const double *__restrict__ pphi, const double *__restrict__ pr,
 // memory, and a mode costs 12 FP64 operations: e^{i Phi} = the product of two entries, w = A
 // e^{-i Phi}, and
 //     h += w Y+ + conj(w) Y- = [a Re w - b Im w] + i [g Re w + d Im w]   (a, b, g, d as above).
-// Small blocks (4 samples), so that the last wave is spread evenly.  4001 samples x 1953 modes:
-// see launch_direct for both sides.
+// kPairs: the factor of (l, m) is formed once per sample too, in a table over (l, m): with v = A e^{-i n
+// Phi_r}, c = cos m Phi_phi, s = sin m Phi_phi,
+//     h += [(a c + b s) Re v - (b c - a s) Im v] + i [(g c - d s) Re v + (d c + g s) Im v],
+// and a mode costs 8 operations.
+// Small blocks (4 samples), so that the last wave is spread evenly.  4001 samples x 1953 modes: 814 us
+// with sincospi per mode, 245 with the exponentials' tables, 182 with kPairs.
 constexpr int kTabThreads = 128;
+constexpr int kTabMaxBytes = 12 * 1024;  // a warp, with kPairs
 constexpr int kTabMaxEntries = 512;  // (m_top + 1) + (n_hi - n_lo + 1): 8 KB a warp
 
 struct alignas(16) ModeConstTab {
     double a, b, g, d;
     int m, n, pad[2];  // table entries of m and n
+};
+struct alignas(16) PairConst64 {
+    double a, b, g, d;
 };
 
 __global__ void k_mode_consts_tab(const int *__restrict__ l, const int *__restrict__ m,
@@ -166,10 +174,34 @@ __global__ void k_mode_consts_tab(const int *__restrict__ l, const int *__restri
                           m[i], m_top + 1 + n[i] - n_lo, {0, 0}};
 }
 
+// kPairs: the constants of every (l, m), record (l - 2) (m_top + 1) + m, and each mode's record and n.
+__global__ void k_pair_consts(const int *__restrict__ l, const int *__restrict__ m, const int *__restrict__ n, int N,
+                              double theta, double phi, int l_top, int m_top, int n_lo, int2 *__restrict__ modes,
+                              PairConst64 *__restrict__ pairs)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N) modes[i] = make_int2((l[i] - 2) * (m_top + 1) + m[i], m_top + 1 + n[i] - n_lo);
+    if (i >= (l_top - 1) * (m_top + 1)) return;
+    const int li = 2 + i / (m_top + 1), mi = i % (m_top + 1);
+    if (mi > li) {  // no such mode
+        pairs[i] = PairConst64{};
+        return;
+    }
+    const double2 yp = swsh_m2(li, mi, theta, phi);
+    double2 ym = make_double2(0.0, 0.0);
+    if (mi > 0) {
+        ym = swsh_m2(li, -mi, theta, phi);
+        if (li & 1) ym = make_double2(-ym.x, -ym.y);
+    }
+    pairs[i] = PairConst64{yp.x + ym.x, yp.y - ym.y, yp.y + ym.y, yp.x - ym.x};
+}
+
+// tables: the modes' ModeConstTab, or (kPairs) n_pairs PairConst64, then int2 per mode.
+template <bool kPairs>
 __global__ void __launch_bounds__(kTabThreads)
 k_direct_tab(const double *__restrict__ pphi, const double *__restrict__ pr,
              const double *__restrict__ are, const double *__restrict__ aim, long long ns, int N,
-             const ModeConstTab *__restrict__ mc, int m_top, int n_lo, int entries, double scale,
+             const void *__restrict__ tables, int n_pairs, int m_top, int n_lo, int entries, double scale,
              void *__restrict__ out, int out_c64)
 {
     extern __shared__ __align__(16) double2 dir_tab[];
@@ -177,29 +209,57 @@ k_direct_tab(const double *__restrict__ pphi, const double *__restrict__ pr,
     const int lane = threadIdx.x & 31;
     const long long i = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;  // sample
     if (i >= ns) return;  // a whole warp
-    double2 *tab = dir_tab + (threadIdx.x >> 5) * entries;
+    double2 *tab = dir_tab + (threadIdx.x >> 5) * (entries + (kPairs ? 2 * n_pairs : 0));
     const double xp = reduce_2pi(pphi[i]) * kInv2Pi, xr = reduce_2pi(pr[i]) * kInv2Pi;
     const double fphi = xp - rint(xp), fr = xr - rint(xr);
-    for (int e = lane; e < entries; e += 32) {
-        const double x = e <= m_top ? e * fphi : (double)(n_lo + e - m_top - 1) * fr;
+    // (of n and -n one is computed: the table of a range about zero takes half the sincospi)
+    const int n_hi = n_lo + entries - m_top - 2, a0 = n_lo < 0 && n_hi > 0 ? 0 : n_lo;
+    const int a1 = a0 < 0 ? n_hi : max(n_hi, -n_lo);
+    for (int e = lane; e < m_top + 2 + a1 - a0; e += 32) {
+        const int a = a0 + e - m_top - 1;
+        const double x = e <= m_top ? e * fphi : (double)a * fr;
         double s, c;
         sincospi(2.0 * (x - rint(x)), &s, &c);
-        tab[e] = make_double2(c, s);
+        if (e <= m_top || a <= n_hi) tab[e <= m_top ? e : m_top + 1 + a - n_lo] = make_double2(c, s);
+        if (e > m_top && a0 == 0 && -a >= n_lo) tab[m_top + 1 - a - n_lo] = make_double2(c, -s);
     }
     __syncwarp();
     const double *ar = are + (size_t)i * N, *ai = aim + (size_t)i * N;
     double hr = 0.0, hi = 0.0;
+    if constexpr (kPairs) {
+        const PairConst64 *pc = static_cast<const PairConst64 *>(tables);
+        const int2 *md = reinterpret_cast<const int2 *>(pc + n_pairs);
+        double2 *fac = tab + entries;
+        for (int p = lane; p < n_pairs; p += 32) {
+            const PairConst64 y = pc[p];
+            const double2 e = tab[p % (m_top + 1)];
+            fac[2 * p] = make_double2(fma(y.a, e.x, y.b * e.y), fma(y.b, e.x, -y.a * e.y));
+            fac[2 * p + 1] = make_double2(fma(y.g, e.x, -y.d * e.y), fma(y.d, e.x, y.g * e.y));
+        }
+        __syncwarp();
 #pragma unroll 4
-    for (int j = lane; j < N; j += 32) {
-        const double vr = __ldcs(ar + j), vi = __ldcs(ai + j);
-        const double2 y0 = *reinterpret_cast<const double2 *>(&mc[j].a);
-        const double2 y1 = *reinterpret_cast<const double2 *>(&mc[j].g);
-        const int2 mn = *reinterpret_cast<const int2 *>(&mc[j].m);
-        const double2 p = tab[mn.x], q = tab[mn.y];
-        const double co = fma(p.x, q.x, -p.y * q.y), s = fma(p.y, q.x, p.x * q.y);
-        const double wr = fma(vr, co, vi * s), wi = fma(vi, co, -vr * s);
-        hr = fma(wr, y0.x, fma(-wi, y0.y, hr));
-        hi = fma(wr, y1.x, fma(wi, y1.y, hi));
+        for (int j = lane; j < N; j += 32) {
+            const double vr = __ldcs(ar + j), vi = __ldcs(ai + j);
+            const int2 k = md[j];
+            const double2 q = tab[k.y], f = fac[2 * k.x], g = fac[2 * k.x + 1];
+            const double wr = fma(vr, q.x, vi * q.y), wi = fma(vi, q.x, -vr * q.y);
+            hr = fma(wr, f.x, fma(-wi, f.y, hr));
+            hi = fma(wr, g.x, fma(wi, g.y, hi));
+        }
+    } else {
+        const ModeConstTab *mc = static_cast<const ModeConstTab *>(tables);
+#pragma unroll 4
+        for (int j = lane; j < N; j += 32) {
+            const double vr = __ldcs(ar + j), vi = __ldcs(ai + j);
+            const double2 y0 = *reinterpret_cast<const double2 *>(&mc[j].a);
+            const double2 y1 = *reinterpret_cast<const double2 *>(&mc[j].g);
+            const int2 mn = *reinterpret_cast<const int2 *>(&mc[j].m);
+            const double2 p = tab[mn.x], q = tab[mn.y];
+            const double co = fma(p.x, q.x, -p.y * q.y), s = fma(p.y, q.x, p.x * q.y);
+            const double wr = fma(vr, co, vi * s), wi = fma(vi, co, -vr * s);
+            hr = fma(wr, y0.x, fma(-wi, y0.y, hr));
+            hi = fma(wr, y1.x, fma(wi, y1.y, hi));
+        }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -476,12 +536,25 @@ cudaError_t launch_direct(const double *pphi, const double *pr, const double *ar
     // the tables pay wherever they hold fewer exponentials than there are modes
     const int entries = m_top + 1 + n_hi - n_lo + 1;
     if (fp64 && entries <= kTabMaxEntries && entries < N && ns > 0) {
+        const int per = kTabThreads / 32;
+        const unsigned blocks = (unsigned)((ns + per - 1) / per);
+        // factors of (l, m): eight operations a pair and sample save four a mode, where there are more
+        // than twice as many modes (and the tables stay within 12 KB a sample and the caller's scratch)
+        const int bytes = (entries + 2 * pairs) * (int)sizeof(double2);
+        if (N > 2 * pairs && bytes <= kTabMaxBytes &&
+            sizeof(PairConst64) * pairs + sizeof(int2) * (size_t)N <= direct_mode_const_bytes(N)) {
+            auto *pc = static_cast<PairConst64 *>(mode_consts);
+            const int n_thr = N > pairs ? N : pairs;
+            k_pair_consts<<<(n_thr + 63) / 64, 64, 0, st>>>(l, m, n, N, theta, phi, l_top, m_top, n_lo,
+                                                            reinterpret_cast<int2 *>(pc + pairs), pc);
+            k_direct_tab<true><<<blocks, kTabThreads, per * bytes, st>>>(pphi, pr, are, aim, ns, N, pc, pairs, m_top,
+                                                                       n_lo, entries, scale, out, out_c64);
+            return cudaGetLastError();
+        }
         auto *mc = static_cast<ModeConstTab *>(mode_consts);
         k_mode_consts_tab<<<(N + 63) / 64, 64, 0, st>>>(l, m, n, N, theta, phi, m_top, n_lo, mc);
-        const int per = kTabThreads / 32;
-        const int smem = per * entries * (int)sizeof(double2);
-        k_direct_tab<<<(unsigned)((ns + per - 1) / per), kTabThreads, smem, st>>>(
-            pphi, pr, are, aim, ns, N, mc, m_top, n_lo, entries, scale, out, out_c64);
+        k_direct_tab<false><<<blocks, kTabThreads, per * entries * (int)sizeof(double2), st>>>(
+            pphi, pr, are, aim, ns, N, mc, 0, m_top, n_lo, entries, scale, out, out_c64);
         return cudaGetLastError();
     }
     // one wave of resident blocks (8 warps, i.e. 8 samples, per block per round)

@@ -162,3 +162,23 @@ def test_direct_mixed_ring_edges(gpu_ctx, ms, ns_range, ns, shift):
     assert gpu_ctx.sync_status() == F.FEW_OK
     o = oracle.direct_dense(pphi, pr, modes, are, aim, 0.9, 2.1)
     assert oracle.mismatch(to_host(out), o) <= MIXED_MISMATCH
+
+
+@pytest.mark.parametrize("ls,ms,ns_range,extra", [
+    ([5], [0, 3], range(-3, 5), 0),     # 16 records, 16 modes: the factors of (l, m) not tabulated
+    ([5], [0, 3], range(-8, 9), -1),    # 33 modes: tabulated, n about zero, unequal ends
+    ([5], [0, 3], range(-8, 9), -2),    # 32 modes: not
+    ([2, 5], [0, 2], range(-40, -2), 0),  # n of one sign
+    ([2, 5], [1, 2], range(0, 30), 0),
+    ([32], [32], range(-1000, 1001), 0),  # tables too large for either
+    ([32], [0, 32], range(-100, 101), 0)])
+def test_direct_fp64_pair_table_edges(gpu_ctx, ls, ms, ns_range, extra):
+    """Both sides of the choice of a table over (l, m), and the tables' n ranges."""
+    rng = np.random.default_rng(8)
+    modes = np.asarray([(l, m, n) for l in ls for m in ms if m <= l for n in ns_range], dtype=np.int32)
+    modes = modes[:len(modes) + extra]
+    pphi, pr = rng.uniform(-1e5, 1e5, (2, 6))
+    are, aim = rng.standard_normal((2, 6, len(modes)))
+    g = _gpu_direct(gpu_ctx, pphi, pr, are, aim, modes, 0.9, 2.1, F.FEW_FP64)
+    o = oracle.direct_dense(pphi, pr, modes, are, aim, 0.9, 2.1)
+    assert rel_l2(g, o) <= FP64_REL_L2
