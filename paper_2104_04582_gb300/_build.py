@@ -24,7 +24,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CFLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
           f"-I{os.path.join(ROOT, 'include')}", f"-I{CSRC}"]
 SOURCES = ["api.cpp", "spline.cu", "fold.cu", "sum.cu", "tcsum.cu", "tcsum64.cu", "anchor.cu", "selftest.cu", "noalloc.cu",
-           "select.cu", "direct.cu", "rb.cu"]
+           "select.cu", "direct.cu", "rb.cu", "rb64.cu"]
 HEADERS = ["fewsum_internal.h", "phase_eval.cuh", "harmonics.cuh", "convert.cuh", "async.cuh",
            "tcgen05.cuh", "tctile.cuh", "fold_tc.cuh", "launch.cuh"]
 

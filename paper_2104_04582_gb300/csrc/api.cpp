@@ -830,7 +830,8 @@ few_status few_ctx_create(few_ctx **out, int device, size_t hbm_budget_bytes)
     if (cudaMalloc(&c->d_err, sizeof(unsigned)) != cudaSuccess) return fail(FEW_ERR_NOMEM);
     if (cudaMemset(c->d_err, 0, sizeof(unsigned)) != cudaSuccess) return fail(FEW_ERR_CUDA);
     if (sum_configure() != cudaSuccess || tc_configure() != cudaSuccess ||
-        tc64_configure() != cudaSuccess || direct_configure() != cudaSuccess)
+        tc64_configure() != cudaSuccess || direct_configure() != cudaSuccess ||
+        rb64_configure() != cudaSuccess)
         return fail(FEW_ERR_CUDA);
     for (auto &e : c->tev)
         if (cudaEventCreate(&e) != cudaSuccess) return fail(FEW_ERR_CUDA);
@@ -1301,6 +1302,8 @@ struct few_basis {
     const float2 *gt32 = nullptr;
     const int *bexp = nullptr;
     const unsigned char *bpack = nullptr;
+    const int *bexp64 = nullptr;
+    const unsigned char *bpack64 = nullptr;  // digit slices (null: no room for them)
 };
 
 few_status few_basis_create(few_ctx *ctx, const double *b_re, const double *b_im, int Nb, int N,
@@ -1320,8 +1323,15 @@ few_status few_basis_create(few_ctx *ctx, const double *b_re, const double *b_im
     const size_t g64 = align_up(sizeof(double2) * (size_t)Nb * Nb, 256);
     const size_t g32 = align_up(sizeof(float2) * (size_t)Nb * Nb, 256);
     const size_t ex = align_up(sizeof(int) * (size_t)L.modes_padded, 256);
+    const size_t ex64 = align_up(sizeof(int) * (size_t)rb64_modes(N), 256);
+    const size_t plain = align_up(2 * b_bytes + g64 + g32 + ex + L.bpack_bytes, 256);
     void *d = nullptr;
-    few_status st = dev_alloc(ctx, 2 * b_bytes + g64 + g32 + ex + L.bpack_bytes, s, &d);
+    bool digits = true;
+    few_status st = dev_alloc(ctx, plain + ex64 + rb64_basis_bytes(Nb, N), s, &d);
+    if (st) {
+        digits = false;
+        st = dev_alloc(ctx, plain, s, &d);
+    }
     if (st) return st;
     unsigned char *p = static_cast<unsigned char *>(d);
     double *bre = reinterpret_cast<double *>(p), *bim = reinterpret_cast<double *>(p + b_bytes);
@@ -1338,7 +1348,11 @@ few_status few_basis_create(few_ctx *ctx, const double *b_re, const double *b_im
     auto *gt32 = reinterpret_cast<float2 *>(p + 2 * b_bytes + g64);
     int *bexp = reinterpret_cast<int *>(p + 2 * b_bytes + g64 + g32);
     unsigned char *bpack = p + 2 * b_bytes + g64 + g32 + ex;
-    if (!st && launch_rb_basis(bre, bim, Nb, N, gt64, gt32, bexp, bpack, ctx->sm_count, s) != cudaSuccess) {
+    int *bexp64 = reinterpret_cast<int *>(p + plain);
+    unsigned char *bpack64 = p + plain + ex64;
+    if (!st && (launch_rb_basis(bre, bim, Nb, N, gt64, gt32, bexp, bpack, ctx->sm_count, s) != cudaSuccess ||
+                (digits &&
+                 launch_rb64_basis(bre, bim, Nb, N, bexp64, bpack64, ctx->sm_count, s) != cudaSuccess))) {
         (void)cudaGetLastError();
         st = FEW_ERR_CUDA;
     }
@@ -1357,6 +1371,8 @@ few_status few_basis_create(few_ctx *ctx, const double *b_re, const double *b_im
     b->gt32 = gt32;
     b->bexp = bexp;
     b->bpack = bpack;
+    b->bexp64 = digits ? bexp64 : nullptr;
+    b->bpack64 = digits ? bpack64 : nullptr;
     ctx->bases.insert(b);
     *out = b;
     return FEW_OK;
@@ -1392,15 +1408,26 @@ few_status few_rb_amplitudes(few_ctx *ctx, const few_basis *b, const double *are
     const bool fp64 = prec == FEW_FP64;
     const RbLayout L = rb_layout(b->Nb, b->N, M);
     const size_t sc_bytes = align_up(2 * sizeof(double) * (size_t)M, 256);  // scale, then q
-    const size_t ex_bytes = fp64 ? 0 : align_up(sizeof(int) * (size_t)L.rows_padded, 256);
+    bool digits = fp64 && b->bpack64;
+    size_t ex_bytes = 0, pack_bytes = 0;
+    if (!fp64 || digits) {
+        ex_bytes = align_up(sizeof(int) * (size_t)(fp64 ? rb64_rows(M) : L.rows_padded), 256);
+        pack_bytes = fp64 ? rb64_coef_bytes(b->Nb, M) : L.apack_bytes;
+    }
     void *d = nullptr;
-    few_status st = dev_alloc(ctx, sc_bytes + ex_bytes + (fp64 ? 0 : L.apack_bytes), s, &d);
+    few_status st = dev_alloc(ctx, sc_bytes + ex_bytes + pack_bytes, s, &d);
+    if (st && digits) {  // no room for the digits: the plain chain
+        digits = false;
+        ex_bytes = 0;
+        st = dev_alloc(ctx, sc_bytes, s, &d);
+    }
     if (st) return st;
     unsigned char *p = static_cast<unsigned char *>(d);
     auto &lane = ctx->lanes[ctx->lane_next++ % 4];
     cudaError_t e = launch_rb(are, aim, M, b->Nb, b->N, nu, fp64, b->bre, b->bim, b->gt64, b->gt32,
                               b->bexp, b->bpack, reinterpret_cast<double *>(p),
-                              reinterpret_cast<int *>(p + sc_bytes), p + sc_bytes + ex_bytes, ore,
+                              reinterpret_cast<int *>(p + sc_bytes), p + sc_bytes + ex_bytes,
+                              digits ? b->bexp64 : nullptr, digits ? b->bpack64 : nullptr, ore,
                               oim, ctx->d_err, ctx->sm_count, s, lane.s, lane.fork, lane.join);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();

@@ -301,12 +301,32 @@ struct RbLayout {
     size_t bpack_bytes = 0, apack_bytes = 0;
 };
 RbLayout rb_layout(int Nb, int N, int M);
+// FP64 amplitudes from digit slices (rb64.cu).
+struct Rb64Args {
+    const unsigned char *bpack, *apack;
+    const int *bexp, *aexp;
+    const double *are, *aim, *bre, *bim;  // for the outputs left to the plain chain
+    const double *scale;                  // [M] or null
+    double *out_re, *out_im;
+    int M, N, Nb, steps, tiles, per;
+    unsigned *err;
+};
+size_t rb64_basis_bytes(int Nb, int N);
+size_t rb64_coef_bytes(int Nb, int M);
+int rb64_rows(int M);    // padded counts
+int rb64_modes(int N);
+cudaError_t rb64_configure();
+cudaError_t launch_rb64_basis(const double *bre, const double *bim, int Nb, int N, int *bexp, unsigned char *pack,
+                              int sm_count, cudaStream_t st);
+// after_scale: the kernel launched before it on `st` forms the scale.
+cudaError_t launch_rb64(Rb64Args a, unsigned char *apack, int *aexp, bool after_scale, cudaStream_t st);
 cudaError_t launch_rb_basis(const double *bre, const double *bim, int Nb, int N, double2 *gt64,
                             float2 *gt32, int *bexp, unsigned char *bpack, int sm_count, cudaStream_t st);
 cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N, const double *nu,
                       bool fp64, const double *bre, const double *bim, const double2 *gt64,
                       const float2 *gt32, const int *bexp, const unsigned char *bpack, double *scale,
-                      int *aexp, unsigned char *apack, double *ore, double *oim, unsigned *err,
+                      int *aexp, unsigned char *apack, const int *bexp64, const unsigned char *bpack64,
+                      double *ore, double *oim, unsigned *err,
                       int sm_count, cudaStream_t st, cudaStream_t side, cudaEvent_t fork_ev,
                       cudaEvent_t join_ev);
 // Maximum resident CTAs per SM of the summation kernel for a configuration (0 if invalid).

@@ -7,7 +7,8 @@
 // basis Gram matrix, ||alpha B||^2 = sum_jl alpha_j conj(alpha_l) G_jl with G = B B^H, so the
 // scale is known before the product and no second pass over the output is needed.
 //
-// FP64 path: a tiled complex GEMM on the FP64 pipe.
+// FP64 path: exact integer digit slices on the tensor cores (rb64.cu); on the FP64 pipe (k_rb_fp64) in a
+// context without room for the slices.
 // Mixed path: the complex product as one real GEMM on the tcgen05 tensor cores,
 //     [Re A_i, Im A_i] = s sum_q a_q Bhat_q,(2i, 2i+1),  a = [Re alpha | Im alpha] (2 Nb),
 //     Bhat_q,2i = (Re B_qi | -Im B_qi),  Bhat_q,2i+1 = (Im B_qi | Re B_qi),
@@ -738,35 +739,48 @@ k_rb_fp64(const double *__restrict__ are, const double *__restrict__ aim, const 
     }
 }
 
-// The renormalisation of the FP64 path, one block per knot: warp w forms q_k's terms of j = 32 w +
-// lane, t_j = sum_l G_jl conj(alpha_l) with coalesced rows of the transposed Gram matrix, and the
-// warps' sums are added in order: s_k = nu_k / sqrt(q_k).  (k_rb_quad leaves 100 knots to 8 blocks:
-// most of the chip's FP64 pipes idle, and two more launches.)
-__global__ void __launch_bounds__(FEW_MAX_BASIS)
-k_rb_scale64(const double *__restrict__ are, const double *__restrict__ aim, int Nb,
+// The renormalisation of the FP64 path, one block per knot: q_k = sum_jl Re(alpha_j G_jl conj(alpha_l)), s_k =
+// nu_k / sqrt(q_k).  G is Hermitian: with the rows in groups of at most 32, a warp a group, a group's
+// square of G counts once and what is left of it twice.  Four sets of warps share the columns, for
+// loads in flight; partial sums are added in order.  (FP64 pipe: 100 knots of 99 vectors 35 us as one
+// set over whole rows, bound by the loads' latency; 19 us so.)
+constexpr int kScaleSets = 4;
+
+__global__ void __launch_bounds__(FEW_MAX_BASIS * kScaleSets)
+k_rb_scale64(const double *__restrict__ are, const double *__restrict__ aim, int Nb, int groups,
              const double2 *__restrict__ gt, const double *__restrict__ nu,
              double *__restrict__ scale, unsigned *__restrict__ err)
 {
     __shared__ double2 a[FEW_MAX_BASIS];
-    __shared__ double part[FEW_MAX_BASIS / 32];
-    const int k = blockIdx.x, j = threadIdx.x;
-    if (j < Nb) a[j] = make_double2(are[(size_t)k * Nb + j], aim[(size_t)k * Nb + j]);
+    __shared__ double part[FEW_MAX_BASIS / 32 * kScaleSets];
+    pdl_launch_dependents();  // the pack, if it is launched so
+    const int k = blockIdx.x, tid = threadIdx.x, w = tid >> 5, group = w % groups, set = w / groups;
+    for (int j = tid; j < Nb; j += blockDim.x) a[j] = make_double2(are[(size_t)k * Nb + j], aim[(size_t)k * Nb + j]);
     __syncthreads();
-    double tr[2] = {0.0, 0.0}, ti[2] = {0.0, 0.0};
-    const int jj = min(j, Nb - 1);
+    const int rows = (Nb + groups - 1) / groups, first = group * rows, end = min(first + rows, Nb);
+    const int j = first + (tid & 31), jj = min(j, Nb - 1);
+    double q = 0.0;
+#pragma unroll
+    for (int twice = 1; twice >= 0; --twice) {  // the columns before the group's own, then those
+        const int l1 = twice ? first : end;
+        double tr[2] = {0.0, 0.0}, ti[2] = {0.0, 0.0};
 #pragma unroll 4
-    for (int l = 0; l < Nb; ++l) {
-        const double2 g = __ldg(gt + (size_t)l * Nb + jj), x = a[l];
-        tr[l & 1] = fma(g.x, x.x, fma(g.y, x.y, tr[l & 1]));
-        ti[l & 1] = fma(g.y, x.x, fma(-g.x, x.y, ti[l & 1]));
+        for (int l = (twice ? 0 : first) + set, i = 0; l < l1; l += kScaleSets, ++i) {
+            const double2 g = __ldg(gt + (size_t)l * Nb + jj), x = a[l];
+            tr[i & 1] = fma(g.x, x.x, fma(g.y, x.y, tr[i & 1]));
+            ti[i & 1] = fma(g.y, x.x, fma(-g.x, x.y, ti[i & 1]));
+        }
+        if (j < end) {
+            const double p = a[j].x * (tr[0] + tr[1]) - a[j].y * (ti[0] + ti[1]);
+            q += twice ? 2.0 * p : p;
+        }
     }
-    double q = j < Nb ? a[j].x * (tr[0] + tr[1]) - a[j].y * (ti[0] + ti[1]) : 0.0;
     for (int o = 16; o > 0; o >>= 1) q += __shfl_down_sync(0xffffffffu, q, o);
-    if ((j & 31) == 0) part[j >> 5] = q;
+    if ((tid & 31) == 0) part[w] = q;
     __syncthreads();
-    if (j == 0) {
+    if (tid == 0) {
         q = 0.0;
-        for (int w = 0; w < (int)blockDim.x / 32; ++w) q += part[w];
+        for (int i = 0; i < (int)blockDim.x / 32; ++i) q += part[i];
         const double v = nu[k];
         if (!(v >= 0.0) || !isfinite(v)) atomicOr(err, ERRBIT_NONFINITE);
         scale[k] = q > 0.0 ? v / sqrt(q) : 0.0;
@@ -804,7 +818,8 @@ cudaError_t launch_rb_basis(const double *bre, const double *bim, int Nb, int N,
 cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N, const double *nu,
                       bool fp64, const double *bre, const double *bim, const double2 *gt64,
                       const float2 *gt32, const int *bexp, const unsigned char *bpack, double *scale,
-                      int *aexp, unsigned char *apack, double *ore, double *oim, unsigned *err,
+                      int *aexp, unsigned char *apack, const int *bexp64, const unsigned char *bpack64,
+                      double *ore, double *oim, unsigned *err,
                       int sm_count, cudaStream_t st, cudaStream_t side, cudaEvent_t fork_ev,
                       cudaEvent_t join_ev)
 {
@@ -844,7 +859,8 @@ cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         sc = scale;
     } else if (nu && fp64) {
-        k_rb_scale64<<<M, (Nb + 31) / 32 * 32, 0, ss>>>(are, aim, Nb, gt64, nu, scale, err);
+        const int groups = (Nb + 31) / 32;
+        k_rb_scale64<<<M, 32 * groups * kScaleSets, 0, ss>>>(are, aim, Nb, groups, gt64, nu, scale, err);
         sc = scale;
     } else if (nu) {
         double *q = scale + M;  // the caller's scratch holds scale [M] then q [M]
@@ -858,6 +874,23 @@ cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N
         sc = scale;
     }
     if (fork && (e = cudaEventRecord(join_ev, side)) != cudaSuccess) return fail(e);
+    if (fp64 && bpack64) {  // (the plain chain: a context without room for the digits)
+        Rb64Args a{};
+        a.bpack = bpack64;
+        a.bexp = bexp64;
+        a.are = are;
+        a.aim = aim;
+        a.bre = bre;
+        a.bim = bim;
+        a.out_re = ore;
+        a.out_im = oim;
+        a.M = M;
+        a.N = N;
+        a.Nb = Nb;
+        a.err = err;
+        a.scale = sc;
+        return launch_rb64(a, apack, aexp, sc != nullptr, st);
+    }
     if (fp64) {
         const unsigned grid = (unsigned)((N + kRb64Threads - 1) / kRb64Threads) *
                               (unsigned)((M + kRb64Max - 1) / kRb64Max);

@@ -201,3 +201,44 @@ def test_rb_mixed_store_edges(gpu_ctx, M, N, Nb, shift):
             assert torch.all(o[:2 + shift] == 7.0) and torch.all(o[2 + shift + M * N:] == 7.0)
     finally:
         F.few_basis_release(gpu_ctx.handle, h)
+
+
+@pytest.mark.parametrize("M,Nb,N,kind", [
+    (1, 102, 43200, "plain"), (64, 102, 640, "plain"), (65, 103, 641, "plain"), (130, 192, 321, "plain"),
+    (200, 256, 130, "plain"), (300, 9, 1600, "plain"), (70, 60, 1025, "ranges"), (70, 60, 1025, "special"),
+    (1, 1, 1, "plain"), (127, 13, 64, "plain")])
+def test_rb_fp64_digit_slices(gpu_ctx, M, Nb, N, kind):
+    """Tiles and parts of the digit-slice product, element by element; rows and columns whose entries span
+    30 decades or are not finite or far from one go to the plain chain.  Bound: both operands to 2^-62 of
+    their largest entry with sums of magnitudes above 2^-7 of the two, or FP64's own (2 Nb roundings):
+    below 1e-13 of the sum of magnitudes."""
+    import torch
+    rng = np.random.default_rng(M + Nb + N)
+    alpha = rng.standard_normal((M, Nb)) + 1j * rng.standard_normal((M, Nb))
+    basis = rng.standard_normal((Nb, N)) + 1j * rng.standard_normal((Nb, N))
+    if kind == "ranges":
+        alpha *= 10.0 ** rng.uniform(-30, 0, (M, Nb))
+        basis *= 10.0 ** rng.uniform(-30, 0, (Nb, N))
+        alpha[3], basis[:, 5] = 0.0, 0.0
+        alpha[4] *= 1e130
+        basis[:, 7] *= 1e-130
+    if kind == "special":
+        alpha[2, 1], alpha[9, 0], basis[4, 3], basis[0, 70] = np.nan, np.inf, np.inf, np.nan
+    h = F.few_basis_create(gpu_ctx.handle, basis.real, basis.imag, RT.current_stream())
+    try:
+        out = [torch.full((M * N + 2,), 7.0, dtype=torch.float64, device="cuda") for _ in range(2)]
+        re, im = (o[1:-1].view(M, N) for o in out)
+        F.few_rb_amplitudes(gpu_ctx.handle, h, _dev(alpha.real), _dev(alpha.imag), re, im, None, F.FEW_FP64,
+                            RT.current_stream())
+        torch.cuda.synchronize()
+        assert gpu_ctx.sync_status() == F.FEW_OK
+        g = to_host(re) + 1j * to_host(im)
+        assert all(float(o[0]) == float(o[-1]) == 7.0 for o in out)
+    finally:
+        F.few_basis_release(gpu_ctx.handle, h)
+    with np.errstate(all="ignore"):
+        ref = alpha.real @ basis.real - alpha.imag @ basis.imag + 1j * (alpha.real @ basis.imag + alpha.imag @ basis.real)
+        bound = 1e-13 * (np.abs(alpha) @ np.abs(basis))
+    bad = ~np.isfinite(alpha).all(axis=1)[:, None] | ~np.isfinite(basis).all(axis=0)[None, :]
+    assert np.all(np.abs(g - ref)[~bad] <= bound[~bad])
+    assert not np.isfinite(g[bad]).any()
