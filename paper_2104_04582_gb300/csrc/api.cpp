@@ -293,8 +293,9 @@ few_status plan_slots(const int *l, const int *m, const int *n, int N, SlotPlan 
     }
     const int n_lo = *std::min_element(R.lo.begin(), R.lo.end());
     const int n_hi = *std::max_element(R.hi.begin(), R.hi.end());
-    P.n_mid = n_lo + (n_hi - n_lo) / 2;
-    const int half = n_hi - P.n_mid;
+    // (the fold mirrors row m into row -m about n = 0: any other centre is for m = 0 alone)
+    P.n_mid = R.m_top > 0 ? 0 : n_lo + (n_hi - n_lo) / 2;
+    const int half = std::max(n_hi - P.n_mid, P.n_mid - n_lo);
     P.m_top = R.m_top;
     if (R.m_top < kTcMaxPairs && half <= kTcMaxHalf) {
         P.tc_pairs = R.m_top + 1;

@@ -35,6 +35,8 @@ SETS = {
     "n_range_63": _modes([0, 1], range(-31, 32)),          # the whole basis
     "n_range_64": _modes([0], range(-32, 32)),             # an even range: half-width 32, scalar
     "n_shifted": _modes([0], range(40, 90)),               # m = 0 only: a centre far from zero
+    "m0_wider_one_way": np.concatenate([_modes([0], range(-23, 23)), _modes([2], range(-5, 7))]),
+    "m0_one_sided": np.concatenate([_modes([0], range(-31, -9)), _modes([1, 4], range(-3, 4))]),
     "rows_21": _modes(range(11), [-2, 0, 5], l=10),
     "rows_22_empty": _modes([0, 10], [-30, 30], l=10),     # empty rows in between
     "rows_23": _modes(range(12), [0, 1], l=11),            # too many rows: scalar
