@@ -4,8 +4,8 @@
 Headline workload (the configuration the metric is quoted on): one 1-yr waveform at dt = 10 s
 (3,155,760 samples), K = 100 knots, the full 3843-mode Schwarzschild grid (l = 2..10,
 m = 0..l, n = -30..30), synthetic seeded inputs.  A step is one pass of the whole hot path
-with the knot data resident in HBM: spline build (all 7688 splines), harmonics, fold, phase
-anchors and the per-sample mode sum, written to a device buffer.
+with the knot data resident in HBM: spline build (all 7688 splines), fold (with the harmonics and
+the tile records) and the per-sample mode sum, written to a device buffer.
 
 Default arm (--impl gb300): the mixed-precision path; beside it, on the same GPU and in the same
 JSON line: the plain FP64 path on the same waveform, the end-to-end call with host buffers, the
@@ -45,11 +45,9 @@ WORKLOAD = ("1-yr waveform, dt=10 s (3,155,760 samples), K=100 knots, 3843 modes
             "(l=2..10, m=0..l, n=-30..30), m<0 by symmetry")
 # DRAM bytes (read + write) of one summation launch on this workload, from the ncu capture
 # summarised in profiles/k_sum_mixed_1yr_3843modes.md; used only while the kernel source is the
-# one that was profiled (hash of the code of sum.cu + phase_eval.cuh + async.cuh, comments
-# left out) and the launch shape (R, threads) is the profiled one.  The stage size is left out: it changes how the L2-resident slot
-# tables are staged, not which bytes come from DRAM (the tables and anchors once, the output
-# still in L2 when the launch ends).
-PROFILED_TRAFFIC = {"source_sha256_16": "c81bdd4aa4270df9", "tile": (8, 256), "bytes": 13583360 + 0}
+# one that was profiled (hash of the code of tcsum.cu + tctile.cuh + fold_tc.cuh + tcgen05.cuh +
+# async.cuh, comments left out).
+PROFILED_TRAFFIC = {"source_sha256_16": "031caa8b50580095", "bytes": 7667712 + 0}
 FP32_LANES_PER_SM = 128   # FP32 FMA lanes per SM (4 sub-partitions x 32)
 FP64_FMA_PER_SM_CLK = 2   # FP64 FMA per SM per clock on GB300 (1.25 TFLOP/s at 152 SMs, 2.07 GHz)
 
@@ -92,7 +90,8 @@ def _code_hash(paths) -> str:
 def _kernel_source_hash() -> str:
     """Code hash of the summation kernel's sources (the key of a profiled traffic figure)."""
     d = os.path.join(ROOT, "paper_2104_04582_gb300", "csrc")
-    return _code_hash([os.path.join(d, f) for f in ("sum.cu", "phase_eval.cuh", "async.cuh")])
+    return _code_hash([os.path.join(d, f) for f in ("tcsum.cu", "tctile.cuh", "fold_tc.cuh",
+                                               "tcgen05.cuh", "async.cuh")])
 
 
 def _peaks_file():
@@ -285,8 +284,11 @@ def bench_rb(ctx, M, N, stream, sh):
     gbs = nbytes / (ms * 1e-3) / 1e9
     alg_flops = 8.0 * M * Nb * N  # complex product: 4 real multiply-adds per term
     n_kb = -(-(6 * Nb) // 64)  # three split products of depth 2 Nb
-    # transposed tiles: 256 knots x 128 output columns (64 modes, real and imaginary)
-    exec_flops = 2.0 * (-(-M // 256) * 256) * (-(-N // 64) * 128) * (n_kb * 64)
+    # transposed tiles: 256 knots x 128 output columns (two groups of 32 modes, real and imaginary; the
+    # groups start 28 modes apart where N is not a multiple of four)
+    step = 28 if N % 4 else 32
+    groups = 1 if N <= 32 else -(-(N - 32 + step) // step)
+    exec_flops = 2.0 * (-(-M // 256) * 256) * ((groups + 1) // 2 * 128) * (n_kb * 64)
     return {"knots": M, "basis": Nb, "modes": N, "prec": "mixed (split fp16 on tcgen05)",
             "ms": ms, "amplitudes_per_s": M * N / (ms * 1e-3),
             "roofline": {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s",
@@ -390,8 +392,8 @@ def _in_flight(ctx, sets, streams, steps):
 
 
 def bench_step_c2(args, ctx, w, dev, stream, sh, flush, prec, rank, world, tune_cache):
-    """The headline step on the one-year workload: spline build + harmonics + fold + anchors +
-    mode sum, knot data resident in HBM, timed with `args.in_flight` waveforms in flight (also
+    """The headline step on the one-year workload: spline build + fold (with harmonics
+    and tile records) + mode sum, knot data resident in HBM, timed with `args.in_flight` waveforms in flight (also
     timed one at a time, L2 flushed before each).  Returns the timed steps and kernel figures."""
     import torch
     from paper_2104_04582_gb300 import fewsum as F
@@ -471,7 +473,7 @@ def bench_step_c2(args, ctx, w, dev, stream, sh, flush, prec, rank, world, tune_
                tile=tuple(tile), tile_tuned_now=tuned_now,
                kernel_ms={"build": statistics.median(k[0] for k in kt),
                           "harmonics": statistics.median(k[1] for k in kt),
-                          "fold_and_anchors": statistics.median(k[2] for k in kt),
+                          "fold_and_records": statistics.median(k[2] for k in kt),
                           "sum": statistics.median(k[3] for k in kt)},
                sum_ms=[float(k[3]) for k in kt if k[3] > 0])
     del out
@@ -600,7 +602,7 @@ C2_MODE_SAMPLES = 3843 * 3155760
 def bench_batched_c3(ctx, dev, stream, sh, flush, n_waves, reps, tune_cache, oracle_windows=4,
                      in_flight=1):
     """256 waveforms of 0.25-2 yr, K 50-150, power-selected 10-3843 modes, mixed precision:
-    spline rebuild of every trajectory + harmonics + fold + anchors + one persistent summation
+    spline rebuild of every trajectory + fold + one persistent summation
     launch, captured once as a CUDA graph and replayed; tile chosen by the autotuner on a
     16-waveform sub-batch."""
     import torch
@@ -700,8 +702,8 @@ def bench_batched_c3(ctx, dev, stream, sh, flush, n_waves, reps, tune_cache, ora
            "modes_min_median_max": [int(min(x.N for x in ws)), int(statistics.median(x.N for x in ws)),
                                     int(max(x.N for x in ws))],
            "tile": list(tile), "tile_tuned_in_this_run": tuned_now,
-           "launches_per_step": 5, "graph": True, "precision": "mixed",
-           "step": "spline rebuild of all 256 trajectories + harmonics + fold + phase anchors + "
+           "launches_per_step": 3, "graph": True, "precision": "mixed",
+           "step": "spline rebuild of all 256 trajectories + fold (with harmonics and tile records) + "
                    "one persistent summation launch, replayed as one CUDA graph",
            "host_setup_s": setup_s, "plan_and_capture_s": plan_s, "accuracy": acc}
     if flight:
@@ -777,7 +779,7 @@ def bench_stress_c5(ctx, dev, stream, sh, reps, tune_cache, in_flight=1):
            "slot_samples_per_s": slots * w.n_samples / (m * 1e-3),
            "mismatch_vs_fp64_gpu_full_series": 1.0 - overlap, "tile": list(tile),
            "tile_tuned_in_this_run": tuned_now,
-           "step": "spline build + harmonics + fold + phase anchors + mode sum, complex64 output"}
+           "step": "spline build + fold (with harmonics and tile records) + mode sum, complex64 output"}
     if flight:
         res["in_flight"] = flight
     del a, out, out64
@@ -1014,39 +1016,28 @@ def assemble_line(args, res, ms, world):
     slots = res["slots"]
     dp = res.get("device_peaks") or {}
     kms = statistics.mean(res["sum_ms"]) if res["sum_ms"] else float("nan")
-    # algorithmic arithmetic of the summation kernel: one complex cubic (6 FMA) and one complex
-    # Horner step (4 FMA) per (harmonic slot, sample); an FMA is 2 flops
-    flops = 20.0 * slots * w.n_samples
+    # multiply-adds of the summation's tensor-core products: every sample by 16 ks basis values and 16
+    # columns per pair of rows (m, -m), three fp16 products (mixed) or 28 digit products (FP64)
+    pairs = int(w.modes[:, 1].max()) + 1
+    half = int(abs(w.modes[:, 2]).max())
+    flops = 2.0 * w.n_samples * (16 * pairs) * (16 * (half // 8 + 1)) * (3 if fp32 else 28)
     achieved = flops / (kms * 1e-3) / 1e12
     clocks = res["clocks"] or {}
-    peak = dp.get("fp32_tflops" if fp32 else "fp64_tflops", float("nan"))
+    peak = float(_peaks_file().get("bf16_tflops", 0.0)) or 1900.0
     traffic = None
     if (fp32 and PROFILED_TRAFFIC["bytes"] and
-            _kernel_source_hash() == PROFILED_TRAFFIC["source_sha256_16"] and
-            tuple(res.get("tile"))[:2] == PROFILED_TRAFFIC["tile"]):
+            _kernel_source_hash() == PROFILED_TRAFFIC["source_sha256_16"]):
         traffic = PROFILED_TRAFFIC["bytes"]
-    roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+    roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak, "traffic": traffic, "traffic_unit": "bytes per launch",
-            "kernel": "k_sum<float,R> (mixed)" if fp32 else "k_sum<double,R> (fp64)",
+            "kernel": "k_sum_tc<KS> (mixed)" if fp32 else "k_sum_tc64<KS> (fp64)",
             "kernel_ms": kms, "flops_per_launch": flops,
-            "peak_source": ("nominal FP32 FMA: " if fp32 else "nominal FP64 FMA: ") +
-                           dp.get("source", "") + " (ALU-bound kernel: neither HBM nor tensor peak applies)",
-            "tile": list(res["tile"]), "tile_tuned_in_this_run": res["tile_tuned_now"]}
-    probe = res["peaks"]
-    if probe:
-        key = "fp32_fma_per_s" if fp32 else "fp64_fma_per_s"
-        if key in probe:
-            pm = 2 * probe[key] / 1e12
-            roof["peak_probe_tflops"] = pm
-            roof["frac_of_probe"] = achieved / pm
-        if fp32 and "fp32_fma_3reg_per_s" in probe:
-            p3 = 2 * probe["fp32_fma_3reg_per_s"] / 1e12
-            roof["peak_register_operand_tflops"] = p3
-            roof["frac_of_register_operand_rate"] = achieved / p3
-        if fp32 and "fp32_fma_summation_block_per_s" in probe:
-            pb = 2 * probe["fp32_fma_summation_block_per_s"] / 1e12
-            roof["peak_summation_block_tflops"] = pb
-            roof["frac_of_summation_block_rate"] = achieved / pb
+            "peak_source": "measured cuBLAS bf16 rate of this GPU model (burst); the products are fp16 with "
+                           "FP32 accumulation, which runs at the same rate",
+            "scalar_chain_tflops": 20.0 * slots * w.n_samples / (kms * 1e-3) / 1e12,
+            "scalar_chain_note": "the work of one complex cubic and one complex multiply-add per harmonic "
+                                 "slot and sample, which the products replace, against %.1f TFLOP/s nominal"
+                                 % dp.get("fp32_tflops" if fp32 else "fp64_tflops", float("nan"))}
     if clocks.get("sm_mhz") and dp.get("sm_max_mhz"):
         roof["frac_at_measured_clock"] = achieved / (peak * clocks["sm_mhz"] / dp["sm_max_mhz"])
     value = aggregate_value(ms, world)
@@ -1054,16 +1045,17 @@ def assemble_line(args, res, ms, world):
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32" if fp32 else "f64",
-        "precision": ("mixed: FP64 phase splines and mod-2pi reduction (at anchors every 16 "
-                      "samples, FP32 in-group increments); FP32 amplitudes, exponential powers "
-                      "and accumulation") if fp32 else "fp64 throughout",
+        "precision": ("mixed: FP64 phase splines, phases in 64-bit fixed point (exact modulo one turn); "
+                      "FP32 amplitudes and exponential powers, multiplied as two fp16 parts each with "
+                      "FP32 accumulation") if fp32 else
+                     "fp64 (the contraction in exact 56-bit integer digits, 64-bit fixed point after it)",
         "data": "synthetic",
         "config": {"workload": WORKLOAD, "seed": W.SEEDS["C2"], "knots": w.K, "modes": w.N,
                    "samples": w.n_samples, "harmonic_slots": slots,
                    "l2": ("not flushed: the steps rotate over %d sets of knot data, spline data "
                           "and output (~300 MB, more than L2)" % IN_FLIGHT_SETS
                           if args.in_flight > 1 else "flushed (256 MB write) between timed steps"),
-                   "step": "spline build + harmonics + fold + phase anchors + mode sum, inputs "
+                   "step": "spline build + fold (with harmonics and tile records) + mode sum, inputs "
                            "resident in HBM",
                    "in_flight": ("%d waveforms in flight on %d streams (independent waveforms "
                                  "overlap: the next one's kernels fill SMs the previous "
@@ -1073,7 +1065,7 @@ def assemble_line(args, res, ms, world):
         "mode_samples_per_s": world * w.N * w.n_samples / (ms * 1e-3),
         "kernel_ms": res["kernel_ms"],
         "roofline": roof,
-        "gpu_launches": (5 if fp32 else 4) * args.steps,
+        "gpu_launches": (3 if fp32 else 4) * args.steps,
         "clocks": clocks or None,
         "e2e": res["e2e"],
     }

@@ -184,7 +184,9 @@ typedef struct few_request {
 
 /*
  * Compute one waveform (Sec. 3.C interpolated summation of the Sec. 4 sum).  Validates and
- * plans on the host, then queues the harmonic, fold and summation kernels on `stream`.
+ * plans on the host, then queues the fold (with the harmonics; FEW_FP64: a kernel before it) and the
+ * summation on `stream`.  Mode sets with m <= 10 and |n| <= 31 (m = 0 alone: any n range of 63) are
+ * summed on the tensor cores, others, and requests whose scratch fits only so, by a scalar chain.
  * n_samples == 0 is a no-op.  Errors: FEW_ERR_INVALID_ARG, FEW_ERR_STATE, FEW_ERR_RANGE,
  * FEW_ERR_LIMIT, FEW_ERR_BUDGET, FEW_ERR_NOMEM, FEW_ERR_CUDA.
  */
@@ -196,13 +198,14 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream);
  * real-time pipeline that reserves all device memory at start-up, or code under a policy that
  * forbids cudaMalloc (and the synchronisation it can imply) on the call path.  It computes
  * what few_waveform computes for the same request (either frame), but keeps its scratch (plan,
- * harmonic table, folded coefficients and, for FEW_MIXED, the phase anchors) in one fixed device
+ * folded coefficients or operand tables, phase anchors or tile records) in one fixed device
  * array of FEW_NOALLOC_SCRATCH_BYTES that is part of the library image (reserved on every GPU
  * that loads the library, until the process exits) and calls no allocator of any kind.
  *   req->out_where must be FEW_MEM_DEVICE; the trajectory and the output buffer are the
  *   caller's, as for few_waveform.
  * Limits: the request's scratch must fit in FEW_NOALLOC_SCRATCH_BYTES and K <= 4096; otherwise
- *   it returns FEW_ERR_LIMIT without queuing work.  The scratch is about 64 x slots x (K - 1)
+ *   it returns FEW_ERR_LIMIT without queuing work.  The limit is on the scalar chain's scratch (a
+ *   tensor-core plan is taken where it fits too), which is about 64 x slots x (K - 1)
  *   bytes for FEW_FP64; for FEW_MIXED 32 x slots x (K - 1) bytes plus 3 bytes per output sample
  *   (the phase anchors), plus a few KB.  The one-year 3843-mode waveform (K = 100,
  *   3,155,760 samples) fits in both precisions; the four-year one at dt = 2 s does not.
@@ -290,11 +293,14 @@ few_status few_basis_release(few_ctx *ctx, few_basis *basis);
  *     must be finite and >= 0; others latch FEW_ERR_INVALID_ARG (see few_sync_status).
  *   amp_re_dev, amp_im_dev [M][N]: device memory, overwritten; the layout few_traj_set_data
  *     reads (FEW_MEM_DEVICE), so a trajectory's amplitudes can be produced in place.
- *   prec: FEW_FP64 (complex GEMM on the FP64 pipe) or FEW_MIXED (one real GEMM on the tensor
+ *   prec: FEW_FP64 (exact 62-bit digit products on the tensor cores, one rounding to FP64; outputs whose
+ *     sum of magnitudes is far below the product of the largest entries, or with entries that are not
+ *     finite or not within 2^+-400, by FP64 arithmetic) or FEW_MIXED (one real GEMM on the tensor
  *     cores: fp16 operands split two ways after exact power-of-two scaling of each knot's row and
  *     each mode's column, three partial products, FP32 accumulation; error near FP32 rounding of
  *     the row's and column's largest terms).
- * Asynchronous on `stream`; scratch (M x 16 bytes, plus about M x Nb x 12 bytes for FEW_MIXED)
+ * Asynchronous on `stream`; scratch (M x 16 bytes, plus about M x Nb x 12 bytes for FEW_MIXED and x 36
+ * for FEW_FP64, which without room for it runs on the FP64 pipe)
  * comes from the context's pool.  M = 0 is a no-op.
  */
 few_status few_rb_amplitudes(few_ctx *ctx, const few_basis *basis, const double *alpha_re_dev,
@@ -342,7 +348,8 @@ few_status few_sync_status(few_ctx *ctx);
 few_status few_selftest_wait_expiry(few_ctx *ctx, unsigned limit_us, void *stream);
 
 /*
- * Tile configuration of the summation kernel for one precision:
+ * Tile configuration of the scalar summation chain for one precision (the tensor-core summation has
+ * none):
  *   samples_per_thread (R, the sample tile: a pass covers threads x R consecutive samples):
  *     FEW_FP64: 1 or 2; FEW_MIXED: 2, 4 or 8;
  *   threads_per_block: 128 or 256;
@@ -362,7 +369,7 @@ few_status few_get_tiles(few_ctx *ctx, int prec, int *samples_per_thread, int *t
  * Per-kernel device timing.  With timing enabled, the library records a CUDA event pair on the
  * launch stream around each kernel it queues.  few_last_timing waits for the most recent pairs
  * and returns their durations in ms: ms[0] spline build (last few_traj_set_data), ms[1]
- * harmonics, ms[2] fold, ms[3] summation (last few_waveform or few_batch_run without a graph).
+ * harmonics (next to nothing where the fold forms them), ms[2] fold, ms[3] summation (last few_waveform or few_batch_run without a graph).
  * Entries never recorded are returned as -1.
  */
 few_status few_ctx_set_timing(few_ctx *ctx, int enable);

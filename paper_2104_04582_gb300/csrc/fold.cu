@@ -74,11 +74,10 @@ __global__ void __launch_bounds__(kYlmThreads) k_ylm(const PlanHdr *__restrict__
 
 // The plan in the parameters: the harmonics need nothing of an earlier kernel, only their store waits;
 // the last block copies the plan to the device for the kernels that follow.
-template <bool FP64>
 __global__ void __launch_bounds__(kYlmThreads) k_ylm_param(const __grid_constant__ PlanParam plan)
 {
     pdl_launch_dependents();
-    ylm_thread<FP64>(*reinterpret_cast<const PlanHdr *>(plan.bytes), true);
+    ylm_thread<true>(*reinterpret_cast<const PlanHdr *>(plan.bytes), true);
     tc_store_plan(plan);
 }
 
@@ -87,7 +86,7 @@ cudaError_t launch_ylm(const PlanHdr *hdr_dev, const PlanParam *plan, int total_
 {
     if (total_pairs <= 0) return cudaSuccess;
     const int threads = 2 * total_pairs, grid = (threads + kYlmThreads - 1) / kYlmThreads;
-    if (plan) return launch_pdl(fp64 ? k_ylm_param<true> : k_ylm_param<false>, grid, kYlmThreads, 0, st, *plan);
+    if (plan) return launch_pdl(k_ylm_param, grid, kYlmThreads, 0, st, *plan);
     return launch_pdl(fp64 ? k_ylm<true> : k_ylm<false>, grid, kYlmThreads, 0, st, hdr_dev);
 }
 

@@ -42,7 +42,7 @@ __device__ inline T jacobi_p(int n, int a, int b, T x)
 // FP64: the same recurrence and ratio without a division per step (a division is ~30 operations of
 // the narrow FP64 pipe, all on the critical path).  The recurrence is carried as p_k = q_k / s_k, s_k
 // the product of the divisors, and divided once; products stay below 1e170 for l <= 32.
-// One FP64 harmonic of l <= 10: ~40 us with a division per step, see k_ylm.
+// One FP64 harmonic of l <= 10: 36 us with a division per step (k_ylm, 3843 modes), 18 with one.
 __device__ inline double jacobi_p(int n, int a, int b, double x)
 {
     if (n == 0) return 1.0;

@@ -20,7 +20,7 @@
 // sample) are in units of 2^-64 turn, so that wrap-around arithmetic is the exact reduction modulo
 // one turn and z_r^8 and z_r^{n_mid} come from exact integer multiples of the
 // phases instead of powers of rounded exponentials.  Measured error against a 64-bit restatement
-// over the one-year 3843-mode waveform: see the table beside k_sum_tc.
+// over the one-year 3843-mode waveform: 1.7e-7 to 2.9e-7 over seeds (the scalar chain: 2.3e-6).
 //
 // Work decomposition: tiles of 128 samples (one per tensor-memory lane) that start at multiples of
 // 128 within a segment; a persistent CTA per SM takes a contiguous run of tiles.  Four warpgroups
@@ -237,6 +237,11 @@ __device__ __forceinline__ void load_table(const TileRec *__restrict__ recs, int
 // its basis in registers while the slot's other warpgroup waits for its MMAs, and stores it while
 // that one drains them.
 // KS: K steps of the plan's widest n range (a wave with fewer uses the first of them).
+// One year, 3843 modes: 104 us (the scalar chain 1,417), 1,154 cycles a tile = twelve N = 176 MMAs of 96,
+// the tensor cores 90 % active.  Sets of fewer rows run at 430 to 700 ns a tile whatever their size:
+// there the chain of a slot bounds it (issue ~900 cycles, the MMAs' tail ~440, loads to the release
+// of the accumulator ~500, wake-up ~350).  Six warpgroups of 80 registers: 133 us; factors before
+// the issue: 122; MMAs in tile order by a token: 114.
 template <int KS>
 __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restrict__ hp)
 {

@@ -21,6 +21,10 @@
 // columns) and two accumulator sets of one row pair (7 x 16 columns each): the MMAs of one pair run
 // while the previous pair's sums are formed.  Two warpgroups take the tiles in turn; one prepares its
 // exponentials while the other's MMAs run.
+// One year, 3843 modes: 1.89 ms (the scalar chain 66.6), ~22,000 cycles a tile: 13,000 of MMAs (tensor cores
+// 44 % active), the rest the forming of sums, ~1,700 a row pair by one warp a scheduler (issue 47 %).
+// Both warpgroups on every tile (half of the rows each): 2.03 ms.  Error against 64-bit phases 1.6e-13
+// to 2.4e-13 over seeds (the scalar chain 3.5e-13 to 4.0e-13).
 #include <cuda_fp16.h>
 
 #include "fewsum_internal.h"
