@@ -29,10 +29,9 @@
 
 namespace fewsum {
 
-constexpr int kFactorThreads = 32;  // one warp: per-knot loops strided, one thread per block
+constexpr int kFactorThreads = 128;
 
-// Partitioned factorisation of the reduced not-a-knot matrix of one knot grid (one warp; O(K)
-// work, each block's elimination on its own thread), rows k = 1..K-2 with diagonal dg(k), lower
+// Partitioned factorisation of the reduced not-a-knot matrix of one knot grid (O(K) work), rows k = 1..K-2 with diagonal dg(k), lower
 // coefficient sub(k) = h_k (k >= 2) and upper sup(k) = h_{k-1} (k <= K-3).  The rows are split into P blocks separated by single rows (the
 // separators): block b spans rows start_b .. start_b + size_b - 1, separator b + 1 is the row
 // after it.  With x_sigma the separators' unknowns, block b's rows solve
@@ -60,134 +59,187 @@ constexpr int kFactorThreads = 32;  // one warp: per-knot loops strided, one thr
 //     lo_{K-1} s_{K-2}
 // (the end rows divided by h_1 and hc).  K >= 4, so rows 1 and K-2 are distinct, and neither is
 // a separator.
+//
+// Bound by latency: an FP64 instruction of one warp holds its scheduler for 64 cycles and a division is
+// about ten of them, so what can be done side by side is: everything is kept in shared memory, per-knot
+// work takes four warps, a block's elimination two lanes, one of which divides the next multiplier
+// and the other 1 by the same pivot (then the responses v and w, a lane each), the separators'
+// likewise, and the end rows' quotients a lane each in another warp.  K = 100: 42 us as one warp on
+// global memory with a thread a block, 18 us so; the same operations on the same numbers.
 __global__ void __launch_bounds__(kFactorThreads) k_factor(const double *__restrict__ t, int K,
                                                              FactorArrays f)
 {
-    if (blockIdx.x != 0) return;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    double *h = f.h, *ip = f.ip, *fl = f.lo, *fu = f.up, *fv = f.v, *fx = f.x, *ra = f.ra,
-           *rb = f.rb;
-    const int S = K - 1, n = K - 2;
-    // knot widths and cleared arrays (every thread a stride of k)
-    for (int k = tid; k < S; k += nt) {
-        h[k] = t[k + 1] - t[k];
-        f.inv_h[k] = 1.0 / h[k];
-    }
-    for (int k = tid; k < K; k += nt) ip[k] = fl[k] = fu[k] = fv[k] = fx[k] = ra[k] = rb[k] = 0.0;
-    constexpr int NS = kBuildParts - 1;
-    for (int i = tid; i < NS * NS; i += nt) f.sinv[i] = 0.0;
-    __syncthreads();
-    auto dg = [&](int k) {
-        if (k == 1) return h[0] + h[1];
-        if (k == K - 2) return h[K - 3] + h[K - 2];
-        return 2.0 * (h[k - 1] + h[k]);
-    };
-    auto sub = [&](int k) { return k >= 2 ? h[k] : 0.0; };
-    auto sup = [&](int k) { return k <= K - 3 ? h[k - 1] : 0.0; };
-    for (int k = 2 + tid; k <= K - 3; k += nt) {
-        ra[k] = 3.0 * h[k] * f.inv_h[k - 1];
-        rb[k] = 3.0 * h[k - 1] * f.inv_h[k];
-    }
-    const double h0 = h[0], h1 = h[1], hc = h[K - 3], hd = h[K - 2];
-    if (tid == 0) {
-        ra[1] = h1 * h1 / (h0 * (h0 + h1));
-        rb[1] = h0 * (2.0 * h0 + 3.0 * h1) / (h1 * (h0 + h1));
-        ra[K - 2] = hd * (3.0 * hc + 2.0 * hd) / (hc * (hc + hd));
-        rb[K - 2] = hc * hc / (hd * (hc + hd));
-    }
+    extern __shared__ double fac[];
+    double *h = fac, *ih = fac + K, *dg = fac + 2 * K, *ip = fac + 3 * K, *fl = fac + 4 * K, *fv = fac + 5 * K;
+    double *fx = ih;  // (1/h is not needed once ra and rb are formed)
+    __shared__ double s_ends[10];
+    const int tid = threadIdx.x, lane = tid & 31, S = K - 1, n = K - 2;
+    for (int k = tid; k < S; k += kFactorThreads) h[k] = t[k + 1] - t[k];
     // the partition (every thread derives the same)
     int P = (n + 1) / 2;
     if (P > kBuildParts) P = kBuildParts;
     if (P < 1) P = 1;
     const int nb = n - (P - 1), base = nb / P, extra = nb % P;
-    int start[kBuildParts + 1];
-    int k = 1;
-    for (int b = 0; b < P; ++b) {
-        start[b] = k;
-        k += base + (b < extra ? 1 : 0) + 1;  // block rows, then its right separator
-    }
-    start[P] = K - 1;
+    auto start = [&](int b) { return b == P ? K - 1 : 1 + b * (base + 1) + min(b, extra); };
     if (tid == 0) {
         f.parts[0] = P;
-        for (int b = 0; b <= P; ++b) f.parts[1 + b] = start[b];
+        for (int b = 0; b <= P; ++b) f.parts[1 + b] = start(b);
     }
     __syncthreads();
-    // each block's elimination, responses and scaled rows: independent, one thread per block
-    for (int b = tid; b < P; b += nt) {
-        const int a = start[b], e = (b + 1 < P ? start[b + 1] - 1 : K - 1) - 1;
-        double p = dg(a);
-        ip[a] = 1.0 / p;
-        for (int r = a + 1; r <= e; ++r) {  // fl holds the Thomas multipliers for now
-            const double m = sub(r) / p;
-            p = dg(r) - m * sup(r - 1);
-            fl[r] = m;
-            ip[r] = 1.0 / p;
+    auto sub = [&](int k) { return k >= 2 ? h[k] : 0.0; };
+    auto sup = [&](int k) { return k <= K - 3 ? h[k - 1] : 0.0; };
+    for (int k = tid; k < K; k += kFactorThreads) {
+        if (k < S) {
+            f.h[k] = h[k];
+            f.inv_h[k] = ih[k] = 1.0 / h[k];
         }
-        if (b > 0) {  // v_b = A_b^-1 sub(a) e_first
-            fv[a] = sub(a);
-            for (int r = a + 1; r <= e; ++r) fv[r] = -fl[r] * fv[r - 1];
-            fv[e] *= ip[e];
-            for (int r = e - 1; r >= a; --r) fv[r] = (fv[r] - sup(r) * fv[r + 1]) * ip[r];
-        }
-        if (b + 1 < P) {  // w_b = A_b^-1 sup(e) e_last
-            fx[e] = sup(e) * ip[e];
-            for (int r = e - 1; r >= a; --r) fx[r] = -sup(r) * fx[r + 1] * ip[r];
-        }
-        for (int r = a; r <= e; ++r) {  // the pivot-scaled rows
-            fl[r] = r > a ? sub(r) * ip[r] : 0.0;
-            fu[r] = sup(r) * ip[r];
-            ra[r] *= ip[r];
-            rb[r] *= ip[r];
-        }
+        dg[k] = k == 0 || k == K - 1 ? 0.0
+                : k == 1             ? h[0] + h[1]
+                : k == K - 2         ? h[K - 3] + h[K - 2]
+                                     : 2.0 * (h[k - 1] + h[k]);
+        ip[k] = fl[k] = fv[k] = 0.0;
     }
     __syncthreads();
-    // the separator system's elimination (sequential, P - 1 <= 7 rows) and the end slopes
-    if (tid == 0) {
-        double piv = 0.0, cup_prev = 0.0;
-        for (int i = 1; i < P; ++i) {
-            const int sg = start[i] - 1, L = sg - 1, F = sg + 1;
-            const double D = dg(sg) - sub(sg) * fx[L] - sup(sg) * fv[F];
-            const double clo = -sub(sg) * fv[L], cup = -sup(sg) * fx[F];
-            double mu = 0.0;
-            if (i == 1) {
-                piv = D;
-            } else {
-                mu = clo / piv;
-                piv = D - mu * cup_prev;
+    // the end rows' quotients
+    if (tid >= 32 && lane < 10) {
+        const double h0 = h[0], h1 = h[1], hc = h[K - 3], hd = h[K - 2];
+        double num, den;
+        switch (lane) {
+        case 0: num = h1 * h1, den = h0 * (h0 + h1); break;                             // ra_1
+        case 1: num = h0 * (2.0 * h0 + 3.0 * h1), den = h1 * (h0 + h1); break;          // rb_1
+        case 2: num = hd * (3.0 * hc + 2.0 * hd), den = hc * (hc + hd); break;          // ra_{K-2}
+        case 3: num = hc * hc, den = hd * (hc + hd); break;                             // rb_{K-2}
+        case 4: num = 2.0 * h1 + 3.0 * h0, den = h0 * (h0 + h1); break;                 // ra_0
+        case 5: num = h0 * h0, den = h1 * h1 * (h0 + h1); break;                        // rb_0
+        case 6: num = h0 + h1, den = h1; break;                                         // lo_0
+        case 7: num = hd * hd, den = hc * hc * (hc + hd); break;                        // ra_{K-1}
+        case 8: num = 2.0 * hc + 3.0 * hd, den = hd * (hc + hd); break;                 // rb_{K-1}
+        default: num = hc + hd, den = hc; break;                                        // lo_{K-1}
+        }
+        if (tid < 64) s_ends[lane] = num / den;
+    }
+    // ra, rb of the inner rows (divided by the pivots at the end)
+    for (int k = 2 + tid; k <= K - 3; k += kFactorThreads) {
+        f.ra[k] = 3.0 * h[k] * ih[k - 1];
+        f.rb[k] = 3.0 * h[k - 1] * ih[k];
+    }
+    __syncthreads();
+    for (int k = tid; k < K; k += kFactorThreads) fx[k] = 0.0;  // (was 1/h)
+    __syncthreads();
+    if (tid < 32) {
+        // each block's elimination and responses: lanes 2 b and 2 b + 1
+        const int b = min(lane >> 1, P - 1), a = start(b), e = (b + 1 < P ? start(b + 1) - 1 : K - 1) - 1;
+        const bool mine = lane < 2 * P, first = (lane & 1) == 0;
+        const int most = base + (extra ? 1 : 0);
+        double p = dg[a], v = b > 0 ? sub(a) : 0.0;
+        if (mine && first) fv[a] = v;
+        for (int i = 1; i <= most; ++i) {
+            const int r = min(a + i, e);
+            const bool row = a + i <= e, last = a + i == e + 1;
+            const double q = (first ? sub(r) : 1.0) / p;  // the multiplier of row r; the last pivot's inverse
+            const double m = __shfl_sync(0xffffffffu, q, lane & ~1);
+            if (mine && !first && (row || last)) ip[a + i - 1] = q;
+            if (row) {
+                p = dg[r] - m * sup(r - 1);
+                v = -m * v;
+                if (mine && first) {
+                    fl[r] = m;
+                    fv[r] = v;
+                }
             }
-            fv[sg] = mu;
-            ip[sg] = 1.0 / piv;
-            fx[sg] = cup;
-            cup_prev = cup;
         }
-        ra[0] = (2.0 * h1 + 3.0 * h0) / (h0 * (h0 + h1));
-        rb[0] = h0 * h0 / (h1 * h1 * (h0 + h1));
-        fl[0] = (h0 + h1) / h1;
-        ra[K - 1] = hd * hd / (hc * hc * (hc + hd));
-        rb[K - 1] = (2.0 * hc + 3.0 * hd) / (hd * (hc + hd));
-        fl[K - 1] = (hc + hd) / hc;
+        __syncwarp();
+        double x = first ? fv[e] : b + 1 < P ? sup(e) : 0.0;
+        x *= ip[e];
+        double *resp = first ? fv : fx;
+        __syncwarp();
+        if (mine) resp[e] = x;
+        for (int i = 1; i < most; ++i) {
+            const int r = e - i;
+            if (r >= a) {
+                x = fma(-sup(r), x, first ? fv[r] : 0.0) * ip[r];
+                if (mine) resp[r] = x;
+            }
+        }
+        __syncwarp();
+        // the separator system's elimination (at most 7 rows): row i = lane + 1 formed side by side
+        const int sg = lane + 1 < P ? start(lane + 1) - 1 : 1;
+        double D = 0.0, clo = 0.0, cup = 0.0;
+        if (lane + 1 < P) {
+            D = dg[sg] - sub(sg) * fx[sg - 1] - sup(sg) * fv[sg + 1];
+            clo = -sub(sg) * fv[sg - 1];
+            cup = -sup(sg) * fx[sg + 1];
+        }
+        double piv = __shfl_sync(0xffffffffu, D, 0), cup_prev = __shfl_sync(0xffffffffu, cup, 0);
+        double mu_own = 0.0, inv_own = 0.0;
+        for (int i = 1; i < P; ++i) {  // row i's inverse pivot and row i + 1's multiplier
+            const double cn = __shfl_sync(0xffffffffu, clo, i), Dn = __shfl_sync(0xffffffffu, D, i);
+            const double q = (first ? cn : 1.0) / piv;
+            const double mu = __shfl_sync(0xffffffffu, q, 0), inv = __shfl_sync(0xffffffffu, q, 1);
+            if (lane == i - 1) inv_own = inv;
+            if (lane == i) mu_own = mu;
+            piv = Dn - mu * cup_prev;
+            cup_prev = __shfl_sync(0xffffffffu, cup, i);
+        }
+        if (lane + 1 < P) {
+            fv[sg] = mu_own;
+            ip[sg] = inv_own;
+            fx[sg] = cup;
+        }
+        __syncwarp();
+        // the separator system's inverse, column m from the unit right-hand side e_m (one lane per
+        // column; entries past P - 1 are zero): every lane of a spline then forms its right
+        // separator's slope as one short dot product instead of a chain of 3 (P - 1) dependent
+        // operations
+        constexpr int NS = kBuildParts - 1;
+        const int m = lane + 1;
+        if (m <= NS) {
+            double gp[kBuildParts], X = 0.0;
+#pragma unroll
+            for (int i = 1; i <= NS; ++i) {
+                if (i >= P) break;
+                const double gi = i == m ? 1.0 : 0.0;
+                gp[i] = i == 1 ? gi : gi - fv[start(i) - 1] * gp[i - 1];
+            }
+#pragma unroll
+            for (int i = NS; i >= 1; --i) {
+                double out = 0.0;
+                if (i < P && m < P) {
+                    X = (gp[i] - fx[start(i) - 1] * X) * ip[start(i) - 1];
+                    out = X;
+                }
+                f.sinv[(i - 1) * NS + (m - 1)] = out;
+            }
+        }
     }
     __syncthreads();
-    // the separator system's inverse, column m from the unit right-hand side e_m (one thread per
-    // column; entries past P - 1 stay zero): every lane of a spline then forms its right
-    // separator's slope as one short dot product instead of a chain of 3 (P - 1) dependent
-    // operations
-    for (int m = 1 + tid; m < P; m += nt) {
-        double gp[kBuildParts], X[kBuildParts + 1];
-        for (int i = 1; i < P; ++i) {
-            const double gi = i == m ? 1.0 : 0.0;
-            gp[i] = i == 1 ? gi : gi - fv[start[i] - 1] * gp[i - 1];
+    // the pivot-scaled rows, and everything to the trajectory's arrays
+    for (int k = tid; k < K; k += kFactorThreads) {
+        bool sep = false, head = false;
+        for (int b = 0; b < P; ++b) {
+            sep |= b > 0 && k == start(b) - 1;
+            head |= k == start(b);
         }
-        X[P] = 0.0;
-        for (int i = P - 1; i >= 1; --i)
-            X[i] = (gp[i] - fx[start[i] - 1] * X[i + 1]) * ip[start[i] - 1];
-        for (int i = 1; i < P; ++i) f.sinv[(i - 1) * NS + (m - 1)] = X[i];
+        const bool end = k == 0 || k == K - 1, row = !end && !sep;
+        const double q = ip[k];
+        double ra = end ? s_ends[k == 0 ? 4 : 7] : k == 1 ? s_ends[0] : k == K - 2 ? s_ends[2] : f.ra[k];
+        double rb = end ? s_ends[k == 0 ? 5 : 8] : k == 1 ? s_ends[1] : k == K - 2 ? s_ends[3] : f.rb[k];
+        f.ra[k] = row ? ra * q : ra;
+        f.rb[k] = row ? rb * q : rb;
+        f.lo[k] = end ? s_ends[k == 0 ? 6 : 9] : row && !head ? sub(k) * q : 0.0;
+        f.up[k] = row ? sup(k) * q : 0.0;
+        f.ip[k] = q;
+        f.v[k] = fv[k];
+        f.x[k] = fx[k];
     }
 }
 
 cudaError_t launch_factor(const double *t, int K, const FactorArrays &f, cudaStream_t st)
 {
-    k_factor<<<1, kFactorThreads, 0, st>>>(t, K, f);
+    const cudaError_t e = cudaFuncSetAttribute(k_factor, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               6 * FEW_MAX_KNOTS * (int)sizeof(double));
+    if (e != cudaSuccess) return e;
+    k_factor<<<1, kFactorThreads, 6 * K * (int)sizeof(double), st>>>(t, K, f);
     return cudaGetLastError();
 }
 
