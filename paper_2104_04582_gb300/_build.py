@@ -26,7 +26,7 @@ CFLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler",
 SOURCES = ["api.cpp", "spline.cu", "fold.cu", "sum.cu", "tcsum.cu", "tcsum64.cu", "anchor.cu", "selftest.cu", "noalloc.cu",
            "select.cu", "direct.cu", "rb.cu", "rb64.cu"]
 HEADERS = ["fewsum_internal.h", "phase_eval.cuh", "harmonics.cuh", "convert.cuh", "async.cuh",
-           "tcgen05.cuh", "tctile.cuh", "fold_tc.cuh", "launch.cuh"]
+           "tcgen05.cuh", "tctile.cuh", "fold_tc.cuh", "launch.cuh", "rb_scale.cuh"]
 
 
 def nvcc() -> str:

@@ -1351,7 +1351,8 @@ few_status few_basis_create(few_ctx *ctx, const double *b_re, const double *b_im
     unsigned char *bpack = p + 2 * b_bytes + g64 + g32 + ex;
     int *bexp64 = reinterpret_cast<int *>(p + plain);
     unsigned char *bpack64 = p + plain + ex64;
-    if (!st && (launch_rb_basis(bre, bim, Nb, N, gt64, gt32, bexp, bpack, ctx->sm_count, s) != cudaSuccess ||
+    if (!st && (launch_rb_exponents(bre, bim, Nb, N, L.modes_padded, bexp, digits ? bexp64 : nullptr, s) != cudaSuccess ||
+                launch_rb_basis(bre, bim, Nb, N, gt64, gt32, bexp, bpack, ctx->sm_count, s) != cudaSuccess ||
                 (digits &&
                  launch_rb64_basis(bre, bim, Nb, N, bexp64, bpack64, ctx->sm_count, s) != cudaSuccess))) {
         (void)cudaGetLastError();

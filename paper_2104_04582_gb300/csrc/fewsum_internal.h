@@ -316,12 +316,15 @@ size_t rb64_coef_bytes(int Nb, int M);
 int rb64_rows(int M);    // padded counts
 int rb64_modes(int N);
 cudaError_t rb64_configure();
-cudaError_t launch_rb64_basis(const double *bre, const double *bim, int Nb, int N, int *bexp, unsigned char *pack,
+// The basis columns' scaling exponents of both products (bexp64 null: of the mixed one).
+cudaError_t launch_rb_exponents(const double *bre, const double *bim, int Nb, int N, int n_exp, int *bexp, int *bexp64,
+                                cudaStream_t st);
+cudaError_t launch_rb64_basis(const double *bre, const double *bim, int Nb, int N, const int *bexp, unsigned char *pack,
                               int sm_count, cudaStream_t st);
 // after_scale: the kernel launched before it on `st` forms the scale.
 cudaError_t launch_rb64(Rb64Args a, unsigned char *apack, int *aexp, bool after_scale, cudaStream_t st);
 cudaError_t launch_rb_basis(const double *bre, const double *bim, int Nb, int N, double2 *gt64,
-                            float2 *gt32, int *bexp, unsigned char *bpack, int sm_count, cudaStream_t st);
+                            float2 *gt32, const int *bexp, unsigned char *bpack, int sm_count, cudaStream_t st);
 cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N, const double *nu,
                       bool fp64, const double *bre, const double *bim, const double2 *gt64,
                       const float2 *gt32, const int *bexp, const unsigned char *bpack, double *scale,

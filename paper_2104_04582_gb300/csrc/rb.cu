@@ -45,6 +45,7 @@
 #include "convert.cuh"
 #include "fewsum_internal.h"
 #include "launch.cuh"
+#include "rb_scale.cuh"
 #include "tcgen05.cuh"
 
 namespace fewsum {
@@ -63,8 +64,6 @@ constexpr uint32_t kRbStageBytes = kRbABytes + kRbBBytes;
 // table, so lanes at different segments need no divergent constant-memory reads.
 __host__ __device__ constexpr int part_a(int g) { return g == 2 ? 1 : 0; }
 __host__ __device__ constexpr int part_b(int g) { return g == 1 ? 1 : 0; }
-constexpr int kRbMaxExp = 100;  // bound on the power-of-two scaling exponents
-
 __host__ __device__ constexpr uint32_t core_offset(int r, int c)
 {
     return (uint32_t)(r >> 3) * 1024u + (uint32_t)(c >> 3) * 128u + (uint32_t)(r & 7) * 16u +
@@ -85,14 +84,6 @@ __device__ __forceinline__ uint32_t pack2(__half a, __half b)
 
 // 2^e as a float, |e| <= kRbMaxExp.
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
-
-// Exponent e with m 2^e in [2^14, 2^15) for m > 0 (0 for m = 0), clamped to +-kRbMaxExp.
-__device__ __forceinline__ int scale_exp(float m)
-{
-    if (!(m > 0.0f)) return 0;
-    const int e = 14 - (int)((__float_as_uint(m) >> 23) & 0xffu) + 127;
-    return e > kRbMaxExp ? kRbMaxExp : (e < -kRbMaxExp ? -kRbMaxExp : e);
-}
 
 // ---- basis set-up -------------------------------------------------------------------------
 
@@ -123,20 +114,6 @@ __global__ void k_rb_gram(const double *__restrict__ bre, const double *__restri
         gt64[(size_t)l * Nb + j] = make_double2(tr, ti);
         gt32[(size_t)l * Nb + j] = make_float2((float)tr, (float)ti);
     }
-}
-
-// Scaling exponent of each mode's basis column: bexp[i] puts max_j max(|Re B_ji|, |Im B_ji|)
-// into [2^14, 2^15); padded modes get 0.
-__global__ void k_rb_bexp(const double *__restrict__ bre, const double *__restrict__ bim, int Nb,
-                          int N, int n_modes_padded, int *__restrict__ bexp)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_modes_padded) return;
-    double m = 0.0;
-    if (i < N)
-        for (int j = 0; j < Nb; ++j)
-            m = fmax(m, fmax(fabs(bre[(size_t)j * N + i]), fabs(bim[(size_t)j * N + i])));
-    bexp[i] = scale_exp((float)m);
 }
 
 // Basis operand (the MMA's A side), scaled, split and packed: row r of basis tile b is the real
@@ -806,11 +783,10 @@ RbLayout rb_layout(int Nb, int N, int M)
 }
 
 cudaError_t launch_rb_basis(const double *bre, const double *bim, int Nb, int N, double2 *gt64,
-                            float2 *gt32, int *bexp, unsigned char *bpack, int sm_count, cudaStream_t st)
+                            float2 *gt32, const int *bexp, unsigned char *bpack, int sm_count, cudaStream_t st)
 {
     const RbLayout L = rb_layout(Nb, N, 0);
     k_rb_gram<<<Nb * Nb, 128, 0, st>>>(bre, bim, Nb, N, gt64, gt32);
-    k_rb_bexp<<<(L.modes_padded + 127) / 128, 128, 0, st>>>(bre, bim, Nb, N, L.modes_padded, bexp);
     k_rb_pack_b<<<sm_count * 8, 256, 0, st>>>(bre, bim, Nb, N, L.n_kb, L.n_tiles, L.step, bexp, bpack);
     return cudaGetLastError();
 }

@@ -25,6 +25,7 @@
 #include "async.cuh"
 #include "fewsum_internal.h"
 #include "launch.cuh"
+#include "rb_scale.cuh"
 #include "tcgen05.cuh"
 
 namespace fewsum {
@@ -35,26 +36,11 @@ constexpr int kDigits = 8, kRows = 128, kKnots = 64;       // slices; tile
 constexpr int kA = kRows * 32, kB = kKnots * 32;            // bytes of one slice of 16 columns
 constexpr int kStages = 4, kStage = kDigits * (kA + kB);     // 48 KB
 constexpr int kSumSteps = 12, kSumColumns = 204;              // K steps of a part; columns that need no parts
-constexpr int kPlain = 10000;                                // exponent of a row or column for the plain chain
 constexpr int kEpiWarps = 8, kThreads = 32 * (kEpiWarps + 2);  // and producer, MMAs
 constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(kKnots >> 3) << 17) | ((uint32_t)(kRows >> 4) << 24);
 constexpr float kSmall = 128.0f;                             // 2^-5 in units of the top digits' products
 
-// Exponent e with m 2^e in [1/2, 1) for m > 0 (0 for m = 0); kPlain outside 2^+-400.
-__device__ __forceinline__ int scale_exp64(double m)
-{
-    if (m == 0.0) return 0;
-    const int e = (int)((unsigned)__double2hiint(m) >> 20 & 0x7ffu);
-    if (e < 1023 - 400 || e > 1023 + 400) return kPlain;
-    return 1022 - e;
-}
 __device__ __forceinline__ double pow2_64(int e) { return __hiloint2double((1023 + e) << 20, 0); }
-
-// |x| as an integer that orders as the magnitudes do, infinities and NaN above all numbers.
-__device__ __forceinline__ unsigned long long mag(double x)
-{
-    return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
-}
 
 // Two bytes digit + 128 as fp16 integers: 0x64 byte is 1024 + byte.
 __device__ __forceinline__ uint32_t digits2(uint32_t b0, uint32_t b1)
@@ -90,17 +76,39 @@ __host__ __device__ constexpr int core64(int r, int c) { return (r >> 3) * 256 +
 
 }  // namespace
 
-// Scaling exponent of each mode's basis column.
-__global__ void k_rb64_bexp(const double *__restrict__ bre, const double *__restrict__ bim, int Nb, int N,
-                            int modes_padded, int *__restrict__ bexp)
+// Scaling exponents of each mode's basis column: for the mixed product's split (bexp) and for the digit
+// slices (bexp64, or null); 0 past the last mode.  Eight warps share the basis vectors of 32 modes (a thread
+// a mode left the chip idle: 45 us for 3843 modes of 99 vectors, 5 so).
+constexpr int kColWarps = 8;
+
+__global__ void __launch_bounds__(32 * kColWarps)
+k_rb_col_exp(const double *__restrict__ bre, const double *__restrict__ bim, int Nb, int N, int n_exp, int n_exp64,
+             int *__restrict__ bexp, int *__restrict__ bexp64)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= modes_padded) return;
-    unsigned long long m = 0;
-    if (i < N)
-        for (int j = 0; j < Nb; ++j)
-            m = max(m, max(mag(bre[(size_t)j * N + i]), mag(bim[(size_t)j * N + i])));
-    bexp[i] = scale_exp64(__longlong_as_double((long long)m));
+    __shared__ double s_max[kColWarps][32];
+    __shared__ unsigned long long s_mag[kColWarps][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    double m = 0.0;
+    unsigned long long g = 0;
+    if (i < N) {
+#pragma unroll 4
+        for (int j = w; j < Nb; j += kColWarps) {
+            const double x = bre[(size_t)j * N + i], y = bim[(size_t)j * N + i];
+            m = fmax(m, fmax(fabs(x), fabs(y)));
+            g = max(g, max(mag(x), mag(y)));
+        }
+    }
+    s_max[w][lane] = m;
+    s_mag[w][lane] = g;
+    __syncthreads();
+    if (w > 0) return;
+#pragma unroll
+    for (int k = 1; k < kColWarps; ++k) {
+        m = fmax(m, s_max[k][lane]);
+        g = max(g, s_mag[k][lane]);
+    }
+    if (i < n_exp) bexp[i] = scale_exp((float)m);
+    if (bexp64 && i < n_exp64) bexp64[i] = scale_exp64(__longlong_as_double((long long)g));
 }
 
 // Basis slices: tile t holds [steps][8][4 KB], then the magnitudes [steps][4 KB].  Row r is the real (r < 64)
@@ -369,11 +377,18 @@ cudaError_t rb64_configure()
     return cudaFuncSetAttribute(k_rb64_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, kStages * kStage);
 }
 
-cudaError_t launch_rb64_basis(const double *bre, const double *bim, int Nb, int N, int *bexp, unsigned char *pack,
+cudaError_t launch_rb_exponents(const double *bre, const double *bim, int Nb, int N, int n_exp, int *bexp, int *bexp64,
+                                cudaStream_t st)
+{
+    const int modes = rb64_modes(N), most = n_exp > modes ? n_exp : modes;
+    k_rb_col_exp<<<(most + 31) / 32, 32 * kColWarps, 0, st>>>(bre, bim, Nb, N, n_exp, modes, bexp, bexp64);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rb64_basis(const double *bre, const double *bim, int Nb, int N, const int *bexp, unsigned char *pack,
                               int sm_count, cudaStream_t st)
 {
     const int modes = rb64_modes(N);
-    k_rb64_bexp<<<(modes + 127) / 128, 128, 0, st>>>(bre, bim, Nb, N, modes, bexp);
     k_rb64_pack_b<<<sm_count * 8, 256, 0, st>>>(bre, bim, Nb, N, (2 * Nb + 15) / 16, modes / 64, bexp, pack);
     return cudaGetLastError();
 }
