@@ -328,7 +328,7 @@ __global__ void k_mode_words(const int *__restrict__ l, const int *__restrict__ 
 
 __global__ void __launch_bounds__(32 * kRingWarps, 1)
 k_direct_ring(const double *__restrict__ pphi, const double *__restrict__ pr, const double *__restrict__ are,
-              const double *__restrict__ aim, long long ns, int N, const uint4 *__restrict__ tables, int table_bytes,
+              const double *__restrict__ aim, long long ns, int N, const uint4 *tables, int table_bytes,
               double scale, void *__restrict__ out, int out_c64, unsigned *__restrict__ err)
 {
     extern __shared__ __align__(16) unsigned char ring_smem[];

@@ -65,7 +65,7 @@ __device__ __forceinline__ void ylm_thread(const PlanHdr &h, bool wait)
 }
 
 template <bool FP64>
-__global__ void __launch_bounds__(kYlmThreads) k_ylm(const PlanHdr *__restrict__ hp)
+__global__ void __launch_bounds__(kYlmThreads) k_ylm(const PlanHdr *hp)
 {
     pdl_wait();
     pdl_launch_dependents();

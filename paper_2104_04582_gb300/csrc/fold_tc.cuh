@@ -27,10 +27,10 @@ __host__ __device__ constexpr int fold_stride(int ks, size_t size) { return 16 *
 // Y: [n_pairs][2] harmonics Y+, Y- in the arithmetic type.  Needs a barrier before kc is read.
 template <typename T>
 __device__ __forceinline__ void fold_rows(const TrajDev &tr, int s, double scale,
-                                          const typename Pair2<T>::type *__restrict__ Y, T *__restrict__ kc)
+                                          const typename Pair2<T>::type *Y, T *__restrict__ kc)
 {
     const int ks = tr.tc_ks, half = 8 * ks - 1, width = 2 * half + 1, ld = fold_stride(ks, sizeof(T));
-    const double *__restrict__ cs = tr.coef + (size_t)s * tr.J * 4;
+    const double *cs = tr.coef + (size_t)s * tr.J * 4;
     const T hk = fold_cvt(tr.h[s], T()), sc = fold_cvt(scale, T());
     for (int it = threadIdx.x; it < tr.tc_pairs * width; it += blockDim.x) {
         const int p = it / width, off = it - p * width - half, m = tr.m_top - p;

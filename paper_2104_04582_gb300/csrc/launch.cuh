@@ -3,6 +3,11 @@
 // what needs none of that one's results (barriers, tensor memory, harmonics), then waits for its
 // completion.  Every kernel launched by launch_pdl executes pdl_wait() before it reads or writes
 // anything that an earlier kernel may use, in every block.
+//
+// What the kernels before it write is read by ordinary loads: not by __ldg, nor through a const
+// __restrict__ pointer.  Those may take the read-only path, which is specified only for data that does
+// not change while the kernel runs (its blocks are there before that data is), and the compiler may
+// move them up across the wait.
 #pragma once
 
 #include <cuda_runtime.h>

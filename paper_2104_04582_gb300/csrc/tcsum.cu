@@ -129,7 +129,7 @@ __device__ __forceinline__ void fold_tc_block(const PlanHdr &h, bool wait)
     }
 }
 
-__global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *__restrict__ hp)
+__global__ void __launch_bounds__(kTcFoldThreads) k_fold_tc(const PlanHdr *hp)
 {
     pdl_wait();
     pdl_launch_dependents();
@@ -219,13 +219,12 @@ __device__ __forceinline__ void first_powers(unsigned long long f, float2 (&c)[4
 }  // namespace
 
 // Starts the copy of table `n` of the CTA's run (first tile T) into its buffer (one thread).
-__device__ __forceinline__ void load_table(const TileRec *__restrict__ recs, int T, int n,
+__device__ __forceinline__ void load_table(const TileRec *recs, int T, int n,
                                            unsigned char *buf, uint64_t *full)
 {
     const TileRec *r = recs + T;
-    const uint32_t bytes = (uint32_t)tc_table_bytes(__ldg(&r->pairs), __ldg(&r->ks));
-    const unsigned char *src = reinterpret_cast<const unsigned char *>(
-        __ldg(reinterpret_cast<const unsigned long long *>(&r->tab)));
+    const uint32_t bytes = (uint32_t)tc_table_bytes(r->pairs, r->ks);
+    const unsigned char *src = r->tab;
     mbar_arrive_expect_tx(&full[n & 1], bytes);
     for (uint32_t o = 0; o < bytes; o += 16384u)
         bulk_g2s(buf + (n & 1) * kTcMaxTable + o, src + o, min(16384u, bytes - o), &full[n & 1]);
@@ -243,7 +242,7 @@ __device__ __forceinline__ void load_table(const TileRec *__restrict__ recs, int
 // of the accumulator ~500, wake-up ~350).  Six warpgroups of 80 registers: 133 us; factors before
 // the issue: 122; MMAs in tile order by a token: 114.
 template <int KS>
-__global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restrict__ hp)
+__global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *hp)
 {
     extern __shared__ __align__(128) unsigned char tcs[];  // two operand tables
     __shared__ __align__(8) uint64_t b_full[2], d_full[2], d_free[2];
@@ -255,7 +254,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
     pdl_wait();
     pdl_launch_dependents();
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
-    const TileRec *__restrict__ recs = hp->recs;
+    const TileRec *recs = hp->recs;
     const int T0 = hp->tile_cta[blockIdx.x], T1 = hp->tile_cta[blockIdx.x + 1];
     if (T0 >= T1) return;  // uniform across the CTA: no work
     if (warp == 0) {
@@ -275,7 +274,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
         fence_mbar_init();
         s_abort = 0;
         load_table(recs, T0, 0, tcs, b_full);
-        const int next = __ldg(&recs[T0].tile_end);
+        const int next = recs[T0].tile_end;
         if (next < T1) load_table(recs, next, 1, tcs, b_full);
         s_loaded = next < T1 ? 2 : 1;
     }
@@ -288,14 +287,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
     const uint32_t quarter = (uint32_t)(32 * (warp & 3)) << 16;
     const uint32_t d_col = tmem + (uint32_t)slot * kTcDStride;
     const uint32_t e_col = tmem + kTcECol + (uint32_t)slot * kTcEStride;
-    int j = 0, tend = __ldg(&recs[T0].tile_end);  // table of the current tile, and where it ends
+    int j = 0, tend = recs[T0].tile_end;  // table of the current tile, and where it ends
     bool bad = false;
     // This warpgroup's MMAs on table j have completed: release it (lead), and let the last of the
     // warpgroups refill its buffer.  A table is released only once it has landed (also one that the
     // warpgroup had no tile in): its buffer's previous table has then been released by every
     // warpgroup, so neither the count nor a parity wait can be taken for the previous table's.
     auto release_table = [&]() {
-        const int next = __ldg(&recs[tend].tile_end);  // end of table j + 1, first tile of j + 2
+        const int next = recs[tend].tile_end;  // end of table j + 1, first tile of j + 2
         if (lead && !bad) {
             if (!mbar_wait_bounded(&b_full[j & 1], (j >> 1) & 1)) {
                 bad = true;
@@ -315,7 +314,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
     // own line of shared memory
     const TileRec *rp = reinterpret_cast<const TileRec *>(s_rec[warp]);
     uint32_t next_word = 0;
-    if (T0 + group < T1) next_word = __ldg(reinterpret_cast<const uint32_t *>(recs + T0 + group) + (tid & 31));
+    if (T0 + group < T1) next_word = reinterpret_cast<const uint32_t *>(recs + T0 + group)[tid & 31];
 #pragma unroll 1
     for (int T = T0 + group; T < T1; T += kTcGroups) {
         s_rec[warp][tid & 31] = next_word;
@@ -394,10 +393,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_sum_tc(const PlanHdr *__restr
         }
         // while the MMAs run: this sample's factors
         const float2 uu = *reinterpret_cast<const float2 *>(&rp->u0);
-        const float inv = __ldg(static_cast<const float *>(rp->seg));
+        const float inv = *static_cast<const float *>(rp->seg);
         void *out = rp->out;
         if (T + kTcGroups < T1)
-            next_word = __ldg(reinterpret_cast<const uint32_t *>(recs + T + kTcGroups) + (tid & 31));
+            next_word = reinterpret_cast<const uint32_t *>(recs + T + kTcGroups)[tid & 31];
         const float u = fmaf((float)(i - span.y), uu.y, uu.x);
         float zs, zc;
         sincos_fixed((uint32_t)(fphi >> 32), zs, zc);

@@ -164,7 +164,7 @@ __device__ __forceinline__ void fold_tc64_block(const PlanHdr &h)
     }
 }
 
-__global__ void __launch_bounds__(kT64FoldThreads) k_fold_tc64(const PlanHdr *__restrict__ hp)
+__global__ void __launch_bounds__(kT64FoldThreads) k_fold_tc64(const PlanHdr *hp)
 {
     pdl_launch_dependents();
     fold_tc64_block(*hp);
@@ -350,7 +350,7 @@ __device__ __forceinline__ void issue_pair(int issuer, uint32_t d, uint32_t e, u
 // the run): e_full[g] the basis of group g's tile is stored; done[g] its MMAs have completed (the
 // operand columns are free); d_full[b], d_empty[b] accumulator set b = chunk & 1.
 template <int KS>
-__global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__restrict__ hp)
+__global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *hp)
 {
     extern __shared__ __align__(128) unsigned char tcs64[];  // the operand table
     __shared__ __align__(8) uint64_t b_full, d_full[2], d_empty[2], e_full[kT64Groups], done[kT64Groups];
@@ -359,7 +359,7 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
     pdl_wait();
     pdl_launch_dependents();
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);  // uniform
-    const TileRec *__restrict__ recs = hp->recs;
+    const TileRec *recs = hp->recs;
     const int T0 = hp->tile_cta[blockIdx.x], T1 = hp->tile_cta[blockIdx.x + 1];
     if (T0 >= T1) return;  // uniform across the CTA: no work
     if (warp == 0) {
@@ -393,17 +393,16 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
         uint32_t chunk = 0;
         bool ok = true;
         for (int T = T0; T < T1 && ok; ++T) {
-            const int4 shape = __ldg(reinterpret_cast<const int4 *>(&recs[T].pairs));
+            const int4 shape = *reinterpret_cast<const int4 *>(&recs[T].pairs);
             const int pairs = __shfl_sync(0xffffffffu, shape.x, 0), ks = __shfl_sync(0xffffffffu, shape.y, 0);
             const int g = (T - T0) & 1;
             if (T == tend) {  // the table's first tile: the previous one's MMAs must have completed
-                tend = __ldg(&recs[T].tile_end);
+                tend = recs[T].tile_end;
                 ++table;
                 if (T > T0) ok = warp_ok(mbar_wait_bounded(&done[g ^ 1], (uint32_t)(T - 1 - T0) >> 1 & 1u));
                 if (ok && issuer == 0 && (tid & 31) == 0) {
                     const uint32_t bytes = (uint32_t)tc64_table_bytes(pairs, ks);
-                    const unsigned char *src = reinterpret_cast<const unsigned char *>(
-                        __ldg(reinterpret_cast<const unsigned long long *>(&recs[T].tab)));
+                    const unsigned char *src = recs[T].tab;
                     mbar_arrive_expect_tx(&b_full, bytes);
                     for (uint32_t o = 0; o < bytes; o += 16384u)
                         bulk_g2s(tcs64 + o, src + o, min(16384u, bytes - o), &b_full);
@@ -449,22 +448,21 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
 #pragma unroll 1
         for (int T = T0 + group; T < T1; T += kT64Groups) {
             const TileRec *rp = recs + T;
-            const int4 span = __ldg(reinterpret_cast<const int4 *>(&rp->i0));      // i0, s0, s1, tile_end
-            const int4 shape = __ldg(reinterpret_cast<const int4 *>(&rp->pairs));  // pairs, ks, n_mid, c64
+            const int4 span = *reinterpret_cast<const int4 *>(&rp->i0);      // i0, s0, s1, tile_end
+            const int4 shape = *reinterpret_cast<const int4 *>(&rp->pairs);  // pairs, ks, n_mid, c64
             const int pairs = shape.x;
-            for (; counted < T; ++counted) chunk += (uint32_t)__ldg(&recs[counted].pairs);
+            for (; counted < T; ++counted) chunk += (uint32_t)recs[counted].pairs;
             const int i = span.x + lane;
             const uint32_t v = (uint32_t)max(i - max(span.x, span.y), 0);
             TileRec ph;
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                reinterpret_cast<int4 *>(&ph)[k] = __ldg(reinterpret_cast<const int4 *>(rp) + k);
-            const int2 lo3 = __ldg(reinterpret_cast<const int2 *>(&rp->u0));  // of c3: phi, r
+                reinterpret_cast<int4 *>(&ph)[k] = reinterpret_cast<const int4 *>(rp)[k];
+            const int2 lo3 = *reinterpret_cast<const int2 *>(&rp->u0);  // of c3: phi, r
             const long long v3 = (long long)(v * v * v);
             const unsigned long long fr = phase_fixed(ph.r, v) + (unsigned long long)(lo3.y * v3 >> 32);
             const unsigned long long fphi = phase_fixed(ph.phi, v) + (unsigned long long)(lo3.x * v3 >> 32);
-            const TcSeg64 *sg = static_cast<const TcSeg64 *>(
-                reinterpret_cast<const void *>(__ldg(reinterpret_cast<const unsigned long long *>(&rp->seg))));
+            const TcSeg64 *sg = static_cast<const TcSeg64 *>(rp->seg);
             // (lanes outside the segment take its first or last sample's u: sums stay in range)
             const double u = (fma((double)min(max(i, span.y), span.z - 1), sg->dt, sg->t0) - sg->tk) * sg->ih;
             const Q62 U = q62(__double2ll_rn(u * 4611686018427387904.0));
@@ -573,7 +571,7 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *__re
                     fs = (double)value(w.s) * 2.168404344971008868e-19 * inv;
                 }
                 const double yr = fma(hr, fc, hi * fs) * sg->inv2, yi = fma(hi, fc, -hr * fs) * sg->inv2;
-                void *out = reinterpret_cast<void *>(__ldg(reinterpret_cast<const unsigned long long *>(&rp->out)));
+                void *out = rp->out;
                 if (shape.w)
                     reinterpret_cast<float2 *>(out)[i] = make_float2((float)yr, (float)yi);
                 else
