@@ -529,6 +529,7 @@ cudaError_t launch_direct(const double *pphi, const double *pr, const double *ar
         k_mode_words<<<(n_thr + 63) / 64, 64, 0, st>>>(l, m, n, N, theta, phi, l_top, m_top, words, recs);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
+        // (reads the caller's arrays beside the plain launch above: launch.cuh)
         return launch_pdl(k_direct_ring, (unsigned)(ns < sm_count ? ns : sm_count), 32 * kRingWarps,
                           (size_t)(kRingBytes + table), st, pphi, pr, are, aim, ns, N,
                           static_cast<const uint4 *>(mode_consts), table, scale, out, out_c64, err);

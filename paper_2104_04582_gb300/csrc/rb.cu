@@ -837,6 +837,8 @@ cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N
     } else if (nu && fp64) {
         const int groups = (Nb + 31) / 32;
         k_rb_scale64<<<M, 32 * groups * kScaleSets, 0, ss>>>(are, aim, Nb, groups, gt64, nu, scale, err);
+        // (launch_rb64's pack leans on this launch: see launch.cuh)
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
         sc = scale;
     } else if (nu) {
         double *q = scale + M;  // the caller's scratch holds scale [M] then q [M]
@@ -847,6 +849,7 @@ cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N
         if (e != cudaSuccess) return fail(e);
         k_rb_quad<<<grid, kQThreads, kQSmem, ss>>>(are, aim, M, Nb, gt32, q);
         k_rb_norm<<<(M + 255) / 256, 256, 0, ss>>>(q, nu, M, scale, err);
+        if ((e = cudaGetLastError()) != cudaSuccess) return fail(e);
         sc = scale;
     }
     if (fork && (e = cudaEventRecord(join_ev, side)) != cudaSuccess) return fail(e);
@@ -876,7 +879,7 @@ cudaError_t launch_rb(const double *are, const double *aim, int M, int Nb, int N
     const int rows = L.m_tiles * kRbTileN;
     const int pgrid = (rows + kRbPackWarps - 1) / kRbPackWarps;
     const unsigned pblocks = pgrid < sm_count * 8 ? pgrid : sm_count * 8;
-    if (tile) {  // beside the scale's kernel
+    if (tile) {  // beside the scale's kernel, whose plain launch it leans on (launch.cuh)
         e = launch_pdl(k_rb_pack_a, pblocks, kRbPackWarps * 32, 0, st, are, aim, M, Nb, L.n_kb, L.m_tiles, apack,
                        aexp);
     } else {

@@ -402,7 +402,7 @@ cudaError_t launch_rb64(Rb64Args a, unsigned char *apack, int *aexp, bool after_
     a.apack = apack;
     a.aexp = aexp;
     cudaError_t e;
-    if (after_scale) {  // beside the scale's kernel
+    if (after_scale) {  // beside the scale's kernel, whose plain launch it leans on (launch.cuh)
         e = launch_pdl(k_rb64_pack_a, (unsigned)(rows / 4), 128u, (size_t)0, st, a.are, a.aim, a.M, a.Nb, a.steps,
                        a.per, apack, aexp);
     } else {

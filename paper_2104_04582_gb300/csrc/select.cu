@@ -636,6 +636,7 @@ cudaError_t launch_mode_select(const double *amp_re, const double *amp_im, int K
     k_mask_zero<<<1, 1024, 0, st>>>(mask, N);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    // (reads the caller's arrays beside the plain launch above: launch.cuh)
     return launch_pdl(k_mode_select, (unsigned)K, (unsigned)threads, (size_t)smem, st, amp_re, amp_im, N, dbl, eps,
                       P, sub, mask);
 }

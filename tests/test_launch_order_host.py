@@ -58,3 +58,27 @@ def test_waveform_kernels_have_no_read_only_loads(name):
     assert "__ldg(" not in SOURCES[name]
     for m in re.finditer(r"const [^;,()]*?\*\s*__restrict__ (\w+)", SOURCES[name]):
         assert m.group(1) == "kc"  # the block's own shared memory
+
+
+def _launches(text):
+    """The launches of a source in their order: 'plain', the dependent kernel's name, or 'checked'."""
+    out = []
+    for m in re.finditer(r"<<<|launch_pdl\(([^,]+),|(launch_rb64)\(|cudaGetLastError\(\)", text):
+        out.append("plain" if m.group(0) == "<<<" else "checked" if m.group(0).startswith("cudaGet")
+                   else (m.group(1) or m.group(2)).strip())
+    return out
+
+
+@pytest.mark.parametrize("name", [f for f in SOURCES if f.endswith(".cu")])
+def test_plain_launch_is_checked_before_a_dependent_one(name):
+    seq = _launches(SOURCES[name])
+    for before, after in zip(seq, seq[1:]):
+        assert not (before == "plain" and after not in ("plain", "checked"))
+
+
+@pytest.mark.parametrize("name,kernel", [("rb.cu", "k_rb_pack_a"), ("rb.cu", "launch_rb64"), ("direct.cu", "k_direct_ring"),
+                                         ("select.cu", "k_mode_select")])
+def test_kernels_that_start_before_their_wait_follow_a_plain_launch(name, kernel):
+    """They touch memory before their wait, which only a plain launch just ahead makes safe."""
+    seq = [s for s in _launches(SOURCES[name]) if s != "checked"]
+    assert seq[seq.index(kernel) - 1] == "plain"
