@@ -1128,18 +1128,8 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream)
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     PlanImage P;
     const size_t out_bytes = (size_t)req->n_samples * (req->out_c64 ? 8 : 16);
-    void *blob = nullptr, *dout = nullptr;  // the plan, its scratch behind it
-    auto plan = [&](bool tc) {
-        P = PlanImage();
-        const few_status e = build_image(ctx, req, 1, tc, P);
-        return e ? e : dev_alloc(ctx, P.blob.size() + P.scratch_bytes, s, &blob);
-    };
-    const bool tc = tc_fits(*req);
-    st = plan(tc);
-    // the tensor-core plan may need more scratch than the scalar one (sparse mode sets)
-    if (tc && (st == FEW_ERR_BUDGET || st == FEW_ERR_NOMEM)) st = plan(false);
-    if (st) return st;
     void *out_dev = req->out;
+    bool staged = false;
     if (req->out_where == FEW_MEM_HOST) {
         // page-locked host memory is addressable from the device (over NVLink-C2C on a Grace
         // host): the summation kernel stores into it directly and the transfer overlaps the
@@ -1150,13 +1140,23 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream)
             out_dev = pa.devicePointer;
         } else {
             (void)cudaGetLastError();
-            if ((st = dev_alloc(ctx, out_bytes, s, &dout))) {
-                dev_free(ctx, blob, s);
-                return st;
-            }
-            out_dev = dout;
+            staged = true;
         }
     }
+    void *blob = nullptr, *dout = nullptr;  // the plan, its scratch behind it; the staged output
+    auto plan = [&](bool tc) {
+        P = PlanImage();
+        few_status e = build_image(ctx, req, 1, tc, P);
+        if (!e) e = dev_alloc(ctx, P.blob.size() + P.scratch_bytes, s, &blob);
+        if (!e && staged && (e = dev_alloc(ctx, out_bytes, s, &dout))) dev_free(ctx, blob, s);
+        return e;
+    };
+    const bool tc = tc_fits(*req);
+    st = plan(tc);
+    // the tensor-core plan may need more scratch than the scalar one (sparse mode sets)
+    if (tc && (st == FEW_ERR_BUDGET || st == FEW_ERR_NOMEM)) st = plan(false);
+    if (st) return st;
+    if (staged) out_dev = dout;
     unsigned char *blob_dev = static_cast<unsigned char *>(blob);
     fill_image(ctx, req, 1, P, blob_dev, blob_dev + P.blob.size(), &out_dev);
     // a small tensor-core plan travels in the fold's parameters: no copy stands between the kernels
@@ -1475,6 +1475,31 @@ few_status few_batch_plan(few_ctx *ctx, const few_request *reqs, int n, unsigned
         delete b;
         return e;
     };
+    // the build jobs first: what is left decides which summation plan fits
+    if (flags & FEW_BATCH_REBUILD_SPLINES) {
+        std::vector<BuildJob> jobs;
+        std::set<const few_traj *> seen;
+        int blocks = 0;
+        for (int q = 0; q < n; ++q) {
+            const few_traj *tr = reqs[q].traj;
+            if (!seen.insert(tr).second) continue;
+            BuildJob j{};
+            j.tr = tr->dev;
+            j.phi_phi = tr->src_phi_phi;
+            j.phi_r = tr->src_phi_r;
+            j.amp_re = tr->src_re;
+            j.amp_im = tr->src_im;
+            j.block_begin = blocks;
+            blocks += (tr->J + kBuildSplines - 1) / kBuildSplines;
+            b->max_knots = std::max(b->max_knots, tr->K);
+            jobs.push_back(j);
+        }
+        if ((st = dev_alloc(ctx, sizeof(BuildJob) * jobs.size(), s, &b->jobs_dev))) return fail(st);
+        if ((st = upload(ctx, b->jobs_dev, jobs.data(), sizeof(BuildJob) * jobs.size(), s)))
+            return fail(st);
+        b->n_jobs = (int)jobs.size();
+        b->build_blocks = blocks;
+    }
     // one part per summation variant
     auto add_part = [&](const std::vector<few_request> &rq, bool tc) -> few_status {
         if (rq.empty()) return FEW_OK;
@@ -1503,30 +1528,6 @@ few_status few_batch_plan(few_ctx *ctx, const few_request *reqs, int n, unsigned
         st = add_part(std::vector<few_request>(reqs, reqs + n), false);
     }
     if (st) return fail(st);
-    if (flags & FEW_BATCH_REBUILD_SPLINES) {
-        std::vector<BuildJob> jobs;
-        std::set<const few_traj *> seen;
-        int blocks = 0;
-        for (int q = 0; q < n; ++q) {
-            const few_traj *tr = reqs[q].traj;
-            if (!seen.insert(tr).second) continue;
-            BuildJob j{};
-            j.tr = tr->dev;
-            j.phi_phi = tr->src_phi_phi;
-            j.phi_r = tr->src_phi_r;
-            j.amp_re = tr->src_re;
-            j.amp_im = tr->src_im;
-            j.block_begin = blocks;
-            blocks += (tr->J + kBuildSplines - 1) / kBuildSplines;
-            b->max_knots = std::max(b->max_knots, tr->K);
-            jobs.push_back(j);
-        }
-        if ((st = dev_alloc(ctx, sizeof(BuildJob) * jobs.size(), s, &b->jobs_dev))) return fail(st);
-        if ((st = upload(ctx, b->jobs_dev, jobs.data(), sizeof(BuildJob) * jobs.size(), s)))
-            return fail(st);
-        b->n_jobs = (int)jobs.size();
-        b->build_blocks = blocks;
-    }
     if (cudaStreamSynchronize(s) != cudaSuccess) return fail(FEW_ERR_CUDA);
     if (!(flags & FEW_BATCH_NO_GRAPH)) {
         cudaStream_t cap = nullptr;

@@ -178,3 +178,42 @@ def test_budget_that_only_the_scalar_plan_fits():
                 # under the small budget the scalar chain ran: the mixed path's gate
                 assert oracle.mismatch(to_host(h), ref) <= MIXED_MISMATCH
             tr.release()
+
+
+@pytest.mark.parametrize("how", ["pageable", "rebuild"])
+def test_budget_with_buffers_beside_the_plan(how):
+    """The same two modes with a buffer next to the plan: staging of a pageable output, or the build jobs
+    of a batch.  A budget that holds the tensor-core plan alone, but not that buffer beside it, still
+    runs the request (by the scalar plan)."""
+    import torch
+    w = W.make_inputs(3.0e6, 4096, 300.0, _modes([2], [-31, 31]), 3)
+    out = np.empty(w.n_samples, dtype=np.complex64)
+
+    def run(ctx, tr):
+        if how == "pageable":
+            out[:] = 0
+            F.few_waveform(ctx.handle, RT.request(tr, out, w.n_samples, w.t0, w.dt, w.theta, w.phi, F.FEW_MIXED,
+                                                  out_where=F.FEW_MEM_HOST), RT.current_stream())
+            return out.astype(np.complex128)
+        dev = RT.alloc_out(w.n_samples, True)
+        req = RT.request(tr, dev, w.n_samples, w.t0, w.dt, w.theta, w.phi, F.FEW_MIXED)
+        b = F.few_batch_plan(ctx.handle, [req], F.FEW_BATCH_REBUILD_SPLINES)
+        F.few_batch_run(ctx.handle, b, RT.current_stream())
+        torch.cuda.synchronize()
+        F.few_batch_release(ctx.handle, b)
+        return to_host(dev)
+
+    with RT.Context(0) as free:
+        tr = RT.from_inputs(free, w)
+        held = free.memory()[0]
+        ref = to_host(RT.waveform_inputs(free, tr, w, F.FEW_MIXED))
+        b = F.few_batch_plan(free.handle, [RT.request(tr, RT.alloc_out(w.n_samples, True), w.n_samples, w.t0, w.dt,
+                                                      w.theta, w.phi, F.FEW_MIXED)], 0)
+        plan = free.memory()[0] - held  # the tensor-core plan
+        F.few_batch_release(free.handle, b)
+        tr.release()
+    with RT.Context(0, held + plan) as ctx:
+        tr = RT.from_inputs(ctx, w)
+        assert oracle.mismatch(run(ctx, tr), ref) <= MIXED_MISMATCH
+        assert ctx.sync_status() == F.FEW_OK
+        tr.release()
