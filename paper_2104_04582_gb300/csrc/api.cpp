@@ -1518,14 +1518,32 @@ few_status few_batch_plan(few_ctx *ctx, const few_request *reqs, int n, unsigned
         part.launch = P.launch;
         return upload(ctx, part.blob_dev, P.blob.data(), P.blob.size(), s);
     };
-    std::vector<few_request> tc_reqs, other;
-    for (int q = 0; q < n; ++q) (tc_fits(reqs[q]) ? tc_reqs : other).push_back(reqs[q]);
-    st = add_part(tc_reqs, true);
-    if (!st) st = add_part(other, false);
-    if ((st == FEW_ERR_BUDGET || st == FEW_ERR_NOMEM) && !tc_reqs.empty()) {
-        // the scalar plan of sparse mode sets needs less scratch
+    // Waves on the tensor cores where they fit.  A plan past the budget moves the waves that save most by
+    // it to the scalar chain (sparse mode sets: their tables are larger than the slots), twice as many
+    // each time.
+    std::vector<int> order;
+    std::vector<char> on_tc(n);
+    for (int q = 0; q < n; ++q)
+        if ((on_tc[q] = tc_fits(reqs[q]))) order.push_back(q);
+    auto saves = [&](int q) {
+        const few_traj *tr = reqs[q].traj;
+        const bool fp64 = reqs[q].prec == FEW_FP64;
+        const int variant = fp64 ? kVariantFp64 : kVariantScalar;
+        const double table = (double)tc_segment_bytes(fp64, tr->plan.tc_pairs, tr->plan.tc_ks);
+        const double recs = (double)sizeof(TileRec) / kTcTile, anchors = (double)sizeof(Anchor) / kAnchorGroup;
+        return tr->S * (table - (double)tr->plan.n_slots * sum_slot_bytes(variant)) +
+               (double)reqs[q].n_samples * (recs - (fp64 ? 0.0 : anchors));
+    };
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return saves(a) > saves(b); });
+    for (size_t moved = 0;;) {
+        std::vector<few_request> tc_reqs, other;
+        for (int q = 0; q < n; ++q) (on_tc[q] ? tc_reqs : other).push_back(reqs[q]);
+        st = add_part(tc_reqs, true);
+        if (!st) st = add_part(other, false);
+        if ((st != FEW_ERR_BUDGET && st != FEW_ERR_NOMEM) || moved == order.size()) break;
         drop_parts();
-        st = add_part(std::vector<few_request>(reqs, reqs + n), false);
+        const size_t next = std::min(order.size(), 2 * moved + 1);
+        for (; moved < next; ++moved) on_tc[order[moved]] = 0;
     }
     if (st) return fail(st);
     if (cudaStreamSynchronize(s) != cudaSuccess) return fail(FEW_ERR_CUDA);

@@ -217,3 +217,49 @@ def test_budget_with_buffers_beside_the_plan(how):
         assert oracle.mismatch(run(ctx, tr), ref) <= MIXED_MISMATCH
         assert ctx.sync_status() == F.FEW_OK
         tr.release()
+
+
+@pytest.mark.parametrize("prec", PRECS)
+def test_budget_moves_only_the_waves_that_do_not_fit(prec):
+    """A batch of one full and three sparse mode sets (two modes on 1500 knots): under a budget that does
+    not hold the sparse sets' tables beside the full one's, the full set keeps its plan, to the bit."""
+    import torch
+    ws = [W.make_inputs(2.0e5, 1500, 200.0, _modes([2], [-31, 31]), 3 + k) for k in range(3)]
+    ws.insert(1, W.make_inputs(2.0e5, 20, 50.0, W.mode_grid(10, 30), 9, 4.0, 60.0))
+
+    def setup(ctx):
+        trs = [RT.from_inputs(ctx, w) for w in ws]
+        outs = [RT.alloc_out(w.n_samples, prec == F.FEW_MIXED) for w in ws]
+        return trs, outs, [RT.request(tr, o, w.n_samples, w.t0, w.dt, w.theta, w.phi, prec)
+                           for tr, o, w in zip(trs, outs, ws)]
+
+    def plan_bytes(ctx, reqs):
+        held = ctx.memory()[0]
+        b = F.few_batch_plan(ctx.handle, reqs, 0)
+        held = ctx.memory()[0] - held
+        F.few_batch_release(ctx.handle, b)
+        return held
+
+    with RT.Context(0) as free:
+        trs, outs, reqs = setup(free)
+        held, both, full = free.memory()[0], plan_bytes(free, reqs), plan_bytes(free, reqs[1:2])
+        refs = [to_host(RT.waveform(free, tr, w.n_samples, w.t0, w.dt, w.theta, w.phi, prec)) for tr, w in zip(trs, ws)]
+        for tr in trs:
+            tr.release()
+    budget = held + full + (both - full) // 2  # the sparse sets by the scalar chain: a third at most
+    with RT.Context(0, budget) as ctx:
+        trs, outs, reqs = setup(ctx)
+        b = F.few_batch_plan(ctx.handle, reqs, 0)
+        F.few_batch_run(ctx.handle, b, RT.current_stream())
+        torch.cuda.synchronize()
+        assert ctx.sync_status() == F.FEW_OK
+        for k, (o, ref) in enumerate(zip(outs, refs)):
+            if k == 1:
+                np.testing.assert_array_equal(to_host(o), ref)
+            elif prec == F.FEW_FP64:
+                assert rel_l2(to_host(o), ref) <= REL[prec]
+            else:
+                assert oracle.mismatch(to_host(o), ref) <= MIXED_MISMATCH
+        F.few_batch_release(ctx.handle, b)
+        for tr in trs:
+            tr.release()
