@@ -43,11 +43,16 @@ constexpr int kTcMaxPairs = 11;  // rows m and -m, max m <= 10: two accumulators
                                  //   pair, beside the operands, in the 512 tensor-memory columns
 constexpr int kTcMaxHalf = 31;  // half-width of the n range: 64 basis values (K)
 constexpr int kTcFoldThreads = 704;
-// Fold blocks that fill tile records: 128 tiles each, until there are four a multiprocessor.
-constexpr int kTcRecTiles = 128;
-inline int tc_record_blocks(int total_tiles, int sm_count)
+// Fold blocks that fill tile records: 128 tiles each, until there are four a multiprocessor.  FP64 (segs:
+// the plan's segments, else 0): no more than 16 segments each on average, since a block forms the coefficients of
+// 32 at a time, in a chain of FP64 operations, and the blocks at the dense end of the knots hold more than the
+// average.  FP64 fold of 100 (1000) knots, 2 modes, 20,000 samples: 66 (208) us with 128 tiles to a block whatever
+// their segments and both phases in a thread, 23 (75) so.
+constexpr int kTcRecTiles = 128, kTcFillSegs = 32;
+inline int tc_record_blocks(int total_tiles, int segs, int sm_count)
 {
-    const int n = (total_tiles + kTcRecTiles - 1) / kTcRecTiles, most = 4 * sm_count;
+    const int t = (total_tiles + kTcRecTiles - 1) / kTcRecTiles, s = (segs + 15) / 16;
+    const int n = t > s ? t : s < total_tiles ? s : total_tiles, most = 4 * sm_count;
     return n < most ? n : most;
 }
 // Everything the summation reads for one tile, one 128-byte line.  Phases of sample a + v, a =

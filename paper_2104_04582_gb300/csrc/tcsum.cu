@@ -504,7 +504,7 @@ cudaError_t launch_fold_tc(const PlanHdr *hdr_dev, const PlanParam *plan, int to
                            int sm_count, cudaStream_t st)
 {
     if (total_tiles <= 0) return cudaSuccess;
-    const unsigned grid = total_segs + tc_record_blocks(total_tiles, sm_count);
+    const unsigned grid = total_segs + tc_record_blocks(total_tiles, 0, sm_count);
     // More segments than multiprocessors: blocks of half the threads, two a multiprocessor, so that one
     // loads while the other packs (24 uneven waveforms, 2,400 segments: 3.17 -> 2.99 ms with the records'
     // share of that); else a thread a frequency, for the latency of the one block.

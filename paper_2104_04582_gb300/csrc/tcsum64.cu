@@ -609,7 +609,7 @@ cudaError_t launch_fold_tc64(const PlanHdr *hdr_dev, int total_segs, int total_t
                              cudaStream_t st)
 {
     if (total_tiles <= 0) return cudaSuccess;
-    const unsigned grid = total_segs + tc_record_blocks(total_tiles, sm_count);
+    const unsigned grid = total_segs + tc_record_blocks(total_tiles, total_segs, sm_count);
     return launch_pdl(k_fold_tc64, grid, kT64FoldThreads, kFold64Smem, st, hdr_dev);
 }
 

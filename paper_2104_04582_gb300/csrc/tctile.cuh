@@ -118,7 +118,6 @@ struct SegFill {
     int s0, s1;
     int pairs, ks, n_mid, c64;
 };
-constexpr int kTcFillSegs = 32;
 
 // x modulo 2 pi (2 pi in two parts; see reduce_2pi).
 __device__ __forceinline__ double tc_reduce(double x)
@@ -202,7 +201,20 @@ __device__ __forceinline__ bool tc_phase_at(const PhaseFill64 &p, const Dd &u, l
 }
 
 template <bool FP64>
-__device__ inline void tc_seg_fill(const PlanHdr &h, const WaveDev &W, int s, SegFill<FP64> &o)
+__device__ __forceinline__ Dd tc_seg_ih(const WaveDev &W, int s)
+{
+    if constexpr (FP64) return dd_div(Dd{1.0, 0.0}, W.tr.h[s]);
+    return Dd{W.tr.inv_h[s], 0.0};
+}
+// Phase p (0 Phi_phi, 1 Phi_r) of segment s.
+template <bool FP64>
+__device__ __forceinline__ void tc_seg_phase(const WaveDev &W, int s, int p, Dd ih, SegFill<FP64> &o)
+{
+    tc_phase_fill(W.tr.coef + (size_t)s * W.tr.J * 4 + 4 * p, W.tr.h[s], ih, W.dt, p ? W.dphi_r : W.dphi_phi, o.p[p]);
+}
+// The rest of segment s.
+template <bool FP64>
+__device__ inline void tc_seg_fill(const PlanHdr &h, const WaveDev &W, int s, Dd ih, SegFill<FP64> &o)
 {
     const TrajDev &tr = W.tr;
     const int *tile_off = tc_local(h, W.tile_off), *seg_start = tc_local(h, W.seg_start);
@@ -213,13 +225,9 @@ __device__ inline void tc_seg_fill(const PlanHdr &h, const WaveDev &W, int s, Se
     o.tk = tr.t[s];
     o.t0 = W.t0;
     o.dt = W.dt;
-    const double ih = tr.inv_h[s], hk = tr.h[s];
-    o.ih = FP64 ? dd_div(Dd{1.0, 0.0}, hk) : Dd{ih, 0.0};
-    const double *c = tr.coef + (size_t)s * tr.J * 4;
-    tc_phase_fill(c, hk, o.ih, W.dt, W.dphi_phi, o.p[0]);
-    tc_phase_fill(c + 4, hk, o.ih, W.dt, W.dphi_r, o.p[1]);
-    o.u0 = (float)((fma((double)o.s0, W.dt, W.t0) - o.tk) * ih);
-    o.du = (float)(W.dt * ih);
+    o.ih = ih;
+    o.u0 = (float)((fma((double)o.s0, W.dt, W.t0) - o.tk) * ih.h);
+    o.du = (float)(W.dt * ih.h);
     o.seg = FP64 ? (const void *)(W.seg64 + s) : (const void *)(W.tab_inv + s);
     o.tab = W.tab + (size_t)s * (FP64 ? tc64_table_bytes(tr.tc_pairs, tr.tc_ks)
                                       : tc_table_bytes(tr.tc_pairs, tr.tc_ks));
@@ -230,16 +238,24 @@ __device__ inline void tc_seg_fill(const PlanHdr &h, const WaveDev &W, int s, Se
     o.c64 = W.out_c64;
 }
 
-// Segment g of the plan for a block's cache; past the last one: no tiles.
+// Segments g0 .. of the plan for a block's cache; past the last one: no tiles.  FP64: a phase a thread (the
+// second phases in another warp, on another scheduler's share of the FP64 pipe).
 template <bool FP64>
-__device__ inline void tc_cache_seg(const PlanHdr &h, int g, SegFill<FP64> &o)
+__device__ inline void tc_cache_segs(const PlanHdr &h, int g0, SegFill<FP64> *seg)
 {
+    constexpr int kThreads = FP64 ? 2 * kTcFillSegs : kTcFillSegs;
+    if (threadIdx.x >= kThreads) return;
+    const int k = threadIdx.x % kTcFillSegs, p = threadIdx.x / kTcFillSegs, g = g0 + k;
     if (g >= h.total_segs) {
-        o.first = o.end = h.total_tiles;
+        if (p == 0) seg[k].first = seg[k].end = h.total_tiles;
         return;
     }
     const WaveDev &W = tc_wave(h, tc_wave_of_seg(h, g));
-    tc_seg_fill<FP64>(h, W, g - W.seg_begin, o);
+    const int s = g - W.seg_begin;
+    const Dd ih = tc_seg_ih<FP64>(W, s);
+    tc_seg_phase<FP64>(W, s, p, ih, seg[k]);
+    if (!FP64) tc_seg_phase<FP64>(W, s, 1, ih, seg[k]);
+    if (p == 0) tc_seg_fill<FP64>(h, W, s, ih, seg[k]);
 }
 
 // The segment s of wave W that holds tile T.
@@ -261,17 +277,14 @@ __device__ inline const WaveDev &tc_find_tile(const PlanHdr &h, int T, int &s)
     return W;
 }
 
+// What a record holds beside the phases.  fin: the phases are finite.
 template <bool FP64>
-__device__ __forceinline__ void tc_store_record(const PlanHdr &h, const SegFill<FP64> &S, int t)
+__device__ __forceinline__ void tc_record_rest(const SegFill<FP64> &S, int t, bool fin, TileRec &r)
 {
-    TileRec r;
     r.i0 = (S.s0 / kTcTile + (t - S.first)) * kTcTile;
     r.s0 = S.s0;
     r.s1 = S.s1;
     r.tile_end = S.end;
-    const auto u = tc_u(S, max(r.i0, r.s0));
-    bool fin = tc_phase_at(S.p[0], u, r.phi);
-    fin = tc_phase_at(S.p[1], u, r.r) && fin;
     if constexpr (FP64) {  // non-finite data reach the output through the segment's factor
         r.u0 = __int_as_float(S.p[0].lo3);
         r.du = __int_as_float(S.p[1].lo3);
@@ -286,7 +299,37 @@ __device__ __forceinline__ void tc_store_record(const PlanHdr &h, const SegFill<
     r.ks = S.ks;
     r.n_mid = S.n_mid;
     r.c64 = S.c64;
+}
+
+template <bool FP64>
+__device__ __forceinline__ auto tc_tile_u(const SegFill<FP64> &S, int t)
+{
+    return tc_u(S, max((S.s0 / kTcTile + (t - S.first)) * kTcTile, S.s0));
+}
+
+__device__ __forceinline__ void tc_store_record(const PlanHdr &h, const SegFill<false> &S, int t)
+{
+    TileRec r;
+    const double u = tc_tile_u(S, t);
+    bool fin = tc_phase_at(S.p[0], u, r.phi);
+    fin = tc_phase_at(S.p[1], u, r.r) && fin;
+    tc_record_rest(S, t, fin, r);
     h.recs[t] = r;
+}
+
+// FP64: phase p of a record, and with the first one the rest.
+__device__ __forceinline__ void tc_store_record(const PlanHdr &h, const SegFill<true> &S, int t, int p)
+{
+    TileRec r;
+    tc_phase_at(S.p[p], tc_tile_u(S, t), r.phi);
+    longlong2 *dst = reinterpret_cast<longlong2 *>(h.recs[t].phi) + 2 * p;
+    dst[0] = make_longlong2(r.phi[0], r.phi[1]);
+    dst[1] = make_longlong2(r.phi[2], r.phi[3]);
+    if (p > 0) return;
+    tc_record_rest(S, t, true, r);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        reinterpret_cast<int4 *>(h.recs + t)[4 + q] = reinterpret_cast<const int4 *>(&r)[4 + q];
 }
 
 // The records of a block after the segments' (an even share of the tiles; seg: kTcFillSegs entries in
@@ -304,24 +347,31 @@ __device__ inline void tc_fill_records(const PlanHdr &h, SegFill<FP64> *seg)
         if (T >= T1) return;
         int s;
         const WaveDev &W = tc_find_tile(h, T, s);
-        SegFill<FP64> S;
-        tc_seg_fill<FP64>(h, W, s, S);
-        tc_store_record<FP64>(h, S, T);
+        SegFill<false> S;
+        const Dd ih = tc_seg_ih<false>(W, s);
+        tc_seg_phase<false>(W, s, 0, ih, S);
+        tc_seg_phase<false>(W, s, 1, ih, S);
+        tc_seg_fill<false>(h, W, s, ih, S);
+        tc_store_record(h, S, T);
         return;
     }
     while (T < T1) {  // uniform
         int s;
         const WaveDev &W = tc_find_tile(h, T, s);
-        if (threadIdx.x < kTcFillSegs) tc_cache_seg<FP64>(h, W.seg_begin + s + threadIdx.x, seg[threadIdx.x]);
+        tc_cache_segs<FP64>(h, W.seg_begin + s, seg);
         __syncthreads();
         const int Te = min(T1, seg[kTcFillSegs - 1].end);
-        for (int t = T + threadIdx.x; t < Te; t += blockDim.x) {
+        for (int i = threadIdx.x; i < (FP64 ? 2 : 1) * (Te - T); i += blockDim.x) {
+            const int p = i >= Te - T, t = T + i - p * (Te - T);
             int k = 0, ke = kTcFillSegs - 1;
             while (k < ke) {  // largest k with first <= t
                 const int mid = (k + ke + 1) >> 1;
                 if (seg[mid].first <= t) k = mid; else ke = mid - 1;
             }
-            tc_store_record<FP64>(h, seg[k], t);
+            if constexpr (FP64)
+                tc_store_record(h, seg[k], t, p);
+            else
+                tc_store_record(h, seg[k], t);
         }
         __syncthreads();
         T = Te;

@@ -263,3 +263,25 @@ def test_budget_moves_only_the_waves_that_do_not_fit(prec):
         F.few_batch_release(ctx.handle, b)
         for tr in trs:
             tr.release()
+
+
+def test_fp64_records_of_many_short_segments(gpu_ctx):
+    """About one sample a segment (many of them empty): blocks that fill tile records meet more segments than
+    they cache at once.  The call stays near its latency (140 us; 400 us while a block took 128 tiles
+    whatever their segments)."""
+    import torch
+    w = W.make_inputs(1.0e4, 1000, 10.0, W.mode_grid(4, 5), 7, 2.0, 8.0)
+    tr = RT.from_inputs(gpu_ctx, w)
+    out = RT.alloc_out(w.n_samples, False)
+    best = float("inf")
+    for _ in range(20):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_FP64, out=out)
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 1e3)
+    assert gpu_ctx.sync_status() == F.FEW_OK
+    assert rel_l2(to_host(out), oracle.waveform_inputs(w, nthreads=oracle_threads())) <= REL[F.FEW_FP64]
+    assert best <= 270.0
+    tr.release()
