@@ -186,7 +186,8 @@ typedef struct few_request {
  * Compute one waveform (Sec. 3.C interpolated summation of the Sec. 4 sum).  Validates and
  * plans on the host, then queues the fold (with the harmonics; FEW_FP64: a kernel before it) and the
  * summation on `stream`.  Mode sets with m <= 10 and |n| <= 31 (m = 0 alone: any n range of 63) are
- * summed on the tensor cores, others, and requests whose scratch fits only so, by a scalar chain.
+ * summed on the tensor cores; others, sets of a few frequencies where that is faster (few_plan_chain),
+ * and requests whose scratch fits only so, by a scalar chain.
  * n_samples == 0 is a no-op.  Errors: FEW_ERR_INVALID_ARG, FEW_ERR_STATE, FEW_ERR_RANGE,
  * FEW_ERR_LIMIT, FEW_ERR_BUDGET, FEW_ERR_NOMEM, FEW_ERR_CUDA.
  */
@@ -389,6 +390,17 @@ few_status few_last_timing(few_ctx *ctx, float *ms);
  */
 few_status few_plan_segments(const double *t_knots, int K, double t0, double dt, int64_t n_samples,
                              int64_t *seg_start);
+
+/*
+ * How few_waveform (and few_batch_plan) compute a request: *tensor_cores = 1 if on the tensor cores, 0 if by
+ * the scalar chain (its mode set is past the tensor cores' limits, or so small that the scalar chain is
+ * faster); and the device memory of its plan either way, to within 16 KB: *scalar_bytes, and *tc_bytes
+ * (0 past the limits).  Any of the three may be NULL.  Validates the modes, knots and samples as
+ * few_waveform does.
+ */
+few_status few_plan_chain(const double *t_knots, int K, const int *l, const int *m, const int *n, int N,
+                          double t0, double dt, int64_t n_samples, int prec, int *tensor_cores,
+                          size_t *scalar_bytes, size_t *tc_bytes);
 
 /*
  * Harmonic slot plan of a mode list: the distinct signed (m, n) frequencies that the m >= 0

@@ -437,12 +437,29 @@ few_status validate_request(const few_request &r, bool need_device_out)
     return FEW_OK;
 }
 
-// Whether a request's mode set fits the tensor-core summation (kTcMaxPairs, kTcMaxHalf).
-bool tc_fits(const few_request &r) { return r.traj->plan.tc_pairs > 0; }
+// Whether a mode set fits the tensor-core summation (kTcMaxPairs, kTcMaxHalf) and it is the faster one.
+// seg: the request's segment ranges [K].
+bool takes_tc(bool fp64, const SlotPlan &P, const std::vector<int64_t> &seg)
+{
+    if (P.tc_pairs == 0) return false;
+    const int K = (int)seg.size();
+    const TcShape s{P.tc_pairs, P.tc_ks, P.n_slots, (int)P.rows.size(), (int)P.mode_pair.size(), K};
+    TcWork w;
+    if (s.slots <= kTcAlwaysSlots)
+        for (int k = 0; k + 1 < K; ++k) w.add(seg[k], seg[k + 1]);
+    return tc_pays(fp64, s, w);
+}
+std::vector<int64_t> request_segments(const few_request &r)
+{
+    std::vector<int64_t> seg(r.traj->K);
+    segments(r.traj->t_host.data(), r.traj->K, r.t0, r.dt, r.n_samples, seg.data());
+    return seg;
+}
 
 // Build the host image of a plan for `n` requests of one precision; tc: by the tensor-core
-// summation (every request fits it).
-few_status build_image(few_ctx *c, const few_request *reqs, int n, bool tc, PlanImage &P)
+// summation (every request's mode set fits it); segs: their segment ranges.
+few_status build_image(few_ctx *c, const few_request *reqs, int n, bool tc, const std::vector<int64_t> *segs,
+                       PlanImage &P)
 {
     P.fp64 = reqs[0].prec == FEW_FP64;
     LaunchPlan &L = P.launch;
@@ -461,12 +478,7 @@ few_status build_image(few_ctx *c, const few_request *reqs, int n, bool tc, Plan
     const int occ = occupancy(c, L.variant, L.R, L.threads, L.smem);
     if (occ <= 0) return FEW_ERR_LIMIT;
     L.grid = c->sm_count * occ;
-    P.seg.resize(n);
-    for (int q = 0; q < n; ++q) {
-        const few_request &r = reqs[q];
-        P.seg[q].resize(r.traj->K);
-        segments(r.traj->t_host.data(), r.traj->K, r.t0, r.dt, r.n_samples, P.seg[q].data());
-    }
+    P.seg.assign(segs, segs + n);
     if (tc) {
         L.variant = P.fp64 ? kVariantTc64 : kVariantTc;
         int64_t tiles = 0;
@@ -1127,6 +1139,7 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream)
     if (!dev_scope.ok) return FEW_ERR_CUDA;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     PlanImage P;
+    const std::vector<int64_t> seg = request_segments(*req);
     const size_t out_bytes = (size_t)req->n_samples * (req->out_c64 ? 8 : 16);
     void *out_dev = req->out;
     bool staged = false;
@@ -1146,12 +1159,12 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream)
     void *blob = nullptr, *dout = nullptr;  // the plan, its scratch behind it; the staged output
     auto plan = [&](bool tc) {
         P = PlanImage();
-        few_status e = build_image(ctx, req, 1, tc, P);
+        few_status e = build_image(ctx, req, 1, tc, &seg, P);
         if (!e) e = dev_alloc(ctx, P.blob.size() + P.scratch_bytes, s, &blob);
         if (!e && staged && (e = dev_alloc(ctx, out_bytes, s, &dout))) dev_free(ctx, blob, s);
         return e;
     };
-    const bool tc = tc_fits(*req);
+    const bool tc = takes_tc(req->prec == FEW_FP64, req->traj->plan, seg);
     st = plan(tc);
     // the tensor-core plan may need more scratch than the scalar one (sparse mode sets)
     if (tc && (st == FEW_ERR_BUDGET || st == FEW_ERR_NOMEM)) st = plan(false);
@@ -1501,11 +1514,12 @@ few_status few_batch_plan(few_ctx *ctx, const few_request *reqs, int n, unsigned
         b->build_blocks = blocks;
     }
     // one part per summation variant
-    auto add_part = [&](const std::vector<few_request> &rq, bool tc) -> few_status {
+    auto add_part = [&](const std::vector<few_request> &rq, const std::vector<std::vector<int64_t>> &sg,
+                        bool tc) -> few_status {
         if (rq.empty()) return FEW_OK;
         const int nr = (int)rq.size();
         PlanImage P;
-        few_status e = build_image(ctx, rq.data(), nr, tc, P);
+        few_status e = build_image(ctx, rq.data(), nr, tc, sg.data(), P);
         if (e) return e;
         b->parts.emplace_back();
         few_batch::Part &part = b->parts.back();
@@ -1523,8 +1537,11 @@ few_status few_batch_plan(few_ctx *ctx, const few_request *reqs, int n, unsigned
     // each time.
     std::vector<int> order;
     std::vector<char> on_tc(n);
-    for (int q = 0; q < n; ++q)
-        if ((on_tc[q] = tc_fits(reqs[q]))) order.push_back(q);
+    std::vector<std::vector<int64_t>> seg(n);
+    for (int q = 0; q < n; ++q) {
+        seg[q] = request_segments(reqs[q]);
+        if ((on_tc[q] = takes_tc(reqs[q].prec == FEW_FP64, reqs[q].traj->plan, seg[q]))) order.push_back(q);
+    }
     auto saves = [&](int q) {
         const few_traj *tr = reqs[q].traj;
         const bool fp64 = reqs[q].prec == FEW_FP64;
@@ -1536,10 +1553,14 @@ few_status few_batch_plan(few_ctx *ctx, const few_request *reqs, int n, unsigned
     };
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return saves(a) > saves(b); });
     for (size_t moved = 0;;) {
-        std::vector<few_request> tc_reqs, other;
-        for (int q = 0; q < n; ++q) (on_tc[q] ? tc_reqs : other).push_back(reqs[q]);
-        st = add_part(tc_reqs, true);
-        if (!st) st = add_part(other, false);
+        std::vector<few_request> rq[2];  // by the scalar chain, on the tensor cores
+        std::vector<std::vector<int64_t>> sg[2];
+        for (int q = 0; q < n; ++q) {
+            rq[on_tc[q]].push_back(reqs[q]);
+            sg[on_tc[q]].push_back(seg[q]);
+        }
+        st = add_part(rq[1], sg[1], true);
+        if (!st) st = add_part(rq[0], sg[0], false);
         if ((st != FEW_ERR_BUDGET && st != FEW_ERR_NOMEM) || moved == order.size()) break;
         drop_parts();
         const size_t next = std::min(order.size(), 2 * moved + 1);
@@ -1702,6 +1723,36 @@ few_status few_plan_segments(const double *t_knots, int K, double t0, double dt,
 {
     if (!seg_start) return FEW_ERR_INVALID_ARG;
     return segments(t_knots, K, t0, dt, n_samples, seg_start);
+}
+
+few_status few_plan_chain(const double *t_knots, int K, const int *l, const int *m, const int *n, int N,
+                          double t0, double dt, int64_t n_samples, int prec, int *tensor_cores,
+                          size_t *scalar_bytes, size_t *tc_bytes)
+{
+    if (prec != FEW_FP64 && prec != FEW_MIXED) return FEW_ERR_INVALID_ARG;
+    SlotPlan P;
+    few_status st = plan_slots(l, m, n, N, P);
+    if (st) return st;
+    std::vector<int64_t> seg(K > 0 ? K : 0);
+    if ((st = segments(t_knots, K, t0, dt, n_samples, seg.data()))) return st;
+    const bool fp64 = prec == FEW_FP64;
+    if (tensor_cores) *tensor_cores = takes_tc(fp64, P, seg) ? 1 : 0;
+    // the layout of build_image; the plan itself: headers, the CTAs' starts, two ints a knot
+    const size_t S = K - 1, plan = 16384 + 2 * sizeof(int) * (size_t)K;
+    const size_t ylm = P.pair_lm.size() * 2 * sizeof(double2);
+    size_t anchors = 0, tiles = 0;
+    for (int k = 0; k + 1 < K; ++k) {
+        anchors += anchors_in_segment((int)seg[k], (int)seg[k + 1]);
+        tiles += tiles_in_segment((int)seg[k], (int)seg[k + 1]);
+    }
+    if (scalar_bytes)
+        *scalar_bytes = plan + ylm + S * P.n_slots * sum_slot_bytes(fp64 ? kVariantFp64 : kVariantScalar) +
+                        (fp64 ? 0 : anchors * sizeof(Anchor));
+    if (tc_bytes)
+        *tc_bytes = P.tc_pairs == 0 ? 0
+                                    : plan + ylm + S * tc_segment_bytes(fp64, P.tc_pairs, P.tc_ks) +
+                                          tiles * sizeof(TileRec);
+    return FEW_OK;
 }
 
 few_status few_mode_slots(const int *l, const int *m, const int *n, int N, int *n_slots, int *n_rows)

@@ -267,6 +267,51 @@ inline int tiles_in_segment(int s_begin, int s_end)
 {
     return s_end > s_begin ? (s_end - 1) / kTcTile - s_begin / kTcTile + 1 : 0;
 }
+// What the choice between the two summations looks at: a mode set and a request's segments.
+struct TcShape {
+    int pairs, ks, slots, rows, modes, K;
+};
+struct TcWork {
+    double samples = 0.0, segs = 0.0, passes = 0.0, tiles = 0.0;  // segments with samples; passes of 256
+    void add(long long s0, long long s1)
+    {
+        if (s1 <= s0) return;
+        samples += (double)(s1 - s0);
+        segs += 1.0;
+        passes += (double)((s1 - s0 + 255) / 256);
+        tiles += tiles_in_segment((int)s0, (int)s1);
+    }
+};
+// Sets of more frequencies are always faster on the tensor cores.
+constexpr int kTcAlwaysSlots = 128;
+// Whether the tensor-core summation is the faster one (not past kTcMaxPairs, kTcMaxHalf).  A tile, a
+// segment's table and an FP64 record cost about the same for one mode as for a hundred, a slot of the scalar
+// chain next to nothing, so sets of a few frequencies stay with the scalar chain where there is enough of the
+// one or the other.  Both sides in us, as measured (tensor cores against scalar):
+//   mixed, long waveforms:  40 M samples, one frequency pair (m, n) = (2, 0): 884, 740; 18 slots: 885, 979;
+//                           3.2 M samples, one pair: 82, 90
+//   FP64, short segments:   one pair: 4096 knots, 20,000 samples 371, 229; 1000 knots, 1,000 samples
+//                           110, 77; 100 knots, 20,000 samples 38, 61; m = 10: 4096 knots, a million samples
+//                           1159, 886; m = 10, n = 0 and 30: 300 knots, 20,000 samples 135, 110;
+//                           99 slots: 4096 knots, 20,000 samples 534, 784
+// The estimates are fits to such times, good to 20 %; where they are near one another the tensor cores, the more
+// exact of the two, are taken (FP64).
+inline bool tc_pays(bool fp64, const TcShape &s, const TcWork &w)
+{
+    if (s.slots > kTcAlwaysSlots) return true;
+    if (!fp64) {
+        const double scalar = 34.0 + 0.037 * w.segs + 1e-6 * w.samples * (16.1 + 0.3 * s.slots + 0.315 * s.rows);
+        const double tc = 13.0 + 0.012 * w.segs + w.tiles * 0.93e-3 * tc_tile_cost(false, s.pairs, s.ks) / 152.0;
+        return tc < scalar;
+    }
+    const double scalar = 36.0 + 0.005 * s.K + w.segs * (0.003 + 0.00015 * s.modes) +
+                          w.passes * (0.03 + 0.0012 * s.slots + 0.00075 * s.rows) +
+                          0.7e-3 * w.samples * (0.27 + 0.018 * s.slots + 0.012 * s.rows);
+    const double tc = (8 * s.K + 2048 <= kPlanParamBytes ? 28.0 : 47.0) +
+                      w.segs * (0.045 + s.pairs * (0.006 + 0.0045 * (s.ks - 1)) + 0.0001 * s.modes) +
+                      w.tiles * (0.6 + 0.85 * s.pairs + 0.7 * (s.ks - 1)) / 152.0;
+    return 0.9 * tc < scalar;
+}
 cudaError_t tc_configure();
 cudaError_t tc64_configure();
 cudaError_t launch_fold_tc64(const PlanHdr *hdr_dev, int total_segs, int total_tiles, int sm_count, cudaStream_t st);

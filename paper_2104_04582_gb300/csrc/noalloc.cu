@@ -149,8 +149,10 @@ extern "C" few_status few_waveform_noalloc(few_ctx *ctx, const few_request *req,
     // and their scales instead of anchors and folded coefficients) is taken where it fits too
     if (blob_plain + fcoef_bytes + ylm_bytes + anc_bytes > kScratchBytes) return FEW_ERR_LIMIT;
     int n_tiles = 0;
-    if (v.tc_pairs > 0)
-        for (int k = 0; k + 1 < K; ++k) n_tiles += tiles_in_segment(seg[k], seg[k + 1]);
+    TcWork work;
+    for (int k = 0; k + 1 < K; ++k) work.add(seg[k], seg[k + 1]);
+    const TcShape shape{v.tc_pairs, v.tc_ks, v.n_slots, v.dev.n_rows, v.dev.N, K};
+    if (v.tc_pairs > 0 && tc_pays(fp64, shape, work)) n_tiles = (int)work.tiles;
     const size_t tab_bytes =
         up((size_t)S * (fp64 ? tc64_table_bytes(v.tc_pairs, v.tc_ks) : tc_table_bytes(v.tc_pairs, v.tc_ks)), 256);
     const size_t inv_bytes = up((size_t)S * (fp64 ? sizeof(TcSeg64) : sizeof(float)), 256);

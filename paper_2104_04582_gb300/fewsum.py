@@ -45,7 +45,7 @@ EXPORTED = [
     "few_get_tiles", "few_plan_segments", "few_mode_slots", "few_ctx_set_timing",
     "few_last_timing", "few_phase_samples", "few_waveform_noalloc",
     "few_mode_select", "few_direct_sum", "few_basis_create", "few_basis_release",
-    "few_rb_amplitudes", "few_selftest_wait_expiry", "few_plan_cta_slices",
+    "few_rb_amplitudes", "few_selftest_wait_expiry", "few_plan_cta_slices", "few_plan_chain",
 ]
 
 
@@ -136,6 +136,9 @@ def load(path: Optional[str] = None) -> ctypes.CDLL:
             "few_plan_segments": (ctypes.c_int, [_dp, ctypes.c_int, ctypes.c_double,
                                                  ctypes.c_double, ctypes.c_int64, _i64p]),
             "few_mode_slots": (ctypes.c_int, [_ip, _ip, _ip, ctypes.c_int, _ip, _ip]),
+            "few_plan_chain": (ctypes.c_int, [_dp, ctypes.c_int, _ip, _ip, _ip, ctypes.c_int, ctypes.c_double,
+                                              ctypes.c_double, ctypes.c_int64, ctypes.c_int, _ip,
+                                              ctypes.POINTER(ctypes.c_size_t), ctypes.POINTER(ctypes.c_size_t)]),
             "few_plan_cta_slices": (ctypes.c_int, [ctypes.c_int, _i64p, _ip, _ip, ctypes.c_int,
                                                    ctypes.c_int, _ip, _ip]),
         }
@@ -378,6 +381,19 @@ def few_plan_segments(t_knots, t0: float, dt: float, n_samples: int) -> np.ndarr
                                   int(n_samples), seg.ctypes.data_as(_i64p))
     _check("few_plan_segments", st)
     return seg
+
+
+def few_plan_chain(t_knots, modes, t0: float, dt: float, n_samples: int, prec: int):
+    """(on the tensor cores?, plan bytes by the scalar chain, plan bytes on the tensor cores or 0) of a
+    request (host only)."""
+    t, md = _f64(t_knots), _i32(modes).reshape(-1, 3)
+    l, m, n = (_i32(md[:, k]) for k in range(3))
+    on, sb, tb = ctypes.c_int(), ctypes.c_size_t(), ctypes.c_size_t()
+    st = load().few_plan_chain(t.ctypes.data_as(_dp), len(t), l.ctypes.data_as(_ip), m.ctypes.data_as(_ip),
+                               n.ctypes.data_as(_ip), len(md), float(t0), float(dt), int(n_samples), int(prec),
+                               ctypes.byref(on), ctypes.byref(sb), ctypes.byref(tb))
+    _check("few_plan_chain", st)
+    return bool(on.value), int(sb.value), int(tb.value)
 
 
 def few_plan_cta_slices(seg_starts, n_slots, grid: int, pass_samples: int):

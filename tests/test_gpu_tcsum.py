@@ -285,3 +285,35 @@ def test_fp64_records_of_many_short_segments(gpu_ctx):
     assert rel_l2(to_host(out), oracle.waveform_inputs(w, nthreads=oracle_threads())) <= REL[F.FEW_FP64]
     assert best <= 270.0
     tr.release()
+
+
+@pytest.mark.parametrize("modes,K,n,prec", [
+    (_modes([2], [0]), 1000, 1000, F.FEW_FP64), (_modes([2], [0]), 100, 20000, F.FEW_FP64),
+    (_modes([2], [0]), 20, 24000000, F.FEW_MIXED), (_modes([2], [0]), 20, 300000, F.FEW_MIXED),
+    (W.mode_grid(4, 5), 60, 50000, F.FEW_MIXED), (_modes([11], [0, 1], l=11), 40, 20000, F.FEW_FP64)])
+def test_requests_take_the_chain_that_few_plan_chain_names(gpu_ctx, modes, K, n, prec):
+    """The memory that a planned batch holds is that of the chain it names, and so are the two entry points'
+    results."""
+    import torch
+    w = W.make_inputs(max(n, K) * 10.0, K, 10.0, modes, 5, 2.0, 8.0, n_samples=n)
+    on, scalar_bytes, tc_bytes = F.few_plan_chain(w.t_knots, w.modes, w.t0, w.dt, n, prec)
+    tr = RT.from_inputs(gpu_ctx, w)
+    out = RT.alloc_out(n, prec == F.FEW_MIXED)
+    req = RT.request(tr, out, n, w.t0, w.dt, w.theta, w.phi, prec)
+    held = gpu_ctx.memory()[0]
+    b = F.few_batch_plan(gpu_ctx.handle, [req], 0)
+    held = gpu_ctx.memory()[0] - held
+    F.few_batch_release(gpu_ctx.handle, b)
+    assert abs(held - (tc_bytes if on else scalar_bytes)) <= 16384 + 1024
+    F.few_waveform(gpu_ctx.handle, req, RT.current_stream())
+    if min(scalar_bytes, tc_bytes or scalar_bytes) < (8 << 20):  # of the 16 MiB that the other entry point has
+        other = torch.empty_like(out)
+        F.few_waveform_noalloc(gpu_ctx.handle, RT.request(tr, other, n, w.t0, w.dt, w.theta, w.phi, prec),
+                               RT.current_stream())
+        np.testing.assert_array_equal(to_host(other), to_host(out))
+    torch.cuda.synchronize()
+    assert gpu_ctx.sync_status() == F.FEW_OK
+    i0, count = n // 3, min(n, 4000)
+    g, o = to_host(out[i0:i0 + count]), oracle.waveform_inputs(w, i0, min(count, n - i0), nthreads=oracle_threads())
+    assert rel_l2(g, o) <= REL[prec] if prec == F.FEW_FP64 else oracle.mismatch(g, o) <= MIXED_MISMATCH
+    tr.release()
