@@ -63,15 +63,17 @@ struct alignas(128) TileRec {
     int i0, s0, s1;       // first sample of lane 0; the segment's samples [s0, s1)
     int tile_end;         // first tile after the segment
     float u0, du;         // mixed: u of sample i is u0 + (i - s0) du; FP64: the next 32 bits (units of
-                          //   2^-96 turn) of the phases' c3, as int bits
+                          //   2^-96 turn) of the two phases' c3, as int bits
     const void *seg;      // mixed: float, inverse of the table's power-of-two scale; FP64: TcSeg64
     const unsigned char *tab;  // the segment's operand table
     void *out;
     int pairs, ks;        // row pairs, K steps of 16 (8 powers of z_r each)
     int n_mid;            // centre of the n range
     int c64;
+    // FP64: pairs also holds ks and c64 (tc64_shape), whose own words hold the next 32 bits of the phases' c2
 };
 static_assert(sizeof(TileRec) == 128, "one line");
+__host__ __device__ inline int tc64_shape(int pairs, int ks, int c64) { return pairs | ks << 8 | c64 << 16; }
 // FP64 tensor-core summation (tcsum64.cu): what a segment's tiles read beside its table.
 constexpr int kTc64Slices = 7;  // 8-bit digits per operand
 struct TcSeg64 {

@@ -393,8 +393,7 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *hp)
         uint32_t chunk = 0;
         bool ok = true;
         for (int T = T0; T < T1 && ok; ++T) {
-            const int4 shape = *reinterpret_cast<const int4 *>(&recs[T].pairs);
-            const int pairs = __shfl_sync(0xffffffffu, shape.x, 0), ks = __shfl_sync(0xffffffffu, shape.y, 0);
+            const int shape = __shfl_sync(0xffffffffu, recs[T].pairs, 0), pairs = shape & 255, ks = shape >> 8 & 255;
             const int g = (T - T0) & 1;
             if (T == tend) {  // the table's first tile: the previous one's MMAs must have completed
                 tend = recs[T].tile_end;
@@ -449,9 +448,9 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *hp)
         for (int T = T0 + group; T < T1; T += kT64Groups) {
             const TileRec *rp = recs + T;
             const int4 span = *reinterpret_cast<const int4 *>(&rp->i0);      // i0, s0, s1, tile_end
-            const int4 shape = *reinterpret_cast<const int4 *>(&rp->pairs);  // pairs, ks, n_mid, c64
-            const int pairs = shape.x;
-            for (; counted < T; ++counted) chunk += (uint32_t)recs[counted].pairs;
+            const int4 shape = *reinterpret_cast<const int4 *>(&rp->pairs);  // tc64_shape, c2's (phi), n_mid, c2's (r)
+            const int pairs = shape.x & 255;
+            for (; counted < T; ++counted) chunk += (uint32_t)(recs[counted].pairs & 255);
             const int i = span.x + lane;
             const uint32_t v = (uint32_t)max(i - max(span.x, span.y), 0);
             TileRec ph;
@@ -459,9 +458,9 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *hp)
             for (int k = 0; k < 4; ++k)
                 reinterpret_cast<int4 *>(&ph)[k] = reinterpret_cast<const int4 *>(rp)[k];
             const int2 lo3 = *reinterpret_cast<const int2 *>(&rp->u0);  // of c3: phi, r
-            const long long v3 = (long long)(v * v * v);
-            const unsigned long long fr = phase_fixed(ph.r, v) + (unsigned long long)(lo3.y * v3 >> 32);
-            const unsigned long long fphi = phase_fixed(ph.phi, v) + (unsigned long long)(lo3.x * v3 >> 32);
+            const long long v2 = (long long)(v * v), v3 = (long long)(v * v * v);
+            const unsigned long long fr = phase_fixed(ph.r, v) + (unsigned long long)((lo3.y * v3 + shape.w * v2) >> 32);
+            const unsigned long long fphi = phase_fixed(ph.phi, v) + (unsigned long long)((lo3.x * v3 + shape.y * v2) >> 32);
             const TcSeg64 *sg = static_cast<const TcSeg64 *>(rp->seg);
             // (lanes outside the segment take its first or last sample's u: sums stay in range)
             const double u = (fma((double)min(max(i, span.y), span.z - 1), sg->dt, sg->t0) - sg->tk) * sg->ih;
@@ -572,7 +571,7 @@ __global__ void __launch_bounds__(kT64Threads, 1) k_sum_tc64(const PlanHdr *hp)
                 }
                 const double yr = fma(hr, fc, hi * fs) * sg->inv2, yi = fma(hi, fc, -hr * fs) * sg->inv2;
                 void *out = rp->out;
-                if (shape.w)
+                if (shape.x >> 16)
                     reinterpret_cast<float2 *>(out)[i] = make_float2((float)yr, (float)yi);
                 else
                     reinterpret_cast<double2 *>(out)[i] = make_double2(yr, yi);

@@ -82,6 +82,16 @@ __device__ __forceinline__ long long dd_turns_fixed(const Dd &a)
     return (long long)((unsigned long long)turns_fixed(a.h) + (unsigned long long)turns_fixed(a.l));
 }
 
+// The same with the next 32 bits (units of 2^-96 turn).
+__device__ __forceinline__ long long tc_fixed96(const Dd &a, int &lo)
+{
+    const double x = (a.h - rint(a.h)) * 18446744073709551616.0, y = a.l * 18446744073709551616.0;
+    const long long cx = __double2ll_rn(x), cy = __double2ll_rn(y);
+    const double r = (x - (double)cx) + (y - (double)cy), k = rint(r);
+    lo = __double2int_rn((r - k) * 4294967296.0);
+    return (long long)((unsigned long long)cx + (unsigned long long)cy + (unsigned long long)(long long)k);
+}
+
 __device__ __forceinline__ int tc_wave_of_seg(const PlanHdr &h, int g)
 {
     int lo = 0, hi = h.n_waves - 1;
@@ -101,7 +111,7 @@ struct PhaseFill {  // the phase c, its derivative per sample d, half the second
     double c[4], d[3], q[2];
     long long c3;
 };
-struct PhaseFill64 {  // the same in pairs; v^3 reaches 2^21, so c3 also has its next 32 bits (2^-96 turn)
+struct PhaseFill64 {  // the same in pairs; v^3 reaches 2^21, so c3 also has its next 32 bits (2^-96 turn; c2: tc_fixed96)
     Dd c[4], d[3], q[2];
     long long c3;
     int lo3;
@@ -166,10 +176,7 @@ __device__ inline void tc_phase_fill(const double *y, double h, Dd ih, double dt
     o.d[2] = dd_scale(c3, 3.0);
     o.q[0] = dd_mul(o.q[0], w);
     o.q[1] = dd_mul(o.d[2], w);
-    const Dd f = dd_mul(dd_mul(c3, w), w);
-    const double x3 = (f.h - rint(f.h)) * 18446744073709551616.0;
-    o.c3 = __double2ll_rn(x3);
-    o.lo3 = __double2int_rn(((x3 - (double)o.c3) + f.l * 18446744073709551616.0) * 4294967296.0);
+    o.c3 = tc_fixed96(dd_mul(dd_mul(c3, w), w), o.lo3);
 }
 
 __device__ __forceinline__ double tc_u(const SegFill<false> &S, int i)
@@ -190,14 +197,15 @@ __device__ __forceinline__ bool tc_phase_at(const PhaseFill &p, double u, long l
     o[3] = p.c3;
     return (__double2hiint(f) & 0x7ff00000) != 0x7ff00000;
 }
-__device__ __forceinline__ bool tc_phase_at(const PhaseFill64 &p, const Dd &u, long long (&o)[4])
+// lo2: c2's next 32 bits.  v^2 reaches 2^14: rounded to 2^-64 turn, c2 alone was wrong by up to 3e-15 rad at a
+// tile's end, n times that in the n-th power, which showed wherever the phases themselves are small.
+__device__ __forceinline__ void tc_phase_at(const PhaseFill64 &p, const Dd &u, long long (&o)[4], int &lo2)
 {
     o[0] = dd_turns_fixed(
         dd_add(dd_mul(dd_add(dd_mul(dd_add(dd_mul(p.c[3], u), p.c[2]), u), p.c[1]), u), p.c[0]));
     o[1] = dd_turns_fixed(dd_add(dd_mul(dd_add(dd_mul(p.d[2], u), p.d[1]), u), p.d[0]));
-    o[2] = dd_turns_fixed(dd_add(dd_mul(p.q[1], u), p.q[0]));
+    o[2] = tc_fixed96(dd_add(dd_mul(p.q[1], u), p.q[0]), lo2);
     o[3] = p.c3;
-    return true;
 }
 
 template <bool FP64>
@@ -320,16 +328,19 @@ __device__ __forceinline__ void tc_store_record(const PlanHdr &h, const SegFill<
 // FP64: phase p of a record, and with the first one the rest.
 __device__ __forceinline__ void tc_store_record(const PlanHdr &h, const SegFill<true> &S, int t, int p)
 {
-    TileRec r;
-    tc_phase_at(S.p[p], tc_tile_u(S, t), r.phi);
-    longlong2 *dst = reinterpret_cast<longlong2 *>(h.recs[t].phi) + 2 * p;
-    dst[0] = make_longlong2(r.phi[0], r.phi[1]);
-    dst[1] = make_longlong2(r.phi[2], r.phi[3]);
+    TileRec r, &dst = h.recs[t];
+    int lo2;
+    tc_phase_at(S.p[p], tc_tile_u(S, t), r.phi, lo2);
+    longlong2 *c = reinterpret_cast<longlong2 *>(dst.phi) + 2 * p;
+    c[0] = make_longlong2(r.phi[0], r.phi[1]);
+    c[1] = make_longlong2(r.phi[2], r.phi[3]);
+    (p ? dst.c64 : dst.ks) = lo2;
     if (p > 0) return;
     tc_record_rest(S, t, true, r);
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-        reinterpret_cast<int4 *>(h.recs + t)[4 + q] = reinterpret_cast<const int4 *>(&r)[4 + q];
+    for (int q = 4; q < 7; ++q) reinterpret_cast<int4 *>(&dst)[q] = reinterpret_cast<const int4 *>(&r)[q];
+    dst.pairs = tc64_shape(r.pairs, r.ks, r.c64);
+    dst.n_mid = r.n_mid;
 }
 
 // The records of a block after the segments' (an even share of the tiles; seg: kTcFillSegs entries in

@@ -317,3 +317,35 @@ def test_requests_take_the_chain_that_few_plan_chain_names(gpu_ctx, modes, K, n,
     g, o = to_host(out[i0:i0 + count]), oracle.waveform_inputs(w, i0, min(count, n - i0), nthreads=oracle_threads())
     assert rel_l2(g, o) <= REL[prec] if prec == F.FEW_FP64 else oracle.mismatch(g, o) <= MIXED_MISMATCH
     tr.release()
+
+
+@pytest.mark.parametrize("span", [1e-4, 2e-2, 1.0])
+def test_fp64_phase_of_one_frequency(gpu_ctx, span):
+    """One frequency (n = 31, m = 0) over a small phase `span` (rad, quadratic in time: the splines reproduce
+    it): the sample's phase against extended precision.  The expansion's coefficients c0 and c1 are rounded
+    to 2^-65 turn, the latter times 127 samples and n: 31 x 127 x 2^-65 x 2 pi = 7e-16; sine and cosine,
+    digits and sums 2^-50; the phases themselves and the oracle of this test 31 x 2^-53 x span: 4e-15 +
+    4e-15 span in all.  (c2 rounded likewise: 31 x 127^2 x 2^-65 x 2 pi = 8.5e-14.)"""
+    import torch
+    K, n, dt = 60, 20000, 10.0
+    w = W.make_inputs(n * dt, K, dt, _modes([0], [31]), 3, n_samples=n)
+    LD = np.longdouble
+
+    def phase(t):
+        x = np.asarray(t, dtype=LD) / LD(n * dt)
+        return LD(span) * (LD(0.3) + LD(0.5) * x + LD(0.2) * x * x)
+
+    w.phi_r = phase(w.t_knots).astype(np.float64)
+    w.phi_phi = np.zeros(K)
+    w.amp_re, w.amp_im = np.ones((K, 1)), np.zeros((K, 1))
+    assert F.few_plan_chain(w.t_knots, w.modes, w.t0, dt, n, F.FEW_FP64)[0]
+    tr = RT.from_inputs(gpu_ctx, w)
+    h = to_host(RT.waveform_inputs(gpu_ctx, tr, w, F.FEW_FP64))
+    torch.cuda.synchronize()
+    assert gpu_ctx.sync_status() == F.FEW_OK
+    tr.release()
+    a = -31 * (phase(np.arange(n) * dt) - phase(0.0))
+    c, s = np.cos(a), np.sin(a)
+    re, im = LD(h[0].real), LD(h[0].imag)
+    err = np.hypot(h.real - (re * c - im * s), h.imag - (re * s + im * c)) / np.hypot(re, im)
+    assert float(err.max()) <= 4e-15 + 4e-15 * span
