@@ -242,3 +242,39 @@ def test_rb_fp64_digit_slices(gpu_ctx, M, Nb, N, kind):
     bad = ~np.isfinite(alpha).all(axis=1)[:, None] | ~np.isfinite(basis).all(axis=0)[None, :]
     assert np.all(np.abs(g - ref)[~bad] <= bound[~bad])
     assert not np.isfinite(g[bad]).any()
+
+
+@pytest.mark.parametrize("kind", ["unit", "blocks"])
+def test_rb_fp64_localised_basis(gpu_ctx, kind):
+    """A localised basis (each mode in one vector, or in a few neighbouring ones) and decaying coefficients:
+    most outputs are below the digit product's guard and take the plain chain.  Bound of
+    test_rb_fp64_digit_slices; and the call stays below the 1.7 ms that the plain chain of every output
+    takes (it took 2.6 ms with one output at a time in flight a thread)."""
+    import torch
+    M, Nb, N = 400, 99, 3843
+    rng = np.random.default_rng(5)
+    alpha = (rng.standard_normal((M, Nb)) + 1j * rng.standard_normal((M, Nb))) * np.exp(-np.arange(Nb) / 5.0)
+    basis = rng.standard_normal((Nb, N)) + 1j * rng.standard_normal((Nb, N))
+    place = np.abs(np.arange(N)[None, :] * Nb // N - np.arange(Nb)[:, None])
+    basis *= (place == 0) if kind == "unit" else np.exp(-place)
+    nu = rng.uniform(0.5, 2.0, M)
+    h = F.few_basis_create(gpu_ctx.handle, basis.real, basis.imag, RT.current_stream())
+    try:
+        dev = [_dev(alpha.real), _dev(alpha.imag), _dev(nu)]
+        re, im = (torch.empty(M, N, dtype=torch.float64, device="cuda") for _ in range(2))
+        best = float("inf")
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            F.few_rb_amplitudes(gpu_ctx.handle, h, dev[0], dev[1], re, im, dev[2], F.FEW_FP64, RT.current_stream())
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b) * 1e3)
+        assert gpu_ctx.sync_status() == F.FEW_OK
+        plain = alpha @ basis
+        s = (nu / np.linalg.norm(plain, axis=1))[:, None]
+        g = to_host(re) + 1j * to_host(im)
+        assert np.all(np.abs(g - s * plain) <= 1e-13 * s * (np.abs(alpha) @ np.abs(basis)) + 1e-300)
+        assert best <= 1700.0
+    finally:
+        F.few_basis_release(gpu_ctx.handle, h)
