@@ -275,7 +275,9 @@ few_status few_direct_sum(few_ctx *ctx, const double *phi_phi_dev, const double 
  *     until that work completes).  1 <= Nb <= FEW_MAX_BASIS, N >= 1.
  * The library keeps an FP64 copy of B, the Gram matrix B B^H (for the renormalisation) and the
  * scaled, split, packed fp16 operand of the tensor-core product, about 16 x Nb x N + 12 x Nb x N
- * bytes.
+ * bytes; and, while there is room, the digit slices of the FEW_FP64 product, about 72 x Nb x N bytes more.
+ * The slices are given up (after a wait for the device) when another allocation of the context finds no
+ * room, unless a captured graph uses them; FEW_FP64 amplitudes then run on the FP64 pipe.
  * Asynchronous on `stream`; the handle is usable on any stream ordered after it.
  * Errors: FEW_ERR_INVALID_ARG, FEW_ERR_LIMIT (Nb too large), FEW_ERR_BUDGET, FEW_ERR_NOMEM,
  * FEW_ERR_CUDA.

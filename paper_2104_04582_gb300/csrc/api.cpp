@@ -92,6 +92,24 @@ struct PinnedPool {
 struct few_traj;
 struct few_batch;
 
+// Reduced basis (Sec. 3.E): FP64 B, its transposed Gram matrix in FP64 and FP32, and the split
+// fp16 operand of the tensor-core product, in one device allocation; the FP64 product's digit slices in
+// another, which is given up when the context has no room for something else (give_up_slices).
+struct few_basis {
+    few_ctx *ctx = nullptr;
+    int Nb = 0, N = 0;
+    void *dmem = nullptr;
+    const double *bre = nullptr, *bim = nullptr;
+    const double2 *gt64 = nullptr;
+    const float2 *gt32 = nullptr;
+    const int *bexp = nullptr;
+    const unsigned char *bpack = nullptr;
+    void *slices = nullptr;  // exponents, then the slices (null: no room for them)
+    const int *bexp64 = nullptr;
+    const unsigned char *bpack64 = nullptr;
+    mutable bool captured = false;  // a captured graph of the caller's reads the slices: they stay
+};
+
 struct few_ctx {
     int device = 0;
     int sm_count = 0;
@@ -134,7 +152,7 @@ struct NvtxRange {
     NvtxRange &operator=(const NvtxRange &) = delete;
 };
 
-few_status dev_alloc(few_ctx *c, size_t bytes, cudaStream_t st, void **out)
+few_status try_alloc(few_ctx *c, size_t bytes, cudaStream_t st, void **out)
 {
     *out = nullptr;
     if (bytes == 0) bytes = 256;
@@ -149,6 +167,38 @@ few_status dev_alloc(few_ctx *c, size_t bytes, cudaStream_t st, void **out)
     c->in_use += bytes;
     c->sizes[*out] = bytes;
     return FEW_OK;
+}
+
+void dev_free(few_ctx *c, void *p, cudaStream_t st);
+
+// Frees the digit slices of the context's bases (the FP64 amplitudes then take the plain chain), once all
+// work that may read them has ended.  False if there are none to free, or while `st` is being captured.
+bool give_up_slices(few_ctx *c, cudaStream_t st)
+{
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    const bool known = cudaStreamIsCapturing(st, &capture) == cudaSuccess;
+    bool any = false;
+    for (const few_basis *b : c->bases) any |= b->slices && !b->captured;
+    if (!known || capture != cudaStreamCaptureStatusNone || !any || cudaDeviceSynchronize() != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    for (few_basis *b : c->bases) {
+        if (!b->slices || b->captured) continue;
+        dev_free(c, b->slices, c->internal);
+        b->slices = nullptr;
+        b->bexp64 = nullptr;
+        b->bpack64 = nullptr;
+    }
+    cudaStreamSynchronize(c->internal);
+    return true;
+}
+
+few_status dev_alloc(few_ctx *c, size_t bytes, cudaStream_t st, void **out)
+{
+    few_status e = try_alloc(c, bytes, st, out);
+    if ((e == FEW_ERR_BUDGET || e == FEW_ERR_NOMEM) && give_up_slices(c, st)) e = try_alloc(c, bytes, st, out);
+    return e;
 }
 
 void dev_free(few_ctx *c, void *p, cudaStream_t st)
@@ -1305,21 +1355,6 @@ few_status few_direct_sum(few_ctx *ctx, const double *pphi, const double *pr, co
     return st;
 }
 
-// Reduced basis (Sec. 3.E): FP64 B, its transposed Gram matrix in FP64 and FP32, and the split
-// bf16 operand of the tensor-core product, in one device allocation.
-struct few_basis {
-    few_ctx *ctx = nullptr;
-    int Nb = 0, N = 0;
-    void *dmem = nullptr;
-    const double *bre = nullptr, *bim = nullptr;
-    const double2 *gt64 = nullptr;
-    const float2 *gt32 = nullptr;
-    const int *bexp = nullptr;
-    const unsigned char *bpack = nullptr;
-    const int *bexp64 = nullptr;
-    const unsigned char *bpack64 = nullptr;  // digit slices (null: no room for them)
-};
-
 few_status few_basis_create(few_ctx *ctx, const double *b_re, const double *b_im, int Nb, int N,
                             few_mem where, void *stream, few_basis **out)
 {
@@ -1339,14 +1374,10 @@ few_status few_basis_create(few_ctx *ctx, const double *b_re, const double *b_im
     const size_t ex = align_up(sizeof(int) * (size_t)L.modes_padded, 256);
     const size_t ex64 = align_up(sizeof(int) * (size_t)rb64_modes(N), 256);
     const size_t plain = align_up(2 * b_bytes + g64 + g32 + ex + L.bpack_bytes, 256);
-    void *d = nullptr;
-    bool digits = true;
-    few_status st = dev_alloc(ctx, plain + ex64 + rb64_basis_bytes(Nb, N), s, &d);
-    if (st) {
-        digits = false;
-        st = dev_alloc(ctx, plain, s, &d);
-    }
+    void *d = nullptr, *slices = nullptr;
+    few_status st = dev_alloc(ctx, plain, s, &d);
     if (st) return st;
+    const bool digits = try_alloc(ctx, ex64 + rb64_basis_bytes(Nb, N), s, &slices) == FEW_OK;
     unsigned char *p = static_cast<unsigned char *>(d);
     double *bre = reinterpret_cast<double *>(p), *bim = reinterpret_cast<double *>(p + b_bytes);
     const size_t bytes = sizeof(double) * (size_t)Nb * N;
@@ -1362,8 +1393,8 @@ few_status few_basis_create(few_ctx *ctx, const double *b_re, const double *b_im
     auto *gt32 = reinterpret_cast<float2 *>(p + 2 * b_bytes + g64);
     int *bexp = reinterpret_cast<int *>(p + 2 * b_bytes + g64 + g32);
     unsigned char *bpack = p + 2 * b_bytes + g64 + g32 + ex;
-    int *bexp64 = reinterpret_cast<int *>(p + plain);
-    unsigned char *bpack64 = p + plain + ex64;
+    int *bexp64 = static_cast<int *>(slices);
+    unsigned char *bpack64 = static_cast<unsigned char *>(slices) + ex64;
     if (!st && (launch_rb_exponents(bre, bim, Nb, N, L.modes_padded, bexp, digits ? bexp64 : nullptr, s) != cudaSuccess ||
                 launch_rb_basis(bre, bim, Nb, N, gt64, gt32, bexp, bpack, ctx->sm_count, s) != cudaSuccess ||
                 (digits &&
@@ -1372,6 +1403,7 @@ few_status few_basis_create(few_ctx *ctx, const double *b_re, const double *b_im
         st = FEW_ERR_CUDA;
     }
     if (st) {
+        dev_free(ctx, slices, s);
         dev_free(ctx, d, s);
         return st;
     }
@@ -1380,6 +1412,7 @@ few_status few_basis_create(few_ctx *ctx, const double *b_re, const double *b_im
     b->Nb = Nb;
     b->N = N;
     b->dmem = d;
+    b->slices = slices;
     b->bre = bre;
     b->bim = bim;
     b->gt64 = gt64;
@@ -1399,6 +1432,7 @@ few_status few_basis_release(few_ctx *ctx, few_basis *b)
     std::lock_guard<std::recursive_mutex> lk(ctx->mu);
     DeviceScope dev_scope(ctx->device);
     cudaDeviceSynchronize();
+    dev_free(ctx, b->slices, ctx->internal);
     dev_free(ctx, b->dmem, ctx->internal);
     cudaStreamSynchronize(ctx->internal);
     (void)cudaGetLastError();
@@ -1430,13 +1464,18 @@ few_status few_rb_amplitudes(few_ctx *ctx, const few_basis *b, const double *are
         pack_bytes = fp64 ? rb64_coef_bytes(b->Nb, M) : L.apack_bytes;
     }
     void *d = nullptr;
-    few_status st = dev_alloc(ctx, sc_bytes + ex_bytes + pack_bytes, s, &d);
-    if (st && digits) {  // no room for the digits: the plain chain
+    few_status st = FEW_OK;
+    if (digits && try_alloc(ctx, sc_bytes + ex_bytes + pack_bytes, s, &d)) {  // no room: the plain chain
         digits = false;
-        ex_bytes = 0;
-        st = dev_alloc(ctx, sc_bytes, s, &d);
+        ex_bytes = pack_bytes = 0;
     }
+    if (!d) st = dev_alloc(ctx, sc_bytes + ex_bytes + pack_bytes, s, &d);
     if (st) return st;
+    if (digits && !b->captured) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(s, &capture) != cudaSuccess) (void)cudaGetLastError();
+        b->captured = capture != cudaStreamCaptureStatusNone;
+    }
     unsigned char *p = static_cast<unsigned char *>(d);
     auto &lane = ctx->lanes[ctx->lane_next++ % 4];
     cudaError_t e = launch_rb(are, aim, M, b->Nb, b->N, nu, fp64, b->bre, b->bim, b->gt64, b->gt32,

@@ -278,3 +278,77 @@ def test_rb_fp64_localised_basis(gpu_ctx, kind):
         assert best <= 1700.0
     finally:
         F.few_basis_release(gpu_ctx.handle, h)
+
+
+def _slices_case(rng, M=40, Nb=99, N=3843):
+    alpha = rng.standard_normal((M, Nb)) + 1j * rng.standard_normal((M, Nb))
+    basis = rng.standard_normal((Nb, N)) + 1j * rng.standard_normal((Nb, N))
+    return alpha, basis, rng.uniform(0.5, 2.0, M)
+
+
+def _room_for_basis_alone(basis, modes, knots):
+    """Bytes that a context holds for a basis (with its digit slices) and for a trajectory."""
+    with RT.Context(0) as free:
+        h = F.few_basis_create(free.handle, basis.real, basis.imag, RT.current_stream())
+        held = free.memory()[0]
+        tr = RT.Trajectory(free, knots, modes)
+        traj = free.memory()[0] - held
+        tr.release()
+        F.few_basis_release(free.handle, h)
+    return held, traj
+
+
+@pytest.mark.parametrize("prec", [F.FEW_FP64, F.FEW_MIXED])
+def test_rb_slices_give_way_to_other_allocations(prec):
+    """A budget that holds a basis with its FP64 digit slices, or the basis and a trajectory: the trajectory
+    is not refused, and the basis' amplitudes stay what they were (FP64 by the plain chain)."""
+    import torch
+    alpha, basis, nu = _slices_case(np.random.default_rng(8))
+    modes, knots = W.mode_grid(10, 10), W.knot_times(1e6, 200)
+    held, traj = _room_for_basis_alone(basis, modes, knots)
+    with RT.Context(0, held + traj // 4) as ctx:
+        h = F.few_basis_create(ctx.handle, basis.real, basis.imag, RT.current_stream())
+        assert ctx.memory()[0] == held
+        tr = RT.Trajectory(ctx, knots, modes)
+        assert ctx.memory()[0] < held + traj
+        re, im = (torch.empty(len(nu), basis.shape[1], dtype=torch.float64, device="cuda") for _ in range(2))
+        F.few_rb_amplitudes(ctx.handle, h, _dev(alpha.real), _dev(alpha.imag), re, im, _dev(nu), prec,
+                            RT.current_stream())
+        torch.cuda.synchronize()
+        assert ctx.sync_status() == F.FEW_OK
+        _check_rows(to_host(re) + 1j * to_host(im), oracle.rb_amplitudes(alpha, basis, nu), alpha, basis, nu, prec)
+        tr.release()
+        F.few_basis_release(ctx.handle, h)
+
+
+def test_rb_slices_of_a_captured_call_stay():
+    """A captured graph reads the slices: they are kept, the trajectory is refused, and the replay is right."""
+    import torch
+    alpha, basis, nu = _slices_case(np.random.default_rng(9))
+    modes, knots = W.mode_grid(10, 10), W.knot_times(1e6, 200)
+    held, traj = _room_for_basis_alone(basis, modes, knots)
+    with RT.Context(0, held + traj // 4) as ctx:
+        h = F.few_basis_create(ctx.handle, basis.real, basis.imag, RT.current_stream())
+        dev = [_dev(alpha.real), _dev(alpha.imag), _dev(nu)]
+        re, im = (torch.zeros(len(nu), basis.shape[1], dtype=torch.float64, device="cuda") for _ in range(2))
+
+        def call():
+            F.few_rb_amplitudes(ctx.handle, h, dev[0], dev[1], re, im, dev[2], F.FEW_FP64, RT.current_stream())
+
+        call()
+        torch.cuda.synchronize()
+        ref = to_host(re) + 1j * to_host(im)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            call()
+        with pytest.raises(F.FewError) as e:
+            RT.Trajectory(ctx, knots, modes)
+        assert e.value.status == F.FEW_ERR_BUDGET
+        re.zero_()
+        im.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert ctx.sync_status() == F.FEW_OK
+        np.testing.assert_array_equal(to_host(re) + 1j * to_host(im), ref)
+        del g
+        F.few_basis_release(ctx.handle, h)
