@@ -111,12 +111,16 @@ class Server:
         fut: cf.Future = cf.Future()
         try:
             need = req.out_bytes() + self.engine.scratch_bytes(req)
+            least = need
+            if need > self.budget and hasattr(self.engine, "least_scratch_bytes"):
+                least = req.out_bytes() + self.engine.least_scratch_bytes(req)
         except Exception as e:  # noqa: BLE001 -- e.g. an unknown trajectory without knot data
             fut.set_exception(AdmissionError(f"request cannot be sized: {e}"))
             return fut
-        if need > self.budget:
-            fut.set_exception(AdmissionError(f"request needs {need} bytes > budget {self.budget}"))
+        if least > self.budget:
+            fut.set_exception(AdmissionError(f"request needs {least} bytes > budget {self.budget}"))
             return fut
+        need = min(need, self.budget)  # a request whose smaller plan alone fits runs by itself
         job = _Job(req, fut, time.perf_counter(), need)
         with self._cv:
             if self._stop:
@@ -340,21 +344,26 @@ class GpuEngine:
         self.tiles[req.prec] = tuple(choice)
         return tuple(choice)
 
-    def scratch_bytes(self, req: Request) -> int:
-        """Plan scratch of `req` (called by Server.submit for every request, which also lets
-        the engine note the knot data a request brings)."""
+    def _plan(self, req: Request) -> tuple:
+        """few_plan_chain of `req`: (tensor cores?, plan bytes by the scalar chain, on the tensor cores)."""
         tr = self.trajs.get(req.traj_key)
         if req.traj_inputs is not None and tr is None:
             self._announced.setdefault(req.traj_key, req.traj_inputs)
-        if tr is not None:
-            K, N, slots = tr.info
-        else:  # not created yet: sized from its knot data
-            w = self._announced.get(req.traj_key)
-            if w is None:
-                raise KeyError(f"unknown trajectory {req.traj_key!r} and no knot data")
-            K, slots = len(w.t_knots), F.few_mode_slots(w.modes)[0]
-        elem = 8 if req.prec == F.FEW_FP64 else 4
-        return (K - 1) * slots * 8 * elem + 64 * 1024
+        src = tr if tr is not None else self._announced.get(req.traj_key)
+        if src is None:
+            raise KeyError(f"unknown trajectory {req.traj_key!r} and no knot data")
+        return F.few_plan_chain(src.t_knots, src.modes, req.t0, req.dt, req.n_samples, req.prec)
+
+    def scratch_bytes(self, req: Request) -> int:
+        """Plan scratch of `req` by the chain it takes (called by Server.submit for every request, which
+        also lets the engine note the knot data a request brings)."""
+        on_tc, scalar, tc = self._plan(req)
+        return (tc if on_tc else scalar) + 64 * 1024
+
+    def least_scratch_bytes(self, req: Request) -> int:
+        """The same by the scalar chain where that is less: what a context with a budget falls back to."""
+        on_tc, scalar, tc = self._plan(req)
+        return (min(tc, scalar) if on_tc else scalar) + 64 * 1024
 
     def alloc_out(self, req: Request):
         torch = self.torch
