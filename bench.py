@@ -414,7 +414,8 @@ def bench_step_c2(args, ctx, w, dev, stream, sh, flush, prec, rank, world, tune_
     step()
     torch.cuda.synchronize()
     tile, tuned_now = tune.ensure(ctx.handle, lambda: F.few_waveform(ctx.handle, req, sh), prec,
-                                  slots, w.n_samples, tune_cache)
+                                  slots, w.n_samples, tune_cache,
+                                  requests=[(w.t_knots, w.modes, w.t0, w.dt, w.n_samples, prec)])
     for _ in range(args.warmup):
         step()
     torch.cuda.synchronize()
@@ -625,7 +626,8 @@ def bench_batched_c3(ctx, dev, stream, sh, flush, n_waves, reps, tune_cache, ora
         ctx.handle, lambda b: F.few_batch_run(ctx.handle, b, sh), F.FEW_MIXED, sub_slots,
         sub_samples, tune_cache,
         prepare=lambda: F.few_batch_plan(ctx.handle, sub, F.FEW_BATCH_NO_GRAPH),
-        cleanup=lambda b: (torch.cuda.synchronize(), F.few_batch_release(ctx.handle, b)))
+        cleanup=lambda b: (torch.cuda.synchronize(), F.few_batch_release(ctx.handle, b)),
+        requests=[(x.t_knots, x.modes, x.t0, x.dt, x.n_samples, F.FEW_MIXED) for x in ws[:16]])
     t_plan = time.perf_counter()
     bh = F.few_batch_plan(ctx.handle, reqs, F.FEW_BATCH_REBUILD_SPLINES)
     plan_s = time.perf_counter() - t_plan
@@ -735,7 +737,8 @@ def bench_stress_c5(ctx, dev, stream, sh, reps, tune_cache, in_flight=1):
     req = RT.request(tr, out, w.n_samples, w.t0, w.dt, w.theta, w.phi, F.FEW_MIXED)
     slots = tr.info[2]
     tile, tuned_now = tune.ensure(ctx.handle, lambda: F.few_waveform(ctx.handle, req, sh),
-                                  F.FEW_MIXED, slots, w.n_samples, tune_cache)
+                                  F.FEW_MIXED, slots, w.n_samples, tune_cache,
+                                  requests=[(w.t_knots, w.modes, w.t0, w.dt, w.n_samples, F.FEW_MIXED)])
 
     def step():
         F.few_traj_set_data(ctx.handle, tr.handle, *dev_in, stream=sh)
@@ -1232,7 +1235,7 @@ def main():
                     help="samples of the direct-summation measurement (0: skip)")
     ap.add_argument("--batch", type=int, default=256,
                     help="waveforms of the batched measurement (0: skip)")
-    ap.add_argument("--tune-cache", default=os.path.join(ROOT, "build", "fewsum_tiles.json"),
+    ap.add_argument("--tune-cache", default=os.path.join(ROOT, "build", "fewsum_scalar_tiles.json"),
                     help="tile cache of the autotuner ('' to tune without caching)")
     args = ap.parse_args()
     args.warmup = max(3, args.warmup)

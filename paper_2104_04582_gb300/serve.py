@@ -329,7 +329,8 @@ class GpuEngine:
 
     def tune_tiles(self, req: Request, cache_path: Optional[str] = tune.DEFAULT_CACHE) -> tuple:
         """Install the tile of `req`'s workload bucket (tuning on a cache miss, timed on `req`
-        itself) for its precision; every later group of that precision runs with it."""
+        itself) for its precision; every later group of that precision runs with it.  A request that is
+        summed on the tensor cores has no tile and leaves the context's as it is."""
         torch = self.torch
         tr = self._ensure_traj(req, self.streams[0])
         torch.cuda.synchronize()
@@ -339,7 +340,8 @@ class GpuEngine:
                             req.phi, req.scale, req.prec, req.c64(), F.FEW_MEM_DEVICE,
                             req.dphi_phi0, req.dphi_r0)
         run = lambda: F.few_waveform(self.ctx.handle, rq, int(torch.cuda.current_stream().cuda_stream))
-        choice, _ = tune.ensure(self.ctx.handle, run, req.prec, slots, req.n_samples, cache_path)
+        choice, _ = tune.ensure(self.ctx.handle, run, req.prec, slots, req.n_samples, cache_path,
+                                requests=[(tr.t_knots, tr.modes, req.t0, req.dt, req.n_samples, req.prec)])
         torch.cuda.synchronize()
         self.tiles[req.prec] = tuple(choice)
         return tuple(choice)

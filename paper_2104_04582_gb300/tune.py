@@ -1,7 +1,9 @@
-"""Autotuner for the summation kernel's tile shape.
+"""Autotuner for the tile shape of the scalar summation chain.
 
-The summation kernel is tunable in three ways that change speed but never results (every sample
-is summed by one thread in a fixed order, so all choices are bit-identical):
+The scalar chain's kernel is tunable in three ways that change speed but never results (every sample
+is summed by one thread in a fixed order, so all choices are bit-identical).  The tensor-core summation
+has no tile: a workload that is summed there (few_plan_chain) says nothing about the candidates, so
+`ensure` leaves the context's tiles alone for it.
 
 * samples per thread R (the segment tile: one pass covers threads x R consecutive samples),
 * threads per block (128 or 256),
@@ -12,7 +14,7 @@ is summed by one thread in a fixed order, so all choices are bit-identical):
 best of), picks the fastest, installs it in the context, and records it in a JSON cache keyed by
 (precision, slot-count bucket, samples bucket); `apply_cached()` installs a cached choice and
 `ensure()` does either, so that a caller (the batched path, the serving engine, the benchmark)
-runs every workload with a tuned tile.
+runs every workload that has a tile with a tuned one.
 """
 from __future__ import annotations
 
@@ -28,7 +30,8 @@ CANDIDATES = {
     F.FEW_MIXED: [(r, t, s) for r in (2, 4, 8) for t in (128, 256) for s in (256, 512, 1024)],
 }
 
-DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "fewsum_tiles.json")
+# (a name of its own: files of earlier versions also hold winners among candidates that made no difference)
+DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "fewsum_scalar_tiles.json")
 
 
 def bucket(prec: int, n_slots: int, n_samples: int) -> str:
@@ -125,13 +128,23 @@ def apply_cached(ctx_handle: int, prec: int, n_slots: int, n_samples: int,
     return choice
 
 
+def has_tile(requests) -> bool:
+    """Whether any of the requests, (t_knots, modes, t0, dt, n_samples, prec) each, is summed by the scalar
+    chain."""
+    return any(not F.few_plan_chain(*r)[0] for r in requests)
+
+
 def ensure(ctx_handle: int, run, prec: int, n_slots: int, n_samples: int,
            cache_path: Optional[str] = DEFAULT_CACHE, repeats: int = 2,
            prepare: Optional[Callable[[], Any]] = None,
-           cleanup: Optional[Callable[[Any], None]] = None) -> Tuple[Tuple[int, int, int], bool]:
-    """Install the cached tile for this workload bucket, tuning with `run` on a miss.
+           cleanup: Optional[Callable[[Any], None]] = None,
+           requests: Optional[Sequence] = None) -> Tuple[Tuple[int, int, int], bool]:
+    """Install the cached tile for this workload bucket, tuning with `run` on a miss.  requests (see
+    has_tile): what `run` computes; if none of it has a tile, the installed one stays.
 
     Returns (choice, tuned_now)."""
+    if requests is not None and not has_tile(requests):
+        return tuple(F.few_get_tiles(ctx_handle, prec)), False
     if cache_path:
         c = apply_cached(ctx_handle, prec, n_slots, n_samples, cache_path)
         if c is not None:
