@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(kRbMmaThreads, 1) k_rb_mma(RbMmaArgs a)
             // the lanes whose modes fill whole 32-byte sectors of the row, and the row's two ends
             const bool overlap = a.step < 32, first = group == 0, last = group >= a.groups - 1;
             const bool live = group < a.groups && mode < a.N;
-            const int at0 = (int)(reinterpret_cast<uintptr_t>(dst) >> 3) + m0;
+            const unsigned at0 = (unsigned)(reinterpret_cast<uintptr_t>(dst) >> 3) + (unsigned)m0;  // modulo 2^32
             const float fb = pow2f(-a.bexp[mode]);  // undo the column scaling (exact)
             for (int c = c_first; c < (nn + 31) / 32; c += kRbEpiPerQuarter) {
                 float v[32];
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(kRbMmaThreads, 1) k_rb_mma(RbMmaArgs a)
                 bool on[4];  // of knots kc + j, by j mod 4
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int off = overlap ? -(at0 + (kc + j) * a.N) & 3 : 0;
+                    const int off = overlap ? (int)(0u - (at0 + (unsigned)(kc + j) * (unsigned)a.N) & 3u) : 0;
                     on[j] = live && (first || lane >= off) && (last || lane < off + a.step);
                 }
                 double *row = dst + (size_t)kc * a.N + mode;

@@ -352,3 +352,36 @@ def test_rb_slices_of_a_captured_call_stay():
         np.testing.assert_array_equal(to_host(re) + 1j * to_host(im), ref)
         del g
         F.few_basis_release(ctx.handle, h)
+
+
+@pytest.mark.parametrize("prec", [F.FEW_MIXED, F.FEW_FP64])
+def test_rb_more_outputs_than_2_to_the_31(gpu_ctx, prec):
+    """559,200 knots of 3841 modes (2 x 17 GB): the rows' places in memory past 2^31 elements, around that
+    boundary and at both ends."""
+    import torch
+    M, N, Nb = 559200, 3841, 2
+    assert M * N > 2 ** 31
+    if torch.cuda.mem_get_info()[0] < 48 << 30:
+        pytest.skip("needs 48 GB")
+    rng = np.random.default_rng(2)
+    basis = rng.standard_normal((Nb, N)) + 1j * rng.standard_normal((Nb, N))
+    are, aim = (_dev(rng.standard_normal((M, Nb))) for _ in range(2))
+    bre, bim = _dev(basis.real), _dev(basis.imag)
+    re, im = (torch.full((M, N), 7.0, dtype=torch.float64, device="cuda") for _ in range(2))
+    h = F.few_basis_create(gpu_ctx.handle, basis.real, basis.imag, RT.current_stream())
+    try:
+        F.few_rb_amplitudes(gpu_ctx.handle, h, are, aim, re, im, None, prec, RT.current_stream())
+        torch.cuda.synchronize()
+        assert gpu_ctx.sync_status() == F.FEW_OK
+        edge = 2 ** 31 // N
+        for k0 in (0, edge - 1000, M - 3000):
+            s = slice(k0, k0 + 3000)
+            bound = (FP64_GAMMA if prec == F.FEW_FP64 else MIXED_GAMMA) * torch.linalg.vector_norm(
+                (are[s].abs() + aim[s].abs()) @ (bre.abs() + bim.abs()), dim=1)
+            for g, o in ((re, are[s] @ bre - aim[s] @ bim), (im, are[s] @ bim + aim[s] @ bre)):
+                assert torch.all(torch.linalg.vector_norm(g[s] - o, dim=1) <= bound)
+        assert not torch.any(re[::997] == 7.0) and not torch.any(im[::997] == 7.0)
+    finally:
+        F.few_basis_release(gpu_ctx.handle, h)
+        del re, im
+        torch.cuda.empty_cache()
