@@ -196,6 +196,14 @@ __global__ void k_pair_consts(const int *__restrict__ l, const int *__restrict__
     pairs[i] = PairConst64{yp.x + ym.x, yp.y - ym.y, yp.y + ym.y, yp.x - ym.x};
 }
 
+// The n from which the table's exponentials are computed up (0: and mirrored), and how many there are.
+__host__ __device__ inline int tab_first(int n_lo, int n_hi) { return n_lo < 0 && n_hi > 0 ? 0 : n_lo; }
+__host__ __device__ inline int tab_count(int m_top, int n_lo, int n_hi)
+{
+    const int a0 = tab_first(n_lo, n_hi), a1 = a0 == 0 && -n_lo > n_hi ? -n_lo : n_hi;
+    return m_top + 2 + a1 - a0;
+}
+
 // tables: the modes' ModeConstTab, or (kPairs) n_pairs PairConst64, then int2 per mode.
 template <bool kPairs>
 __global__ void __launch_bounds__(kTabThreads)
@@ -212,11 +220,12 @@ k_direct_tab(const double *__restrict__ pphi, const double *__restrict__ pr,
     double2 *tab = dir_tab + (threadIdx.x >> 5) * (entries + (kPairs ? 2 * n_pairs : 0));
     const double xp = reduce_2pi(pphi[i]) * kInv2Pi, xr = reduce_2pi(pr[i]) * kInv2Pi;
     const double fphi = xp - rint(xp), fr = xr - rint(xr);
-    // (of n and -n one is computed: the table of a range about zero takes half the sincospi)
-    const int n_hi = n_lo + entries - m_top - 2, a0 = n_lo < 0 && n_hi > 0 ? 0 : n_lo;
-    const int a1 = a0 < 0 ? n_hi : max(n_hi, -n_lo);
-    for (int e = lane; e < m_top + 2 + a1 - a0; e += 32) {
-        const int a = a0 + e - m_top - 1;
+    // (of n and -n one is computed: the table of a range about zero takes half the sincospi; lanes past the end
+    // repeat the last entry: lanes a pass apart went through the unrolled loop one group after the other, 64
+    // modes of 33 exponentials, 60,000 samples: 580 us, 458 so)
+    const int n_hi = n_lo + entries - m_top - 2, a0 = tab_first(n_lo, n_hi), count = tab_count(m_top, n_lo, n_hi);
+    for (int e0 = 0; e0 < count; e0 += 32) {
+        const int e = min(e0 + lane, count - 1), a = a0 + e - m_top - 1;
         const double x = e <= m_top ? e * fphi : (double)a * fr;
         double s, c;
         sincospi(2.0 * (x - rint(x)), &s, &c);
@@ -534,9 +543,11 @@ cudaError_t launch_direct(const double *pphi, const double *pr, const double *ar
                           (size_t)(kRingBytes + table), st, pphi, pr, are, aim, ns, N,
                           static_cast<const uint4 *>(mode_consts), table, scale, out, out_c64, err);
     }
-    // the tables pay wherever they hold fewer exponentials than there are modes
-    const int entries = m_top + 1 + n_hi - n_lo + 1;
-    if (fp64 && entries <= kTabMaxEntries && entries < N && ns > 0) {
+    // The tables pay where a warp fills them in fewer passes than the modes take (60,000 samples, 33 to 64 modes:
+    // one pass 447 -> 340 us, two 447 -> 458), and in as many for few samples, by blocks of four instead of eight
+    // (4,000: 12 modes 39 -> 38, 250 modes and 225 exponentials 127 -> 119; 16,000: 96 -> 99, 402 -> 403 and more).
+    const int entries = m_top + 1 + n_hi - n_lo + 1, passes = (tab_count(m_top, n_lo, n_hi) + 31) / 32;
+    if (fp64 && entries <= kTabMaxEntries && entries < N && (passes < (N + 31) / 32 || ns <= 32ll * sm_count) && ns > 0) {
         const int per = kTabThreads / 32;
         const unsigned blocks = (unsigned)((ns + per - 1) / per);
         // factors of (l, m): eight operations a pair and sample save four a mode, where there are more

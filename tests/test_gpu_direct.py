@@ -182,3 +182,43 @@ def test_direct_fp64_pair_table_edges(gpu_ctx, ls, ms, ns_range, extra):
     g = _gpu_direct(gpu_ctx, pphi, pr, are, aim, modes, 0.9, 2.1, F.FEW_FP64)
     o = oracle.direct_dense(pphi, pr, modes, are, aim, 0.9, 2.1)
     assert rel_l2(g, o) <= FP64_REL_L2
+
+
+@pytest.mark.parametrize("off", [0, 1])
+@pytest.mark.parametrize("ls,ns_range,N", [
+    ((3, 4, 5), range(-3, 3), 12), ((3, 4, 5), range(-3, 3), 32),  # one pass of either
+    ((3, 4, 5), range(-3, 3), 33),   # one pass for the tables, two for the modes
+    ((2, 3), range(4, 36), 128),     # two (35 exponentials: most lanes have one) and four
+    ((2, 3), range(4, 36), 36),      # two of either
+])
+def test_direct_fp64_table_passes(gpu_ctx, ls, ns_range, N, off):
+    """Both sides of the choice by passes and samples, and a last pass of the tables that few lanes have."""
+    import torch
+    ns = 32 * torch.cuda.get_device_properties(0).multi_processor_count + off
+    rng = np.random.default_rng(9)
+    modes = np.asarray([(l, m, n) for l in ls for m in (1, 2) for n in ns_range][:N], dtype=np.int32)
+    assert len(modes) == N
+    pphi, pr = rng.uniform(-1e5, 1e5, (2, ns))
+    are, aim = rng.standard_normal((2, ns, N))
+    g = _gpu_direct(gpu_ctx, pphi, pr, are, aim, modes, 0.9, 2.1, F.FEW_FP64)
+    o = oracle.direct_dense(pphi, pr, modes, are, aim, 0.9, 2.1, 1.0, oracle_threads())
+    assert rel_l2(g, o) <= FP64_REL_L2
+
+
+def test_direct_fp64_long_tables_time(gpu_ctx):
+    """64 modes of 33 exponentials (n of one sign), 60,000 samples: 447 us an exponential a mode, 580 by the tables."""
+    import torch
+    ns, modes = 60000, np.asarray([(l, 0, n) for l in (2, 3) for n in range(32)], dtype=np.int32)
+    x = torch.rand(2, ns, dtype=torch.float64, device="cuda") * 1e5
+    a = torch.randn(2, ns, 64, dtype=torch.float64, device="cuda")
+    out = torch.empty(ns, dtype=torch.complex128, device="cuda")
+    best = 1e9
+    for _ in range(20):
+        t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        t0.record()
+        F.few_direct_sum(gpu_ctx.handle, x[0], x[1], a[0], a[1], modes, 0.9, 2.1, out, 1.0, F.FEW_FP64,
+                         RT.current_stream())
+        t1.record()
+        t1.synchronize()
+        best = min(best, t0.elapsed_time(t1))
+    assert best < 0.52
