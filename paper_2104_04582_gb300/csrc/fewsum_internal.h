@@ -298,6 +298,10 @@ constexpr int kTcAlwaysSlots = 128;
 //                           99 slots: 4096 knots, 20,000 samples 534, 784
 // The estimates are fits to such times, good to 20 %; where they are near one another the tensor cores, the more
 // exact of the two, are taken (FP64).
+// A batch's waveforms share the launches, and what they add to it decides: 48 FP64 waveforms of 50 knots and 300
+// samples, two modes of m = 10: 402, 176; one pair, 300 knots, 3,000 samples: 1179, 685.  A request takes the same
+// chain alone and in a batch (its results do not depend on the others), so the tensor cores must also add at most a
+// tenth more there (fits to 10 %).
 inline bool tc_pays(bool fp64, const TcShape &s, const TcWork &w)
 {
     if (s.slots > kTcAlwaysSlots) return true;
@@ -312,7 +316,13 @@ inline bool tc_pays(bool fp64, const TcShape &s, const TcWork &w)
     const double tc = (8 * s.K + 2048 <= kPlanParamBytes ? 28.0 : 47.0) +
                       w.segs * (0.045 + s.pairs * (0.006 + 0.0045 * (s.ks - 1)) + 0.0001 * s.modes) +
                       w.tiles * (0.6 + 0.85 * s.pairs + 0.7 * (s.ks - 1)) / 152.0;
-    return 0.9 * tc < scalar;
+    if (0.9 * tc >= scalar || w.passes == 0.0) return false;
+    const double fill = w.samples / w.passes;  // samples a pass
+    const double adds_scalar = 0.033 * w.segs + w.passes / 152.0 * (1.0 + 0.188 * s.slots + 0.11 * s.rows +
+                                                                    fill * (0.0356 + 0.00277 * s.slots + 0.00172 * s.rows));
+    const double adds_tc = w.segs * (0.0433 + s.pairs * (0.0047 + 0.0052 * (s.ks - 1))) +
+                           w.tiles * (0.0127 + 0.004 * s.pairs + (0.0046 + 0.0002 * s.pairs) * (s.ks - 1));
+    return adds_tc < 1.1 * adds_scalar;
 }
 cudaError_t tc_configure();
 cudaError_t tc64_configure();

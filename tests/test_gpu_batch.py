@@ -139,3 +139,32 @@ def test_batch_of_256_uneven_waveforms(gpu_ctx):
     F.few_batch_release(gpu_ctx.handle, b)
     for tr in trs:
         tr.release()
+
+
+def test_fp64_batch_of_few_modes(gpu_ctx):
+    """48 FP64 waveforms of two modes (m = 10) on 49 short segments: each as alone and as the oracle's, and the
+    graph's time (about 180 us by the scalar chain, 400 us on the tensor cores)."""
+    import torch
+    modes = np.array([[10, 10, 0], [10, 10, 1]], dtype=np.int32)
+    ws = [W.make_inputs(3000.0, 50, 10.0, modes, 31 + q, n_samples=300) for q in range(48)]
+    trs = [RT.from_inputs(gpu_ctx, w) for w in ws]
+    outs = [RT.alloc_out(300, False) for _ in ws]
+    b = F.few_batch_plan(gpu_ctx.handle, [RT.request(tr, o, 300, w.t0, w.dt, w.theta, w.phi, F.FEW_FP64, w.scale)
+                                          for tr, o, w in zip(trs, outs, ws)])
+    best = 1e9
+    for _ in range(20):
+        t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        t0.record()
+        F.few_batch_run(gpu_ctx.handle, b, RT.current_stream())
+        t1.record()
+        t1.synchronize()
+        best = min(best, t0.elapsed_time(t1))
+    assert gpu_ctx.sync_status() == F.FEW_OK
+    for w, tr, o in zip(ws, trs, outs):
+        h = to_host(o)
+        np.testing.assert_array_equal(_alone(gpu_ctx, tr, w, F.FEW_FP64), h)
+        assert rel_l2(h, oracle.waveform_inputs(w, nthreads=oracle_threads())) <= FP64_REL_L2
+    F.few_batch_release(gpu_ctx.handle, b)
+    for tr in trs:
+        tr.release()
+    assert best < 0.28

@@ -77,3 +77,19 @@ def test_refusals(modes, K, n, dt, status):
     with pytest.raises(F.FewError) as e:
         F.few_plan_chain(W.knot_times(1e3, 10), np.asarray(PAIR, dtype=np.int32), 0.0, 1.0, 10, 7)
     assert e.value.status == F.FEW_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("modes,K,n,tc", [
+    # FP64, measured us of 48 waveforms in one graph (6 for 2000 knots), tensor cores against scalar
+    ([(10, 10, 0), (10, 10, 1)], 50, 300, False),   # 402, 176
+    ([(10, 10, 0), (10, 10, 30)], 50, 2000, False), # 952, 492
+    ([(10, 10, 0), (10, 10, 30)], 300, 60000, True),  # 6945, 7976 (one: 171, 292)
+    (PAIR, 300, 3000, False),                       # 1179, 685
+    (PAIR, 300, 60000, True),                       # 1685, 1897
+    (PAIR, 10, 2000, True),                         # 81, 103
+    (PAIR, 10, 200, False),                         # 68, 49
+    ([(2, 2, -30), (2, 2, 30), (2, 1, 3)], 50, 300, True),  # 382, 567
+    ([(2, 2, -30), (2, 2, 30), (2, 1, 3)], 2000, 2000, True),  # 1415, 2107
+])
+def test_line_between_the_chains_in_batches(modes, K, n, tc):
+    assert _chain(modes, K, n, FP64)[0] == tc
