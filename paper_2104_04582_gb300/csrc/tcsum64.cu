@@ -8,8 +8,8 @@
 //
 // Both operands are fixed-point numbers of 7 signed 8-bit digits (units of 2^-54; the table scaled
 // by the power of two that brings its largest entry into [1/2, 1)), held as fp16 integers.  The
-// products of digits i and j with i + j = o <= 6 are summed in accumulator o: at most 61 x 98304
-// < 2^23, so the FP32 accumulators are exact integers.  What is left out (o >= 7) and the operands'
+// products of digits i and j with i + j = o <= 6 are summed in accumulator o: at most 63 x 98304
+// < 2^23 (order_bound), so the FP32 accumulators are exact integers.  What is left out (o >= 7) and the operands'
 // rounding are below 2^-50 of the table's largest entry, as is FP64's own rounding of such a sum.
 // The accumulators are put together as 64-bit integers, and the cubic in u and Horner's rules in
 // z_phi and its conjugate run in 64-bit fixed point too (a product costs ~6 instructions; an FP64
@@ -278,6 +278,16 @@ __device__ __forceinline__ void store_digits(uint32_t e_addr, const Cq (&z)[8])
 #pragma unroll
     for (int q = 0; q < kTc64Slices; ++q) tc_st8(e_addr + kT64EStride * q, w[q]);
 }
+
+// Largest magnitude of accumulator o: the basis has 2 kTcMaxHalf + 1 values (sin 0 is left out), digits are at most
+// 128, and the top ones at most 64, because neither operand exceeds 1 = 64 x 2^48 units of 2^-54 (the table by
+// its scale, the basis as a cosine or sine).  join_orders relies on both bounds; the first holds by 1.6 %.
+constexpr int order_bound(int o)
+{
+    return (2 * kTcMaxHalf + 1) * (o == 0 ? 64 * 64 : 2 * 64 * 128 + (o - 1) * 128 * 128);
+}
+static_assert(kTc64Slices == 7 && order_bound(4) < 1 << 22, "orders 0 .. 4 stay in 1.5 2^23's low mantissa bits");
+static_assert(order_bound(kTc64Slices - 1) < 1 << 23, "the FP32 accumulators are exact integers");
 
 // The sums of one column pair (even, odd row), orders 0 .. 6, as 64-bit integers 4 sum_o S_o
 // 2^(40 - 8 o) (two guard bits): orders 0 .. 4 exact (|S_o| < 2^22: the 1.5 2^23 addition leaves the
