@@ -117,8 +117,8 @@ struct few_ctx {
     size_t in_use = 0;
     cudaMemPool_t pool = nullptr;
     cudaStream_t internal = nullptr;
-    // second streams for work beside a call's main chain (the phase anchors beside the
-    // harmonics and the fold; the reduced-basis scale beside its pack), each with its fork and
+    // second streams for work beside a call's main chain (the scalar chain's phase anchors beside its
+    // harmonics and fold; the reduced-basis scale of more than 128 vectors beside its pack), each with its fork and
     // join events; taken in turn, so calls on different user streams seldom share one
     struct SideLane {
         cudaStream_t s = nullptr;

@@ -18,10 +18,10 @@
 // 3 x 2 Nb sums them all.  fp16's narrow exponent range is handled by exact power-of-two
 // scaling: each knot's coefficient row and each mode's basis column are scaled so that their
 // largest magnitude lies in [2^14, 2^15) before the split, and the epilogue multiplies the
-// accumulator back by both inverse powers and by the knot's renormalisation s (so the scale's
-// kernels run beside the coefficient pack, on a second stream, and are joined before the
-// product).  An entry far below its row or column maximum keeps
-// an absolute error near 2^-24 of that maximum.
+// accumulator back by both inverse powers and by the knot's renormalisation s (so the scale's kernels run
+// beside the coefficient pack: as dependent launches up to 128 vectors, on a second stream above, and end
+// before the product).  An entry far below its row or column maximum keeps an absolute error near 2^-24 of
+// that maximum.
 //
 // The product is computed transposed, A^T = Bhat^T a^T: the MMA's M side (tensor-memory lanes)
 // is 128 real output columns of two groups of 32 modes (rows 0-63 the real parts, 64-127 the
@@ -228,14 +228,16 @@ k_rb_quad(const double *__restrict__ are, const double *__restrict__ aim, int M,
     }
 }
 
-// Mixed path, Nb <= 128: the renormalisation scale in one kernel, one wave.  A block takes
-// kTRows knots; their FP32 coefficients and the whole FP32 Gram matrix (j padded to 128) sit in
-// shared memory.  The sum over l is split among kTParts thread groups (l = part mod kTParts);
+// Mixed path, Nb <= 128: the renormalisation scale in one kernel.  A block takes kTRows knots; their FP32
+// coefficients and the whole FP32 Gram matrix (j padded to a multiple of 16) sit in shared memory.  The sum over l is
+// split among kTParts thread groups (l = part mod kTParts);
 // within a group thread (rg, jg) owns knots 4 rg .. 4 rg + 3 and j = jg + 16 t, t < T = ceil(Nb / 16),
 // so 12 shared-memory reads (half of them broadcasts) feed 128 multiply-adds per l (T = 8).  The 16 threads of
 // a knot group share a half-warp and reduce their partial q_k by shuffles; the groups' partials
 // are added in group order and s_k = nu_k / sqrt(q_k) written directly (0 for q_k = 0; a
-// non-finite or negative nu_k latches ERRBIT_NONFINITE).
+// non-finite or negative nu_k latches ERRBIT_NONFINITE).  A block needs most of a multiprocessor's shared memory at
+// 128 vectors, so one is resident: 44 rows are what 528 threads take by fours, and leave 6,400 knots in one wave of
+// 152 (146 blocks; 48 rows would be 134 of 9 % more work).  Any number of knots runs in such waves.
 constexpr int kTRows = 44, kTGroup = (kTRows / 4) * 16, kTParts = 3;
 constexpr int kTThreads = kTGroup * kTParts;
 constexpr int kTMaxBasis = 128;
@@ -256,7 +258,7 @@ k_rb_scale_tile(const double *__restrict__ are, const double *__restrict__ aim, 
     const int jg = local & 15, rg = local >> 4;
     const int k0 = blockIdx.x * kTRows;
     // staging: the Gram matrix by asynchronous copies, all in flight, while the coefficients (9 loads of
-    // each array in flight a thread) pass through registers
+    // each array in flight a thread: 44 rows of up to 108 vectors in one round) pass through registers
     for (int l = tid / 16; l < Nb; l += kTThreads / 16) {
 #pragma unroll
         for (int t = 0; t < T; ++t) {

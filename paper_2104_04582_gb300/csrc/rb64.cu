@@ -12,14 +12,15 @@
 // rounding, 2^-53 of sum |alpha B| and more, unless that sum is far below the product of the largest
 // entries.  That is checked for every output: a ninth product, of the top digits' magnitudes, bounds the
 // sum of magnitudes, and an output where it is below 2^-5, or whose row or column has entries that
-// are not finite or not within 2^+-400, is computed by the plain FP64 chain (k_rb_fp64) in its place.
+// are not finite or not within 2^+-400, is computed by an FP64 chain in the product's own epilogue.
 //
 // A CTA forms one tile of 64 modes (128 real columns: tensor-memory lanes) x up to 64 knots (an even share
 // of them): eight accumulators of 64 columns fill tensor memory.  The operands' digits of 16 columns (48 KB) are one stage of a ring
 // filled by bulk copies.  Shared memory bounds the products (an MMA reads 6 KB: 48 cycles), then the
 // conversions of the sums.  100 knots x 99 vectors x 3843 modes, whole call: 305 us with the
 // FP64 chain, 51 us here, and 6.4e-16 -> 1.0e-16 from quadruple precision; 374 x 170 x 3843 1808 -> 257 us,
-// 100 x 20 x 200 35 -> 29 us, so the plain chain is left only where there is no memory for the slices.
+// 100 x 20 x 200 35 -> 29 us, so k_rb_fp64 (rb.cu) is left only where there is no memory for the
+// slices.
 #include <cuda_fp16.h>
 
 #include "async.cuh"

@@ -1,6 +1,6 @@
 // tcsum.cu -- the mixed-precision mode sum on the tensor cores (arXiv:2104.04582 Sec. 3.C, Sec. 4).
 //
-// With K_{m,n}(u) = sum_d c_{m,n,d} u^d the folded cubic of a signed frequency (fold_slot.cuh),
+// With K_{m,n}(u) = sum_d c_{m,n,d} u^d the folded cubic of a signed frequency (fold_tc.cuh),
 // n = n_mid + b and theta = Phi_r, the sum over n of one row m is, degree by degree,
 //     sum_n c_{m,n,d} e^{-i n theta} = e^{-i n_mid theta} [ sum_{b >= 0} X_{m,b,d} cos(b theta)
 //                                                        + Y_{m,b,d} sin(b theta) ],
@@ -236,7 +236,8 @@ __device__ __forceinline__ void load_table(const TileRec *recs, int T, int n,
 // its basis in registers while the slot's other warpgroup waits for its MMAs, and stores it while
 // that one drains them.
 // KS: K steps of the plan's widest n range (a wave with fewer uses the first of them).
-// One year, 3843 modes: 104 us (the scalar chain 1,417), 1,154 cycles a tile = twelve N = 176 MMAs of 96,
+// One year, 3843 modes: 109-111 us a launch, 104 from the first CTA's start to the last one's end (the scalar
+// chain 1,417), 1,154 cycles a tile = twelve N = 176 MMAs of 96,
 // the tensor cores 90 % active.  Sets of fewer rows run at 430 to 700 ns a tile whatever their size:
 // there the chain of a slot bounds it (issue ~900 cycles, the MMAs' tail ~440, loads to the release
 // of the accumulator ~500, wake-up ~350).  Six warpgroups of 80 registers: 133 us; factors before
