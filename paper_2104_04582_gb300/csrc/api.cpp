@@ -760,7 +760,7 @@ void fill_image(few_ctx *c, const few_request *reqs, int n, PlanImage &P, unsign
 }
 
 // Queue a plan's kernels on `st`.  Errors are returned after everything queued has been joined.
-// plan: a tensor-core plan that travels in the fold's parameters instead of being at hdr_dev already.
+// plan: a plan that travels in the first kernel's parameters instead of being at hdr_dev already (not kVariantScalar).
 cudaError_t launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, const PlanParam *plan, const LaunchPlan &P,
                            cudaStream_t st, bool mark)
 {
@@ -810,7 +810,7 @@ cudaError_t launch_kernels(few_ctx *c, const PlanHdr *hdr_dev, const PlanParam *
         return err;
     };
     tm(1, false);
-    if ((e = joined(launch_ylm(hdr_dev, nullptr, P.total_pairs, fp64, st))) != cudaSuccess) return e;
+    if ((e = joined(launch_ylm(hdr_dev, plan, P.total_pairs, fp64, st))) != cudaSuccess) return e;
     tm(1, true);
     tm(2, false);
     if ((e = joined(launch_fold(hdr_dev, P.total_fold, fp64, st))) != cudaSuccess) return e;
@@ -1222,9 +1222,10 @@ few_status few_waveform(few_ctx *ctx, const few_request *req, void *stream)
     if (staged) out_dev = dout;
     unsigned char *blob_dev = static_cast<unsigned char *>(blob);
     fill_image(ctx, req, 1, P, blob_dev, blob_dev + P.blob.size(), &out_dev);
-    // a small tensor-core plan travels in the fold's parameters: no copy stands between the kernels
+    // a small plan travels in the first kernel's parameters: no copy stands between the kernels, and the call can be
+    // captured (mixed scalar plans are read by two streams' first kernels: they are copied)
     std::unique_ptr<PlanParam> param;
-    if (is_tc(P.launch.variant) && P.blob.size() <= (size_t)kPlanParamBytes) param.reset(new (std::nothrow) PlanParam);
+    if (P.launch.variant != kVariantScalar && P.blob.size() <= (size_t)kPlanParamBytes) param.reset(new (std::nothrow) PlanParam);
     if (param) {
         std::memcpy(param->bytes, P.blob.data(), P.blob.size());
         param->dev = blob_dev;

@@ -168,3 +168,47 @@ def test_fp64_batch_of_few_modes(gpu_ctx):
     for tr in trs:
         tr.release()
     assert best < 0.28
+
+
+@pytest.mark.parametrize("modes", [[(10, 10, 0), (10, 10, 1)], [(2, 2, 0)], [(11, 11, 0)]])
+def test_fp64_call_of_the_scalar_chain_is_captured(gpu_ctx, modes):
+    """A spline build and an FP64 waveform by the scalar chain (few modes, or past the tensor cores' limits) in a
+    graph of the caller's: replays take new knot data and equal the direct call, whatever other calls come between."""
+    import torch
+    md = np.array(modes, dtype=np.int32)
+    w = W.make_inputs(3000.0, 50, 10.0, md, 61, n_samples=300)
+    assert not F.few_plan_chain(w.t_knots, md, w.t0, w.dt, 300, F.FEW_FP64)[0]
+    tr, other = RT.from_inputs(gpu_ctx, w), RT.from_inputs(gpu_ctx, W.tiny_inputs(3, K=9, n_samples=5000))
+    out, o2 = RT.alloc_out(300, False), RT.alloc_out(5000, False)
+    req = RT.request(tr, out, 300, w.t0, w.dt, w.theta, w.phi, F.FEW_FP64, w.scale)
+    stream = torch.cuda.Stream()
+
+    def call(s):
+        tr.set_data_device(tr._dev_inputs, s)
+        F.few_waveform(gpu_ctx.handle, req, s)
+
+    call(stream.cuda_stream)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        g.capture_begin(capture_error_mode="thread_local")
+        call(stream.cuda_stream)
+        g.capture_end()
+    for factor in (1.0, 1.5):
+        tr._dev_inputs[2].mul_(factor)
+        torch.cuda.synchronize()
+        call(stream.cuda_stream)
+        torch.cuda.synchronize()
+        want = to_host(out)
+        for _ in range(3):
+            RT.waveform(gpu_ctx, other, 5000, 0.0, 10.0, 0.4, 0.2, F.FEW_FP64, out=o2)
+        out.zero_()
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            g.replay()
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(to_host(out), want)
+    assert gpu_ctx.sync_status() == F.FEW_OK
+    del g
+    tr.release()
+    other.release()
